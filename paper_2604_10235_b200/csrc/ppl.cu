@@ -9,16 +9,24 @@
 // (maximum, sum) in base 2 that is rescaled only when a vector raises the maximum; the threads'
 // pairs are merged with shuffles.  One exponential pair in three is evaluated on the FMA pipe
 // (the special-function unit alone would be as slow as the memory for 2-byte logits).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "cc_internal.cuh"
 #include "exp2_poly.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace cc {
 
 namespace {
 
 constexpr int kThreads = 512;
+constexpr int kVecWidth = 8;              // logits a thread takes at a time
+constexpr int kMeanThreads = 128;
+constexpr int kRankThreads = 512;
+constexpr int kMaxParts = 8;              // CTAs that share a row at most
+constexpr int kCtasPerSm = 3;             // resident CTAs of ppl_nll_kernel per SM (registers)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -89,22 +97,37 @@ template <> struct Vec<uint16_t> {       // bf16 bit patterns
 };
 template <typename T> constexpr int kBatch = sizeof(T) == 2 ? 8 : 4;   // 128 bytes per thread in flight
 
+// Rows [0, whole) have a CTA each; every later row is shared by the `parts` CTAs of a cluster
+// (parts divides `whole`, so clusters never mix the two), which merge their pairs in the first
+// one's shared memory.  A row may start anywhere on the element grid: the values before its first
+// and after its last 16-byte boundary (at most fourteen) are read one by one.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t stride_chunk,
-               int64_t stride_token, int vectors, const int32_t* __restrict__ targets,
+               int64_t stride_token, int whole, int parts, const int32_t* __restrict__ targets,
                float* __restrict__ nll, DeviceStatus* status) {
   __shared__ float sm_m[kThreads / 32], sm_s[kThreads / 32];
-  const int row = blockIdx.x, chunk = row / num_tokens, t = row % num_tokens;
+  __shared__ float2 sm_part[kMaxParts];
+  pdl_launch_dependents();
+  const bool split = (int)blockIdx.x >= whole;
+  const int part = split ? ((int)blockIdx.x - whole) % parts : 0;
+  const int row = split ? whole + ((int)blockIdx.x - whole) / parts : (int)blockIdx.x;
+  const int n_parts = split ? parts : 1;
+  if (split) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
+  pdl_wait();
+  const int chunk = row / num_tokens, t = row % num_tokens;
   const T* x = logits + (int64_t)chunk * stride_chunk + (int64_t)t * stride_token;
   Running r{-INFINITY, 0.f};
-  const int n_vec = vectors ? vocab / 8 : 0;   // rows off the 16-byte grid are read value by value
-  int i = threadIdx.x;
+  const int head = min(vocab, (int)((16u - (unsigned)((uintptr_t)x & 15u)) & 15u) / (int)sizeof(T));
+  const T* xv = x + head;
+  const int n_vec = (vocab - head) / kVecWidth;
+  int i = (int)((int64_t)n_vec * part / n_parts) + threadIdx.x;
+  const int i_end = (int)((int64_t)n_vec * (part + 1) / n_parts);
   constexpr int kB = kBatch<T>;
-  for (; i + (kB - 1) * kThreads < n_vec; i += kB * kThreads) {
+  for (; i + (kB - 1) * kThreads < i_end; i += kB * kThreads) {
     Vec<T> raw[kB];
 #pragma unroll
-    for (int u = 0; u < kB; ++u) raw[u].load(x + (int64_t)(i + u * kThreads) * 8);
+    for (int u = 0; u < kB; ++u) raw[u].load(xv + (int64_t)(i + u * kThreads) * kVecWidth);
 #pragma unroll
     for (int u = 0; u < kB; ++u) {
       float v[8];
@@ -112,15 +135,19 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
       r.add8(v);
     }
   }
-  for (; i < n_vec; i += kThreads) {
+  for (; i < i_end; i += kThreads) {
     Vec<T> raw;
-    raw.load(x + (int64_t)i * 8);
+    raw.load(xv + (int64_t)i * kVecWidth);
     float v[8];
     raw.get(v);
     r.add8(v);
   }
-  // the up to seven values after the last whole vector
-  for (int j = n_vec * 8 + threadIdx.x; j < vocab; j += kThreads) r.merge(Vec<T>::one(x + j) * kLog2e, 1.0f);
+  // the values before the first and after the last whole vector
+  if (part == 0) {
+    const int tail = head + n_vec * kVecWidth;
+    for (int j = threadIdx.x; j < head + vocab - tail; j += kThreads)
+      r.merge(Vec<T>::one(x + (j < head ? j : tail + j - head)) * kLog2e, 1.0f);
+  }
 
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -128,9 +155,20 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) { sm_m[warp] = r.m; sm_s[warp] = r.s; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Running all{-INFINITY, 0.f};
+  Running all{-INFINITY, 0.f};
+  if (threadIdx.x == 0)
     for (int w = 0; w < kThreads / 32; ++w) all.merge(sm_m[w], sm_s[w]);
+  if (split) {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // the first CTA has started
+    if (threadIdx.x == 0)
+      *cg::this_cluster().map_shared_rank(&sm_part[part], 0) = make_float2(all.m, all.s);
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (part != 0) return;
+    if (threadIdx.x == 0)
+      for (int k = 1; k < parts; ++k) all.merge(sm_part[k].x, sm_part[k].y);
+  }
+  if (threadIdx.x == 0) {
     const int target = targets[t];
     float out = __int_as_float(0x7fc00000);                   // NaN for an invalid token id
     if (target >= 0 && target < vocab)
@@ -141,31 +179,44 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
   }
 }
 
-// mean over the query positions, summed in order
-__global__ void ppl_mean_kernel(const float* __restrict__ nll, int num_chunks, int num_tokens,
-                                float* __restrict__ score) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+// mean over the query positions, summed in order: one warp per chunk, 32 values per load
+__global__ void __launch_bounds__(kMeanThreads)
+ppl_mean_kernel(const float* __restrict__ nll, int num_chunks, int num_tokens, float* __restrict__ score) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int c = blockIdx.x * (kMeanThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (c >= num_chunks) return;
   float acc = 0.f;
-  for (int t = 0; t < num_tokens; ++t) acc = __fadd_rn(acc, nll[(int64_t)c * num_tokens + t]);
-  score[c] = __fdiv_rn(acc, (float)num_tokens);
+  for (int t0 = 0; t0 < num_tokens; t0 += 32) {
+    const float v = t0 + lane < num_tokens ? nll[(int64_t)c * num_tokens + t0 + lane] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      const float x = __shfl_sync(0xffffffffu, v, k);
+      if (t0 + k < num_tokens) acc = __fadd_rn(acc, x);
+    }
+  }
+  if (lane == 0) score[c] = __fdiv_rn(acc, (float)num_tokens);
 }
 
-// rank of every chunk by (score, index); the k best are written in rank order
-__global__ void __launch_bounds__(1024)
+// rank of every chunk by (score, index); the k best are written in rank order.  A warp ranks one
+// chunk against all others.
+__global__ void __launch_bounds__(kRankThreads)
 select_chunks_kernel(const float* __restrict__ score, int num_chunks, int k, int32_t* __restrict__ chosen) {
   extern __shared__ float key[];
-  for (int i = threadIdx.x; i < num_chunks; i += blockDim.x) {
+  pdl_launch_dependents();
+  pdl_wait();
+  for (int i = threadIdx.x; i < num_chunks; i += kRankThreads) {
     const float s = score[i];
     key[i] = s != s ? INFINITY : s;                           // NaN ranks last
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < num_chunks; i += blockDim.x) {
-    const float mine = key[i];
-    int rank = 0;
-    for (int j = 0; j < num_chunks; ++j) rank += key[j] < mine || (key[j] == mine && j < i);
-    if (rank < k) chosen[rank] = i;
-  }
+  const int i = blockIdx.x * (kRankThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= num_chunks) return;
+  const float mine = key[i];
+  int rank = 0;
+  for (int j = lane; j < num_chunks; j += 32) rank += key[j] < mine || (key[j] == mine && j < i);
+  rank = __reduce_add_sync(0xffffffffu, rank);
+  if (lane == 0 && rank < k) chosen[rank] = i;
 }
 
 }  // namespace
@@ -174,27 +225,30 @@ cudaError_t launch_ppl_scores(const Launch& L, const void* logits, bool is_f32, 
                               int num_tokens, int vocab, int64_t stride_chunk, int64_t stride_token,
                               const int32_t* targets, float* nll, float* score) {
   const int rows = num_chunks * num_tokens;
-  const int64_t per16 = is_f32 ? 4 : 8;
-  const int vectors = (uintptr_t)logits % 16 == 0 && stride_token % per16 == 0 && stride_chunk % per16 == 0;
-  if (is_f32)
-    ppl_nll_kernel<float><<<rows, kThreads, 0, L.stream>>>((const float*)logits, num_tokens, vocab,
-                                                           stride_chunk, stride_token, vectors, targets,
-                                                           nll, L.status);
-  else
-    ppl_nll_kernel<uint16_t><<<rows, kThreads, 0, L.stream>>>((const uint16_t*)logits, num_tokens,
-                                                              vocab, stride_chunk, stride_token,
-                                                              vectors, targets, nll, L.status);
-  cudaError_t e = cudaGetLastError();
+  // A row is a few hundred KB, so whole rows quantise badly: the rows that do not fill a last wave
+  // of CTAs (all of them, when there are few) are split over clusters as wide as that wave allows
+  // (not below 8192 values per CTA).
+  const int slots = L.sm_count * kCtasPerSm;
+  int whole = rows / slots * slots, parts = 1;
+  while (parts < kMaxParts && (rows - whole) * parts * 2 <= slots && vocab / (parts * 2) >= 8192) parts *= 2;
+  if (parts == 1) whole = rows;
+  whole -= whole % parts;
+  const unsigned grid = (unsigned)(whole + (rows - whole) * parts);
+  const cudaError_t e = is_f32
+      ? launch_pdl(ppl_nll_kernel<float>, dim3(grid), dim3(kThreads), 0, L.stream, parts, (const float*)logits,
+                   num_tokens, vocab, stride_chunk, stride_token, whole, parts, targets, nll, L.status)
+      : launch_pdl(ppl_nll_kernel<uint16_t>, dim3(grid), dim3(kThreads), 0, L.stream, parts,
+                   (const uint16_t*)logits, num_tokens, vocab, stride_chunk, stride_token, whole, parts, targets,
+                   nll, L.status);
   if (e != cudaSuccess) return e;
-  ppl_mean_kernel<<<(num_chunks + 127) / 128, 128, 0, L.stream>>>(nll, num_chunks, num_tokens, score);
-  return cudaGetLastError();
+  return launch_pdl(ppl_mean_kernel, dim3((num_chunks + kMeanThreads / 32 - 1) / (kMeanThreads / 32)),
+                    dim3(kMeanThreads), 0, L.stream, 1, nll, num_chunks, num_tokens, score);
 }
 
 cudaError_t launch_select_chunks(const Launch& L, const float* score, int num_chunks, int k,
                                  int32_t* chosen) {
-  select_chunks_kernel<<<1, 1024, (size_t)num_chunks * sizeof(float), L.stream>>>(score, num_chunks, k,
-                                                                                 chosen);
-  return cudaGetLastError();
+  return launch_pdl(select_chunks_kernel, dim3((num_chunks + kRankThreads / 32 - 1) / (kRankThreads / 32)),
+                    dim3(kRankThreads), (size_t)num_chunks * sizeof(float), L.stream, 1, score, num_chunks, k, chosen);
 }
 
 }  // namespace cc
