@@ -122,7 +122,7 @@ __device__ __forceinline__ void add_batch(Running& run, const Vec<T> (&r)[kN]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const uint64_t x = fma2(r[u].pair(i), c2, nm);
-      acc[i & 1] = add2(acc[i & 1], (u * 4 + i) % kPolyPairs == 1 ? ex2_pair_fma(x) : ex2_pair_sfu(x));
+      acc[i & 1] = add2(acc[i & 1], kN * 4 >= kPolyPairs && (u * 4 + i) % kPolyPairs == 1 ? ex2_pair_fma(x) : ex2_pair_sfu(x));
     }
   float a, b;
   unpack2(add2(acc[0], acc[1]), a, b);
