@@ -1,5 +1,6 @@
 // C-ABI layer of libcodecomp: argument checks, batch geometry, workspace carving, launches.
 #include <math.h>
+#include <stddef.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
@@ -44,7 +45,42 @@ struct Plan {
   Geometry g;
   // workspace layout (byte offsets)
   size_t off_scores, off_fused, off_score_ws, off_select_ws, total;
+  // cc_compress_layers runs up to `group` layers per launch; their intermediates follow `total`:
+  // scores and fused values of the layers after the first, then the score kernel's statistics
+  int group;
+  size_t off_group, off_group_ws, grand_total;
 };
+
+// Layers per launch of cc_compress_layers.  Launches that share a prologue, a pipeline fill and a
+// tail are what short prompts gain from (32 layers of 4096 tokens: see score_tc.cu); beyond an
+// L2 full of keys the second pass would find none of them in L2 any more, and one layer of that
+// size fills the GPU for long enough on its own.
+constexpr size_t kGroupKeyBytes = 96u << 20;
+int layers_per_launch(const cc_layer_desc* d, const BatchTable& bt, const Geometry& g) {
+  if (d->compute_mode != CC_MODE_BF16 || d->fill_mode != CC_FILL_ATTENTION || bt.n_tot == 0 || bt.b_tot == 0 ||
+      select_cluster_size(bt, g.hkv) == 0)
+    return 1;
+  const size_t key_bytes = (size_t)bt.n_tot * g.hkv * kHeadDim * 2;
+  size_t n = kGroupKeyBytes / key_bytes;
+  if (n > (size_t)(CC_MAX_SEQS / bt.num_seqs)) n = CC_MAX_SEQS / bt.num_seqs;
+  if (n > (size_t)kMaxLayers) n = kMaxLayers;
+  return n < 1 ? 1 : (int)n;
+}
+
+// The table of a launch over `layers` layers of the batch.
+void repeat_layers(const BatchTable& one, int layers, BatchTable* bt) {
+  const int S = one.num_seqs;
+  memcpy(bt, &one, offsetof(BatchTable, seq) + S * sizeof(SeqInfo));
+  for (int l = 1; l < layers; ++l)
+    for (int s = 0; s < S; ++s) {
+      SeqInfo& q = bt->seq[l * S + s];
+      q = one.seq[s];
+      q.layer = l;
+      q.tile_off += l * one.tiles_per_head;
+    }
+  bt->num_seqs = layers * S;
+  bt->tiles_per_head = layers * one.tiles_per_head;
+}
 
 // B^span = min(B, max(B_min, floor(rho * B)))  (Section 4.4, "Span selection under budget")
 int span_cap(int budget, double ratio, int span_min) {
@@ -99,9 +135,10 @@ int build_plan(cc_ctx* ctx, const cc_layer_desc* d, Plan* p) {
       d->kv_stride_tok < kHeadDim)
     return fail(ctx, CC_ERR_INVALID_ARG, "strides smaller than head_dim");
 
-  memset(p, 0, sizeof(*p));
   BatchTable& bt = p->bt;
   Geometry& g = p->g;
+  memset(&bt, 0, offsetof(BatchTable, seq));
+  memset(&g, 0, sizeof(g));
   bt.num_seqs = d->num_seqs > 0 ? d->num_seqs : 1;
   bt.page_size = ps;
   bt.chunk = d->chunk_size > 1 ? d->chunk_size : 1;
@@ -124,6 +161,8 @@ int build_plan(cc_ctx* ctx, const cc_layer_desc* d, Plan* p) {
     q.n_tiles = (n + kTileKeys - 1) / kTileKeys;
     q.out_page_off = (int)page;
     q.span_cap = span_cap(b, d->span_ratio, d->span_min);
+    q.src = s;
+    q.layer = 0;
     tok += n;
     item += q.n_items;
     slot += b;
@@ -169,14 +208,23 @@ int build_plan(cc_ctx* ctx, const cc_layer_desc* d, Plan* p) {
   off += align256(sw);
   p->off_select_ws = off; off += align256(select_ws_bytes(bt, g));
   p->total = off > 256 ? off : 256;
+  p->group = layers_per_launch(d, bt, g);
+  p->off_group = p->total;
+  p->off_group_ws = p->off_group + (size_t)(p->group - 1) * p->off_score_ws;
+  p->grand_total = p->total;
+  if (p->group > 1) {
+    BatchTable all;
+    repeat_layers(bt, p->group, &all);
+    p->grand_total = p->off_group_ws + align256(score_tc_ws_bytes(all, g, ctx->sm_count));
+  }
   return CC_OK;
 }
 
-int check_ws(cc_ctx* ctx, const Plan& p, void* ws, size_t ws_bytes) {
+int check_ws(cc_ctx* ctx, size_t need, void* ws, size_t ws_bytes) {
   if (!ws) return fail(ctx, CC_ERR_WORKSPACE, "workspace is NULL");
   if ((uintptr_t)ws % 256) return fail(ctx, CC_ERR_WORKSPACE, "workspace is not 256-byte aligned");
-  if (ws_bytes < p.total)
-    return fail(ctx, CC_ERR_WORKSPACE, "workspace has %zu bytes, %zu needed", ws_bytes, p.total);
+  if (ws_bytes < need)
+    return fail(ctx, CC_ERR_WORKSPACE, "workspace has %zu bytes, %zu needed", ws_bytes, need);
   return CC_OK;
 }
 
@@ -188,18 +236,18 @@ Launch make_launch(cc_ctx* ctx, void* stream) {
   return L;
 }
 
-int run_score(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const void* q, const void* k,
-              float* scores, float* lse, char* ws, void* stream) {
-  if (p.bt.n_tot == 0) return CC_OK;
+int run_score(cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp,
+              float* lse, char* score_ws, void* stream) {
+  if (bt.n_tot == 0) return CC_OK;
   const Launch L = make_launch(ctx, stream);
   if (d->compute_mode == CC_MODE_FP32) {
-    cudaError_t e = launch_score_simt(L, p.bt, p.g, q, k, scores, lse, ws + p.off_score_ws);
+    cudaError_t e = launch_score_simt(L, bt, g, lp.q[0], lp.k[0], lp.scores[0], lse, score_ws);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "score (fp32 mode) launch");
     return CC_OK;
   }
   int drv = 0;
-  cudaError_t e = launch_score_tc(L, p.bt, p.g, q, k, scores, lse, ws + p.off_score_ws,
-                                  ctx->encode_tiled, (int64_t)d->pool_pages * d->page_size, &drv);
+  cudaError_t e = launch_score_tc(L, bt, g, lp, lse, score_ws, ctx->encode_tiled,
+                                  (int64_t)d->pool_pages * d->page_size, &drv);
   if (drv != 0) return fail(ctx, CC_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", drv);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "score (tensor-core) launch");
   return CC_OK;
@@ -219,48 +267,48 @@ int run_fuse(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const float* sc
   return CC_OK;
 }
 
-int run_select(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const float* fused,
-               const float* prior, int32_t* idx, int32_t* count, char* ws, void* stream) {
+int run_select(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const LayerPtrs& lp, const float* prior,
+               char* ws, void* stream) {
   const int cluster = select_cluster_size(p.bt, p.g.hkv);
   cudaError_t e;
   if (cluster > 0)
     e = launch_select_cluster(make_launch(ctx, stream), p.bt, p.g, d->force_threshold, false,
-                              d->pool_kind, d->pool_size, d->alpha, d->beta, nullptr,
-                              const_cast<float*>(fused), prior, idx, count, cluster);
+                              d->pool_kind, d->pool_size, d->alpha, d->beta, lp, prior, cluster);
   else
-    e = launch_select(make_launch(ctx, stream), p.bt, p.g, d->force_threshold, fused, prior, idx,
-                      count, ws + p.off_select_ws);
+    e = launch_select(make_launch(ctx, stream), p.bt, p.g, d->force_threshold, lp.fused[0], prior, lp.idx[0],
+                      lp.count[0], ws + p.off_select_ws);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "select launch");
   return CC_OK;
 }
 
 // pooling + prior fusion + selection in one launch (items of every sequence fit a cluster)
-int run_fuse_select(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, int cluster,
-                    const float* scores, const float* prior, float* fused, int32_t* idx,
-                    int32_t* count, void* stream) {
-  cudaError_t e = launch_select_cluster(make_launch(ctx, stream), p.bt, p.g, d->force_threshold,
-                                        true, d->pool_kind, d->pool_size, d->alpha, d->beta,
-                                        scores, fused, prior, idx, count, cluster);
+int run_fuse_select(cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, const Geometry& g, int cluster,
+                    const LayerPtrs& lp, const float* prior, void* stream) {
+  cudaError_t e = launch_select_cluster(make_launch(ctx, stream), bt, g, d->force_threshold, true, d->pool_kind,
+                                        d->pool_size, d->alpha, d->beta, lp, prior, cluster);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "fuse + select launch");
   return CC_OK;
 }
 
-int run_compact(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const void* k, const void* v,
-                const int32_t* idx, void* k_out, void* v_out, const int32_t* free_pages,
-                int32_t* out_page_table, void* stream) {
-  if (p.bt.page_size > 0) {
+// What the compaction of one layer needs beside the plan.
+int check_compact(cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, const void* k, const void* v,
+                  const void* k_out, const void* v_out, const int32_t* free_pages, const int32_t* out_page_table) {
+  if (bt.page_size > 0) {
     if (!free_pages || !out_page_table)
       return fail(ctx, CC_ERR_INVALID_ARG, "paged compaction needs free_pages and out_page_table");
-    for (int s = 0; s < p.bt.num_seqs; ++s) {
-      const int used = (p.bt.seq[s].keep + p.bt.page_size - 1) / p.bt.page_size;
+    for (int s = 0; s < bt.num_seqs; ++s) {
+      const int used = (bt.seq[s].keep + bt.page_size - 1) / bt.page_size;
       if (used > d->out_page_table_stride)
         return fail(ctx, CC_ERR_INVALID_ARG, "out_page_table_stride too small for sequence %d", s);
     }
   } else if (k_out == k || v_out == v) {
     return fail(ctx, CC_ERR_INVALID_ARG, "in-place compaction is not supported");
   }
-  cudaError_t e = launch_compact(make_launch(ctx, stream), p.bt, p.g, k, v, idx, k_out, v_out,
-                                 free_pages, out_page_table);
+  return CC_OK;
+}
+
+int run_compact(cc_ctx* ctx, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp, void* stream) {
+  cudaError_t e = launch_compact(make_launch(ctx, stream), bt, g, lp);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "compact launch");
   return CC_OK;
 }
@@ -349,7 +397,7 @@ int cc_poll_status(cc_ctx* ctx, void* stream, int* device_status) {
 size_t cc_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc) {
   Plan p;
   if (build_plan(const_cast<cc_ctx*>(ctx), desc, &p) != CC_OK) return 0;
-  return p.total;
+  return p.grand_total;
 }
 
 int cc_score_window(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win, const void* k,
@@ -360,8 +408,13 @@ int cc_score_window(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win, c
   if (!q_win || !k || !scores) return fail(ctx, CC_ERR_INVALID_ARG, "NULL tensor pointer");
   if ((uintptr_t)q_win % 16 || (uintptr_t)k % 16)
     return fail(ctx, CC_ERR_INVALID_ARG, "q_win and k must be 16-byte aligned");
-  if ((rc = check_ws(ctx, p, ws, ws_bytes)) != CC_OK) return rc;
-  return run_score(ctx, desc, p, q_win, k, scores, lse, (char*)ws, stream);
+  if ((rc = check_ws(ctx, p.total, ws, ws_bytes)) != CC_OK) return rc;
+  LayerPtrs lp;
+  lp.n = 1;
+  lp.q[0] = q_win;
+  lp.k[0] = k;
+  lp.scores[0] = scores;
+  return run_score(ctx, desc, p.bt, p.g, lp, lse, (char*)ws + p.off_score_ws, stream);
 }
 
 int cc_fuse_prior_pool(cc_ctx* ctx, const cc_layer_desc* desc, const float* scores,
@@ -381,8 +434,14 @@ int cc_topk_select(cc_ctx* ctx, const cc_layer_desc* desc, const float* fused, c
   if (rc != CC_OK) return rc;
   if (!fused || !prior || !count || (!idx && p.bt.b_tot > 0))
     return fail(ctx, CC_ERR_INVALID_ARG, "NULL tensor pointer");
-  if ((rc = check_ws(ctx, p, ws, ws_bytes)) != CC_OK) return rc;
-  return run_select(ctx, desc, p, fused, prior, idx, count, (char*)ws, stream);
+  if ((rc = check_ws(ctx, p.total, ws, ws_bytes)) != CC_OK) return rc;
+  LayerPtrs lp;
+  lp.n = 1;
+  lp.scores[0] = nullptr;
+  lp.fused[0] = const_cast<float*>(fused);
+  lp.idx[0] = idx;
+  lp.count[0] = count;
+  return run_select(ctx, desc, p, lp, prior, (char*)ws, stream);
 }
 
 int cc_topk_select_static(cc_ctx* ctx, const cc_layer_desc* desc, const float* fused,
@@ -416,36 +475,60 @@ int cc_compact_kv(cc_ctx* ctx, const cc_layer_desc* desc, const void* k, const v
   if (!k || !v || !idx || !k_out || !v_out) return fail(ctx, CC_ERR_INVALID_ARG, "NULL tensor pointer");
   if ((uintptr_t)k % 16 || (uintptr_t)v % 16 || (uintptr_t)k_out % 16 || (uintptr_t)v_out % 16)
     return fail(ctx, CC_ERR_INVALID_ARG, "K/V pointers must be 16-byte aligned");
-  return run_compact(ctx, desc, p, k, v, idx, k_out, v_out, free_pages, out_page_table, stream);
+  if ((rc = check_compact(ctx, desc, p.bt, k, v, k_out, v_out, free_pages, out_page_table)) != CC_OK) return rc;
+  LayerPtrs lp;
+  lp.n = 1;
+  lp.k[0] = k;
+  lp.v[0] = v;
+  lp.k_out[0] = k_out;
+  lp.v_out[0] = v_out;
+  lp.idx[0] = const_cast<int32_t*>(idx);
+  lp.free_pages[0] = free_pages;
+  lp.out_page_table[0] = out_page_table;
+  return run_compact(ctx, p.bt, p.g, lp, stream);
 }
 
 namespace {
 
-// One layer of the fused step with a plan that is already built and checked.
-int compress_one(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, const void* q_win,
-                 const void* k, const void* v, const float* prior, void* k_out, void* v_out,
-                 int32_t* idx, int32_t* count, const int32_t* free_pages, int32_t* out_page_table,
-                 char* w, void* stream) {
+// The pointers of one layer, checked, as entry l of a launch.
+int take_layer(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, int l, const void* q_win, const void* k,
+               const void* v, const float* prior, void* k_out, void* v_out, int32_t* idx, int32_t* count,
+               const int32_t* free_pages, int32_t* out_page_table, LayerPtrs* lp) {
   if (!q_win || !k || !v || !prior || !count || (p.bt.b_tot > 0 && (!k_out || !v_out || !idx)))
     return fail(ctx, CC_ERR_INVALID_ARG, "NULL tensor pointer");
-  if ((uintptr_t)q_win % 16 || (uintptr_t)k % 16 || (uintptr_t)v % 16 || (uintptr_t)k_out % 16 ||
-      (uintptr_t)v_out % 16)
+  if (((uintptr_t)q_win | (uintptr_t)k | (uintptr_t)v | (uintptr_t)k_out | (uintptr_t)v_out) % 16)
     return fail(ctx, CC_ERR_INVALID_ARG, "tensor pointers must be 16-byte aligned");
+  lp->q[l] = q_win;
+  lp->k[l] = k;
+  lp->v[l] = v;
+  lp->k_out[l] = k_out;
+  lp->v_out[l] = v_out;
+  lp->idx[l] = idx;
+  lp->count[l] = count;
+  lp->free_pages[l] = free_pages;
+  lp->out_page_table[l] = out_page_table;
+  return CC_OK;
+}
+
+// The fused step of the layers of `lp`; bt is the plan's table repeated for them.
+int compress(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, const BatchTable& bt, const LayerPtrs& lp,
+             const float* prior, char* score_ws, char* w, void* stream) {
   int rc;
-  float* scores = (float*)(w + p.off_scores);
-  float* fused = (float*)(w + p.off_fused);
   const bool nearest = desc->fill_mode == CC_FILL_NEAREST;   // the scores play no part then
-  if (!nearest && (rc = run_score(ctx, desc, p, q_win, k, scores, nullptr, w, stream)) != CC_OK) return rc;
-  const int cluster = select_cluster_size(p.bt, p.g.hkv);
+  if (!nearest && (rc = run_score(ctx, desc, bt, p.g, lp, nullptr, score_ws, stream)) != CC_OK) return rc;
+  const int cluster = select_cluster_size(bt, p.g.hkv);
   if (cluster > 0 && !nearest) {
-    rc = run_fuse_select(ctx, desc, p, cluster, scores, prior, fused, idx, count, stream);
-    if (rc != CC_OK) return rc;
+    if ((rc = run_fuse_select(ctx, desc, bt, p.g, cluster, lp, prior, stream)) != CC_OK) return rc;
   } else {
-    if ((rc = run_fuse(ctx, desc, p, scores, prior, fused, stream)) != CC_OK) return rc;
-    if ((rc = run_select(ctx, desc, p, fused, prior, idx, count, w, stream)) != CC_OK) return rc;
+    if ((rc = run_fuse(ctx, desc, p, lp.scores[0], prior, lp.fused[0], stream)) != CC_OK) return rc;
+    if ((rc = run_select(ctx, desc, p, lp, prior, w, stream)) != CC_OK) return rc;
   }
-  if (p.bt.b_tot == 0) return CC_OK;
-  return run_compact(ctx, desc, p, k, v, idx, k_out, v_out, free_pages, out_page_table, stream);
+  if (bt.b_tot == 0) return CC_OK;
+  for (int l = 0; l < lp.n; ++l)
+    if ((rc = check_compact(ctx, desc, p.bt, lp.k[l], lp.v[l], lp.k_out[l], lp.v_out[l], lp.free_pages[l],
+                            lp.out_page_table[l])) != CC_OK)
+      return rc;
+  return run_compact(ctx, bt, p.g, lp, stream);
 }
 
 }  // namespace
@@ -457,9 +540,15 @@ int cc_compress_layer(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win,
   Plan p;
   int rc = build_plan(ctx, desc, &p);
   if (rc != CC_OK) return rc;
-  if ((rc = check_ws(ctx, p, ws, ws_bytes)) != CC_OK) return rc;
-  return compress_one(ctx, desc, p, q_win, k, v, prior, k_out, v_out, idx, count, free_pages,
-                      out_page_table, (char*)ws, stream);
+  if ((rc = check_ws(ctx, p.total, ws, ws_bytes)) != CC_OK) return rc;
+  char* w = (char*)ws;
+  LayerPtrs lp;
+  lp.n = 1;
+  lp.scores[0] = (float*)(w + p.off_scores);
+  lp.fused[0] = (float*)(w + p.off_fused);
+  rc = take_layer(ctx, desc, p, 0, q_win, k, v, prior, k_out, v_out, idx, count, free_pages, out_page_table, &lp);
+  if (rc != CC_OK) return rc;
+  return compress(ctx, desc, p, p.bt, lp, prior, w + p.off_score_ws, w, stream);
 }
 
 int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
@@ -477,11 +566,25 @@ int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
     return fail(ctx, CC_ERR_INVALID_ARG, "NULL pointer array");
   if (p.bt.page_size > 0 && (!free_pages || !out_page_table))
     return fail(ctx, CC_ERR_INVALID_ARG, "paged compaction needs free_pages and out_page_table");
-  if ((rc = check_ws(ctx, p, ws, ws_bytes)) != CC_OK) return rc;
-  for (int l = 0; l < n_layers; ++l) {
-    rc = compress_one(ctx, desc, p, q_win[l], k[l], v[l], prior, k_out[l], v_out[l], idx[l], count[l],
-                      free_pages ? free_pages[l] : nullptr, out_page_table ? out_page_table[l] : nullptr,
-                      (char*)ws, stream);
+  if ((rc = check_ws(ctx, p.grand_total, ws, ws_bytes)) != CC_OK) return rc;
+  char* w = (char*)ws;
+  const int groups = (n_layers + p.group - 1) / p.group;
+  BatchTable bt;
+  for (int i = 0; i < groups; ++i) {
+    const int l0 = (int)((long long)n_layers * i / groups), l1 = (int)((long long)n_layers * (i + 1) / groups);
+    LayerPtrs lp;
+    lp.n = l1 - l0;
+    for (int l = l0; l < l1; ++l) {
+      const int e = l - l0, slot = l1 - 1 - l;     // the group's last layer uses the first slot of the workspace
+      char* base = slot == 0 ? w : w + p.off_group + (size_t)(slot - 1) * p.off_score_ws;
+      lp.scores[e] = (float*)(base + p.off_scores);
+      lp.fused[e] = (float*)(base + p.off_fused);
+      rc = take_layer(ctx, desc, p, e, q_win[l], k[l], v[l], prior, k_out[l], v_out[l], idx[l], count[l],
+                      free_pages ? free_pages[l] : nullptr, out_page_table ? out_page_table[l] : nullptr, &lp);
+      if (rc != CC_OK) return rc;
+    }
+    if (i == 0 || lp.n * p.bt.num_seqs != bt.num_seqs) repeat_layers(p.bt, lp.n, &bt);
+    rc = compress(ctx, desc, p, bt, lp, prior, w + (lp.n > 1 ? p.off_group_ws : p.off_score_ws), w, stream);
     if (rc != CC_OK) return rc;
   }
   return CC_OK;

@@ -26,11 +26,16 @@ struct SeqInfo {
   int n_tiles;       // ceil(n / kTileKeys)
   int out_page_off;  // first entry of free_pages used by the sequence
   int span_cap;      // B_span, or -1 when protected tokens are not capped
-  int pad_;
+  int src;           // index of the sequence in the caller's batch (row of the page tables, Q, counts)
+  int layer;         // entry of the launch's pointer arrays (several layers in one launch)
 };
 
+// Several layers of a batch go through one launch as further entries of the table: entry
+// layer * S + s is sequence s of that layer, its offsets into the per-layer arrays unchanged.
+constexpr int kMaxLayers = 16;       // layers per launch
+
 struct BatchTable {
-  int num_seqs;
+  int num_seqs;      // entries: sequences x layers of the launch
   int page_size;     // 0 = contiguous
   int chunk;         // >= 1
   int n_tot, m_tot, b_tot;
@@ -76,6 +81,23 @@ struct Launch {
   int sm_count;
 };
 
+// Lets a kernel use all of an SM's shared memory; asked of the runtime once per kernel and device.
+constexpr int kSmemPerCta = 232448;      // 227 KB
+template <class... KArgs>
+cudaError_t allow_smem(void (*kernel)(KArgs...)) {
+  struct Seen { const void* kernel; int device; };
+  static thread_local Seen seen[16];
+  static thread_local int n_seen = 0;
+  int device = -1;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  for (int i = 0; i < n_seen; ++i)
+    if (seen[i].kernel == (const void*)kernel && seen[i].device == device) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
+  if (e == cudaSuccess && n_seen < 16) seen[n_seen++] = Seen{(const void*)kernel, device};
+  return e;
+}
+
 // Programmatic dependent launch: every kernel of the library lets its successor in the stream
 // start its prologue early (pdl_launch_dependents at the top) and touches global memory only
 // after pdl_wait, which returns once the preceding kernels have completed and flushed.
@@ -115,11 +137,28 @@ size_t score_simt_ws_bytes(const BatchTable& bt, const Geometry& g, int sm_count
 cudaError_t launch_score_simt(const Launch& L, const BatchTable& bt, const Geometry& g,
                               const void* q, const void* k, float* scores, float* lse, void* ws);
 
+// Device pointers of the layers of a launch (entry l: what the caller gave for that layer).
+struct LayerPtrs {
+  int n;
+  const void* q[kMaxLayers];
+  const void* k[kMaxLayers];
+  const void* v[kMaxLayers];
+  void* k_out[kMaxLayers];
+  void* v_out[kMaxLayers];
+  int32_t* idx[kMaxLayers];
+  int32_t* count[kMaxLayers];
+  const int32_t* free_pages[kMaxLayers];
+  int32_t* out_page_table[kMaxLayers];
+  float* scores[kMaxLayers];
+  float* fused[kMaxLayers];
+};
+
 size_t score_tc_ws_bytes(const BatchTable& bt, const Geometry& g, int sm_count);
 // encode = cuTensorMapEncodeTiled entry point; err receives a CUresult-like code on failure
+// (reads q, k and scores of the layers; lse: one layer only)
 cudaError_t launch_score_tc(const Launch& L, const BatchTable& bt, const Geometry& g,
-                            const void* q, const void* k, float* scores, float* lse, void* ws,
-                            void* encode_fn, int64_t pool_rows, int* drv_err);
+                            const LayerPtrs& lp, float* lse, void* ws, void* encode_fn,
+                            int64_t pool_rows, int* drv_err);
 
 // fused[h][j] = -(distance of token j to the closest token with prior >= threshold), every head
 cudaError_t launch_nearest_fill(const Launch& L, const BatchTable& bt, const Geometry& g,
@@ -138,11 +177,11 @@ cudaError_t launch_select(const Launch& L, const BatchTable& bt, const Geometry&
 // (pooling and prior fusion done in the same launch).  select_cluster_size returns the CTAs per
 // (sequence, head) to use, or 0 when a sequence has too many items for it.
 int select_cluster_size(const BatchTable& bt, int hkv);
+// (reads scores, fused, idx and count of the layers)
 cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const Geometry& g,
                                   float force_threshold, bool fused_input, int pool_kind,
-                                  int pool_size, float alpha, float beta, const float* scores,
-                                  float* fused, const float* prior, int32_t* idx, int32_t* count,
-                                  int cluster);
+                                  int pool_size, float alpha, float beta, const LayerPtrs& lp,
+                                  const float* prior, int cluster);
 
 // variant of launch_select whose scratch is a static device array (no workspace argument)
 int64_t select_static_capacity();
@@ -150,9 +189,7 @@ cudaError_t launch_select_static(const Launch& L, const BatchTable& bt, const Ge
                                  float force_threshold, const float* fused, const float* prior,
                                  int32_t* idx, int32_t* count, int device);
 
-cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g,
-                           const void* k, const void* v, const int32_t* idx, void* k_out,
-                           void* v_out, const int32_t* free_pages, int32_t* out_page_table);
+cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp);
 
 // chunk selection by query-conditioned perplexity (Section 4.1)
 cudaError_t launch_ppl_scores(const Launch& L, const void* logits, bool is_f32, int num_chunks,

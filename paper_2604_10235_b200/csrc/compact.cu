@@ -24,6 +24,16 @@ __device__ __forceinline__ void st_stream(uint4* p, uint4 v) {
                :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+struct CompactPtrs {          // per layer of the launch
+  const uint16_t* k[kMaxLayers];
+  const uint16_t* v[kMaxLayers];
+  const int32_t* idx[kMaxLayers];
+  const int32_t* free_pages[kMaxLayers];
+  uint16_t* k_out[kMaxLayers];
+  uint16_t* v_out[kMaxLayers];
+  int32_t* out_page_table[kMaxLayers];
+};
+
 // A group of 16 threads owns a unit = (slot, run of heads_per_group consecutive heads): the
 // destination rows of a unit are adjacent, its page look-up on the output side is done once, and
 // no division by the head count is needed (units per slot = 1 << hc_shift).  The rows of a unit
@@ -34,11 +44,8 @@ __device__ __forceinline__ void st_stream(uint4* p, uint4 v) {
 template <int kUnroll>
 __global__ void __launch_bounds__(kThreads)
 compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
-               const uint16_t* __restrict__ k, const uint16_t* __restrict__ v,
-               const int32_t* __restrict__ idx, uint16_t* __restrict__ k_out,
-               uint16_t* __restrict__ v_out, const int32_t* __restrict__ free_pages,
-               int32_t* __restrict__ out_page_table, DeviceStatus* status,
-               int heads_per_group, int hc_shift) {
+               const __grid_constant__ CompactPtrs P, DeviceStatus* status, int heads_per_group,
+               int hc_shift) {
   pdl_launch_dependents();
   pdl_wait();
   int s = 0, local = blockIdx.x;              // sequence of this block, block index within it
@@ -48,6 +55,10 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
     local -= nb;
   }
   const SeqInfo& q = bt.seq[s];
+  const uint16_t* __restrict__ k = P.k[q.layer];
+  const uint16_t* __restrict__ v = P.v[q.layer];
+  const int32_t* __restrict__ idx = P.idx[q.layer];
+  const int32_t* __restrict__ free_pages = P.free_pages[q.layer];
   const int lane = threadIdx.x % kLanesPerRow;
   const int grp = threadIdx.x / kLanesPerRow;
   const int ps = bt.page_size;
@@ -63,16 +74,18 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
         report_error(status, CC_ERR_DEVICE_FLAG, 503);
         page = -1;
       }
-      out_page_table[(int64_t)s * g.out_page_table_stride + i] = page;
+      P.out_page_table[q.layer][(int64_t)q.src * g.out_page_table_stride + i] = page;
     }
   }
 
   const int units = q.keep << hc_shift;          // fits: keep * heads indexes an int32 array
   const int hc_mask = (1 << hc_shift) - 1;
   const int64_t head_step = ps == 0 ? g.out_stride_head : g.kv_stride_head;
-  const int32_t* pt = ps > 0 ? g.page_table + (int64_t)s * g.page_table_stride : nullptr;
+  const int32_t* pt = ps > 0 ? g.page_table + (int64_t)q.src * g.page_table_stride : nullptr;
   const int u = local * kRowsPerBlock + grp;
   if (u < units) {
+    uint16_t* __restrict__ k_out = P.k_out[q.layer];
+    uint16_t* __restrict__ v_out = P.v_out[q.layer];
     const int slot = u >> hc_shift;
     const int h0 = (u & hc_mask) * heads_per_group;
     int64_t dst0;                                  // destination row of (slot, head 0)
@@ -137,9 +150,17 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
 
 }  // namespace
 
-cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g,
-                           const void* k, const void* v, const int32_t* idx, void* k_out,
-                           void* v_out, const int32_t* free_pages, int32_t* out_page_table) {
+cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp) {
+  CompactPtrs P = {};
+  for (int l = 0; l < lp.n; ++l) {
+    P.k[l] = (const uint16_t*)lp.k[l];
+    P.v[l] = (const uint16_t*)lp.v[l];
+    P.idx[l] = lp.idx[l];
+    P.free_pages[l] = lp.free_pages[l];
+    P.k_out[l] = (uint16_t*)lp.k_out[l];
+    P.v_out[l] = (uint16_t*)lp.v_out[l];
+    P.out_page_table[l] = lp.out_page_table[l];
+  }
   int64_t slots = 0;
   for (int s = 0; s < bt.num_seqs; ++s) slots += bt.seq[s].keep;
   // Heads per unit: all heads of a slot when the batch still fills the GPU that way (fewest
@@ -159,9 +180,7 @@ cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry
     blocks += max((int64_t)1, (((int64_t)bt.seq[s].keep << hc_shift) + kRowsPerBlock - 1) / kRowsPerBlock);
   dim3 grid((unsigned)blocks);
   auto kern = hpg >= 4 ? compact_kernel<4> : (hpg >= 2 ? compact_kernel<2> : compact_kernel<1>);
-  return launch_pdl(kern, grid, dim3(kThreads), 0, L.stream, 1, bt, g, (const uint16_t*)k,
-                    (const uint16_t*)v, idx, (uint16_t*)k_out, (uint16_t*)v_out, free_pages,
-                    out_page_table, L.status, hpg, hc_shift);
+  return launch_pdl(kern, grid, dim3(kThreads), 0, L.stream, 1, bt, g, P, L.status, hpg, hc_shift);
 }
 
 }  // namespace cc

@@ -75,7 +75,6 @@ struct TcParams {
   int n_sub;           // pass 1: 128-row blocks; pass 2: column chunks
   int sub_cols;        // pass 2: rows per column chunk (multiple of 16, <= 128)
   float2* part;        // [(grid + problems)][rows_pad] (max, sum) in the log2 domain
-  float* scores;
   float* lse;
   int64_t pool_rows;
   // K tile in shared memory.  Contiguous cache: two panels of 64 channels, each 128 rows of 128
@@ -84,6 +83,13 @@ struct TcParams {
   // 2048 bytes apart, second panel 1 KB on), whatever the page size.
   uint32_t k_sbo16;      // stride between 8-row groups of a panel, in 16-byte units
   uint32_t k_panel16;    // offset of the second panel, in 16-byte units
+};
+
+// Tensor maps and score arrays of the layers of a launch.
+template <int LAYERS>
+struct TcLayers {
+  CUtensorMap q[LAYERS], k[LAYERS];
+  float* scores[LAYERS];
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -288,11 +294,11 @@ __device__ __forceinline__ int cta_of_tile(int t, const TcParams& P) {
 // ------------------------------------------------------------------ the kernel
 // CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of
 // that code.
-template <int PASS, bool CAUSAL>
+template <int PASS, bool CAUSAL, int LAYERS>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ Geometry g,
-                const __grid_constant__ TcParams P, const __grid_constant__ CUtensorMap q_map,
-                const __grid_constant__ CUtensorMap k_map, DeviceStatus* status) {
+                const __grid_constant__ TcParams P, const __grid_constant__ TcLayers<LAYERS> M,
+                DeviceStatus* status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t q_bytes = (uint32_t)P.rows_pad * 256u;
@@ -307,8 +313,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
 
   if (threadIdx.x == 32) {
     // fetch the two TMA descriptors (kernel parameters) while the barriers are being set up
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&q_map)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&k_map)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&M.q[0])) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&M.k[0])) : "memory");
   }
   if (threadIdx.x == 0) {
     for (int i = 0; i < kMaxStages; ++i) {
@@ -364,6 +370,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       else           asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(k_policy));
       for (int t = t_begin; t < t_end; ++t, cur.advance(bt, g.hkv)) {
         const SeqInfo& sq = bt.seq[cur.s];
+        const int layer = LAYERS > 1 ? sq.layer : 0;
+        const CUtensorMap* q_map = &M.q[layer];
+        const CUtensorMap* k_map = &M.k[layer];
         if (cur.problem(g.hkv) != cur_problem) {
           if (cur_problem >= 0) {
             const bool got = lane != 0 || wait_bar(pipe, &misc->bar.q_empty, qe_phase, 10);
@@ -374,8 +383,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           if (lane == 0) {
             const uint32_t qb = smem_u32(&misc->bar.q_full);
             mbar_expect_tx(qb, q_bytes);
-            tma_load_4d(smem_u32(q_smem), &q_map, qb, 0, cur.h * g.group, 0, cur.s);
-            tma_load_4d(smem_u32(q_smem) + q_panel, &q_map, qb, 64, cur.h * g.group, 0, cur.s);
+            tma_load_4d(smem_u32(q_smem), q_map, qb, 0, cur.h * g.group, 0, sq.src);
+            tma_load_4d(smem_u32(q_smem) + q_panel, q_map, qb, 64, cur.h * g.group, 0, sq.src);
           }
         }
         const int key0 = cur.local * kTileKeys;
@@ -384,7 +393,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         if (ps > 0) {
           const int valid = min(kTileKeys, sq.n - key0);
           mine = lane < (valid + ps - 1) / ps;
-          if (mine) page_id = g.page_table[(int64_t)cur.s * g.page_table_stride + key0 / ps + lane];
+          if (mine) page_id = g.page_table[(int64_t)sq.src * g.page_table_stride + key0 / ps + lane];
         }
         {
           const bool got = lane != 0 || wait_bar(pipe, &misc->bar.empty[stage], phase ^ 1, 11);
@@ -395,8 +404,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         if (ps == 0) {
           if (lane == 0) {
             mbar_expect_tx(fb, kStageBytes);
-            tma_load_3d_hint(dst, &k_map, fb, 0, cur.h, sq.tok_off + key0, k_policy);
-            tma_load_3d_hint(dst + kPanelBytes, &k_map, fb, 64, cur.h, sq.tok_off + key0, k_policy);
+            tma_load_3d_hint(dst, k_map, fb, 0, cur.h, sq.tok_off + key0, k_policy);
+            tma_load_3d_hint(dst + kPanelBytes, k_map, fb, 64, cur.h, sq.tok_off + key0, k_policy);
           }
         } else {
           const bool good = mine && page_id >= 0 && ((int64_t)page_id + 1) * ps <= P.pool_rows;
@@ -407,7 +416,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           if (lane == 0) mbar_expect_tx(fb, (uint32_t)__popc(good_mask) * (uint32_t)ps * 256u);
           __syncwarp();
           if (good)      // the page's rows, both panels, in one copy
-            tma_load_5d_hint(dst + (uint32_t)lane * (uint32_t)ps * 256u, &k_map, fb,
+            tma_load_5d_hint(dst + (uint32_t)lane * (uint32_t)ps * 256u, k_map, fb,
                              page_id * (ps >> 3), cur.h, k_policy);
         }
         if (++stage == P.n_stages) { stage = 0; phase ^= 1; }
@@ -620,7 +629,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     int sub = set % n_sub, t = t_begin + set / n_sub;
     uint32_t par = 0;
     int prob_end = t_begin, first_tile = 0, n_cur = 0;
-    int64_t out_base = 0;
+    float* out = nullptr;
     const uint32_t full_bar = smem_u32(&misc->bar.acc_full[set]);
     const uint32_t empty_bar = smem_u32(&misc->bar.acc_empty[set]);
     const uint32_t acc_addr = lane_addr + (uint32_t)set * kBufCols;
@@ -641,7 +650,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           cur_problem = cur.problem(g.hkv);
           prob_end = min(t_end, first_tile + sq.n_tiles);
           n_cur = sq.n;
-          out_base = (int64_t)cur.h * bt.n_tot + sq.tok_off;
+          out = M.scores[LAYERS > 1 ? sq.layer : 0] + (int64_t)cur.h * bt.n_tot + sq.tok_off;
         } while (t >= prob_end);
         if (done) break;
       }
@@ -781,11 +790,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
             if (!dead && row_in_tile < valid) {
               float u = u_acc;
               for (int k = 0; k < n_sub - 1; ++k) u += misc->u_part[slot][k][row_in_tile];
-              P.scores[out_base + key0 + row_in_tile] = u;
+              out[key0 + row_in_tile] = u;
             }
           }
         } else if (!dead && row_in_tile < valid) {
-          P.scores[out_base + key0 + row_in_tile] = u_acc;
+          out[key0 + row_in_tile] = u_acc;
         }
       }
       sub += ds;
@@ -850,84 +859,85 @@ size_t score_tc_ws_bytes(const BatchTable& bt, const Geometry& g, int sm_count) 
   return (entries * pl.P.rows_pad * sizeof(float2) + 255) / 256 * 256;
 }
 
-cudaError_t launch_score_tc(const Launch& L, const BatchTable& bt, const Geometry& g,
-                            const void* q, const void* k, float* scores, float* lse, void* ws,
-                            void* encode_fn, int64_t pool_rows, int* drv_err) {
-  *drv_err = 0;
-  TcPlan pl = make_plan(bt, g, L.sm_count);
-  if (!pl.ok) return cudaErrorInvalidConfiguration;
-  TcParams& P = pl.P;
-  P.part = (float2*)ws;
-  P.scores = scores;
-  P.lse = lse;
-  P.pool_rows = bt.page_size > 0 ? pool_rows : (int64_t)bt.n_tot;
+namespace {
 
-  EncodeTiledFn encode = (EncodeTiledFn)encode_fn;
-  CUtensorMap q_map, k_map;
+// The tensor maps of one layer.
+CUresult encode_maps(EncodeTiledFn encode, const BatchTable& bt, const Geometry& g, const TcParams& P, int num_seqs,
+                     const void* q, const void* k, CUtensorMap* q_map, CUtensorMap* k_map) {
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   {
-    const int S = bt.num_seqs;
-    cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.hq, (cuuint64_t)g.window, (cuuint64_t)S};
+    const cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.hq, (cuuint64_t)g.window, (cuuint64_t)num_seqs};
     int64_t seq_stride = g.q_stride_seq;
-    if (S == 1 || seq_stride <= 0) seq_stride = g.q_stride_row * g.window;
-    cuuint64_t strides[3] = {(cuuint64_t)g.q_stride_head * 2, (cuuint64_t)g.q_stride_row * 2,
-                             (cuuint64_t)seq_stride * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)g.group, (cuuint32_t)P.w_pad, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = encode(&q_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(q), dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { *drv_err = (int)r; return cudaErrorUnknown; }
+    if (num_seqs == 1 || seq_stride <= 0) seq_stride = g.q_stride_row * g.window;
+    const cuuint64_t strides[3] = {(cuuint64_t)g.q_stride_head * 2, (cuuint64_t)g.q_stride_row * 2,
+                                   (cuuint64_t)seq_stride * 2};
+    const cuuint32_t box[4] = {64, (cuuint32_t)g.group, (cuuint32_t)P.w_pad, 1};
+    const CUresult r = encode(q_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(q), dims, strides, box,
+                              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return r;
   }
   if (bt.page_size > 0) {
     // A page (page_size tokens, a multiple of 8, starting at a multiple of 8 rows) as one box: 64
     // channels x 8 tokens x 2 panels x page_size / 8 groups of one head.  In shared memory that is
     // page_size / 8 blocks of 2 KB, each the eight rows of the first panel followed by the eight
     // rows of the second: two copies per page become one (a 16-token page: 4 KB per copy).
-    cuuint64_t dims[5] = {64, 8, 2, (cuuint64_t)(P.pool_rows / 8), (cuuint64_t)g.hkv};
-    cuuint64_t strides[4] = {(cuuint64_t)g.kv_stride_tok * 2, 128, (cuuint64_t)g.kv_stride_tok * 16,
-                             (cuuint64_t)g.kv_stride_head * 2};
-    cuuint32_t box[5] = {64, 8, 2, (cuuint32_t)(bt.page_size / 8), 1};
-    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    CUresult r = encode(&k_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(k), dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { *drv_err = (int)r; return cudaErrorUnknown; }
-    P.k_sbo16 = 2048u >> 4;
-    P.k_panel16 = 1024u >> 4;
-  } else {
-    cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.hkv, (cuuint64_t)P.pool_rows};
-    cuuint64_t strides[2] = {(cuuint64_t)g.kv_stride_head * 2, (cuuint64_t)g.kv_stride_tok * 2};
-    cuuint32_t box[3] = {64, 1, (cuuint32_t)kTileKeys};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = encode(&k_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(k), dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { *drv_err = (int)r; return cudaErrorUnknown; }
-    P.k_sbo16 = 1024u >> 4;
-    P.k_panel16 = kPanelBytes >> 4;
+    const cuuint64_t dims[5] = {64, 8, 2, (cuuint64_t)(P.pool_rows / 8), (cuuint64_t)g.hkv};
+    const cuuint64_t strides[4] = {(cuuint64_t)g.kv_stride_tok * 2, 128, (cuuint64_t)g.kv_stride_tok * 16,
+                                   (cuuint64_t)g.kv_stride_head * 2};
+    const cuuint32_t box[5] = {64, 8, 2, (cuuint32_t)(bt.page_size / 8), 1};
+    return encode(k_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(k), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
+  const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.hkv, (cuuint64_t)P.pool_rows};
+  const cuuint64_t strides[2] = {(cuuint64_t)g.kv_stride_head * 2, (cuuint64_t)g.kv_stride_tok * 2};
+  const cuuint32_t box[3] = {64, 1, (cuuint32_t)kTileKeys};
+  return encode(k_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(k), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
 
-  auto pass1 = g.causal ? score_tc_kernel<1, true> : score_tc_kernel<1, false>;
-  auto pass2 = g.causal ? score_tc_kernel<2, true> : score_tc_kernel<2, false>;
-  cudaError_t e;
-  e = cudaFuncSetAttribute(pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem_bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem_bytes);
+template <int LAYERS>
+cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp,
+                          const TcPlan& pl, EncodeTiledFn encode, int* drv_err) {
+  TcParams P = pl.P;
+  TcLayers<LAYERS> M;
+  for (int l = 0; l < lp.n; ++l) {
+    const CUresult r = encode_maps(encode, bt, g, P, bt.num_seqs / lp.n, lp.q[l], lp.k[l], &M.q[l], &M.k[l]);
+    if (r != CUDA_SUCCESS) { *drv_err = (int)r; return cudaErrorUnknown; }
+    M.scores[l] = lp.scores[l];
+  }
+  auto pass1 = g.causal ? score_tc_kernel<1, true, LAYERS> : score_tc_kernel<1, false, LAYERS>;
+  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS> : score_tc_kernel<2, false, LAYERS>;
+  cudaError_t e = allow_smem(pass1);
+  if (e == cudaSuccess) e = allow_smem(pass2);
   if (e != cudaSuccess) return e;
 
   P.n_sub = (P.rows_pad + 127) / 128;
   P.sub_cols = 0;
-  e = launch_pdl(pass1, dim3(P.grid), dim3(kThreads), pl.smem_bytes, L.stream, 1, bt, g, P, q_map,
-                 k_map, L.status);
+  e = launch_pdl(pass1, dim3(P.grid), dim3(kThreads), pl.smem_bytes, L.stream, 1, bt, g, P, M, L.status);
   if (e != cudaSuccess) return e;
-
-  P.n_sub = (P.rows_pad + 127) / 128;
   P.sub_cols = ((P.rows_pad + P.n_sub - 1) / P.n_sub + 15) / 16 * 16;
-  return launch_pdl(pass2, dim3(P.grid), dim3(kThreads), pl.smem_bytes, L.stream, 1, bt, g, P, q_map,
-                    k_map, L.status);
+  return launch_pdl(pass2, dim3(P.grid), dim3(kThreads), pl.smem_bytes, L.stream, 1, bt, g, P, M, L.status);
+}
+
+}  // namespace
+
+cudaError_t launch_score_tc(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp,
+                            float* lse, void* ws, void* encode_fn, int64_t pool_rows, int* drv_err) {
+  *drv_err = 0;
+  TcPlan pl = make_plan(bt, g, L.sm_count);
+  if (!pl.ok) return cudaErrorInvalidConfiguration;
+  pl.P.part = (float2*)ws;
+  pl.P.lse = lse;
+  pl.P.pool_rows = bt.page_size > 0 ? pool_rows : (int64_t)bt.n_tot;
+  // 8-row groups and panels of a K tile in shared memory (see TcParams)
+  pl.P.k_sbo16 = (bt.page_size > 0 ? 2048u : 1024u) >> 4;
+  pl.P.k_panel16 = (bt.page_size > 0 ? 1024u : kPanelBytes) >> 4;
+  EncodeTiledFn encode = (EncodeTiledFn)encode_fn;
+  return lp.n > 1 ? launch_passes<kMaxLayers>(L, bt, g, lp, pl, encode, drv_err)
+                  : launch_passes<1>(L, bt, g, lp, pl, encode, drv_err);
 }
 
 }  // namespace cc

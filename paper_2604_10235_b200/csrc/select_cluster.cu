@@ -42,6 +42,7 @@ struct Shared {
   unsigned xchg[2][kMaxCluster][4];   // [buffer copy][source CTA][word]: written by the peers
   unsigned warp_a[kWarps];
   unsigned warp_b[kWarps];
+  unsigned warp_lo[kWarps], warp_hi[kWarps];
   unsigned bcast[4];
 };
 
@@ -53,13 +54,12 @@ struct ClusterParams {
   int stage_u;               // the slice's raw scores are staged in shared memory before pooling
   int pool_kind, pool_size;
   float alpha, beta;
-  const float* scores;
-  float* fused_out;
-  // plain
-  const float* fused_in;
   const float* prior;
-  int32_t* idx;
-  int32_t* count;
+  // per layer of the launch
+  const float* scores[kMaxLayers];    // FUSED only
+  float* fused[kMaxLayers];           // FUSED: written; plain: read
+  int32_t* idx[kMaxLayers];
+  int32_t* count[kMaxLayers];
 };
 
 __host__ __device__ __forceinline__ int padded(int li) { return li + (li >> 5); }
@@ -180,7 +180,7 @@ struct Ctx {
       lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
       hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
-    __shared__ unsigned w_lo[kWarps], w_hi[kWarps];
+    unsigned *w_lo = sm->warp_lo, *w_hi = sm->warp_hi;
     if (lane == 0) { w_lo[warp] = lo; w_hi[warp] = hi; }
     unsigned eb, ta, tb;
     block_scan2(a, 0u, ea, eb, ta, tb);      // its barriers also publish w_lo / w_hi
@@ -328,7 +328,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   const int cta_items = cta_hi - cta_lo;
   uint8_t* flags = reinterpret_cast<uint8_t*>(keys + padded(kThreads * per) + 1);
   const float* p = P.prior + q.tok_off;
-  int32_t* out = P.idx + (int64_t)h * bt.b_tot + q.idx_off;
+  int32_t* out = P.idx[q.layer] + (int64_t)h * bt.b_tot + q.idx_off;
   const unsigned keep = (unsigned)q.keep;
   const float theta = P.theta;
 
@@ -352,8 +352,8 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 
   // ---- load: keys and protected flags of the CTA's slice (coalesced over the block)
   if (FUSED) {
-    const float* u = P.scores + (int64_t)h * bt.n_tot + q.tok_off;
-    float* fo = P.fused_out + (int64_t)h * bt.m_tot + q.item_off;
+    const float* u = P.scores[q.layer] + (int64_t)h * bt.n_tot + q.tok_off;
+    float* fo = P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off;
     const int half = (cs == 1 && P.pool_kind != CC_POOL_NONE) ? P.pool_size / 2 : 0;
     float* us = reinterpret_cast<float*>(flags + ((kThreads * per + 15) / 16) * 16);
     if (cs == 1) {
@@ -440,7 +440,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
       flags[li] = pr >= theta ? 1 : 0;
     }
   } else {
-    const float* f = P.fused_in + (int64_t)h * bt.m_tot + q.item_off;
+    const float* f = P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off;
 #pragma unroll 1
     for (int li = threadIdx.x; li < cta_items; li += kThreads) {
       keys[padded(li)] = mono_key(f[cta_lo + li]);
@@ -571,7 +571,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   }
   for (int i = (int)keep + c.rank * kThreads + threadIdx.x; i < q.budget; i += c.C * kThreads)
     out[i] = -1;
-  if (c.rank == 0 && threadIdx.x == 0) P.count[s * P.hkv + h] = (int)keep;
+  if (c.rank == 0 && threadIdx.x == 0) P.count[q.layer][q.src * P.hkv + h] = (int)keep;
   // no CTA may leave while a peer can still read its shared memory
   if (c.C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -615,9 +615,8 @@ int select_cluster_size(const BatchTable& bt, int hkv) {
 
 cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const Geometry& g,
                                   float force_threshold, bool fused_input, int pool_kind,
-                                  int pool_size, float alpha, float beta, const float* scores,
-                                  float* fused, const float* prior, int32_t* idx, int32_t* count,
-                                  int cluster) {
+                                  int pool_size, float alpha, float beta, const LayerPtrs& lp,
+                                  const float* prior, int cluster) {
   ClusterParams P;
   P.cluster = cluster;
   P.hkv = g.hkv;
@@ -626,12 +625,13 @@ cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const G
   P.pool_size = pool_kind == CC_POOL_NONE ? 1 : pool_size;
   P.alpha = alpha;
   P.beta = beta;
-  P.scores = scores;
-  P.fused_out = fused;
-  P.fused_in = fused;
   P.prior = prior;
-  P.idx = idx;
-  P.count = count;
+  for (int l = 0; l < lp.n; ++l) {
+    P.scores[l] = lp.scores[l];
+    P.fused[l] = lp.fused[l];
+    P.idx[l] = lp.idx[l];
+    P.count[l] = lp.count[l];
+  }
   const int per = bt.max_items > 0 ? (bt.max_items + cluster * kThreads - 1) / (cluster * kThreads) : 1;
   // token-level fused form: stage the slice's raw scores while they fit beside keys and flags
   P.stage_u = fused_input && bt.chunk == 1 && kThreads * per <= kStagedItems ? 1 : 0;
@@ -639,7 +639,7 @@ cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const G
   const bool chunked = bt.chunk > 1;
   auto kern = fused_input ? (chunked ? select_cluster_kernel<true, true> : select_cluster_kernel<true, false>)
                           : (chunked ? select_cluster_kernel<false, true> : select_cluster_kernel<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(cluster, g.hkv, bt.num_seqs), dim3(kThreads), smem, L.stream, cluster, bt, P);
 }
