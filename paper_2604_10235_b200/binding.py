@@ -9,6 +9,8 @@ missing or a call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import math
 import os
 from typing import Optional, Sequence
@@ -63,11 +65,17 @@ class cc_layer_desc(C.Structure):
 
 
 _LIB = None
+_CALL = None          # the extension's call(fn, spec, *args): see csrc/py_call.cpp
+# arguments of the entry points that are called through it, after the context and the descriptor
+_SPEC = {"cc_score_window": b"iittttwi", "cc_fuse_prior_pool": b"iittti", "cc_topk_select": b"iittttwi",
+         "cc_topk_select_static": b"iitttti", "cc_compact_kv": b"iippttttti",
+         "cc_compress_layer": b"iittptttttttwi", "cc_compress_layers": b"iiiLLLtLLLLLLwi",
+         "cc_ppl_chunk_scores": b"itiiiiiittti", "cc_select_chunks": b"itiiti"}
 
 
 def load_library(path: Optional[str] = None) -> C.CDLL:
     """Loads (building first if the sources are newer) the in-tree shared library."""
-    global _LIB
+    global _LIB, _CALL
     if _LIB is not None and path is None:
         return _LIB
     if path is None:
@@ -76,7 +84,7 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
             try:
                 _build.build()
             except Exception as exc:                      # no nvcc: a stale library is still usable
-                if not os.path.exists(path):
+                if not os.path.exists(path) or not os.path.exists(_build.CALL_PATH):
                     raise RuntimeError(f"libcodecomp.so is missing and cannot be built: {exc}")
     lib = C.CDLL(path)
     vp, i32, sz = C.c_void_p, C.c_int32, C.c_size_t
@@ -109,6 +117,12 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     for name in EXPORTS:
         if name not in ("cc_status_string", "cc_last_error", "cc_workspace_bytes"):
             getattr(lib, name).restype = C.c_int
+    lib.addresses = {name: C.cast(getattr(lib, name), vp).value for name in _SPEC}
+    if _CALL is None:
+        loader = importlib.machinery.ExtensionFileLoader("_cccall", _build.CALL_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_cccall", loader))
+        loader.exec_module(module)
+        _CALL = module.call
     if path == _build.LIB_PATH:
         _LIB = lib
     return lib
@@ -133,6 +147,12 @@ class Context:
         if rc != CC_OK:
             raise CodecompError(rc, self.lib.cc_status_string(rc).decode())
         self.handle = h
+
+    def call(self, name: str, desc: "Desc", *args) -> None:
+        """Calls entry point ``name`` with this context, the descriptor and the arguments."""
+        rc = _CALL(self.lib.addresses[name], _SPEC[name], self.handle.value, C.addressof(desc.c), *args)
+        if rc:
+            self.check(rc)
 
     def close(self) -> None:
         if getattr(self, "handle", None):
@@ -239,40 +259,37 @@ class Desc:
         return sum((n + ch - 1) // ch for n in self.lens)
 
 
-def _stream(stream: Optional[int]) -> C.c_void_p:
+def _raw(stream: Optional[int]) -> int:
+    """The stream as an integer; None is torch's current stream."""
     if stream is None:
-        stream = torch.cuda.current_stream().cuda_stream
-    return C.c_void_p(stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream
 
 
-def _ptr(t: Optional[torch.Tensor], pinned_ok: bool = False) -> C.c_void_p:
-    """Address of a CUDA tensor; with ``pinned_ok`` also of a page-locked host tensor (its address
-    is valid on the device: the V rows of a compaction may be gathered straight from it)."""
+def _stream(stream: Optional[int]) -> C.c_void_p:
+    return C.c_void_p(_raw(stream))
+
+
+def _ptr(t: Optional[torch.Tensor]) -> C.c_void_p:
     if t is None:
         return C.c_void_p(0)
-    if not t.is_cuda and not (pinned_ok and t.is_pinned()):
-        raise ValueError("libcodecomp takes CUDA tensors only" +
-                         (" (or page-locked host memory here)" if pinned_ok else ""))
+    if not t.is_cuda:
+        raise ValueError("libcodecomp takes CUDA tensors only")
     return C.c_void_p(t.data_ptr())
 
 
 def cc_score_window(ctx: Context, desc: Desc, q_win, k, scores, lse=None, ws=None, stream=None):
     ws = ctx.workspace(desc) if ws is None else ws
-    ctx.check(ctx.lib.cc_score_window(ctx.handle, C.byref(desc.c), _ptr(q_win), _ptr(k),
-                                      _ptr(scores), _ptr(lse), _ptr(ws), ws.numel(),
-                                      _stream(stream)))
+    ctx.call("cc_score_window", desc, q_win, k, scores, lse, ws, _raw(stream))
 
 
 def cc_fuse_prior_pool(ctx: Context, desc: Desc, scores, prior, fused, stream=None):
-    ctx.check(ctx.lib.cc_fuse_prior_pool(ctx.handle, C.byref(desc.c), _ptr(scores), _ptr(prior),
-                                         _ptr(fused), _stream(stream)))
+    ctx.call("cc_fuse_prior_pool", desc, scores, prior, fused, _raw(stream))
 
 
 def cc_topk_select(ctx: Context, desc: Desc, fused, prior, idx, count, ws=None, stream=None):
     ws = ctx.workspace(desc) if ws is None else ws
-    ctx.check(ctx.lib.cc_topk_select(ctx.handle, C.byref(desc.c), _ptr(fused), _ptr(prior),
-                                     _ptr(idx), _ptr(count), _ptr(ws), ws.numel(),
-                                     _stream(stream)))
+    ctx.call("cc_topk_select", desc, fused, prior, idx, count, ws, _raw(stream))
 
 
 def cc_topk_select_static(ctx: Context, desc: Desc, fused, prior, idx, count, stream=None):
@@ -281,15 +298,13 @@ def cc_topk_select_static(ctx: Context, desc: Desc, fused, prior, idx, count, st
     (CC_STATIC_SELECT_MAX_ITEMS bytes per GPU, shared by every call, so overlapping calls must
     be ordered by the caller); larger batches raise CodecompError(CC_ERR_UNSUPPORTED).  The
     first call on a device resolves the array's address and belongs outside stream capture."""
-    ctx.check(ctx.lib.cc_topk_select_static(ctx.handle, C.byref(desc.c), _ptr(fused), _ptr(prior),
-                                            _ptr(idx), _ptr(count), _stream(stream)))
+    ctx.call("cc_topk_select_static", desc, fused, prior, idx, count, _raw(stream))
 
 
 def cc_compact_kv(ctx: Context, desc: Desc, k, v, idx, k_out, v_out, free_pages=None,
                   out_page_table=None, stream=None):
-    ctx.check(ctx.lib.cc_compact_kv(ctx.handle, C.byref(desc.c), _ptr(k, True), _ptr(v, True), _ptr(idx),
-                                    _ptr(k_out), _ptr(v_out), _ptr(free_pages),
-                                    _ptr(out_page_table), _stream(stream)))
+    """k and v may be page-locked host tensors (their addresses are valid on the device)."""
+    ctx.call("cc_compact_kv", desc, k, v, idx, k_out, v_out, free_pages, out_page_table, _raw(stream))
 
 
 def cc_structural_score(ctx: Context, desc: Desc, idx, prior, threshold: float, score,
@@ -305,14 +320,17 @@ def cc_ppl_chunk_scores(ctx: Context, logits: torch.Tensor, targets: torch.Tenso
     chunks, t, v = logits.shape
     assert logits.stride(2) == 1
     dtype = CC_F32 if logits.dtype == torch.float32 else CC_BF16
-    ctx.check(ctx.lib.cc_ppl_chunk_scores(ctx.handle, _ptr(logits), dtype, chunks, t, v,
-                                          logits.stride(0), logits.stride(1), _ptr(targets),
-                                          _ptr(nll), _ptr(score), _stream(stream)))
+    rc = _CALL(ctx.lib.addresses["cc_ppl_chunk_scores"], _SPEC["cc_ppl_chunk_scores"], ctx.handle.value, logits,
+               dtype, chunks, t, v, logits.stride(0), logits.stride(1), targets, nll, score, _raw(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def cc_select_chunks(ctx: Context, score: torch.Tensor, k: int, chosen: torch.Tensor, stream=None):
-    ctx.check(ctx.lib.cc_select_chunks(ctx.handle, _ptr(score), score.numel(), k, _ptr(chosen),
-                                       _stream(stream)))
+    rc = _CALL(ctx.lib.addresses["cc_select_chunks"], _SPEC["cc_select_chunks"], ctx.handle.value, score,
+               score.numel(), k, chosen, _raw(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def _host(a: np.ndarray):
@@ -358,10 +376,8 @@ def cc_select_spans(starts, ends, scores, protected, n: int, budget: int, span_r
 def cc_compress_layer(ctx: Context, desc: Desc, q_win, k, v, prior, k_out, v_out, idx, count,
                       free_pages=None, out_page_table=None, ws=None, stream=None):
     ws = ctx.workspace(desc) if ws is None else ws
-    ctx.check(ctx.lib.cc_compress_layer(ctx.handle, C.byref(desc.c), _ptr(q_win), _ptr(k), _ptr(v, True),
-                                        _ptr(prior), _ptr(k_out), _ptr(v_out), _ptr(idx),
-                                        _ptr(count), _ptr(free_pages), _ptr(out_page_table),
-                                        _ptr(ws), ws.numel(), _stream(stream)))
+    ctx.call("cc_compress_layer", desc, q_win, k, v, prior, k_out, v_out, idx, count, free_pages,
+             out_page_table, ws, _raw(stream))
 
 
 def cc_exp_rate_probe(ctx: Context, from_tmem: bool, iters: int = 4000, stream=None) -> float:
@@ -372,24 +388,13 @@ def cc_exp_rate_probe(ctx: Context, from_tmem: bool, iters: int = 4000, stream=N
     return float(rate.value)
 
 
-def _ptr_array(tensors):
-    """Host array of the device pointers of a list of tensors (None -> NULL array)."""
-    if tensors is None:
-        return None
-    arr = (C.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
-    return arr
-
-
 def cc_compress_layers(ctx: Context, desc: Desc, q_win, k, v, prior, k_out, v_out, idx, count,
                        free_pages=None, out_page_table=None, ws=None, stream=None):
     """cc_compress_layer for a list of layers in one call: every tensor argument except ``prior``
     and ``ws`` is a list with one tensor per layer."""
     ws = ctx.workspace(desc) if ws is None else ws
-    n = len(k)
-    arrays = [_ptr_array(x) for x in (q_win, k, v)]
-    outs = [_ptr_array(x) for x in (k_out, v_out, idx, count, free_pages, out_page_table)]
-    ctx.check(ctx.lib.cc_compress_layers(ctx.handle, C.byref(desc.c), n, *arrays, _ptr(prior), *outs,
-                                         _ptr(ws), ws.numel(), _stream(stream)))
+    ctx.call("cc_compress_layers", desc, len(k), q_win, k, v, prior, k_out, v_out, idx, count, free_pages,
+             out_page_table, ws, _raw(stream))
 
 
 def cc_workspace_views(ctx: Context, desc: Desc, ws: torch.Tensor):

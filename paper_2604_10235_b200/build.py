@@ -1,16 +1,18 @@
-"""Builds libcodecomp.so (sm_100a) from csrc/ with nvcc, in-tree."""
+"""Builds libcodecomp.so (sm_100a) and the extension that calls it from Python, in-tree, with nvcc."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB_DIR = os.path.join(HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libcodecomp.so")
+CALL_PATH = os.path.join(LIB_DIR, "_cccall.so")        # Python extension that marshals the calls
 SOURCES = ["api.cu", "score_simt.cu", "score_tc.cu", "fuse_pool.cu", "select.cu", "select_cluster.cu", "compact.cu",
            "str_score.cu", "planner.cu", "ppl.cu", "exp_probe.cu"]
 
@@ -23,9 +25,9 @@ def nvcc_path() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(CALL_PATH):
         return True
-    built = os.path.getmtime(LIB_PATH)
+    built = min(os.path.getmtime(LIB_PATH), os.path.getmtime(CALL_PATH))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps.append(os.path.join(ROOT, "include", "codecomp.h"))
     return any(os.path.getmtime(d) > built for d in deps)
@@ -44,7 +46,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
               "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if verbose:
         common += ["-Xptxas", "-v"]
-    procs = []
+    call = [nvcc, "-shared", "-cudart", "none", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
+            "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "py_call.cpp"), "-o", CALL_PATH]
+    procs = [("py_call.cpp", subprocess.Popen(call, stdout=subprocess.PIPE, stderr=subprocess.STDOUT,
+                                              text=True))]
     objs = []
     for src in SOURCES:
         obj = os.path.join(obj_dir, src.replace(".cu", ".o"))
