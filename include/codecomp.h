@@ -210,8 +210,9 @@ int cc_compress_layer(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win,
  * v_out, idx, count (and, for the paged layout, free_pages and out_page_table; NULL otherwise)
  * are HOST arrays of n_layers device pointers, entry l being what cc_compress_layer takes for
  * layer l.  The descriptor is checked and the workspace carved once; the layers share the
- * workspace (they run one after the other on the stream), so the intermediates left in it are
- * those of the last layer.  Results are those of n_layers separate calls, bit for bit. */
+ * workspace, and the intermediates left where cc_workspace_views finds them are those of the last
+ * layer.  Results are those of n_layers separate calls; short layers run several to a launch, where
+ * the sums of a row's softmax may be added up in another order (last place of an f32 score). */
 int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
                        const void* const* q_win, const void* const* k, const void* const* v,
                        const float* prior, void* const* k_out, void* const* v_out,

@@ -118,6 +118,18 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
   return ok;
 }
+// Up to 64 probes in a short loop (a suspended thread is woken by every arrival in the CTA,
+// whatever the barrier, so waiting threads go round often); whether the phase completed.
+__device__ __forceinline__ bool mbar_spin(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\tmov.u32 n, 64;\n"
+      "W%=:\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "@p bra D%=;\n\tsub.u32 n, n, 1;\n\tsetp.ne.u32 q, n, 0;\n\t@q bra W%=;\n"
+      "D%=:\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -165,6 +177,18 @@ __device__ __forceinline__ void tc_fence_after() {
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                ::"r"(bar) : "memory");
+}
+// One lane of the warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t yes;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(yes));
+  return yes != 0;
+}
+__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
@@ -239,23 +263,131 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-__device__ __noinline__ bool wait_bar(const Pipe& p, uint64_t* bar, uint32_t parity, int where) {
+// Every lane of the warp waits; the answer is the same in all of them.
+__device__ __forceinline__ bool warp_wait(const Pipe& p, uint64_t* bar, uint32_t parity, int where) {
   const uint32_t b = smem_u32(bar);
-  for (int i = 0; i < 64; ++i)
-    if (mbar_try_wait(b, parity)) return true;
-  const unsigned long long t0 = global_ns();
+  if (__all_sync(0xffffffffu, mbar_try_wait(b, parity))) return true;
+  unsigned long long t0 = 0;
   for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 8; ++i) {
-      if (mbar_try_wait(b, parity)) return true;
-      __nanosleep(200);
-    }
-    if (p.misc->abort_flag) return false;
-    if (global_ns() - t0 > 50ull * 1000 * 1000) break;
+    if (__all_sync(0xffffffffu, mbar_spin(b, parity))) return true;
+    if (__any_sync(0xffffffffu, p.misc->abort_flag)) return false;
+    const unsigned long long now = global_ns();
+    if (t0 == 0) t0 = now;
+    if (__any_sync(0xffffffffu, now - t0 > 50ull * 1000 * 1000)) break;
   }
   p.misc->abort_flag = 1;
-  report_error(p.status, CC_ERR_TIMEOUT, where);
+  if ((threadIdx.x & 31) == 0) report_error(p.status, CC_ERR_TIMEOUT, where);
+  __syncwarp();
   return false;
+}
+
+// ------------------------------------------------------------------ the four drains
+// One accumulator buffer through a warp, 32 columns at a time.  The common forms and the masked ones
+// are loops of their own, so that the common ones hold no range tests and no moves of values that
+// only the others overwrite.  Bound by the exponentials and the issue slots around them: 14.9
+// (pass 1) and 13.5 (pass 2) exponentials per clock per SM on a large batch, against 18.5 for
+// this loop alone; 189 instructions per chunk over all warps of the CTA (227 before).
+__device__ __forceinline__ void hand_back(uint32_t empty_bar, int lane) {
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(empty_bar);
+}
+
+// pass 1, all 128 keys count.  The reference of the exponentials only has to be near the row
+// maximum, not equal to it: it is replaced when a value lies more than 2^64 above it.
+__device__ __forceinline__ void drain_keys(uint32_t addr, uint32_t empty_bar, int lane, float c, uint64_t c2,
+                                           float& m_run, float& l_run) {
+  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
+  for (int cc0 = 0; cc0 < kTileKeys; cc0 += 32) {
+    uint32_t v[32];
+    tmem_ld32(addr + (uint32_t)cc0, v);
+    tmem_wait_ld();
+    if (cc0 + 32 == kTileKeys) hand_back(empty_bar, lane);
+    const float mx = max32(v) * c;
+    const bool renew = m_run == -INFINITY || mx > m_run + 64.0f;
+    if (__any_sync(0xffffffffu, renew)) {
+      if (renew) {
+        if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
+        acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
+        m_run = mx;
+      }
+    }
+    exp_accumulate<false, 32>(v, c2, pack2(-m_run, -m_run), 0u, acc);
+  }
+  l_run += acc_total(acc);
+}
+
+// pass 1, keys from valid_r on (a bound of the thread's own) do not count
+// (returns the row's new reference and sum)
+__device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empty_bar, int lane, float c, int valid_r,
+                                                 float m_run, float l_run) {
+  const uint64_t c2 = pack2(c, c);
+  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
+  for (int cc0 = 0; cc0 < kTileKeys; cc0 += 32) {
+    uint32_t v[32];
+    __syncwarp();                       // the rows of a warp skip different chunks
+    tmem_ld32(addr + (uint32_t)cc0, v);
+    tmem_wait_ld();
+    if (cc0 + 32 == kTileKeys) hand_back(empty_bar, lane);
+    if (cc0 >= valid_r) continue;
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
+    const float mx = max32(v) * c;
+    if (m_run == -INFINITY || mx > m_run + 64.0f) {
+      if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
+      acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
+      m_run = mx;
+    }
+    exp_accumulate<false, 32>(v, c2, pack2(-m_run, -m_run), 0u, acc);
+  }
+  return make_float2(m_run, l_run + acc_total(acc));
+}
+
+// pass 2: nc columns (a multiple of 16), -L_r of the first at shared-space address nl
+__device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, int lane, uint64_t c2, uint32_t nl,
+                                            int nc) {
+  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
+  for (int cc0 = 0; cc0 + 32 <= nc; cc0 += 32) {
+    uint32_t v[32];
+    tmem_ld32(addr + (uint32_t)cc0, v);               // stays inside the 128-column buffer
+    tmem_wait_ld();
+    if (cc0 + 32 == nc) hand_back(empty_bar, lane);
+    exp_accumulate<true, 32>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
+  }
+  if (nc & 16) {
+    uint32_t v[32];
+    tmem_ld32(addr + (uint32_t)(nc - 16), v);
+    tmem_wait_ld();
+    hand_back(empty_bar, lane);
+    exp_accumulate<true, 16>(v, c2, 0ull, nl + 4u * (uint32_t)(nc - 16), acc);
+  }
+  return acc_total(acc);
+}
+
+// pass 2, columns before first_col (a bound of the thread's own) do not count
+// (returns the sum)
+__device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty_bar, int lane, float c, uint32_t nl,
+                                                int nc, int first_col) {
+  const uint64_t c2 = pack2(c, c);
+  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
+  for (int cc0 = 0; cc0 < nc; cc0 += 32) {
+    uint32_t v[32];
+    __syncwarp();
+    tmem_ld32(addr + (uint32_t)cc0, v);
+    tmem_wait_ld();
+    if (cc0 + 32 >= nc) hand_back(empty_bar, lane);
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (cc0 + i < first_col) v[i] = 0xc61c4000u;     // -1e4: exponential ~ 0
+    if (cc0 + 32 <= nc) exp_accumulate<true, 32>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
+    else                exp_accumulate<true, 16>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
+  }
+  return acc_total(acc);
 }
 
 // Walks the tiles of a CTA's span in (sequence, head, tile) order.
@@ -308,7 +440,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   Misc* misc = reinterpret_cast<Misc*>(k_smem + (size_t)P.n_stages * kStageBytes);
   Pipe pipe{misc, status};
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the warp index as a value the compiler knows to be the same in all lanes: the MMA issuer's
+  // descriptors then live in uniform registers
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int t_begin = span_begin(blockIdx.x, P), t_end = span_begin(blockIdx.x + 1, P);
 
   if (threadIdx.x == 32) {
@@ -341,7 +475,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = misc->tmem_base;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, misc->tmem_base, 0);
   // Pass 1 reads Q and K, which the launch before it in the stream may have produced: every
   // thread waits for that launch, and only then lets pass 2 be scheduled, so that whatever runs
   // after pass 1 has begun finds the caller's inputs complete.  The launch before pass 2 is
@@ -355,13 +489,13 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
 
   if (warp == 0) {
     // ================================================================ TMA producer
-    // The whole warp walks the tile list; lane 0 waits and issues the copies of contiguous K.
-    // With a paged cache every lane owns one page of the tile: it reads the page id (before the
-    // wait for the stage, so the load is covered), checks it and issues the two copies of its
-    // page, so the page-table look-ups of a tile are one parallel load instead of a chain.
+    // The whole warp walks the tile list; one lane issues the copies.  With a paged cache every
+    // lane reads and checks the id of one page of the tile (before the wait for the stage, so the
+    // load is covered): the page-table look-ups of a tile are one parallel load, not a chain.
     {
       TileCursor cur;
       cur.locate(bt, g.hkv, t_begin);
+      const bool elected = elect_one();
       int stage = 0, cur_problem = -1;
       uint32_t phase = 0, qe_phase = 0;
       const int ps = bt.page_size;
@@ -375,12 +509,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         const CUtensorMap* k_map = &M.k[layer];
         if (cur.problem(g.hkv) != cur_problem) {
           if (cur_problem >= 0) {
-            const bool got = lane != 0 || wait_bar(pipe, &misc->bar.q_empty, qe_phase, 10);
-            if (!__all_sync(0xffffffffu, got)) break;
+            if (!warp_wait(pipe, &misc->bar.q_empty, qe_phase, 10)) break;
             qe_phase ^= 1;
           }
           cur_problem = cur.problem(g.hkv);
-          if (lane == 0) {
+          if (elected) {
             const uint32_t qb = smem_u32(&misc->bar.q_full);
             mbar_expect_tx(qb, q_bytes);
             tma_load_4d(smem_u32(q_smem), q_map, qb, 0, cur.h * g.group, 0, sq.src);
@@ -395,14 +528,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           mine = lane < (valid + ps - 1) / ps;
           if (mine) page_id = g.page_table[(int64_t)sq.src * g.page_table_stride + key0 / ps + lane];
         }
-        {
-          const bool got = lane != 0 || wait_bar(pipe, &misc->bar.empty[stage], phase ^ 1, 11);
-          if (!__all_sync(0xffffffffu, got)) break;
-        }
+        if (!warp_wait(pipe, &misc->bar.empty[stage], phase ^ 1, 11)) break;
         const uint32_t fb = smem_u32(&misc->bar.full[stage]);
         const uint32_t dst = smem_u32(k_smem) + (uint32_t)stage * kStageBytes;
         if (ps == 0) {
-          if (lane == 0) {
+          if (elected) {
             mbar_expect_tx(fb, kStageBytes);
             tma_load_3d_hint(dst, k_map, fb, 0, cur.h, sq.tok_off + key0, k_policy);
             tma_load_3d_hint(dst + kPanelBytes, k_map, fb, 64, cur.h, sq.tok_off + key0, k_policy);
@@ -411,27 +541,33 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           const bool good = mine && page_id >= 0 && ((int64_t)page_id + 1) * ps <= P.pool_rows;
           if (mine && !good) report_error(status, CC_ERR_DEVICE_FLAG, 12);
           const unsigned good_mask = __ballot_sync(0xffffffffu, good);
-          // the stage completes when the bytes of the good pages have landed; the expectation is
-          // registered before any lane issues a copy
-          if (lane == 0) mbar_expect_tx(fb, (uint32_t)__popc(good_mask) * (uint32_t)ps * 256u);
-          __syncwarp();
-          if (good)      // the page's rows, both panels, in one copy
-            tma_load_5d_hint(dst + (uint32_t)lane * (uint32_t)ps * 256u, k_map, fb,
-                             page_id * (ps >> 3), cur.h, k_policy);
+          // the stage completes when the bytes of the good pages have landed; one lane issues the
+          // copies, so that their operands are uniform
+          if (elected) mbar_expect_tx(fb, (uint32_t)__popc(good_mask) * (uint32_t)ps * 256u);
+          for (unsigned left = good_mask; left; left &= left - 1) {
+            const int p = __ffs(left) - 1;
+            const int id = __shfl_sync(0xffffffffu, page_id, p);
+            if (elected)       // the page's rows, both panels, in one copy
+              tma_load_5d_hint(dst + (uint32_t)p * (uint32_t)ps * 256u, k_map, fb, id * (ps >> 3), cur.h, k_policy);
+          }
         }
         if (++stage == P.n_stages) { stage = 0; phase ^= 1; }
       }
     }
   } else if (warp == 1 || (kIssuers == 2 && warp == kMmaWarpB)) {
     // ================================================================ MMA issuers
-    // The serial instruction stream of a thread that issues tcgen05.mma (waits, descriptor
-    // words, eight multiplications and a commit per item) is long, so there are two issuers;
-    // items go to them in pairs (0, 1 -> first; 2, 3 -> second; ...); both wait for every K
-    // tile and both hand it back.  Descriptors are formed by adding small constants
-    // to a base word, the accumulate flag is a compile-time predicate, and the tile bookkeeping
-    // is a countdown instead of a cursor walk.
+    // The whole warp walks the items and waits; one elected lane issues the multiplications.  With
+    // all of it inside `if (lane == 0)` the compiler cannot know that the operands of tcgen05.mma
+    // (uniform registers) are the same in all lanes and wraps each one in a loop over the lanes:
+    // that was 30 of the 227 instructions the SM issued per 32-column chunk of a warp, and as long
+    // a serial stream between a buffer's return and its refill (llama3_8b shape, both passes:
+    // 52.1 -> 49.4 us together with the waits and the single issuing lane of the K copies).
+    // Two issuers still refill a little sooner than one (chunk batch 190 against 194 us); items go
+    // to them in pairs (0, 1 -> first; 2, 3 -> second; ...); both wait for every K tile and both
+    // hand it back.  Descriptors are formed by adding small constants to a base word, and the tile
+    // bookkeeping is a countdown instead of a cursor walk.
     const int my_half = warp == 1 ? 0 : 1;
-    if (lane == 0) {
+    {
       TileCursor cur;
       cur.locate(bt, g.hkv, t_begin);
       int left = cur.n_tiles - cur.local;          // tiles of the current (sequence, head) still to do
@@ -452,19 +588,17 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       const uint32_t idesc_last =
           PASS == 1 ? idesc_full
                     : instr_desc(128, (uint32_t)(P.rows_pad - (P.n_sub - 1) * P.sub_cols));
-      const uint32_t full0 = smem_u32(&misc->bar.full[0]), empty0 = smem_u32(&misc->bar.empty[0]);
+      const uint32_t empty0 = smem_u32(&misc->bar.empty[0]);
       const uint32_t accf0 = smem_u32(&misc->bar.acc_full[0]);
-      const uint32_t acce0 = smem_u32(&misc->bar.acc_empty[0]);
+      const bool elected = elect_one();
       bool ok = true;
       for (int t = t_begin; t < t_end && ok; ++t) {
         if (need_q) {
-          if (!wait_bar(pipe, &misc->bar.q_full, qf_phase, 20)) break;
+          if (!warp_wait(pipe, &misc->bar.q_full, qf_phase, 20)) break;
           qf_phase ^= 1;
           need_q = false;
         }
-        if (!mbar_try_wait(full0 + 8u * (uint32_t)stage, phase) &&
-            !wait_bar(pipe, &misc->bar.full[stage], phase, 21))
-          break;
+        if (!warp_wait(pipe, &misc->bar.full[stage], phase, 21)) break;
         tc_fence_after();
         const uint32_t k_lo = k_lo0 + (uint32_t)stage * (kStageBytes >> 4);
 #pragma unroll 1
@@ -472,8 +606,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           if (kIssuers == 2 && (int)((item >> 1) & 1u) != my_half) continue;
           const uint32_t buf = item & (kBufs - 1);
           const uint32_t par = ((item >> 2) & 1u) ^ 1u;
-          if (!mbar_try_wait(acce0 + 8u * buf, par) &&
-              !wait_bar(pipe, &misc->bar.acc_empty[buf], par, 22)) {
+          if (!warp_wait(pipe, &misc->bar.acc_empty[buf], par, 22)) {
             ok = false;
             break;
           }
@@ -481,34 +614,24 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           const uint32_t d_tmem = tmem_base + buf * kBufCols;
           const uint32_t idesc = sub == P.n_sub - 1 ? idesc_last : idesc_full;
           const uint32_t q_lo = q_lo0 + (uint32_t)sub * q_step16;
+          if (elected) {
 #pragma unroll
-          for (int ks = 0; ks < kHeadDim / 16; ++ks) {
-            const uint32_t ql = q_lo + (ks >= 4 ? q_panel16 : 0u) + (uint32_t)(ks & 3) * 2u;
-            const uint32_t kl = k_lo + (ks >= 4 ? P.k_panel16 : 0u) + (uint32_t)(ks & 3) * 2u;
-            const uint32_t al = PASS == 1 ? ql : kl, bl = PASS == 1 ? kl : ql;
-            if (ks == 0) {
-              asm volatile(
-                  "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, 0, 0;\n\t"
-                  "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %5};\n\t"
-                  "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
-                  ::"r"(d_tmem), "r"(al), "r"(bl), "r"(a_hi), "r"(idesc), "r"(b_hi) : "memory");
-            } else {
-              asm volatile(
-                  "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.eq.b32 p, 0, 0;\n\t"
-                  "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %5};\n\t"
-                  "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
-                  ::"r"(d_tmem), "r"(al), "r"(bl), "r"(a_hi), "r"(idesc), "r"(b_hi) : "memory");
+            for (int ks = 0; ks < kHeadDim / 16; ++ks) {
+              const uint32_t ql = q_lo + (ks >= 4 ? q_panel16 : 0u) + (uint32_t)(ks & 3) * 2u;
+              const uint32_t kl = k_lo + (ks >= 4 ? P.k_panel16 : 0u) + (uint32_t)(ks & 3) * 2u;
+              const uint64_t al = PASS == 1 ? ql : kl, bl = PASS == 1 ? kl : ql;
+              umma(d_tmem, al | ((uint64_t)a_hi << 32), bl | ((uint64_t)b_hi << 32), idesc, ks > 0);
             }
+            umma_commit(accf0 + 8u * buf);
           }
-          umma_commit(accf0 + 8u * buf);
         }
         if (!ok) break;
-        umma_commit(empty0 + 8u * (uint32_t)stage);
+        if (elected) umma_commit(empty0 + 8u * (uint32_t)stage);
         if (++stage == P.n_stages) { stage = 0; phase ^= 1; }
         if (--left == 0 && t + 1 < t_end) {
           // the next tile belongs to another (sequence, head): Q may be replaced once the
           // multiplications issued so far have read it
-          umma_commit(smem_u32(&misc->bar.q_empty));
+          if (elected) umma_commit(smem_u32(&misc->bar.q_empty));
           cur.local = cur.n_tiles - 1;
           cur.advance(bt, g.hkv);
           left = cur.n_tiles;
@@ -657,18 +780,14 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       const int key0 = (t - first_tile) * kTileKeys;
       const int valid = min(kTileKeys, n_cur - key0);
       if (!dead) {
-        // every lane probes once; only when the buffer is not full yet does one lane wait
-        if (!__all_sync(0xffffffffu, mbar_try_wait(full_bar, par))) {
-          const bool got = lane != 0 || wait_bar(pipe, &misc->bar.acc_full[set], par, 30);
-          dead = !__all_sync(0xffffffffu, got);
-        }
+        dead = !warp_wait(pipe, &misc->bar.acc_full[set], par, 30);
       }
       par ^= 1u;
       float u_acc = 0.f;
       if (!dead) {
         tc_fence_after();
-        uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-        uint32_t v[32];
+        const bool edge = PASS == 1 ? valid < kTileKeys || (CAUSAL && key0 + kTileKeys > n_cur - g.window + 1)
+                                    : CAUSAL && key0 + kTileKeys > n_cur - g.window + 1;
         if (PASS == 1) {
           // thread = query row (sub * 128 + row_in_tile); columns = the 128 keys of the tile
           float m_run = run_m[0], l_run = run_l[0];
@@ -676,58 +795,20 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
 #pragma unroll
             for (int rb = 1; rb < 4; ++rb) if (rb == sub) { m_run = run_m[rb]; l_run = run_l[rb]; }
           }
-          // keys of the tile this row attends to: all valid ones, or (causal window) those up
-          // to the row's own position n - w + t
-          // (the masked form is a copy of the loop of its own, so that the common one stays lean)
-          const bool masked_tile = CAUSAL && key0 + kTileKeys > n_cur - g.window + 1;
-          auto drain = [&](auto masked) {
-          constexpr bool kMasked = decltype(masked)::value;
-          // a warp whose 32 rows all lie past the padded window (last row block of a row count
-          // that is not a multiple of 128) has nothing to sum: it only hands the buffer back
-          int valid_r = sub * 128 + quad * 32 >= P.rows_pad ? 0 : valid;
-          if (kMasked) {
-            const int t_row = (sub * 128 + row_in_tile) / g.group;
-            if (t_row < g.window) valid_r = min(valid, n_cur - g.window + t_row + 1 - key0);
+          if (!edge) {
+            drain_keys(acc_addr, empty_bar, lane, c, c2, m_run, l_run);
+          } else {
+            // keys of the tile this row attends to: the valid ones, or (causal window) those up to the
+            // row's own position n - w + t
+            int valid_r = valid;
+            if (CAUSAL) {
+              const int t_row = (sub * 128 + row_in_tile) / g.group;
+              if (t_row < g.window) valid_r = min(valid, n_cur - g.window + t_row + 1 - key0);
+            }
+            const float2 st = drain_keys_masked(acc_addr, empty_bar, lane, c, valid_r, m_run, l_run);
+            m_run = st.x;
+            l_run = st.y;
           }
-          // all 128 keys of the tile count for every row of the warp: no per-chunk range tests
-          const bool full_tile = !kMasked && __shfl_sync(0xffffffffu, valid_r, 0) == kTileKeys;
-#pragma unroll 1
-          for (int cc0 = 0; cc0 < kTileKeys; cc0 += 32) {
-            if (kMasked) __syncwarp();            // rows of a masked tile skip different chunks
-            tmem_ld32(acc_addr + (uint32_t)cc0, v);
-            tmem_wait_ld();
-            if (cc0 + 32 == kTileKeys) {             // last read of the buffer: hand it back
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(empty_bar);
-            }
-            if (!full_tile) {
-              if (cc0 >= valid_r) continue;
-              if (cc0 + 32 > valid_r) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
-              }
-            }
-            // The reference of the exponentials only has to be near the row maximum, not equal
-            // to it: it is replaced when a value lies more than 2^64 above it.  The test is a
-            // warp vote where the warp is converged, so that the common case is one uniform branch.
-            const float mx = max32(v) * c;
-            const bool renew = m_run == -INFINITY || mx > m_run + 64.0f;
-            // (the rows of a masked tile skip different chunks, so its lanes are not converged
-            // here and must not vote; everywhere else the warp takes this path as one)
-            if (kMasked ? renew : __any_sync(0xffffffffu, renew)) {
-              if (renew) {
-                if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
-                acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
-                m_run = mx;
-              }
-            }
-            exp_accumulate<false, 32>(v, c2, pack2(-m_run, -m_run), 0u, acc);
-          }
-          };
-          if (CAUSAL && masked_tile) drain(std::true_type{}); else drain(std::false_type{});
-          l_run += acc_total(acc);
           if (rotating) {
 #pragma unroll
             for (int rb = 0; rb < 4; ++rb) if (rb == sub) { run_m[rb] = m_run; run_l[rb] = l_run; }
@@ -740,33 +821,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           const int c0 = sub * P.sub_cols;
           const int nc = min(P.sub_cols, P.rows_pad - c0);        // multiple of 16
           const uint32_t nl = smem_u32(misc->neg_lc + c0);         // -L_r of the item's columns
-          // causal window: key j is seen by the rows t >= j - (n - w), i.e. by the columns
-          // from G * (j - n + w) on; the columns before it contribute nothing
-          const bool masked_tile = CAUSAL && key0 + kTileKeys > n_cur - g.window + 1;
-          auto drain = [&](auto masked) {
-          constexpr bool kMasked = decltype(masked)::value;
-          const int first_col = kMasked ? g.group * (key0 + row_in_tile - n_cur + g.window) : 0;
-#pragma unroll 1
-          for (int cc0 = 0; cc0 < nc; cc0 += 32) {
-            if (kMasked) __syncwarp();
-            tmem_ld32(acc_addr + (uint32_t)cc0, v);               // stays inside the 128-column buffer
-            tmem_wait_ld();
-            if (kMasked && first_col > c0 + cc0) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (c0 + cc0 + i < first_col) v[i] = 0xc61c4000u;   // -1e4: exponential ~ 0
-            }
-            if (cc0 + 32 >= nc) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(empty_bar);
-            }
-            if (cc0 + 32 <= nc) exp_accumulate<true, 32>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
-            else                exp_accumulate<true, 16>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
-          }
-          };
-          if (CAUSAL && masked_tile) drain(std::true_type{}); else drain(std::false_type{});
-          u_acc = acc_total(acc);
+          // causal window: key j is seen by the rows t >= j - (n - w), i.e. by the columns from
+          // G * (j - n + w) on; the columns before it contribute nothing
+          u_acc = edge ? drain_rows_masked(acc_addr, empty_bar, lane, c, nl, nc,
+                                           g.group * (key0 + row_in_tile - n_cur + g.window) - c0)
+                       : drain_rows(acc_addr, empty_bar, lane, c2, nl, nc);
         }
       }
       if (PASS == 2) {
@@ -783,9 +842,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
             if (lane == 0) mbar_arrive(smem_u32(&misc->bar.u_full[slot][quad]));
           } else {
             if (!dead) {
-              const bool got = lane != 0 || wait_bar(pipe, &misc->bar.u_full[slot][quad],
-                                                     (uint32_t)((t - t_begin) >> 3) & 1u, 31);
-              dead = !__all_sync(0xffffffffu, got);
+              dead = !warp_wait(pipe, &misc->bar.u_full[slot][quad], (uint32_t)((t - t_begin) >> 3) & 1u, 31);
             }
             if (!dead && row_in_tile < valid) {
               float u = u_acc;
