@@ -6,18 +6,28 @@
 // output (ascending token indices) are those of select.cu; what differs is where the data
 // lives and how the CTAs cooperate:
 //   * every item is read from global memory once; its order-preserving integer key and its
-//     protected flag stay in shared memory, so the radix descent and the ordered emission never
-//     go back to L2;
-//   * cluster-wide sums, min/max and histograms are exchanged through distributed shared
-//     memory: a CTA publishes into its own buffer, one cluster barrier later every CTA reads all
-//     peers.  Buffers alternate between two copies, which makes one barrier per exchange enough;
-//   * the cut-off is found by an four-step 8-bit radix descent over keys shifted to the range that
-//     is present, and stops early once a bin has to be taken whole;
+//     protected flag stay in shared memory.  A warp owns a run of consecutive items and walks it 32
+//     at a time, so accesses are free of bank conflicts and ordered prefixes are ballots;
+//   * what the CTAs exchange goes through distributed shared memory.  An exchange costs 1 to 2 us
+//     whatever it carries, and at these sizes the kernel's time is mostly a chain of them and of
+//     block barriers, so there are three: (1) protected weight and key range, (2) one histogram of
+//     1024 bins over the range that is present, (3) the keys of the bin that holds the cut-off,
+//     which every CTA then ranks for itself.  A bin usually holds a few dozen keys; one with more
+//     than kCand is looked at again (one value? else a finer histogram).  What the ordered emission
+//     needs to know about the CTAs before it follows from the same three (histograms and
+//     candidates are read per CTA), so no prefix sums are exchanged;
+//   * the passes over all items end with two masks per 32 items, from which the indices are written.
 //   * with FUSED the kernel starts from the raw scores: it pools them (max / avg, or sums them
 //     over a chunk), fuses them with the prior using the same explicitly rounded f32 operations
 //     as fuse_pool.cu, and also stores the fused values.
+// Measured with its launch, replayed alone (four digit rounds of 8 bits with an exchange each, and a
+// contiguous run of items per thread, before): ragged batch of 64 problems, 8 k to 64 k tokens
+// 52.6 -> 28.6 us, 256 problems of 2 k with a cap 19.0 -> 12.6, 32768 tokens x 8 heads 17.3 -> 12.6
+// (7.4 -> 6.4 when the protected tokens fill the budget), 2048 x 2 9.6 -> 6.9.
 #include <cooperative_groups.h>
 #include <string.h>
+
+#include <type_traits>
 
 #include "cc_internal.cuh"
 #include "select_common.cuh"
@@ -28,30 +38,37 @@ namespace cc {
 
 namespace {
 
-constexpr int kThreads = 1024;
-constexpr int kWarps = kThreads / 32;
-constexpr int kDigitBits = 8;
-constexpr int kBins = 1 << kDigitBits;
-constexpr int kCopies = 2;
+constexpr int kBinBits = 10;
+constexpr int kBins = 1 << kBinBits;
+constexpr int kCand = 512;                // candidates of the cut-off bin that are ranked directly
 constexpr int kMaxCluster = 8;
-constexpr int kCtaItems = 32768;          // items one CTA keeps in shared memory
-constexpr int kStagedItems = 16384;       // up to here the raw scores of the slice are staged there too
+constexpr int kMaxWarps = 32;
+constexpr int kCtaItems = 32768;          // items one CTA of 1024 threads keeps in shared memory: 32 per thread
+constexpr int kStep = 4;                  // items a thread pools per part of the slice
+constexpr int kMaxHalf = 32;              // half of the widest pooling window, rounded up
+constexpr int kWords = 6;                 // words of an exchange
 
-struct Shared {
-  unsigned hist[2][kCopies][kBins];
-  unsigned xchg[2][kMaxCluster][4];   // [buffer copy][source CTA][word]: written by the peers
-  unsigned warp_a[kWarps];
-  unsigned warp_b[kWarps];
-  unsigned warp_lo[kWarps], warp_hi[kWarps];
+struct Cand {
+  unsigned key, len;
+};
+
+struct __align__(16) Shared {
+  unsigned hist[2][kBins];                      // alternate between rounds (peers read them)
+  Cand own[kCand];                              // this CTA's candidates (peers read them)
+  Cand all[kCand];                              // the cluster's, in rank order
+  unsigned sub[256];                            // weights of the candidates by their next bits
+  unsigned n_own;
+  unsigned xchg[2][kMaxCluster][kWords];        // [buffer copy][source CTA][word]: written by the peers
+  unsigned warp_x[2][kWords][kMaxWarps];        // block reductions, alternating
   unsigned bcast[4];
 };
 
 struct ClusterParams {
   int cluster;               // CTAs per (sequence, head)
+  int per;                   // steps of 32 items per warp, for the longest sequence
   int hkv;
   float theta;
   // FUSED only
-  int stage_u;               // the slice's raw scores are staged in shared memory before pooling
   int pool_kind, pool_size;
   float alpha, beta;
   const float* prior;
@@ -62,258 +79,376 @@ struct ClusterParams {
   int32_t* count[kMaxLayers];
 };
 
-__host__ __device__ __forceinline__ int padded(int li) { return li + (li >> 5); }
-
-
+template <int THREADS>
 struct Ctx {
+  static constexpr int kWarps = THREADS / 32;
   Shared* sm;
   int C, rank;
-  unsigned phase;          // number of exchanges done so far (selects the buffer copy)
+  unsigned n_xchg, n_red, n_hist;   // exchanges, block reductions, histograms so far (select the copy)
 
   __device__ void sync_all() {
     if (C > 1) cg::this_cluster().sync(); else __syncthreads();
   }
-  __device__ unsigned peer(const unsigned* p, int r) const {
-    if (C == 1) return *p;
-    return *cg::this_cluster().map_shared_rank(const_cast<unsigned*>(p), r);
+  template <class T>
+  __device__ const T* peer(const T* p, int r) const {
+    if (C == 1) return p;
+    return cg::this_cluster().map_shared_rank(const_cast<T*>(p), r);
   }
-
-  // Exchange of up to three words per CTA: threads 0..C-1 each store this CTA's words into one
-  // peer's shared memory (remote stores need no round trip), the cluster barrier publishes them,
-  // and every thread then reads all CTAs' words locally.  Two buffer copies: a CTA writes copy
-  // k & 1 for exchange k only after the barrier of exchange k - 1, which every peer reaches
-  // after it has read exchange k - 2.
-  __device__ unsigned publish(unsigned w0, unsigned w1, unsigned w2) {
-    const unsigned bf = phase++ & 1u;
-    if ((int)threadIdx.x < C) {
-      unsigned* dst = cg::this_cluster().map_shared_rank(&sm->xchg[bf][rank][0], (int)threadIdx.x);
-      dst[0] = w0;
-      dst[1] = w1;
-      dst[2] = w2;
-    }
-    sync_all();
-    return bf;
-  }
-
-  // sum over the block; every thread gets the result
+  // Sum of v over the block.  Two copies of the warp totals: a copy is written again only after
+  // the barrier of the reduction in between, which every warp reaches after it has read it.
   __device__ unsigned block_sum(unsigned v) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v = warp_sum(v);
+    unsigned* w = sm->warp_x[n_red++ & 1u][0];
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) w[warp] = v;
     __syncthreads();
-    if (lane == 0) sm->warp_a[warp] = v;
-    __syncthreads();
-    return warp_sum(sm->warp_a[lane]);
+    return __reduce_add_sync(0xffffffffu, lane < kWarps ? w[lane] : 0u);
   }
-  // sum over all threads of the cluster
-  __device__ unsigned cluster_sum(unsigned v) {
-    v = block_sum(v);
-    if (C == 1) return v;
-    const unsigned b = publish(v, 0u, 0u);
-    unsigned t = 0;
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r)
-      if (r < C) t += sm->xchg[b][r][0];
-    return t;
-  }
-  __device__ void cluster_minmax(unsigned& lo, unsigned& hi) {
+  __device__ void block_sum2(unsigned& a, unsigned& b) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
+    unsigned(*w)[kMaxWarps] = sm->warp_x[n_red++ & 1u];
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    if (lane == 0) { w[0][warp] = a; w[1][warp] = b; }
     __syncthreads();
-    if (lane == 0) { sm->warp_a[warp] = lo; sm->warp_b[warp] = hi; }
-    __syncthreads();
-    lo = sm->warp_a[lane];
-    hi = sm->warp_b[lane];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if (C == 1) return;
-    const unsigned b = publish(lo, hi, 0u);
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) {
-      if (r < C) {
-        lo = min(lo, sm->xchg[b][r][0]);
-        hi = max(hi, sm->xchg[b][r][1]);
-      }
-    }
+    a = __reduce_add_sync(0xffffffffu, lane < kWarps ? w[0][lane] : 0u);
+    b = __reduce_add_sync(0xffffffffu, lane < kWarps ? w[1][lane] : 0u);
   }
-  // exclusive prefix sums over the threads of the block for two counters; tot_* = block totals
-  __device__ void block_scan2(unsigned a, unsigned b, unsigned& ea, unsigned& eb,
-                              unsigned& tot_a, unsigned& tot_b) {
+  // Warp totals a, b (the same in all lanes): sums over the warps before this one.
+  __device__ void warps_before2(unsigned& a, unsigned& b) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned ia = a, ib = b;
+    unsigned(*w)[kMaxWarps] = sm->warp_x[n_red++ & 1u];
+    if (lane == 0) { w[0][warp] = a; w[1][warp] = b; }
+    __syncthreads();
+    a = __reduce_add_sync(0xffffffffu, lane < warp ? w[0][lane] : 0u);
+    b = __reduce_add_sync(0xffffffffu, lane < warp ? w[1][lane] : 0u);
+  }
+  // Sum of a, minimum of b, maximum of e, minimum of d, maximum of f over the block.
+  __device__ void block_totals(unsigned& a, unsigned& b, unsigned& e, unsigned& d, unsigned& f) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned(*w)[kMaxWarps] = sm->warp_x[n_red++ & 1u];
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_min_sync(0xffffffffu, b);
+    e = __reduce_max_sync(0xffffffffu, e);
+    d = __reduce_min_sync(0xffffffffu, d);
+    f = __reduce_max_sync(0xffffffffu, f);
+    if (lane == 0) { w[0][warp] = a; w[1][warp] = b; w[2][warp] = e; w[3][warp] = d; w[4][warp] = f; }
+    __syncthreads();
+    const int i = lane < kWarps ? lane : 0;
+    a = __reduce_add_sync(0xffffffffu, lane < kWarps ? w[0][i] : 0u);
+    b = __reduce_min_sync(0xffffffffu, w[1][i]);
+    e = __reduce_max_sync(0xffffffffu, w[2][i]);
+    d = __reduce_min_sync(0xffffffffu, w[3][i]);
+    f = __reduce_max_sync(0xffffffffu, w[4][i]);
+  }
+  // Exclusive prefix sum over the threads of the block.
+  __device__ unsigned block_scan(unsigned v) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      unsigned ta = __shfl_up_sync(0xffffffffu, ia, o);
-      unsigned tb = __shfl_up_sync(0xffffffffu, ib, o);
-      if (lane >= o) { ia += ta; ib += tb; }
+      const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
     }
+    unsigned* w = sm->warp_x[n_red++ & 1u][0];
+    if (lane == 31) w[warp] = inc;
     __syncthreads();
-    if (lane == 31) { sm->warp_a[warp] = ia; sm->warp_b[warp] = ib; }
-    __syncthreads();
-    const unsigned wa = sm->warp_a[lane], wb = sm->warp_b[lane];
-    unsigned xa = wa, xb = wb;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned ta = __shfl_up_sync(0xffffffffu, xa, o);
-      unsigned tb = __shfl_up_sync(0xffffffffu, xb, o);
-      if (lane >= o) { xa += ta; xb += tb; }
-    }
-    tot_a = __shfl_sync(0xffffffffu, xa, 31);
-    tot_b = __shfl_sync(0xffffffffu, xb, 31);
-    ea = __shfl_sync(0xffffffffu, xa - wa, warp) + ia - a;
-    eb = __shfl_sync(0xffffffffu, xb - wb, warp) + ib - b;
+    return __reduce_add_sync(0xffffffffu, lane < warp ? w[lane] : 0u) + inc - v;
   }
-  // exclusive prefix of one counter over all threads of the cluster, and its cluster total
-  // and, in the same exchange, the cluster-wide minimum of lo and maximum of hi (carried through
-  // the block scan as its second counter's inputs would not do: they are reduced separately)
-  __device__ void cluster_scan_total(unsigned a, unsigned& ea, unsigned& total, unsigned& lo,
-                                     unsigned& hi) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // Words of every CTA to every CTA: thread r < C stores this CTA's into peer r's shared memory
+  // (remote stores need no round trip), the cluster barrier publishes them.  Two buffer copies: a
+  // CTA writes copy k & 1 for exchange k only after the barrier of exchange k - 1, which every
+  // peer reaches after it has read exchange k - 2.
+  __device__ const unsigned (*publish(const unsigned (&w)[kWords]))[kWords] {
+    const unsigned bf = n_xchg++ & 1u;
+    if ((int)threadIdx.x < C) {
+      unsigned* dst = C == 1 ? sm->xchg[bf][0] : cg::this_cluster().map_shared_rank(&sm->xchg[bf][rank][0], (int)threadIdx.x);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      for (int i = 0; i < kWords; ++i) dst[i] = w[i];
     }
-    unsigned *w_lo = sm->warp_lo, *w_hi = sm->warp_hi;
-    if (lane == 0) { w_lo[warp] = lo; w_hi[warp] = hi; }
-    unsigned eb, ta, tb;
-    block_scan2(a, 0u, ea, eb, ta, tb);      // its barriers also publish w_lo / w_hi
-    lo = w_lo[lane];
-    hi = w_hi[lane];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    total = ta;
-    if (C == 1) return;
-    const unsigned bf = publish(ta, lo, hi);
-    total = 0;
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) {
-      if (r < C) {
-        const unsigned v = sm->xchg[bf][r][0];
-        total += v;
-        if (r < rank) ea += v;
-        lo = min(lo, sm->xchg[bf][r][1]);
-        hi = max(hi, sm->xchg[bf][r][2]);
-      }
-    }
-  }
-  // the same over all threads of the cluster (CTA rank major)
-  __device__ void cluster_scan2(unsigned a, unsigned b, unsigned& ea, unsigned& eb) {
-    unsigned ta, tb;
-    block_scan2(a, b, ea, eb, ta, tb);
-    if (C == 1) return;
-    const unsigned bf = publish(ta, tb, 0u);
-#pragma unroll
-    for (int r = 0; r < kMaxCluster - 1; ++r) {
-      if (r < rank) {
-        ea += sm->xchg[bf][r][0];
-        eb += sm->xchg[bf][r][1];
-      }
-    }
+    sync_all();
+    return sm->xchg[bf];
   }
 };
 
-// Finds T over the eligible items such that weight(key > T) < R <= weight(key >= T), with
-// 1 <= R <= total eligible weight.  get(li, key, len) tells whether local item li is
-// eligible.  When `whole_bin` comes back true the descent stopped early: every eligible item
-// with key >= T is taken and nothing is tied.  w_above = weight strictly above the ties.
-template <class Get>
-__device__ void radix_threshold(Ctx& c, int lo, int hi, unsigned R, bool allow_early, Get get,
-                                unsigned& T, unsigned& w_above, bool& whole_bin,
-                                bool range_known = false, unsigned kmin = 0xffffffffu,
-                                unsigned kmax = 0u) {
+// Where the cut-off among a set of items lies.
+struct Cut {
+  unsigned T;             // items with key > T are above it
+  bool whole;             // ... those with key == T too (nothing is tied)
+  unsigned above;         // token weight above it
+  unsigned above_before;  // ... of that in the CTAs before this one
+  unsigned tied_before;   // token weight with key == T in the CTAs before this one
+};
+
+// Finds T such that weight(key > T) < R <= weight(key >= T), 1 <= R <= total weight of the
+// eligible items, whose keys lie in [kmin, kmax].  get(li, key, len) tells whether the local
+// item li is eligible; a warp calls it for its items [lo, hi) 32 at a time.
+template <int THREADS, class Get>
+__device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned kmin, unsigned kmax, unsigned max_len,
+                        bool allow_whole, Get get) {
   Shared& sm = *c.sm;
-  if (!range_known) {
-    for (int li = lo; li < hi; ++li) {
-      unsigned key, len;
-      if (get(li, key, len)) { kmin = min(kmin, key); kmax = max(kmax, key); }
-    }
-    c.cluster_minmax(kmin, kmax);
-  }
+  const int lane = threadIdx.x & 31;
   const unsigned range = kmax - kmin;
-  const int sh = range ? __clz(range) : 0;
-  unsigned prefix = 0, remaining = R;
-  whole_bin = false;
-  const int copy = (threadIdx.x >> 5) & (kCopies - 1);
-  int shift = 32;
+  Cut cut{kmin, false, 0u, 0u, 0u};
+  if (range == 0) {                       // one key value: everything is tied
+    unsigned mine = 0;
+    for (int li = lo + lane; li < hi; li += 32) {
+      unsigned key, len;
+      if (get(li, key, len)) mine += len;
+    }
+    if (c.C == 1) return cut;
+    unsigned w[kWords] = {c.block_sum(mine), 0u, 0u, 0u, 0u, 0u};
+    const unsigned(*x)[kWords] = c.publish(w);
+    for (int r = 0; r < c.rank; ++r) cut.tied_before += x[r][0];
+    return cut;
+  }
+  if (threadIdx.x == 0) sm.n_own = 0;     // (published by the barriers below)
+  if (threadIdx.x < 256) sm.sub[threadIdx.x] = 0;
+  unsigned below = 0;                     // this thread's share of above_before
+  auto before_sums = [&](unsigned gt, unsigned eq) {
+    if (c.C == 1) return;
+    gt += below;
+    c.block_sum2(gt, eq);
+    cut.above_before += gt;
+    cut.tied_before += eq;
+  };
+  const int sh = __clz(range);
+  unsigned prefix = 0, remaining = R;     // resolved high bits of the shifted keys; rank inside them
+  int shift = 32;                         // ... bits [31, shift)
 #pragma unroll 1
-  while (shift > 0 && range) {
-    const int bits = min(kDigitBits, shift);
-    const int hi_shift = shift;             // bits [31, hi_shift) are resolved
+  for (;;) {
+    const int bits = min(kBinBits, shift), top = shift;
     shift -= bits;
-    const unsigned b = c.phase++ & 1u;
-    unsigned* h = &sm.hist[b][0][0];
-#pragma unroll 1
-    for (int i = threadIdx.x; i < kCopies * kBins; i += kThreads) h[i] = 0;
-    __syncthreads();
-    for (int li = lo; li < hi; ++li) {
+    // two copies: a copy is cleared again only after the barrier of the histogram in between
+    unsigned* h = sm.hist[c.n_hist & 1u];
+    if (c.n_hist++ > 0) {                 // (the first one is clear from the start)
+      for (int i = threadIdx.x; i < kBins; i += THREADS) h[i] = 0;
+      __syncthreads();
+    }
+#pragma unroll 4
+    for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len)) continue;
       const unsigned kk = (key - kmin) << sh;
-      const bool match = hi_shift == 32 || (kk >> hi_shift) == (prefix >> hi_shift);
-      if (match) atomicAdd(&sm.hist[b][copy][(kk >> shift) & ((1u << bits) - 1u)], len);
-    }
-    // fold the private copies into copy 0 before the peers look at it
-    __syncthreads();
-    if (threadIdx.x < kBins) {
-      unsigned t = sm.hist[b][0][threadIdx.x];
-#pragma unroll
-      for (int cp = 1; cp < kCopies; ++cp) t += sm.hist[b][cp][threadIdx.x];
-      sm.hist[b][0][threadIdx.x] = t;
+      if (top == 32 || (kk >> top) == (prefix >> top)) atomicAdd(&h[(kk >> shift) & ((1u << bits) - 1u)], len);
     }
     c.sync_all();
-    // thread t (< 256) owns bin 255 - t, so a forward scan walks the keys downwards
-    const int bin0 = kBins - 1 - (int)threadIdx.x;
-    unsigned v0 = 0;
-    if (threadIdx.x < kBins)
+    // Thread t < kBins / 4 owns four bins, counted from the top, so a forward scan walks the keys
+    // down; a peer's four are one 16-byte load (the exchange is paid per request: 4-byte loads by
+    // all threads made this step 4 us long in clusters of eight), and all peers' are requested
+    // before the first is used.
+    constexpr int kOwn = 4;
+    const bool owner = threadIdx.x < kBins / kOwn;
+    const int b0 = owner ? kBins - kOwn - (int)threadIdx.x * kOwn : 0;
+    unsigned n[kOwn] = {0u, 0u, 0u, 0u}, nb[kOwn] = {0u, 0u, 0u, 0u};   // weight per bin: all CTAs, those before this one
+    if (owner) {
+      uint4 v[kMaxCluster];
 #pragma unroll
       for (int r = 0; r < kMaxCluster; ++r)
-        if (r < c.C) v0 += c.peer(&sm.hist[b][0][bin0], r);
-    unsigned excl, d0, d1, d2;
-    c.block_scan2(v0, 0u, excl, d0, d1, d2);
-    if (threadIdx.x < kBins && excl < remaining && remaining <= excl + v0) {
-      sm.bcast[0] = (unsigned)bin0; sm.bcast[1] = remaining - excl; sm.bcast[2] = v0;
+        v[r] = r < c.C ? *reinterpret_cast<const uint4*>(c.peer(h + b0, r)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int r = 0; r < kMaxCluster; ++r) {
+        n[0] += v[r].x; n[1] += v[r].y; n[2] += v[r].z; n[3] += v[r].w;
+        if (r < c.rank) { nb[0] += v[r].x; nb[1] += v[r].y; nb[2] += v[r].z; nb[3] += v[r].w; }
+      }
+    }
+    unsigned sum = 0;
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) sum += n[i];
+    unsigned excl = c.block_scan(sum);
+#pragma unroll
+    for (int i = kOwn - 1; i >= 0; --i) {
+      if (owner && excl < remaining && remaining <= excl + n[i]) {
+        sm.bcast[0] = (unsigned)(b0 + i);
+        sm.bcast[1] = remaining - excl;
+        sm.bcast[2] = n[i];
+        sm.bcast[3] = nb[i];
+      }
+      excl += n[i];
     }
     __syncthreads();
-    prefix |= sm.bcast[0] << shift;
+    const unsigned bin = sm.bcast[0], in_bin = sm.bcast[2], in_bin_before = sm.bcast[3];
     remaining = sm.bcast[1];
-    const unsigned in_bin = sm.bcast[2];
-    __syncthreads();
-    if (allow_early && remaining == in_bin && shift > 0) {
-      whole_bin = true;
-      remaining = 0;
-      break;
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i)
+      if ((unsigned)(b0 + i) > bin) below += nb[i];
+    prefix |= bin << shift;
+    cut.T = kmin + (prefix >> sh);
+    if (allow_whole && remaining == in_bin) {   // the whole bin is above the cut: nothing is tied
+      cut.whole = true;
+      cut.above = R;
+      cut.above_before = in_bin_before;
+      before_sums(0u, 0u);
+      return cut;
+    }
+    cut.above = R - remaining;
+    if (shift == 0) {                     // every bit resolved: the bin is one key value
+      cut.tied_before = in_bin_before;
+      before_sums(0u, 0u);
+      return cut;
+    }
+    if (in_bin <= (unsigned)(kCand - 1) * max_len) break;
+    // a crowded bin is often a single value (equal distances, clamped scores): look before refining
+    unsigned lo_k = 0xffffffffu, hi_k = 0u;
+#pragma unroll 4
+    for (int li = lo + lane; li < hi; li += 32) {
+      unsigned key, len;
+      if (!get(li, key, len) || (((key - kmin) << sh) >> shift) != (prefix >> shift)) continue;
+      lo_k = min(lo_k, key);
+      hi_k = max(hi_k, key);
+    }
+    unsigned a0 = 0u, d0 = 0u, f0 = 0u;
+    c.block_totals(a0, lo_k, hi_k, d0, f0);
+    if (c.C > 1) {
+      const unsigned w[kWords] = {lo_k, hi_k, 0u, 0u, 0u, 0u};
+      const unsigned(*x)[kWords] = c.publish(w);
+      for (int r = 0; r < c.C; ++r) {
+        lo_k = min(lo_k, x[r][0]);
+        hi_k = max(hi_k, x[r][1]);
+      }
+    }
+    if (lo_k == hi_k) {
+      cut.T = lo_k;
+      cut.tied_before = in_bin_before;
+      before_sums(0u, 0u);
+      return cut;
     }
   }
-  T = kmin + (prefix >> sh);
-  w_above = R - remaining;
-  if (whole_bin) w_above = R;
+
+  // the bin's keys, listed per CTA and read by all of them in rank order
+#pragma unroll 4
+  for (int li = lo + lane; li < hi; li += 32) {
+    unsigned key, len;
+    if (!get(li, key, len)) continue;
+    if ((((key - kmin) << sh) >> shift) == (prefix >> shift)) sm.own[atomicAdd(&sm.n_own, 1u)] = Cand{key, len};
+  }
+  c.sync_all();
+  unsigned first[kMaxCluster + 1];        // places of the CTAs' lists in the common one
+  first[0] = 0;
+#pragma unroll
+  for (int r = 0; r < kMaxCluster; ++r) first[r + 1] = r < c.C ? *c.peer(&sm.n_own, r) : 0u;
+#pragma unroll
+  for (int r = 0; r < kMaxCluster; ++r) first[r + 1] += first[r];
+  const unsigned total = first[kMaxCluster];
+  unsigned before = 0;
+#pragma unroll
+  for (int r = 0; r < kMaxCluster; ++r)
+    if (r == c.rank) before = first[r];
+  const int sub_bits = min(8, shift), sub_shift = shift - sub_bits;
+  auto sub_bin = [&](unsigned key) { return (((key - kmin) << sh) >> sub_shift) & ((1u << sub_bits) - 1u); };
+  const bool refine = total > 64;         // narrow a long list down by the next bits before ranking
+  for (unsigned i = threadIdx.x; i < total; i += THREADS) {
+    int r = 0;
+    unsigned at = i;
+#pragma unroll
+    for (int k = 1; k < kMaxCluster; ++k)
+      if (i >= first[k]) { r = k; at = i - first[k]; }
+    const Cand o = c.peer(sm.own, r)[at];
+    sm.all[i] = o;
+    if (refine) atomicAdd(&sm.sub[sub_bin(o.key)], o.len);
+  }
+  __syncthreads();
+  unsigned sub = 0;
+  if (refine) {                           // every warp finds the sub-bin for itself (lane l: bins 255 - 8 l ...)
+    unsigned n8[8], sum = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { n8[i] = sm.sub[255 - 8 * lane - i]; sum += n8[i]; }
+    unsigned inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    unsigned excl = inc - sum;
+    bool found = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (excl < remaining && remaining <= excl + n8[i]) { sub = 255 - 8 * lane - i; found = true; }
+      excl += n8[i];
+    }
+    sub = __shfl_sync(0xffffffffu, sub, __ffs(__ballot_sync(0xffffffffu, found)) - 1);
+  }
+  // a warp ranks one key against all others
+  for (unsigned i = threadIdx.x >> 5; i < total; i += THREADS / 32) {
+    const unsigned key = sm.all[i].key;
+    if (refine && sub_bin(key) != sub) continue;
+    unsigned gt = 0, eq = 0;
+    for (unsigned j = lane; j < total; j += 32) {
+      const Cand o = sm.all[j];
+      gt += o.key > key ? o.len : 0u;
+      eq += o.key == key ? o.len : 0u;
+    }
+    gt = __reduce_add_sync(0xffffffffu, gt);
+    eq = __reduce_add_sync(0xffffffffu, eq);
+    if (lane == 0 && gt < remaining && remaining <= gt + eq) { sm.bcast[0] = key; sm.bcast[1] = gt; }
+  }
+  __syncthreads();
+  cut.T = sm.bcast[0];
+  cut.above += sm.bcast[1];
+  unsigned gt = 0, eq = 0;
+  if (c.C > 1)
+    for (unsigned i = threadIdx.x; i < before; i += THREADS) {
+      const Cand o = sm.all[i];
+      if (o.key > cut.T) gt += o.len;
+      if (o.key == cut.T) eq += o.len;
+    }
+  before_sums(gt, eq);
+  return cut;
+}
+
+// Pooled values of four neighbouring items from the staged scores w4[0] ..: windows of kW taps, the
+// first starting at w4[0].x.  Maxima share the taps all four windows have; averages are
+// left-to-right sums, then one division.
+template <int kW>
+__device__ __forceinline__ void pool4(const float4* w4, int kind, float (&v)[4]) {
+  constexpr int kVecs = (kW + 3 + 3) / 4;
+  float a[4 * kVecs];
+#pragma unroll
+  for (int i = 0; i < kVecs; ++i) {
+    const float4 x = w4[i];
+    a[4 * i] = x.x; a[4 * i + 1] = x.y; a[4 * i + 2] = x.z; a[4 * i + 3] = x.w;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v[j] = a[j];
+    if (kind == CC_POOL_MAX) {
+#pragma unroll
+      for (int d = 1; d < kW; ++d) v[j] = fmaxf(v[j], a[j + d]);
+    } else if (kW > 1) {
+#pragma unroll
+      for (int d = 1; d < kW; ++d) v[j] = __fadd_rn(v[j], a[j + d]);
+      v[j] = __fdiv_rn(v[j], (float)kW);
+    }
+  }
+}
+__device__ __forceinline__ void pool4_any(const float* w, int kind, int width, float (&v)[4]) {
+#pragma unroll 1
+  for (int j = 0; j < 4; ++j) {
+    float x = w[j];
+    for (int d = 1; d < width; ++d) x = kind == CC_POOL_MAX ? fmaxf(x, w[j + d]) : __fadd_rn(x, w[j + d]);
+    const float y = kind == CC_POOL_MAX ? x : __fdiv_rn(x, (float)width);
+    if (j == 0) v[0] = y;
+    if (j == 1) v[1] = y;
+    if (j == 2) v[2] = y;
+    if (j == 3) v[3] = y;
+  }
 }
 
 // CHUNKED instantiations rank fixed chunks of bt.chunk tokens; the others are compiled for
 // token-level items only (bt.chunk == 1), which keeps their code short.
-template <bool FUSED, bool CHUNKED>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool FUSED, bool CHUNKED, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ ClusterParams P) {
   extern __shared__ __align__(16) uint8_t dyn[];
-  Shared* smp = reinterpret_cast<Shared*>(dyn);
-  unsigned* keys = reinterpret_cast<unsigned*>(dyn + sizeof(Shared));
-  Ctx c;
-  c.sm = smp;
+  Shared& sm = *reinterpret_cast<Shared*>(dyn);
+  Ctx<THREADS> c;
+  c.sm = &sm;
   c.C = P.cluster;
   c.rank = P.cluster > 1 ? (int)cg::this_cluster().block_rank() : 0;
-  c.phase = 0;
+  c.n_xchg = c.n_red = c.n_hist = 0;
 
   pdl_launch_dependents();
+  if (c.C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
   // FUSED runs right after the second score pass, which starts only once the caller's inputs
   // are complete: the token-level path reads the prior before it waits for the scores
   const bool early_prior = FUSED && !CHUNKED;
@@ -322,19 +457,18 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   const int h = blockIdx.y, s = blockIdx.z;
   const SeqInfo& q = bt.seq[s];
   const int m = q.n_items, cs = CHUNKED ? bt.chunk : 1;
-  const int per = (m + c.C * kThreads - 1) / (c.C * kThreads);       // items per thread
-  const int cta_lo = min(m, c.rank * kThreads * per);
-  const int cta_hi = min(m, cta_lo + kThreads * per);
-  const int cta_items = cta_hi - cta_lo;
-  uint8_t* flags = reinterpret_cast<uint8_t*>(keys + padded(kThreads * per) + 1);
+  const int slice = (m + c.C * THREADS - 1) / (c.C * THREADS) * THREADS;     // items per CTA, a multiple of 32
+  const int cta_lo = min(m, c.rank * slice), cta_items = min(m, cta_lo + slice) - cta_lo;
+  unsigned* keys = reinterpret_cast<unsigned*>(dyn + sizeof(Shared));
+  uint8_t* flags = reinterpret_cast<uint8_t*>(keys + P.per * THREADS);
   const float* p = P.prior + q.tok_off;
   int32_t* out = P.idx[q.layer] + (int64_t)h * bt.b_tot + q.idx_off;
   const unsigned keep = (unsigned)q.keep;
   const float theta = P.theta;
-
-  // contiguous local range of this thread
-  const int lo = min(cta_items, (int)threadIdx.x * per);
-  const int hi = min(cta_items, lo + per);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the run of items of this warp
+  const int run = slice / (THREADS / 32);
+  const int lo = min(cta_items, warp * run), hi = min(cta_items, lo + run);
 
   auto item_len = [&](int li) -> unsigned {
     if (cs == 1) return 1u;
@@ -350,61 +484,100 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     return pr;
   };
 
+  for (int i = threadIdx.x; i < kBins; i += THREADS) sm.hist[0][i] = 0;
+  // Totals collected while loading: protected weight, key range of the unprotected items (of all
+  // items when a cap may still strip some of their protection), range of the protected items'
+  // priors when there is a cap
+  const bool capped = q.span_cap >= 0;
+  unsigned forced_tokens = 0, forced_before = 0;              // before: in the CTAs before this one
+  unsigned key_lo = 0xffffffffu, key_hi = 0u, pri_lo = 0xffffffffu, pri_hi = 0u;
+  auto tally = [&](unsigned key, float pr, unsigned len) {
+    const bool forced = pr >= theta;
+    if (forced) {
+      forced_tokens += len;
+      if (capped) {
+        const unsigned pk = mono_key(pr);
+        pri_lo = min(pri_lo, pk);
+        pri_hi = max(pri_hi, pk);
+      }
+    }
+    if (!forced || capped) {
+      key_lo = min(key_lo, key);
+      key_hi = max(key_hi, key);
+    }
+    return forced;
+  };
   // ---- load: keys and protected flags of the CTA's slice (coalesced over the block)
   if (FUSED) {
     const float* u = P.scores[q.layer] + (int64_t)h * bt.n_tot + q.tok_off;
-    float* fo = P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off;
     const int half = (cs == 1 && P.pool_kind != CC_POOL_NONE) ? P.pool_size / 2 : 0;
-    float* us = reinterpret_cast<float*>(flags + ((kThreads * per + 15) / 16) * 16);
+    auto fuse = [&](float val, float pr) {
+      return mono_key(__fadd_rn(__fadd_rn(__fmul_rn(P.alpha, val), __fmul_rn(P.beta, pr)), 0.0f));
+    };
+    auto store4 = [&](int l4, const float (&v)[4], float4 pr) {
+      const uint4 k4 = make_uint4(fuse(v[0], pr.x), fuse(v[1], pr.y), fuse(v[2], pr.z), fuse(v[3], pr.w));
+      *reinterpret_cast<uint4*>(keys + l4) = k4;
+      const int left = cta_items - l4;
+      unsigned f = tally(k4.x, pr.x, 1u) ? 1u : 0u;
+      if (left > 1 && tally(k4.y, pr.y, 1u)) f |= 1u << 8;
+      if (left > 2 && tally(k4.z, pr.z, 1u)) f |= 1u << 16;
+      if (left > 3 && tally(k4.w, pr.w, 1u)) f |= 1u << 24;
+      *reinterpret_cast<unsigned*>(flags + l4) = f;
+    };
     if (cs == 1) {
-      // stage u[cta_lo - half, cta_hi + half) (zero outside the sequence) and park the priors in
-      // the key slots; four loads of each are issued before the first store, so the slice
-      // costs a couple of round trips to L2 instead of one per item
-      const int span = cta_items + 2 * half;
+      // The priors are parked in the key slots (loads issued four at a time: the slice costs a
+      // couple of round trips to L2 instead of one per item).
 #pragma unroll 1
-      for (int t0 = threadIdx.x; t0 < cta_items; t0 += 4 * kThreads) {
+      for (int t0 = threadIdx.x; t0 < cta_items; t0 += 4 * THREADS) {
         float b[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) b[k] = t0 + k * kThreads < cta_items ? p[cta_lo + t0 + k * kThreads] : 0.0f;
+        for (int k = 0; k < 4; ++k) b[k] = t0 + k * THREADS < cta_items ? p[cta_lo + t0 + k * THREADS] : 0.0f;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          if (t0 + k * kThreads < cta_items) keys[padded(t0 + k * kThreads)] = __float_as_uint(b[k]);
+          if (t0 + k * THREADS < cta_items) keys[t0 + k * THREADS] = __float_as_uint(b[k]);
       }
       pdl_wait();                                   // the scores are complete from here on
-      if (P.stage_u) {
-#pragma unroll 1
-      for (int t0 = threadIdx.x; t0 < span; t0 += 4 * kThreads) {
-        float a[4];
+      // The scores go through two staging buffers of kStep * THREADS items and the pooling halo
+      // (zero outside the sequence, which is neutral for the maximum too: scores are not
+      // negative); a part is requested while the one before it is pooled.
+      float* us = reinterpret_cast<float*>(flags + P.per * THREADS);
+      const int part = kStep * THREADS, pitch = part + 2 * kMaxHalf;
+      float a[kStep + 1];
+      auto request = [&](int c0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int t = t0 + k * kThreads, j = cta_lo - half + t;
-          a[k] = (t < span && j >= 0 && j < q.n) ? u[j] : 0.0f;
+        for (int k = 0; k <= kStep; ++k) {
+          const int t = threadIdx.x + k * THREADS, j = cta_lo + c0 - half + t;
+          a[k] = (t < part + 2 * half && c0 + t < cta_items + 2 * half && j >= 0 && j < q.n) ? u[j] : 0.0f;
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (t0 + k * kThreads < span) us[t0 + k * kThreads] = a[k];
-      }
-      }
-      __syncthreads();
-    }
-    // raw score at position t of the staged window (token cta_lo - half + t; zero outside the
-    // sequence): from the staging buffer, or straight from global memory through L1 when the
-    // slice is too long to be staged as well
-    const bool staged = P.stage_u != 0;
-    auto uval = [&](int t) -> float {
-      if (staged) return us[t];
-      const int j = cta_lo - half + t;
-      return (j >= 0 && j < q.n) ? u[j] : 0.0f;
-    };
+      };
+      if (cta_items > 0) request(0);
 #pragma unroll 1
-    for (int li = threadIdx.x; li < cta_items; li += kThreads) {
-      const int i = cta_lo + li;
-      float val, pr;
-      if (cs > 1) {
+      for (int c0 = 0, buf = 0; c0 < cta_items; c0 += part, buf ^= 1) {
+        float* ub = us + buf * pitch;
+#pragma unroll
+        for (int k = 0; k <= kStep; ++k)
+          if (threadIdx.x + k * THREADS < part + 2 * half) ub[threadIdx.x + k * THREADS] = a[k];
+        __syncthreads();
+        if (c0 + part < cta_items) request(c0 + part);
+        const int l4 = c0 + 4 * (int)threadIdx.x;
+        if (l4 < cta_items) {
+          const float4 pr = *reinterpret_cast<const float4*>(keys + l4);       // the parked priors
+          const float4* w4 = reinterpret_cast<const float4*>(ub) + threadIdx.x;
+          float v[4];
+          if (half == 3) pool4<7>(w4, P.pool_kind, v);
+          else if (half == 2) pool4<5>(w4, P.pool_kind, v);
+          else if (half == 1) pool4<3>(w4, P.pool_kind, v);
+          else if (half == 0) pool4<1>(w4, P.pool_kind, v);
+          else pool4_any(ub + 4 * threadIdx.x, P.pool_kind, 2 * half + 1, v);
+          store4(l4, v, pr);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int li = threadIdx.x; li < cta_items; li += THREADS) {
         // chunk sum in token order; the loads of eight tokens are issued before they are used
-        const int t0 = i * cs, t1 = min(q.n, t0 + cs);
-        val = 0.0f;
-        pr = -INFINITY;
+        const int t0 = (cta_lo + li) * cs, t1 = min(q.n, t0 + cs);
+        float val = 0.0f, pr = -INFINITY;
         for (int j0 = t0; j0 < t1; j0 += 8) {
           float a[8], b[8];
 #pragma unroll
@@ -420,205 +593,241 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
             }
           }
         }
-      } else {
-        pr = __uint_as_float(keys[padded(li)]);       // parked by this very thread
-        if (half == 0) {
-          val = uval(li);
-        } else if (P.pool_kind == CC_POOL_MAX) {
-          val = uval(li + half);
-          const int a = max(0, i - half), b = min(q.n - 1, i + half);
-          for (int j = a; j <= b; ++j) val = fmaxf(val, uval(j - cta_lo + half));
-        } else {
-          val = uval(li);
-          for (int d = 1; d <= 2 * half; ++d) val = __fadd_rn(val, uval(li + d));
-          val = __fdiv_rn(val, (float)P.pool_size);
-        }
+        keys[li] = fuse(val, pr);
+        flags[li] = tally(keys[li], pr, item_len(li)) ? 1 : 0;
       }
-      const float f = __fadd_rn(__fadd_rn(__fmul_rn(P.alpha, val), __fmul_rn(P.beta, pr)), 0.0f);
-      fo[i] = f;
-      keys[padded(li)] = mono_key(f);
-      flags[li] = pr >= theta ? 1 : 0;
     }
   } else {
     const float* f = P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off;
 #pragma unroll 1
-    for (int li = threadIdx.x; li < cta_items; li += kThreads) {
-      keys[padded(li)] = mono_key(f[cta_lo + li]);
-      flags[li] = item_prior(li) >= theta ? 1 : 0;
+    for (int li = threadIdx.x; li < cta_items; li += THREADS) {
+      const unsigned key = mono_key(f[cta_lo + li]);
+      const float pr = item_prior(li);
+      keys[li] = key;
+      flags[li] = tally(key, pr, item_len(li)) ? 1 : 0;
     }
   }
-  __syncthreads();
 
-  // ---- stage 0: protected weight
-  unsigned wf = 0, free_min = 0xffffffffu, free_max = 0u;   // key range of the unprotected items
-#pragma unroll 1
-  for (int li = lo; li < hi; ++li) {
-    if (flags[li]) {
-      wf += item_len(li);
-    } else {
-      const unsigned key = keys[padded(li)];
-      free_min = min(free_min, key);
-      free_max = max(free_max, key);
+  // ---- stage 0: totals of the cluster (the block reduction's barrier also publishes keys and flags)
+  c.block_totals(forced_tokens, key_lo, key_hi, pri_lo, pri_hi);
+  if (c.C > 1) {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // so have the others
+    const unsigned w[kWords] = {forced_tokens, key_lo, key_hi, pri_lo, pri_hi, 0u};
+    const unsigned(*x)[kWords] = c.publish(w);
+    forced_tokens = 0;
+    for (int r = 0; r < c.C; ++r) {
+      if (r == c.rank) forced_before = forced_tokens;
+      forced_tokens += x[r][0];
+      key_lo = min(key_lo, x[r][1]);
+      key_hi = max(key_hi, x[r][2]);
+      pri_lo = min(pri_lo, x[r][3]);
+      pri_hi = max(pri_hi, x[r][4]);
     }
   }
-  // one exchange yields the sum, its prefix (all the emission needs when the protected items
-  // alone fill the budget: the scan of stage 3 is skipped) and the key range of stage 2
-  unsigned forced_before, forced_tokens;
-  c.cluster_scan_total(wf, forced_before, forced_tokens, free_min, free_max);
-  bool flags_as_counted = true;
 
   // ---- stage 1: cap on protected items (longest prefix by (prior desc, index asc) within B_span)
-  if (q.span_cap >= 0 && forced_tokens > (unsigned)q.span_cap) {
-    flags_as_counted = false;
+  if (capped && forced_tokens > (unsigned)q.span_cap) {
     const unsigned cap = (unsigned)q.span_cap;
-    unsigned t1, above1;
-    bool whole;
-    radix_threshold(c, lo, hi, cap + 1u, false,
-                    [&](int li, unsigned& key, unsigned& len) {
-                      if (!flags[li]) return false;
-                      key = mono_key(item_prior(li));
-                      len = item_len(li);
-                      return true;
-                    }, t1, above1, whole);
-    unsigned tie_w = 0;
-#pragma unroll 1
-    for (int li = lo; li < hi; ++li)
-      if (flags[li] && mono_key(item_prior(li)) == t1) tie_w += item_len(li);
-    unsigned tie_before, dummy;
-    c.cluster_scan2(tie_w, 0u, tie_before, dummy);
-    unsigned kept = 0;
-#pragma unroll 1
-    for (int li = lo; li < hi; ++li) {
-      if (!flags[li]) continue;
-      const unsigned key = mono_key(item_prior(li));
-      const unsigned len = item_len(li);
-      if (key > t1) { kept += len; continue; }
-      if (key == t1) {
-        const bool fits = above1 + tie_before + len <= cap;
-        tie_before += len;
-        if (fits) { kept += len; continue; }
-      }
-      flags[li] = 0;
+    const Cut cut = find_cut(c, lo, hi, cap + 1u, pri_lo, pri_hi, (unsigned)cs, false,
+                             [&](int li, unsigned& key, unsigned& len) {
+                               if (!flags[li]) return false;
+                               key = mono_key(item_prior(li));
+                               len = item_len(li);
+                               return true;
+                             });
+    unsigned ties = 0, none = 0;
+    for (int li = lo + lane; li < hi; li += 32)
+      if (flags[li] && mono_key(item_prior(li)) == cut.T) ties += item_len(li);
+    ties = __reduce_add_sync(0xffffffffu, ties);
+    c.warps_before2(ties, none);
+    unsigned tie_run = cut.tied_before + ties, kept = 0;
+    for (int l0 = lo; l0 < hi; l0 += 32) {
+      const int li = l0 + lane;
+      const bool forced = li < hi && flags[li];
+      const unsigned pk = forced ? mono_key(item_prior(li)) : 0u, len = forced ? item_len(li) : 0u;
+      const unsigned tm = __ballot_sync(0xffffffffu, forced && pk == cut.T);
+      const unsigned before = tie_run + __popc(tm & ((1u << lane) - 1u)) * (unsigned)cs;
+      tie_run += __popc(tm) * (unsigned)cs;
+      if (!forced) continue;
+      if (pk > cut.T || (pk == cut.T && cut.above + before + len <= cap)) kept += len;
+      else flags[li] = 0;
     }
-    forced_tokens = c.cluster_sum(kept);
+    if (cs == 1) {                 // items of one token fill the cap exactly
+      forced_tokens = cap;
+      forced_before = cut.above_before + min(cut.tied_before, cap - cut.above);
+    } else {
+      forced_tokens = c.block_sum(kept);
+      if (c.C > 1) {
+        const unsigned w[kWords] = {forced_tokens, 0u, 0u, 0u, 0u, 0u};
+        const unsigned(*x)[kWords] = c.publish(w);
+        forced_tokens = forced_before = 0;
+        for (int r = 0; r < c.C; ++r) {
+          if (r == c.rank) forced_before = forced_tokens;
+          forced_tokens += x[r][0];
+        }
+      }
+    }
   }
 
   // ---- stage 2: cut-off among the unprotected items
-  bool ties_are_forced, whole_bin = false;
-  unsigned t = 0, tie_budget;
-  if (forced_tokens >= keep) {
-    ties_are_forced = true;          // protected items alone fill the budget: first B in order
-    tie_budget = keep;
-  } else {
-    ties_are_forced = false;
-    unsigned above;
-    radix_threshold(c, lo, hi, keep - forced_tokens, true,
-                    [&](int li, unsigned& key, unsigned& len) {
-                      if (flags[li]) return false;
-                      key = keys[padded(li)];
-                      len = item_len(li);
-                      return true;
-                    }, t, above, whole_bin, flags_as_counted, free_min, free_max);
-    tie_budget = keep - forced_tokens - above;
-  }
-
-  // ---- stage 3: ordered emission
-  const bool reuse_prefix = ties_are_forced && flags_as_counted;
-  unsigned def_w = 0, tie_w = 0;
-  if (!reuse_prefix) {
-#pragma unroll 1
-  for (int li = lo; li < hi; ++li) {
-    const unsigned len = item_len(li);
-    if (flags[li]) {
-      if (ties_are_forced) tie_w += len; else def_w += len;
-    } else if (!ties_are_forced) {
-      const unsigned key = keys[padded(li)];
-      if (key > t || (whole_bin && key == t)) def_w += len; else if (key == t) tie_w += len;
-    }
-  }
-  }
-  unsigned def_before, tie_before;
-  if (reuse_prefix) {
-    def_before = 0;
-    tie_before = forced_before;
-  } else {
-    c.cluster_scan2(def_w, tie_w, def_before, tie_before);
-  }
+  const bool ties_are_forced = forced_tokens >= keep;   // protected items alone fill the budget: first B in order
+  Cut cut{0u, false, 0u, 0u, 0u};
+  if (!ties_are_forced)
+    cut = find_cut(c, lo, hi, keep - forced_tokens, key_lo, key_hi, (unsigned)cs, true,
+                   [&](int li, unsigned& key, unsigned& len) {
+                     if (flags[li]) return false;
+                     key = keys[li];
+                     len = item_len(li);
+                     return true;
+                   });
+  const unsigned tie_budget = ties_are_forced ? keep : keep - forced_tokens - cut.above;
   // last read of a peer's shared memory is done: announce it now, wait for the peers at the
   // very end, and write the indices in between
-  if (c.C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-#pragma unroll 1
-  for (int li = lo; li < hi; ++li) {
-    const unsigned len = item_len(li);
-    unsigned take = 0;
-    bool tie = false;
+  // (relaxed: nothing is published by it, so it need not wait for stores in flight)
+  if (c.C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+
+  // ---- stage 3: ordered emission.  Items kept for sure (def) and the tied ones in sequence order,
+  // until the budget is full
+  auto classify = [&](int li, bool& def, bool& tie) {
+    def = tie = false;
+    if (li >= hi) return;
     if (flags[li]) {
-      if (ties_are_forced) tie = true; else take = len;
+      def = !ties_are_forced;
+      tie = ties_are_forced;
     } else if (!ties_are_forced) {
-      const unsigned key = keys[padded(li)];
-      if (key > t || (whole_bin && key == t)) take = len; else if (key == t) tie = true;
+      const unsigned key = keys[li];
+      def = key > cut.T || (cut.whole && key == cut.T);
+      tie = !cut.whole && key == cut.T;
     }
-    const unsigned pos = def_before + min(tie_before, tie_budget);
-    if (tie) {
-      take = tie_before < tie_budget ? min(len, tie_budget - tie_before) : 0u;
-      tie_before += len;
-    } else {
-      def_before += take;
-    }
+  };
+  // Step k of a warp's run (at most 32 steps) leaves two masks of its 32 items in lane k, and the
+  // indices are written from the masks: the passes over all items end here.  The fused
+  // values are stored on the way, from their keys: earlier, the stores in flight would have to
+  // land before every exchange of the CTAs.
+  float* fo = FUSED ? P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off + cta_lo : nullptr;
+  unsigned defs = 0, ties = 0;
+#pragma unroll 4
+  for (int k = 0; k < run / 32; ++k) {
+    const int li = lo + k * 32 + lane;
+    bool def, tie;
+    classify(li, def, tie);
+    if (FUSED && li < hi) fo[li] = mono_value(keys[li]);
+    const unsigned dm = __ballot_sync(0xffffffffu, def), tm = __ballot_sync(0xffffffffu, tie);
+    if (lane == k) { defs = dm; ties = tm; }
+  }
+  // tokens of this lane's step and of the steps and warps before it
+  const int base = lo + lane * 32, last = m - 1 - cta_lo - base;         // bit of the sequence's last item
+  const unsigned cut_short = CHUNKED && last >= 0 && last < 32 ? (unsigned)(cs - (q.n - (m - 1) * cs)) << 1 : 0u;
+  auto tokens = [&](unsigned mask) {
+    unsigned n = (unsigned)__popc(mask) * (unsigned)cs;
+    if (CHUNKED && cut_short && (mask >> last & 1u)) n -= cut_short >> 1;
+    return n;
+  };
+  const unsigned def_own = tokens(defs), tie_own = tokens(ties);
+  unsigned def_run = def_own, tie_run = tie_own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned a = __shfl_up_sync(0xffffffffu, def_run, o), b = __shfl_up_sync(0xffffffffu, tie_run, o);
+    if (lane >= o) { def_run += a; tie_run += b; }
+  }
+  unsigned def_warps = __shfl_sync(0xffffffffu, def_run, 31), tie_warps = __shfl_sync(0xffffffffu, tie_run, 31);
+  c.warps_before2(def_warps, tie_warps);
+  def_run += def_warps - def_own + (ties_are_forced ? 0u : forced_before) + cut.above_before;
+  tie_run += tie_warps - tie_own + (ties_are_forced ? forced_before : cut.tied_before);
+  auto emit = [&](int li, bool tie, unsigned def_before, unsigned tie_before) {
+    const unsigned len = item_len(li), pos = def_before + min(tie_before, tie_budget);
+    const unsigned take = !tie ? len : (tie_before < tie_budget ? min(len, tie_budget - tie_before) : 0u);
     const int tok0 = (cta_lo + li) * cs;
     for (unsigned k = 0; k < take; ++k)
       if (pos + k < keep) out[pos + k] = tok0 + (int)k;
+    return len;
+  };
+  if (run / 32 > 10) {           // a step per lane
+    for (unsigned left = defs | ties; left; left &= left - 1u) {
+      const int bit = __ffs(left) - 1;
+      const bool tie = ties >> bit & 1u;
+      const unsigned len = emit(base + bit, tie, def_run, tie_run);
+      if (tie) tie_run += len; else def_run += len;
+    }
+  } else {                       // few steps: one after the other, an item per lane
+    const unsigned lt = (1u << lane) - 1u;
+    for (int k = 0; k < run / 32; ++k) {
+      const unsigned dm = __shfl_sync(0xffffffffu, defs, k), tm = __shfl_sync(0xffffffffu, ties, k);
+      const unsigned db = __shfl_sync(0xffffffffu, def_run, k) + __popc(dm & lt) * (unsigned)cs;
+      const unsigned tb = __shfl_sync(0xffffffffu, tie_run, k) + __popc(tm & lt) * (unsigned)cs;
+      if ((dm | tm) >> lane & 1u) emit(lo + k * 32 + lane, tm >> lane & 1u, db, tb);
+    }
   }
-  for (int i = (int)keep + c.rank * kThreads + threadIdx.x; i < q.budget; i += c.C * kThreads)
+  for (int i = (int)keep + c.rank * THREADS + threadIdx.x; i < q.budget; i += c.C * THREADS)
     out[i] = -1;
   if (c.rank == 0 && threadIdx.x == 0) P.count[q.layer][q.src * P.hkv + h] = (int)keep;
   // no CTA may leave while a peer can still read its shared memory
   if (c.C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-size_t cluster_smem_bytes(int per, bool staged, int pool_size) {
-  size_t b = sizeof(Shared);
-  b += ((size_t)padded(kThreads * per) + 1) * 4;          // keys
-  b += ((size_t)kThreads * per + 15) / 16 * 16;           // flags
-  if (staged) b += ((size_t)kThreads * per + 2 * (pool_size / 2) + 4) * 4;
+size_t cluster_smem_bytes(int slots, int threads, bool staging) {
+  size_t b = sizeof(Shared) + (size_t)slots * 5;                   // keys, flags
+  if (staging) b += 2 * (size_t)(kStep * threads + 2 * kMaxHalf) * sizeof(float);
   return (b + 15) / 16 * 16;
+}
+
+struct Shape {
+  int cluster, threads;      // CTAs per (sequence, head), threads per CTA
+};
+
+template <bool FUSED, bool CHUNKED>
+cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, int threads,
+                         size_t smem) {
+  auto kern = threads == 512 ? select_cluster_kernel<FUSED, CHUNKED, 512> : select_cluster_kernel<FUSED, CHUNKED, 1024>;
+  const cudaError_t e = allow_smem(kern);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3(P.cluster, g.hkv, bt.num_seqs), dim3(threads), smem, L.stream, P.cluster, bt, P);
+}
+
+// Time of a launch with clusters of 1 << lc CTAs of `threads` threads, in us, from launches of one wave
+// on a B200 (n = 2048 .. 131072 items, 2 .. 256 problems): a constant that grows with what the
+// exchanges of wider clusters cost, 1 us more for the barriers of 1024 threads, and 0.48 (0.6) us
+// per item of a thread of 512 (1024).  A chunk's tokens count a fifth of an item each.  A CTA of 1024
+// threads fills an SM, CTAs of 512 share it in pairs; a cluster sits inside one GPC, so fewer CTAs run
+// at a time in wide ones.
+double launch_cost(const BatchTable& bt, int hkv, int lc, int threads) {
+  static const double base[4] = {6.1, 7.7, 7.8, 8.6};
+  static const int room[4] = {148, 148, 128, 96};
+  const int c = 1 << lc;
+  const double per_thread = (bt.max_items + (bt.chunk > 1 ? 0.2 * bt.chunk * bt.max_items : 0.0)) / (double)(c * threads);
+  const int ctas = bt.num_seqs * hkv * c, fit = threads == 512 ? 2 * room[lc] : room[lc];
+  const int waves = (ctas + fit - 1) / fit;
+  const double slope = threads == 1024 ? 0.6 : (ctas > room[lc] ? 0.96 : 0.48);
+  return waves * (base[lc] + (threads == 1024 ? 1.0 : 0.0) + slope * per_thread);
+}
+
+// The cheapest shape; cluster 0 when a sequence has more items than the widest cluster holds.
+Shape select_shape(const BatchTable& bt, int hkv) {
+  if (bt.max_items <= 0) return Shape{1, 512};
+  Shape best{0, 0};
+  double best_us = 1e30;
+  for (int lc = 0; lc <= 3; ++lc)
+    for (int threads = 512; threads <= 1024; threads += 512) {
+      // a warp's run has at most 32 steps; CTAs of 512 threads are to fit an SM in pairs
+      if ((bt.max_items + (threads << lc) - 1) / (threads << lc) > 32) continue;
+      const double us = launch_cost(bt, hkv, lc, threads);
+      if (us < best_us) { best_us = us; best = Shape{1 << lc, threads}; }
+    }
+  return best;
 }
 
 }  // namespace
 
-// CTAs per (sequence, head) for the cluster kernel, or 0 when the batch does not fit.
-// A CTA holds up to kCtaItems items (32 per thread; the fused form also stages the raw scores of
-// slices of up to 16 per thread and reads them through L1 beyond that); one CTA of 1024 threads fits per SM, and a
-// cluster is placed inside one GPC, so about 96 CTAs run at a time in clusters of eight, 128 in
-// clusters of four, all 148 otherwise.  Wide clusters finish one (sequence, head) sooner, narrow
-// ones let more of them run at once and pay less per exchange (measured: about 6 + 0.6 x width +
-// items per thread microseconds): the width with the smallest waves x time per wave is taken.
-int select_cluster_size(const BatchTable& bt, int hkv) {
-  if (bt.max_items <= 0) return 1;
-  // in chunk mode a thread reads all tokens of its items, so the width is chosen by tokens
-  const long long work = (long long)bt.max_items * bt.chunk;
-  const long long problems = (long long)bt.num_seqs * hkv;
-  auto per_of = [&](int c) { return (bt.max_items + c * kThreads - 1) / (c * kThreads); };
-  auto cost_of = [&](int c) {
-    const long long room = c == 8 ? 96 : (c == 4 ? 128 : 148);
-    const double waves = (double)((problems * c + room - 1) / room);
-    return waves * (6.0 + 0.6 * c + 1.05 * (double)((work + c * kThreads - 1) / (c * kThreads)));
-  };
-  // widest useful cluster: four items per thread ...
-  int c = 1;
-  while (c < kMaxCluster && (work + c * kThreads - 1) / (c * kThreads) > 4) c *= 2;
-  if (kThreads * per_of(c) > kCtaItems) return 0;
-  // ... narrowed while the batch needs several waves and fewer, longer waves are cheaper
-  while (c > 1 && kThreads * per_of(c / 2) <= kCtaItems && cost_of(c / 2) < cost_of(c)) c /= 2;
-  return c;
-}
+int select_cluster_size(const BatchTable& bt, int hkv) { return select_shape(bt, hkv).cluster; }
 
 cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const Geometry& g,
                                   float force_threshold, bool fused_input, int pool_kind,
                                   int pool_size, float alpha, float beta, const LayerPtrs& lp,
                                   const float* prior, int cluster) {
+  const Shape sh = select_shape(bt, g.hkv);
   ClusterParams P;
-  P.cluster = cluster;
+  P.cluster = sh.cluster;
+  P.per = bt.max_items > 0 ? (bt.max_items + sh.cluster * sh.threads - 1) / (sh.cluster * sh.threads) : 1;
   P.hkv = g.hkv;
   P.theta = force_threshold;
   P.pool_kind = pool_kind;
@@ -632,16 +841,12 @@ cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const G
     P.idx[l] = lp.idx[l];
     P.count[l] = lp.count[l];
   }
-  const int per = bt.max_items > 0 ? (bt.max_items + cluster * kThreads - 1) / (cluster * kThreads) : 1;
-  // token-level fused form: stage the slice's raw scores while they fit beside keys and flags
-  P.stage_u = fused_input && bt.chunk == 1 && kThreads * per <= kStagedItems ? 1 : 0;
-  const size_t smem = cluster_smem_bytes(per, P.stage_u != 0, P.pool_size);
-  const bool chunked = bt.chunk > 1;
-  auto kern = fused_input ? (chunked ? select_cluster_kernel<true, true> : select_cluster_kernel<true, false>)
-                          : (chunked ? select_cluster_kernel<false, true> : select_cluster_kernel<false, false>);
-  cudaError_t e = allow_smem(kern);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(cluster, g.hkv, bt.num_seqs), dim3(kThreads), smem, L.stream, cluster, bt, P);
+  const size_t smem = cluster_smem_bytes(P.per * sh.threads, sh.threads, fused_input && bt.chunk == 1);
+  if (fused_input)
+    return bt.chunk > 1 ? launch_shape<true, true>(L, bt, g, P, sh.threads, smem)
+                        : launch_shape<true, false>(L, bt, g, P, sh.threads, smem);
+  return bt.chunk > 1 ? launch_shape<false, true>(L, bt, g, P, sh.threads, smem)
+                      : launch_shape<false, false>(L, bt, g, P, sh.threads, smem);
 }
 
 }  // namespace cc

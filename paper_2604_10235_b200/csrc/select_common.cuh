@@ -10,6 +10,11 @@ __device__ __forceinline__ unsigned mono_key(float x) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
+// The float of a key (+0.0 for both zeros).
+__device__ __forceinline__ float mono_value(unsigned key) {
+  return __uint_as_float((key & 0x80000000u) ? key & 0x7fffffffu : ~key);
+}
+
 __device__ __forceinline__ unsigned warp_sum(unsigned v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
