@@ -68,6 +68,9 @@ constexpr float kLn2 = 0.6931471805599453f;
 struct TcParams {
   int grid;            // CTAs (same for both passes)
   int total_tiles;     // H_kv * sum of tiles over the sequences
+  int change;          // weight of the start of a (sequence, head) when the spans are cut
+  long long weight;    // of all tiles and starts
+  int halves;          // units of work per tile: 1, or 2 (its row blocks in two halves); HALVES of the kernel
   int rows;            // w * G
   int rows_pad;        // G * w_pad, a multiple of 16
   int w_pad;
@@ -236,6 +239,7 @@ struct Barriers {
   uint64_t q_full, q_empty;
   uint64_t acc_full[kBufs], acc_empty[kBufs];
   uint64_t u_full[8][4];             // pass 2: the other sets' partial sums of (slot, quadrant)
+  uint64_t edge_full[2][4];          // ... of a first / last tile of which the CTA has one half
 };
 
 struct Misc {                        // lives in the last kMiscBytes of dynamic shared memory
@@ -244,7 +248,9 @@ struct Misc {                        // lives in the last kMiscBytes of dynamic 
     float2 xchg[kSets][kMaxRows];    // (max, sum) hand-over: pass 1 per set, pass 2 while merging
     float u_part[8][kSets][kTileKeys];   // pass 2: partial column sums, slot = tile & 7
   };
+  float edge_part[2][kTileKeys];     // pass 2: partial column sums of those tiles
   Barriers bar;
+  long long span[2];                 // first unit of the CTA, first unit behind it
   uint32_t tmem_base;
   volatile int abort_flag;
 };
@@ -416,17 +422,51 @@ struct TileCursor {
   __device__ int problem(int hkv) const { return s * hkv + h; }
 };
 
-__device__ __forceinline__ int span_begin(int b, const TcParams& P) {
-  return (int)(((long long)b * P.total_tiles) / P.grid);
+// The CTAs' spans are runs of units (tiles, or halves of tiles) of equal weight.  A tile weighs 4, and
+// the start of a (sequence, head) weighs P.change besides: a CTA that goes from one to the next
+// replaces Q, drains its pipeline and hands row statistics over.  The first unit of CTA b is the
+// one at weight b * P.weight / grid.
+constexpr int kTileWeight = 4;
+
+// The unit at weight w, counted over all (sequence, head)s.
+template <int HALVES>
+__device__ long long unit_at(const BatchTable& bt, int hkv, const TcParams& P, long long w) {
+  long long unit = 0;
+#pragma unroll 1
+  for (int s = 0; s < bt.num_seqs; ++s) {
+    const int n_tiles = bt.seq[s].n_tiles;
+    if (n_tiles == 0) continue;
+    const unsigned per = (unsigned)(n_tiles * kTileWeight + P.change);       // weight of one head
+    if (w < (long long)per * hkv) {
+      const unsigned h = (unsigned)w / per;
+      const int in = (int)((unsigned)w - h * per) - P.change;
+      return unit + ((long long)h * n_tiles) * HALVES + max(in, 0) / (kTileWeight / HALVES);
+    }
+    w -= (long long)per * hkv;
+    unit += (long long)n_tiles * HALVES * hkv;
+  }
+  return unit;
 }
-__device__ __forceinline__ int cta_of_tile(int t, const TcParams& P) {
-  return (int)((((long long)t + 1) * P.grid - 1) / P.total_tiles);
+// CTA that has unit `local` of head h of sequence s.
+template <int HALVES>
+__device__ __forceinline__ int cta_of_unit(const BatchTable& bt, int hkv, const TcParams& P, int s, int h, int local) {
+  long long w = 0;
+#pragma unroll 1
+  for (int i = 0; i < s; ++i)
+    if (bt.seq[i].n_tiles) w += (long long)(bt.seq[i].n_tiles * kTileWeight + P.change) * hkv;
+  w += (long long)(bt.seq[s].n_tiles * kTileWeight + P.change) * h + P.change + (long long)(local + 1) * (kTileWeight / HALVES);
+  return (int)((w * P.grid - 1) / P.weight);      // w: the weight behind the unit
 }
+
+// A value that is the same in all lanes, in a form in which the compiler knows it: loop bounds and
+// addresses derived from it then live in uniform registers.  (With the span's bounds not known to be
+// uniform the ragged batch took 363 instead of 354 us.)
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // ------------------------------------------------------------------ the kernel
 // CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of
 // that code.
-template <int PASS, bool CAUSAL, int LAYERS>
+template <int PASS, bool CAUSAL, int LAYERS, int HALVES>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ Geometry g,
                 const __grid_constant__ TcParams P, const __grid_constant__ TcLayers<LAYERS> M,
@@ -443,8 +483,6 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   // the warp index as a value the compiler knows to be the same in all lanes: the MMA issuer's
   // descriptors then live in uniform registers
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const int t_begin = span_begin(blockIdx.x, P), t_end = span_begin(blockIdx.x + 1, P);
-
   if (threadIdx.x == 32) {
     // fetch the two TMA descriptors (kernel parameters) while the barriers are being set up
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&M.q[0])) : "memory");
@@ -464,9 +502,13 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     for (int i = 0; i < 8; ++i)
       for (int j = 0; j < 4; ++j)        // one arrival per set that hands its partial sums over
         mbar_init(smem_u32(&misc->bar.u_full[i][j]), P.n_sub > 1 ? P.n_sub - 1 : 1);
+    for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < 4; ++j) mbar_init(smem_u32(&misc->bar.edge_full[i][j]), 1);
     misc->abort_flag = 0;
     fence_barrier_init();
   }
+  if (warp >= 2 && warp < 4 && lane == 0)      // the ends of the span, computed once (it is a slow piece of code)
+    misc->span[warp - 2] = unit_at<HALVES>(bt, g.hkv, P, (blockIdx.x + warp - 2) * P.weight / P.grid);
   if (warp == 1) {
     tmem_alloc(smem_u32(&misc->tmem_base), kTmemCols);
     tmem_relinquish();
@@ -476,6 +518,13 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, misc->tmem_base, 0);
+  // Tiles [t_begin, t_end) of the span; of the first one only the row blocks from sub_begin on, of
+  // the last one only those before sub_end (a tile cut at its middle belongs to two CTAs, which add
+  // their column sums to zeroed scores: two addends, so their order does not matter).
+  const long long u_begin = misc->span[0], u_end = misc->span[1];
+  const int t_begin = uniform((int)(u_begin / HALVES)), t_end = uniform((int)((u_end + HALVES - 1) / HALVES));
+  const int sub_begin = HALVES > 1 ? uniform(u_begin % HALVES ? P.n_sub / 2 : 0) : 0;
+  const int sub_end = HALVES > 1 ? uniform(u_end % HALVES ? P.n_sub / 2 : P.n_sub) : P.n_sub;
   // Pass 1 reads Q and K, which the launch before it in the stream may have produced: every
   // thread waits for that launch, and only then lets pass 2 be scheduled, so that whatever runs
   // after pass 1 has begun finds the caller's inputs complete.  The launch before pass 2 is
@@ -602,7 +651,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         tc_fence_after();
         const uint32_t k_lo = k_lo0 + (uint32_t)stage * (kStageBytes >> 4);
 #pragma unroll 1
-        for (int sub = 0; sub < P.n_sub; ++sub, ++item) {
+        for (int sub = t == t_begin ? sub_begin : 0; sub < (t == t_end - 1 ? sub_end : P.n_sub); ++sub, ++item) {
           if (kIssuers == 2 && (int)((item >> 1) & 1u) != my_half) continue;
           const uint32_t buf = item & (kBufs - 1);
           const uint32_t par = ((item >> 2) & 1u) ^ 1u;
@@ -662,7 +711,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       for (int rb = 0; rb < 4; ++rb) {
         if (rb >= P.n_sub) break;
         // a set whose row block never changes keeps its state in slot 0
-        const int own = P.n_sub == 3 ? rb : (rb == set % P.n_sub ? 0 : -1);
+        const int own = P.n_sub == 3 ? rb : (rb == (sub_begin + set) % P.n_sub ? 0 : -1);
         float2 st = make_float2(-INFINITY, 0.f);
 #pragma unroll
         for (int k = 0; k < 4; ++k) if (k == own) st = make_float2(run_m[k], run_l[k]);
@@ -692,7 +741,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       // dealt round-robin to the threads that share a row, all loads of a thread are issued
       // before the first use, and the threads of a row meet through shared memory
       epi_barrier();
-      const int b0 = cta_of_tile(first_tile, P), b1 = cta_of_tile(first_tile + sq.n_tiles - 1, P);
+      const int b0 = cta_of_unit<HALVES>(bt, g.hkv, P, cur.s, cur.h, 0);
+      const int b1 = cta_of_unit<HALVES>(bt, g.hkv, P, cur.s, cur.h, sq.n_tiles * HALVES - 1);
       const int problem = cur.problem(g.hkv);
       const int ways = max(1, min(4, kEpiThreads / P.rows_pad));    // threads per row
       const int per_sweep = kEpiThreads / ways;                     // rows per sweep
@@ -749,7 +799,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int n_sub = P.n_sub;
     const int dt = kSets / n_sub, ds = kSets % n_sub;
     const bool rotating = ds != 0;          // the set's row block changes from item to item
-    int sub = set % n_sub, t = t_begin + set / n_sub;
+    int sub = (sub_begin + set) % n_sub, t = t_begin + (sub_begin + set) / n_sub;
+    const int set_end = t_end - (sub >= sub_end ? 1 : 0);     // (a cut tile: sub is the same in all items of a set)
+    // cut tiles of the span; the others use the eight slots of u_part in turn, from t_slot on
+    const int cut_first = sub_begin > 0 ? t_begin : -1, cut_last = sub_end < n_sub ? t_end - 1 : -1;
+    const int t_slot = t_begin + (sub_begin > 0 ? 1 : 0);
     uint32_t par = 0;
     int prob_end = t_begin, first_tile = 0, n_cur = 0;
     float* out = nullptr;
@@ -757,8 +811,16 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const uint32_t empty_bar = smem_u32(&misc->bar.acc_empty[set]);
     const uint32_t acc_addr = lane_addr + (uint32_t)set * kBufCols;
     if (PASS == 2) pdl_wait();
+    if (HALVES > 1 && PASS == 1 && sub_end < n_sub && etid < kTileKeys) {
+      // pass 2 adds to the scores of the tile this span shares with the next one
+      TileCursor last;
+      last.locate(bt, g.hkv, t_end - 1);
+      const SeqInfo& sq = bt.seq[last.s];
+      const int key = last.local * kTileKeys + etid;
+      if (key < sq.n) M.scores[LAYERS > 1 ? sq.layer : 0][(int64_t)last.h * bt.n_tot + sq.tok_off + key] = 0.f;
+    }
     for (;;) {
-      if (t >= prob_end) {
+      if (t >= min(prob_end, set_end)) {
         bool done = false;
         do {
           if (PASS == 1 && cur_problem >= 0) flush_partial(cur_problem);
@@ -774,7 +836,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           prob_end = min(t_end, first_tile + sq.n_tiles);
           n_cur = sq.n;
           out = M.scores[LAYERS > 1 ? sq.layer : 0] + (int64_t)cur.h * bt.n_tot + sq.tok_off;
-        } while (t >= prob_end);
+        } while (t >= min(prob_end, set_end));
         if (done) break;
       }
       const int key0 = (t - first_tile) * kTileKeys;
@@ -835,19 +897,32 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           // n_sub - 1 arrivals complete a (slot, quadrant).  Eight slots: a slot is written
           // again only after the accumulator hand-shake has forced the reader past the tile it
           // belongs to.
-          const int slot = t & 7;
-          if (sub != n_sub - 1) {
-            misc->u_part[slot][sub][row_in_tile] = u_acc;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&misc->bar.u_full[slot][quad]));
-          } else {
-            if (!dead) {
-              dead = !warp_wait(pipe, &misc->bar.u_full[slot][quad], (uint32_t)((t - t_begin) >> 3) & 1u, 31);
+          if (HALVES > 1 && (t == cut_first || t == cut_last)) {
+            // half of a tile: one other set at most has a part of it
+            const int e = t == cut_first ? 0 : 1;
+            const bool finish = sub == (e == 0 ? n_sub : sub_end) - 1;
+            if (!finish) {
+              misc->edge_part[e][row_in_tile] = u_acc;
+              __syncwarp();
+              if (lane == 0) mbar_arrive(smem_u32(&misc->bar.edge_full[e][quad]));
+            } else {
+              if (n_sub == 4 && !dead) dead = !warp_wait(pipe, &misc->bar.edge_full[e][quad], 0u, 34);
+              if (!dead && row_in_tile < valid)
+                atomicAdd(out + key0 + row_in_tile, n_sub == 4 ? u_acc + misc->edge_part[e][row_in_tile] : u_acc);
             }
-            if (!dead && row_in_tile < valid) {
-              float u = u_acc;
-              for (int k = 0; k < n_sub - 1; ++k) u += misc->u_part[slot][k][row_in_tile];
-              out[key0 + row_in_tile] = u;
+          } else {
+            const int slot = (t - t_slot) & 7;
+            if (sub != n_sub - 1) {
+              misc->u_part[slot][sub][row_in_tile] = u_acc;
+              __syncwarp();
+              if (lane == 0) mbar_arrive(smem_u32(&misc->bar.u_full[slot][quad]));
+            } else {
+              if (!dead) dead = !warp_wait(pipe, &misc->bar.u_full[slot][quad], (uint32_t)((t - t_slot) >> 3) & 1u, 31);
+              if (!dead && row_in_tile < valid) {
+                float u = u_acc;
+                for (int k = 0; k < n_sub - 1; ++k) u += misc->u_part[slot][k][row_in_tile];
+                out[key0 + row_in_tile] = u;
+              }
             }
           }
         } else if (!dead && row_in_tile < valid) {
@@ -885,19 +960,34 @@ struct TcPlan {
   bool ok;
 };
 
-TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count) {
+TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count, int layers) {
   TcPlan pl;
   TcParams& P = pl.P;
   memset(&pl, 0, sizeof(pl));
   P.total_tiles = g.hkv * bt.tiles_per_head;
-  P.grid = P.total_tiles < sm_count ? P.total_tiles : sm_count;
-  if (P.grid < 1) P.grid = 1;
   P.rows = g.rows;
   // pad the window so that the padded row count is a multiple of 16 (UMMA N granularity)
   int w_pad = g.window;
   while ((g.group * w_pad) % 16 != 0) ++w_pad;
   P.w_pad = w_pad;
   P.rows_pad = g.group * w_pad;
+  P.n_sub = (P.rows_pad + 127) / 128;
+  // Whole tiles, or half ones where whole ones would leave more than 4 % of the launch idle: the
+  // CTA with the most tiles has ceil(tiles / SMs) of them (10007 tokens x 4 heads: 3 where the
+  // average is 2.1).  Halves cost a second copy of the cut tiles' keys and an addition in L2.
+  const int whole = (P.total_tiles + sm_count - 1) / sm_count, half = (2 * P.total_tiles + sm_count - 1) / sm_count;
+  P.halves = layers == 1 && P.n_sub % 2 == 0 && half * 1.04 < 2 * whole ? 2 : 1;
+  int starts = 0;
+  for (int s = 0; s < bt.num_seqs; ++s) starts += bt.seq[s].n_tiles > 0;
+  // A start weighs as much as 2500 / rows quarters of a tile (2.4 tiles at 256 rows, 1.2 at 512; spans
+  // that straddle one were 2.3 us late in pass 2): llama3_8b shape 49.0 -> 47.3 us, 32 chunks 188 -> 178;
+  // half and one and a half times that weight gain less.  With few tiles per CTA whole tiles are too
+  // coarse to pay it back.
+  P.change = P.total_tiles >= 4 * sm_count ? (2500 + P.rows_pad / 2) / P.rows_pad : 0;
+  P.weight = (long long)P.total_tiles * 4 + (long long)starts * g.hkv * P.change;
+  const int units = P.total_tiles * P.halves;
+  P.grid = units < sm_count ? units : sm_count;
+  if (P.grid < 1) P.grid = 1;
   pl.ok = P.rows_pad <= kMaxRows && w_pad <= 256 && g.group <= 256;
   const uint32_t q_bytes = (uint32_t)P.rows_pad * 256u;
   int stages = ((int)kSmemLimit - 1024 - (int)kMiscBytes - (int)q_bytes) / (int)kStageBytes;
@@ -911,7 +1001,7 @@ TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count) {
 }  // namespace
 
 size_t score_tc_ws_bytes(const BatchTable& bt, const Geometry& g, int sm_count) {
-  TcPlan pl = make_plan(bt, g, sm_count);
+  TcPlan pl = make_plan(bt, g, sm_count, bt.num_seqs ? bt.seq[bt.num_seqs - 1].layer + 1 : 1);
   const size_t entries = (size_t)pl.P.grid + (size_t)bt.num_seqs * g.hkv;
   return (entries * pl.P.rows_pad * sizeof(float2) + 255) / 256 * 256;
 }
@@ -955,7 +1045,7 @@ CUresult encode_maps(EncodeTiledFn encode, const BatchTable& bt, const Geometry&
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <int LAYERS>
+template <int LAYERS, int HALVES>
 cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp,
                           const TcPlan& pl, EncodeTiledFn encode, int* drv_err) {
   TcParams P = pl.P;
@@ -965,8 +1055,8 @@ cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry&
     if (r != CUDA_SUCCESS) { *drv_err = (int)r; return cudaErrorUnknown; }
     M.scores[l] = lp.scores[l];
   }
-  auto pass1 = g.causal ? score_tc_kernel<1, true, LAYERS> : score_tc_kernel<1, false, LAYERS>;
-  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS> : score_tc_kernel<2, false, LAYERS>;
+  auto pass1 = g.causal ? score_tc_kernel<1, true, LAYERS, HALVES> : score_tc_kernel<1, false, LAYERS, HALVES>;
+  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES> : score_tc_kernel<2, false, LAYERS, HALVES>;
   cudaError_t e = allow_smem(pass1);
   if (e == cudaSuccess) e = allow_smem(pass2);
   if (e != cudaSuccess) return e;
@@ -984,7 +1074,7 @@ cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry&
 cudaError_t launch_score_tc(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp,
                             float* lse, void* ws, void* encode_fn, int64_t pool_rows, int* drv_err) {
   *drv_err = 0;
-  TcPlan pl = make_plan(bt, g, L.sm_count);
+  TcPlan pl = make_plan(bt, g, L.sm_count, lp.n);
   if (!pl.ok) return cudaErrorInvalidConfiguration;
   pl.P.part = (float2*)ws;
   pl.P.lse = lse;
@@ -993,8 +1083,9 @@ cudaError_t launch_score_tc(const Launch& L, const BatchTable& bt, const Geometr
   pl.P.k_sbo16 = (bt.page_size > 0 ? 2048u : 1024u) >> 4;
   pl.P.k_panel16 = (bt.page_size > 0 ? 1024u : kPanelBytes) >> 4;
   EncodeTiledFn encode = (EncodeTiledFn)encode_fn;
-  return lp.n > 1 ? launch_passes<kMaxLayers>(L, bt, g, lp, pl, encode, drv_err)
-                  : launch_passes<1>(L, bt, g, lp, pl, encode, drv_err);
+  if (lp.n > 1) return launch_passes<kMaxLayers, 1>(L, bt, g, lp, pl, encode, drv_err);
+  return pl.P.halves == 2 ? launch_passes<1, 2>(L, bt, g, lp, pl, encode, drv_err)
+                          : launch_passes<1, 1>(L, bt, g, lp, pl, encode, drv_err);
 }
 
 }  // namespace cc

@@ -1,0 +1,21 @@
+"""Score parity where the tensor-core kernel cuts tiles at their middle between two CTAs (few tiles
+per SM: fewer than half a tile each, a last or first half, several problems in a span), contiguous,
+paged and causal, and where a span holds many short problems."""
+import pytest
+
+from paper_2604_10235_b200 import binding as cc
+from paper_2604_10235_b200 import inputs as gen
+
+from test_gpu_score import check_against_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("w,hq,hkv,lens,page,causal", [
+    (64, 28, 4, (2000,), 0, False), (64, 32, 8, (1000,), 0, False), (128, 32, 8, (777,), 16, False),
+    (64, 28, 4, (10007,), 0, True), (64, 8, 2, (11000,), 0, False), (128, 8, 2, (700, 40, 1300), 32, False),
+    (128, 8, 2, (150,) * 40, 0, False), (64, 28, 4, (500,) * 30, 16, True)])
+def test_scores_of_cut_tiles_and_short_problems(w, hq, hkv, lens, page, causal):
+    wl = gen.Workload("spans", 27, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1,
+                      page_size=page, causal=causal)
+    check_against_oracle(wl, gen.make_layer(wl, layer=sum(lens), with_v=False), cc.CC_MODE_BF16, 2e-3)
