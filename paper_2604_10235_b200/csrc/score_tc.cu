@@ -972,11 +972,12 @@ TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count, int laye
   P.w_pad = w_pad;
   P.rows_pad = g.group * w_pad;
   P.n_sub = (P.rows_pad + 127) / 128;
-  // Whole tiles, or half ones where whole ones would leave more than 4 % of the launch idle: the
-  // CTA with the most tiles has ceil(tiles / SMs) of them (10007 tokens x 4 heads: 3 where the
-  // average is 2.1).  Halves cost a second copy of the cut tiles' keys and an addition in L2.
+  // Whole tiles, or half ones where the CTA with the most whole tiles, ceil(tiles / SMs) of them,
+  // has a tenth more than that in halves (10007 tokens x 4 heads: 3 where the average is 2.1, 2.5 in
+  // halves).  Not below two tiles per SM: half of a lone tile occupies half of the epilogue sets,
+  // and the cut tiles' keys are loaded twice (2546 tokens x 8 heads: 20.2 -> 21.7 us with halves).
   const int whole = (P.total_tiles + sm_count - 1) / sm_count, half = (2 * P.total_tiles + sm_count - 1) / sm_count;
-  P.halves = layers == 1 && P.n_sub % 2 == 0 && half * 1.04 < 2 * whole ? 2 : 1;
+  P.halves = layers == 1 && P.n_sub % 2 == 0 && P.total_tiles > 2 * sm_count && half * 1.1 < 2 * whole ? 2 : 1;
   int starts = 0;
   for (int s = 0; s < bt.num_seqs; ++s) starts += bt.seq[s].n_tiles > 0;
   // A start weighs as much as 2500 / rows quarters of a tile (2.4 tiles at 256 rows, 1.2 at 512; spans

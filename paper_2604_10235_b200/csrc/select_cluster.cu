@@ -38,6 +38,7 @@ namespace cc {
 
 namespace {
 
+constexpr int kUnroll = 2;                // of the passes over a run (deeper grows the code, which is cold here)
 constexpr int kBinBits = 10;
 constexpr int kBins = 1 << kBinBits;
 constexpr int kCand = 512;                // candidates of the cut-off bin that are ranked directly
@@ -205,16 +206,10 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
   if (threadIdx.x == 0) sm.n_own = 0;     // (published by the barriers below)
   if (threadIdx.x < 256) sm.sub[threadIdx.x] = 0;
   unsigned below = 0;                     // this thread's share of above_before
-  auto before_sums = [&](unsigned gt, unsigned eq) {
-    if (c.C == 1) return;
-    gt += below;
-    c.block_sum2(gt, eq);
-    cut.above_before += gt;
-    cut.tied_before += eq;
-  };
   const int sh = __clz(range);
   unsigned prefix = 0, remaining = R;     // resolved high bits of the shifted keys; rank inside them
   int shift = 32;                         // ... bits [31, shift)
+  bool rank_keys = false;                 // the bin's keys have to be listed and ranked
 #pragma unroll 1
   for (;;) {
     const int bits = min(kBinBits, shift), top = shift;
@@ -225,7 +220,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       for (int i = threadIdx.x; i < kBins; i += THREADS) h[i] = 0;
       __syncthreads();
     }
-#pragma unroll 4
+#pragma unroll kUnroll
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len)) continue;
@@ -278,19 +273,17 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       cut.whole = true;
       cut.above = R;
       cut.above_before = in_bin_before;
-      before_sums(0u, 0u);
-      return cut;
+      break;
     }
     cut.above = R - remaining;
     if (shift == 0) {                     // every bit resolved: the bin is one key value
       cut.tied_before = in_bin_before;
-      before_sums(0u, 0u);
-      return cut;
+      break;
     }
-    if (in_bin <= (unsigned)(kCand - 1) * max_len) break;
+    if (in_bin <= (unsigned)(kCand - 1) * max_len) { rank_keys = true; break; }
     // a crowded bin is often a single value (equal distances, clamped scores): look before refining
     unsigned lo_k = 0xffffffffu, hi_k = 0u;
-#pragma unroll 4
+#pragma unroll kUnroll
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len) || (((key - kmin) << sh) >> shift) != (prefix >> shift)) continue;
@@ -310,89 +303,93 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     if (lo_k == hi_k) {
       cut.T = lo_k;
       cut.tied_before = in_bin_before;
-      before_sums(0u, 0u);
-      return cut;
+      break;
     }
   }
+  unsigned gt_before = below, eq_before = 0;
+  if (rank_keys) {
 
-  // the bin's keys, listed per CTA and read by all of them in rank order
-#pragma unroll 4
-  for (int li = lo + lane; li < hi; li += 32) {
-    unsigned key, len;
-    if (!get(li, key, len)) continue;
-    if ((((key - kmin) << sh) >> shift) == (prefix >> shift)) sm.own[atomicAdd(&sm.n_own, 1u)] = Cand{key, len};
-  }
-  c.sync_all();
-  unsigned first[kMaxCluster + 1];        // places of the CTAs' lists in the common one
-  first[0] = 0;
-#pragma unroll
-  for (int r = 0; r < kMaxCluster; ++r) first[r + 1] = r < c.C ? *c.peer(&sm.n_own, r) : 0u;
-#pragma unroll
-  for (int r = 0; r < kMaxCluster; ++r) first[r + 1] += first[r];
-  const unsigned total = first[kMaxCluster];
-  unsigned before = 0;
-#pragma unroll
-  for (int r = 0; r < kMaxCluster; ++r)
-    if (r == c.rank) before = first[r];
-  const int sub_bits = min(8, shift), sub_shift = shift - sub_bits;
-  auto sub_bin = [&](unsigned key) { return (((key - kmin) << sh) >> sub_shift) & ((1u << sub_bits) - 1u); };
-  const bool refine = total > 64;         // narrow a long list down by the next bits before ranking
-  for (unsigned i = threadIdx.x; i < total; i += THREADS) {
-    int r = 0;
-    unsigned at = i;
-#pragma unroll
-    for (int k = 1; k < kMaxCluster; ++k)
-      if (i >= first[k]) { r = k; at = i - first[k]; }
-    const Cand o = c.peer(sm.own, r)[at];
-    sm.all[i] = o;
-    if (refine) atomicAdd(&sm.sub[sub_bin(o.key)], o.len);
-  }
-  __syncthreads();
-  unsigned sub = 0;
-  if (refine) {                           // every warp finds the sub-bin for itself (lane l: bins 255 - 8 l ...)
-    unsigned n8[8], sum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { n8[i] = sm.sub[255 - 8 * lane - i]; sum += n8[i]; }
-    unsigned inc = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += t;
+    // the bin's keys, listed per CTA and read by all of them in rank order
+#pragma unroll kUnroll
+    for (int li = lo + lane; li < hi; li += 32) {
+      unsigned key, len;
+      if (!get(li, key, len)) continue;
+      if ((((key - kmin) << sh) >> shift) == (prefix >> shift)) sm.own[atomicAdd(&sm.n_own, 1u)] = Cand{key, len};
     }
-    unsigned excl = inc - sum;
-    bool found = false;
+    c.sync_all();
+    unsigned first[kMaxCluster + 1];        // places of the CTAs' lists in the common one
+    first[0] = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (excl < remaining && remaining <= excl + n8[i]) { sub = 255 - 8 * lane - i; found = true; }
-      excl += n8[i];
+    for (int r = 0; r < kMaxCluster; ++r) first[r + 1] = r < c.C ? *c.peer(&sm.n_own, r) : 0u;
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r) first[r + 1] += first[r];
+    const unsigned total = first[kMaxCluster];
+    unsigned before = 0;
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r)
+      if (r == c.rank) before = first[r];
+    const int sub_bits = min(8, shift), sub_shift = shift - sub_bits;
+    auto sub_bin = [&](unsigned key) { return (((key - kmin) << sh) >> sub_shift) & ((1u << sub_bits) - 1u); };
+    const bool refine = total > 64;         // narrow a long list down by the next bits before ranking
+    for (unsigned i = threadIdx.x; i < total; i += THREADS) {
+      int r = 0;
+      unsigned at = i;
+#pragma unroll
+      for (int k = 1; k < kMaxCluster; ++k)
+        if (i >= first[k]) { r = k; at = i - first[k]; }
+      const Cand o = c.peer(sm.own, r)[at];
+      sm.all[i] = o;
+      if (refine) atomicAdd(&sm.sub[sub_bin(o.key)], o.len);
     }
-    sub = __shfl_sync(0xffffffffu, sub, __ffs(__ballot_sync(0xffffffffu, found)) - 1);
-  }
-  // a warp ranks one key against all others
-  for (unsigned i = threadIdx.x >> 5; i < total; i += THREADS / 32) {
-    const unsigned key = sm.all[i].key;
-    if (refine && sub_bin(key) != sub) continue;
-    unsigned gt = 0, eq = 0;
-    for (unsigned j = lane; j < total; j += 32) {
-      const Cand o = sm.all[j];
-      gt += o.key > key ? o.len : 0u;
-      eq += o.key == key ? o.len : 0u;
+    __syncthreads();
+    unsigned sub = 0;
+    if (refine) {                           // every warp finds the sub-bin for itself (lane l: bins 255 - 8 l ...)
+      unsigned n8[8], sum = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { n8[i] = sm.sub[255 - 8 * lane - i]; sum += n8[i]; }
+      unsigned inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      unsigned excl = inc - sum;
+      bool found = false;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (excl < remaining && remaining <= excl + n8[i]) { sub = 255 - 8 * lane - i; found = true; }
+        excl += n8[i];
+      }
+      sub = __shfl_sync(0xffffffffu, sub, __ffs(__ballot_sync(0xffffffffu, found)) - 1);
     }
-    gt = __reduce_add_sync(0xffffffffu, gt);
-    eq = __reduce_add_sync(0xffffffffu, eq);
-    if (lane == 0 && gt < remaining && remaining <= gt + eq) { sm.bcast[0] = key; sm.bcast[1] = gt; }
-  }
-  __syncthreads();
-  cut.T = sm.bcast[0];
-  cut.above += sm.bcast[1];
-  unsigned gt = 0, eq = 0;
-  if (c.C > 1)
+    // a warp ranks one key against all others
+    for (unsigned i = threadIdx.x >> 5; i < total; i += THREADS / 32) {
+      const unsigned key = sm.all[i].key;
+      if (refine && sub_bin(key) != sub) continue;
+      unsigned gt = 0, eq = 0;
+      for (unsigned j = lane; j < total; j += 32) {
+        const Cand o = sm.all[j];
+        gt += o.key > key ? o.len : 0u;
+        eq += o.key == key ? o.len : 0u;
+      }
+      gt = __reduce_add_sync(0xffffffffu, gt);
+      eq = __reduce_add_sync(0xffffffffu, eq);
+      if (lane == 0 && gt < remaining && remaining <= gt + eq) { sm.bcast[0] = key; sm.bcast[1] = gt; }
+    }
+    __syncthreads();
+    cut.T = sm.bcast[0];
+    cut.above += sm.bcast[1];
     for (unsigned i = threadIdx.x; i < before; i += THREADS) {
       const Cand o = sm.all[i];
-      if (o.key > cut.T) gt += o.len;
-      if (o.key == cut.T) eq += o.len;
+      if (o.key > cut.T) gt_before += o.len;
+      if (o.key == cut.T) eq_before += o.len;
     }
-  before_sums(gt, eq);
+  }
+  if (c.C > 1) {
+    c.block_sum2(gt_before, eq_before);
+    cut.above_before += gt_before;
+    cut.tied_before += eq_before;
+  }
   return cut;
 }
 
@@ -625,22 +622,31 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     }
   }
 
-  // ---- stage 1: cap on protected items (longest prefix by (prior desc, index asc) within B_span)
-  if (capped && forced_tokens > (unsigned)q.span_cap) {
+  // ---- stage 1: cap on protected items (longest prefix by (prior desc, index asc) within B_span), and
+  // stage 2: cut-off among the unprotected items, through one copy of the search
+  const bool over_cap = capped && forced_tokens > (unsigned)q.span_cap;
+  Cut cut{0u, false, 0u, 0u, 0u};
+#pragma unroll 1
+  for (int stage = over_cap ? 1 : 2; stage <= 2; ++stage) {
+    const bool first = stage == 1;
+    if (!first && forced_tokens >= keep) break;       // protected items alone fill the budget: first B in order
     const unsigned cap = (unsigned)q.span_cap;
-    const Cut cut = find_cut(c, lo, hi, cap + 1u, pri_lo, pri_hi, (unsigned)cs, false,
-                             [&](int li, unsigned& key, unsigned& len) {
-                               if (!flags[li]) return false;
-                               key = mono_key(item_prior(li));
-                               len = item_len(li);
-                               return true;
-                             });
+    cut = find_cut(c, lo, hi, first ? cap + 1u : keep - forced_tokens, first ? pri_lo : key_lo, first ? pri_hi : key_hi,
+                   (unsigned)cs, !first, [&](int li, unsigned& key, unsigned& len) {
+                     if ((flags[li] != 0) != first) return false;
+                     key = first ? mono_key(item_prior(li)) : keys[li];
+                     len = item_len(li);
+                     return true;
+                   });
+    if (!first) break;
     unsigned ties = 0, none = 0;
+#pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32)
       if (flags[li] && mono_key(item_prior(li)) == cut.T) ties += item_len(li);
     ties = __reduce_add_sync(0xffffffffu, ties);
     c.warps_before2(ties, none);
     unsigned tie_run = cut.tied_before + ties, kept = 0;
+#pragma unroll 1
     for (int l0 = lo; l0 < hi; l0 += 32) {
       const int li = l0 + lane;
       const bool forced = li < hi && flags[li];
@@ -668,18 +674,8 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
       }
     }
   }
-
-  // ---- stage 2: cut-off among the unprotected items
-  const bool ties_are_forced = forced_tokens >= keep;   // protected items alone fill the budget: first B in order
-  Cut cut{0u, false, 0u, 0u, 0u};
-  if (!ties_are_forced)
-    cut = find_cut(c, lo, hi, keep - forced_tokens, key_lo, key_hi, (unsigned)cs, true,
-                   [&](int li, unsigned& key, unsigned& len) {
-                     if (flags[li]) return false;
-                     key = keys[li];
-                     len = item_len(li);
-                     return true;
-                   });
+  const bool ties_are_forced = forced_tokens >= keep;
+  if (ties_are_forced) cut = Cut{0u, false, 0u, 0u, 0u};
   const unsigned tie_budget = ties_are_forced ? keep : keep - forced_tokens - cut.above;
   // last read of a peer's shared memory is done: announce it now, wait for the peers at the
   // very end, and write the indices in between
@@ -786,10 +782,11 @@ cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& 
 
 // Time of a launch with clusters of 1 << lc CTAs of `threads` threads, in us, from launches of one wave
 // on a B200 (n = 2048 .. 131072 items, 2 .. 256 problems): a constant that grows with what the
-// exchanges of wider clusters cost, 1 us more for the barriers of 1024 threads, and 0.48 (0.6) us
-// per item of a thread of 512 (1024).  A chunk's tokens count a fifth of an item each.  A CTA of 1024
-// threads fills an SM, CTAs of 512 share it in pairs; a cluster sits inside one GPC, so fewer CTAs run
-// at a time in wide ones.
+// exchanges of wider clusters cost, something for the barriers of 1024 threads (less than in replays
+// of this kernel alone: behind other kernels its code is cold, which more warps hide better), and
+// 0.48 (0.6) us per item of a thread of 512 (1024).  A chunk's tokens count a fifth of an item each.
+// A CTA of 1024 threads fills an SM, CTAs of 512 share it in pairs; a cluster sits inside one GPC, so
+// fewer CTAs run at a time in wide ones.
 double launch_cost(const BatchTable& bt, int hkv, int lc, int threads) {
   static const double base[4] = {6.1, 7.7, 7.8, 8.6};
   static const int room[4] = {148, 148, 128, 96};
@@ -798,7 +795,7 @@ double launch_cost(const BatchTable& bt, int hkv, int lc, int threads) {
   const int ctas = bt.num_seqs * hkv * c, fit = threads == 512 ? 2 * room[lc] : room[lc];
   const int waves = (ctas + fit - 1) / fit;
   const double slope = threads == 1024 ? 0.6 : (ctas > room[lc] ? 0.96 : 0.48);
-  return waves * (base[lc] + (threads == 1024 ? 1.0 : 0.0) + slope * per_thread);
+  return waves * (base[lc] + (threads == 512 ? 0.0 : bt.chunk > 1 ? 1.0 : lc == 0 ? 0.8 : 0.3) + slope * per_thread);
 }
 
 // The cheapest shape; cluster 0 when a sequence has more items than the widest cluster holds.
