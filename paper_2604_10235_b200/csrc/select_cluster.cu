@@ -24,6 +24,10 @@
 // contiguous run of items per thread, before): ragged batch of 64 problems, 8 k to 64 k tokens
 // 52.6 -> 28.6 us, 256 problems of 2 k with a cap 19.0 -> 12.6, 32768 tokens x 8 heads 17.3 -> 12.6
 // (7.4 -> 6.4 when the protected tokens fill the budget), 2048 x 2 9.6 -> 6.9.
+// Loops are rolled unless what they hold in registers is the point: behind the score kernel this
+// kernel's instructions come from L2, and a CTA of a small problem runs each of them once or twice.
+// 75 -> 48 KB of code: whole call on 1691 tokens x 4 heads 22.4 -> 21.3 us, 2048 x 2 20.9 -> 19.9,
+// 8192 with a causal window 41.1 -> 40.1; the widest slices (8192 items per CTA) give back 0.5 us.
 #include <cooperative_groups.h>
 #include <string.h>
 
@@ -38,13 +42,11 @@ namespace cc {
 
 namespace {
 
-constexpr int kUnroll = 2;                // of the passes over a run (deeper grows the code, which is cold here)
 constexpr int kBinBits = 10;
 constexpr int kBins = 1 << kBinBits;
 constexpr int kCand = 512;                // candidates of the cut-off bin that are ranked directly
 constexpr int kMaxCluster = 8;
 constexpr int kMaxWarps = 32;
-constexpr int kCtaItems = 32768;          // items one CTA of 1024 threads keeps in shared memory: 32 per thread
 constexpr int kStep = 4;                  // items a thread pools per part of the slice
 constexpr int kMaxHalf = 32;              // half of the widest pooling window, rounded up
 constexpr int kWords = 6;                 // words of an exchange
@@ -193,6 +195,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
   Cut cut{kmin, false, 0u, 0u, 0u};
   if (range == 0) {                       // one key value: everything is tied
     unsigned mine = 0;
+#pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (get(li, key, len)) mine += len;
@@ -200,6 +203,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     if (c.C == 1) return cut;
     unsigned w[kWords] = {c.block_sum(mine), 0u, 0u, 0u, 0u, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
+#pragma unroll 1
     for (int r = 0; r < c.rank; ++r) cut.tied_before += x[r][0];
     return cut;
   }
@@ -217,10 +221,11 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     // two copies: a copy is cleared again only after the barrier of the histogram in between
     unsigned* h = sm.hist[c.n_hist & 1u];
     if (c.n_hist++ > 0) {                 // (the first one is clear from the start)
+#pragma unroll 1
       for (int i = threadIdx.x; i < kBins; i += THREADS) h[i] = 0;
       __syncthreads();
     }
-#pragma unroll kUnroll
+#pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len)) continue;
@@ -283,7 +288,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     if (in_bin <= (unsigned)(kCand - 1) * max_len) { rank_keys = true; break; }
     // a crowded bin is often a single value (equal distances, clamped scores): look before refining
     unsigned lo_k = 0xffffffffu, hi_k = 0u;
-#pragma unroll kUnroll
+#pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len) || (((key - kmin) << sh) >> shift) != (prefix >> shift)) continue;
@@ -295,6 +300,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     if (c.C > 1) {
       const unsigned w[kWords] = {lo_k, hi_k, 0u, 0u, 0u, 0u};
       const unsigned(*x)[kWords] = c.publish(w);
+#pragma unroll 1
       for (int r = 0; r < c.C; ++r) {
         lo_k = min(lo_k, x[r][0]);
         hi_k = max(hi_k, x[r][1]);
@@ -310,7 +316,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
   if (rank_keys) {
 
     // the bin's keys, listed per CTA and read by all of them in rank order
-#pragma unroll kUnroll
+#pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len)) continue;
@@ -331,6 +337,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     const int sub_bits = min(8, shift), sub_shift = shift - sub_bits;
     auto sub_bin = [&](unsigned key) { return (((key - kmin) << sh) >> sub_shift) & ((1u << sub_bits) - 1u); };
     const bool refine = total > 64;         // narrow a long list down by the next bits before ranking
+#pragma unroll 1
     for (unsigned i = threadIdx.x; i < total; i += THREADS) {
       int r = 0;
       unsigned at = i;
@@ -363,10 +370,12 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       sub = __shfl_sync(0xffffffffu, sub, __ffs(__ballot_sync(0xffffffffu, found)) - 1);
     }
     // a warp ranks one key against all others
+#pragma unroll 1
     for (unsigned i = threadIdx.x >> 5; i < total; i += THREADS / 32) {
       const unsigned key = sm.all[i].key;
       if (refine && sub_bin(key) != sub) continue;
       unsigned gt = 0, eq = 0;
+#pragma unroll 1
       for (unsigned j = lane; j < total; j += 32) {
         const Cand o = sm.all[j];
         gt += o.key > key ? o.len : 0u;
@@ -379,6 +388,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     __syncthreads();
     cut.T = sm.bcast[0];
     cut.above += sm.bcast[1];
+#pragma unroll 1
     for (unsigned i = threadIdx.x; i < before; i += THREADS) {
       const Cand o = sm.all[i];
       if (o.key > cut.T) gt_before += o.len;
@@ -391,44 +401,6 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     cut.tied_before += eq_before;
   }
   return cut;
-}
-
-// Pooled values of four neighbouring items from the staged scores w4[0] ..: windows of kW taps, the
-// first starting at w4[0].x.  Maxima share the taps all four windows have; averages are
-// left-to-right sums, then one division.
-template <int kW>
-__device__ __forceinline__ void pool4(const float4* w4, int kind, float (&v)[4]) {
-  constexpr int kVecs = (kW + 3 + 3) / 4;
-  float a[4 * kVecs];
-#pragma unroll
-  for (int i = 0; i < kVecs; ++i) {
-    const float4 x = w4[i];
-    a[4 * i] = x.x; a[4 * i + 1] = x.y; a[4 * i + 2] = x.z; a[4 * i + 3] = x.w;
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    v[j] = a[j];
-    if (kind == CC_POOL_MAX) {
-#pragma unroll
-      for (int d = 1; d < kW; ++d) v[j] = fmaxf(v[j], a[j + d]);
-    } else if (kW > 1) {
-#pragma unroll
-      for (int d = 1; d < kW; ++d) v[j] = __fadd_rn(v[j], a[j + d]);
-      v[j] = __fdiv_rn(v[j], (float)kW);
-    }
-  }
-}
-__device__ __forceinline__ void pool4_any(const float* w, int kind, int width, float (&v)[4]) {
-#pragma unroll 1
-  for (int j = 0; j < 4; ++j) {
-    float x = w[j];
-    for (int d = 1; d < width; ++d) x = kind == CC_POOL_MAX ? fmaxf(x, w[j + d]) : __fadd_rn(x, w[j + d]);
-    const float y = kind == CC_POOL_MAX ? x : __fdiv_rn(x, (float)width);
-    if (j == 0) v[0] = y;
-    if (j == 1) v[1] = y;
-    if (j == 2) v[2] = y;
-    if (j == 3) v[3] = y;
-  }
 }
 
 // CHUNKED instantiations rank fixed chunks of bt.chunk tokens; the others are compiled for
@@ -477,10 +449,12 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     if (cs == 1) return p[i];
     float pr = p[(int64_t)i * cs];
     const int end = min(q.n, (i + 1) * cs);
+#pragma unroll 1
     for (int j = i * cs + 1; j < end; ++j) pr = fmaxf(pr, p[j]);
     return pr;
   };
 
+#pragma unroll 1
   for (int i = threadIdx.x; i < kBins; i += THREADS) sm.hist[0][i] = 0;
   // Totals collected while loading: protected weight, key range of the unprotected items (of all
   // items when a cap may still strip some of their protection), range of the protected items'
@@ -559,13 +533,29 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
         const int l4 = c0 + 4 * (int)threadIdx.x;
         if (l4 < cta_items) {
           const float4 pr = *reinterpret_cast<const float4*>(keys + l4);       // the parked priors
-          const float4* w4 = reinterpret_cast<const float4*>(ub) + threadIdx.x;
           float v[4];
-          if (half == 3) pool4<7>(w4, P.pool_kind, v);
-          else if (half == 2) pool4<5>(w4, P.pool_kind, v);
-          else if (half == 1) pool4<3>(w4, P.pool_kind, v);
-          else if (half == 0) pool4<1>(w4, P.pool_kind, v);
-          else pool4_any(ub + 4 * threadIdx.x, P.pool_kind, 2 * half + 1, v);
+          // four windows that move one tap on per step; averages are left-to-right sums, then one division
+          const float* w = ub + 4 * threadIdx.x;
+          float4 x = *reinterpret_cast<const float4*>(w);
+          v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+          if (P.pool_kind == CC_POOL_MAX) {
+#pragma unroll 1
+            for (int d = 1; d <= 2 * half; ++d) {
+              x = make_float4(x.y, x.z, x.w, w[d + 3]);
+              v[0] = fmaxf(v[0], x.x); v[1] = fmaxf(v[1], x.y); v[2] = fmaxf(v[2], x.z); v[3] = fmaxf(v[3], x.w);
+            }
+          } else if (half > 0) {
+#pragma unroll 1
+            for (int d = 1; d <= 2 * half; ++d) {
+              x = make_float4(x.y, x.z, x.w, w[d + 3]);
+              v[0] = __fadd_rn(v[0], x.x); v[1] = __fadd_rn(v[1], x.y); v[2] = __fadd_rn(v[2], x.z); v[3] = __fadd_rn(v[3], x.w);
+            }
+#pragma unroll 1
+            for (int j = 0; j < 4; ++j) {       // (rotates: one copy of the division)
+              const float y = __fdiv_rn(v[0], (float)(2 * half + 1));
+              v[0] = v[1]; v[1] = v[2]; v[2] = v[3]; v[3] = y;
+            }
+          }
           store4(l4, v, pr);
         }
       }
@@ -575,6 +565,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
         // chunk sum in token order; the loads of eight tokens are issued before they are used
         const int t0 = (cta_lo + li) * cs, t1 = min(q.n, t0 + cs);
         float val = 0.0f, pr = -INFINITY;
+#pragma unroll 1
         for (int j0 = t0; j0 < t1; j0 += 8) {
           float a[8], b[8];
 #pragma unroll
@@ -612,6 +603,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     const unsigned w[kWords] = {forced_tokens, key_lo, key_hi, pri_lo, pri_hi, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
     forced_tokens = 0;
+#pragma unroll 1
     for (int r = 0; r < c.C; ++r) {
       if (r == c.rank) forced_before = forced_tokens;
       forced_tokens += x[r][0];
@@ -667,6 +659,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
         const unsigned w[kWords] = {forced_tokens, 0u, 0u, 0u, 0u, 0u};
         const unsigned(*x)[kWords] = c.publish(w);
         forced_tokens = forced_before = 0;
+#pragma unroll 1
         for (int r = 0; r < c.C; ++r) {
           if (r == c.rank) forced_before = forced_tokens;
           forced_tokens += x[r][0];
@@ -702,7 +695,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   // land before every exchange of the CTAs.
   float* fo = FUSED ? P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off + cta_lo : nullptr;
   unsigned defs = 0, ties = 0;
-#pragma unroll 4
+#pragma unroll 2
   for (int k = 0; k < run / 32; ++k) {
     const int li = lo + k * 32 + lane;
     bool def, tie;
@@ -734,11 +727,13 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     const unsigned len = item_len(li), pos = def_before + min(tie_before, tie_budget);
     const unsigned take = !tie ? len : (tie_before < tie_budget ? min(len, tie_budget - tie_before) : 0u);
     const int tok0 = (cta_lo + li) * cs;
+#pragma unroll 1
     for (unsigned k = 0; k < take; ++k)
       if (pos + k < keep) out[pos + k] = tok0 + (int)k;
     return len;
   };
   if (run / 32 > 10) {           // a step per lane
+#pragma unroll 1
     for (unsigned left = defs | ties; left; left &= left - 1u) {
       const int bit = __ffs(left) - 1;
       const bool tie = ties >> bit & 1u;
