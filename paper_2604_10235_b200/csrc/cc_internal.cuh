@@ -32,7 +32,7 @@ struct SeqInfo {
 
 // Several layers of a batch go through one launch as further entries of the table: entry
 // layer * S + s is sequence s of that layer, its offsets into the per-layer arrays unchanged.
-constexpr int kMaxLayers = 16;       // layers per launch
+constexpr int kMaxLayers = 32;       // layers per launch
 
 struct BatchTable {
   int num_seqs;      // entries: sequences x layers of the launch
