@@ -53,11 +53,11 @@ struct Plan {
 
 // Layers per launch of cc_compress_layers.  Launches that share a prologue, a pipeline fill and a tail
 // are what short prompts gain from most, and a fuller last wave pays even where the keys of a launch
-// no longer fit L2 (nothing here is bound by reading them twice).  96 MB of keys and 16 layers -> 512 MB
+// no longer fit L2 (nothing here is bound by reading them twice).  96 MB of keys and 16 layers -> 256 MB
 // and 32 layers per launch, us: 32 layers x 4096 tokens x 8 heads 461 -> 442, 32 x 8192 with 32 query
-// tokens 434 -> 352, 8 x 32768 507 -> 403.  The limit bounds the workspace (a 32nd of the keys); the
-// doublings after 256 MB gained 0 to 3 %.
-constexpr size_t kGroupKeyBytes = 512u << 20;
+// tokens 434 -> 359, 8 x 32768 507 -> 405.  The workspace, which a call on one layer gets too, grows by
+// a 32nd of the limit, 8 MB; 512 MB and more gain another 0 to 3 %.
+constexpr size_t kGroupKeyBytes = 256u << 20;
 int layers_per_launch(const cc_layer_desc* d, const BatchTable& bt, const Geometry& g) {
   if (d->compute_mode != CC_MODE_BF16 || d->fill_mode != CC_FILL_ATTENTION || bt.n_tot == 0 || bt.b_tot == 0 ||
       select_cluster_size(bt, g.hkv) == 0)
