@@ -14,6 +14,7 @@
 // arithmetic), f32 154 us = 6.8 TB/s.  Keeping the loads of the next batch in flight during the
 // arithmetic needs 64 registers and costs a resident CTA: slower for bf16 (97 us).
 #include <cooperative_groups.h>
+#include <float.h>
 #include <math.h>
 
 #include "cc_internal.cuh"
@@ -48,18 +49,23 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   return d;
 }
 
+// The maximum starts at the lowest finite value, not at -inf: while a thread has met only -inf (or
+// values that scale to it: masked logits) the arguments x log2(e) - m are then -inf and not
+// -inf + inf.  What the clamp of the FMA-pipe exponentials leaves in the sum meanwhile is multiplied by
+// 0 when the maximum is raised or merged.
+constexpr float kNoMax = -FLT_MAX;
+
 struct Running {
   float m, s;       // maximum (base-2 units) and sum of 2^(x log2(e) - m)
   __device__ __forceinline__ void raise(float top) {
     const float vm = top * kLog2e;
     if (vm > m) {
-      s *= ex2(m - vm);          // m = -inf at the start: the factor is 0 and s is 0
+      s *= ex2(m - vm);          // m = kNoMax at the start: the factor is 0
       m = vm;
     }
   }
   __device__ __forceinline__ void merge(float om, float os) {
     const float nm = fmaxf(m, om);
-    if (nm == -INFINITY) return;
     s = s * ex2(m - nm) + os * ex2(om - nm);
     m = nm;
   }
@@ -150,7 +156,7 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
   pdl_wait();
   const int chunk = row / num_tokens, t = row % num_tokens;
   const T* x = logits + (int64_t)chunk * stride_chunk + (int64_t)t * stride_token;
-  Running r{-INFINITY, 0.f};
+  Running r{kNoMax, 0.f};
   const int head = min(vocab, (int)((16u - (unsigned)((uintptr_t)x & 15u)) & 15u) / (int)sizeof(T));
   const T* xv = x + head;
   const int n_vec = (vocab - head) / kVecWidth;
@@ -187,7 +193,7 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) { sm_m[warp] = r.m; sm_s[warp] = r.s; }
   __syncthreads();
-  Running all{-INFINITY, 0.f};
+  Running all{kNoMax, 0.f};
   if (threadIdx.x == 0)
     for (int w = 0; w < kThreads / 32; ++w) all.merge(sm_m[w], sm_s[w]);
   if (split) {
@@ -204,7 +210,7 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
     const int target = targets[t];
     float out = __int_as_float(0x7fc00000);                   // NaN for an invalid token id
     if (target >= 0 && target < vocab)
-      out = (all.m + log2f(all.s)) * kLn2 - Vec<T>::one(x + target);
+      out = ((all.m > kNoMax ? all.m : -INFINITY) + log2f(all.s)) * kLn2 - Vec<T>::one(x + target);
     else
       report_error(status, CC_ERR_DEVICE_FLAG, 600);
     nll[row] = out;
