@@ -9,7 +9,7 @@
 // they arrive, and keeps a running (maximum, sum) in base 2 that is rescaled only when a pair
 // raises the maximum; the threads' pairs are merged with shuffles.  With 2-byte logits the issue
 // slots come close to the memory time, so scaling and sums are packed f32x2 operations, maxima of
-// bf16 logits are taken on the packed words, and one pair of exponentials in eight is evaluated
+// bf16 logits are taken on the packed words, and (POLY) one pair of exponentials in eight is evaluated
 // on the FMA pipe.  32 x 64 rows of 128256 logits: bf16 90 us = 5.84 TB/s (93 us with scalar
 // arithmetic), f32 154 us = 6.8 TB/s.  Keeping the loads of the next batch in flight during the
 // arithmetic needs 64 registers and costs a resident CTA: slower for bf16 (97 us).
@@ -118,7 +118,7 @@ template <> struct Vec<uint16_t> {       // bf16 bit patterns
   __device__ static float one(const uint16_t* p) { return __uint_as_float((uint32_t)*p << 16); }
 };
 // adds a batch of vectors
-template <typename T, int kN>
+template <bool POLY, typename T, int kN>
 __device__ __forceinline__ void add_batch(Running& run, const Vec<T> (&r)[kN]) {
   run.raise(Vec<T>::top(r));
   const uint64_t c2 = pack2(kLog2e, kLog2e), nm = pack2(-run.m, -run.m);
@@ -128,7 +128,7 @@ __device__ __forceinline__ void add_batch(Running& run, const Vec<T> (&r)[kN]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const uint64_t x = fma2(r[u].pair(i), c2, nm);
-      acc[i & 1] = add2(acc[i & 1], kN * 4 >= kPolyPairs && (u * 4 + i) % kPolyPairs == 1 ? ex2_pair_fma(x) : ex2_pair_sfu(x));
+      acc[i & 1] = add2(acc[i & 1], POLY && kN * 4 >= kPolyPairs && (u * 4 + i) % kPolyPairs == 1 ? ex2_pair_fma(x) : ex2_pair_sfu(x));
     }
   float a, b;
   unpack2(add2(acc[0], acc[1]), a, b);
@@ -140,7 +140,7 @@ template <typename T> constexpr int kBatch = sizeof(T) == 2 ? 8 : 4;   // 128 by
 // (parts divides `whole`, so clusters never mix the two), which merge their pairs in the first
 // one's shared memory.  A row may start anywhere on the element grid: the values before its first
 // and after its last 16-byte boundary (at most fourteen) are read one by one.
-template <typename T>
+template <typename T, bool POLY>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t stride_chunk,
                int64_t stride_token, int whole, int parts, const int32_t* __restrict__ targets,
@@ -172,13 +172,13 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
       Vec<T> taken[kGroup];
 #pragma unroll
       for (int g = 0; g < kGroup; ++g) taken[g] = raw[u + g];
-      add_batch<T, kGroup>(r, taken);
+      add_batch<POLY, T, kGroup>(r, taken);
     }
   }
   for (; i < i_end; i += kThreads) {
     Vec<T> raw[1];
     raw[0].load(xv + (int64_t)i * kVecWidth);
-    add_batch<T, 1>(r, raw);
+    add_batch<POLY, T, 1>(r, raw);
   }
   // the values before the first and after the last whole vector
   if (part == 0) {
@@ -273,10 +273,16 @@ cudaError_t launch_ppl_scores(const Launch& L, const void* logits, bool is_f32, 
   if (parts == 1) whole = rows;
   whole -= whole % parts;
   const unsigned grid = (unsigned)(whole + (rows - whole) * parts);
+  // The FMA pipe's exponentials (relative error 8e-5) are for bf16 rows on the 16-byte grid alone, where
+  // they take 1.6 % off the call (32 x 64 rows of 128256: 94.2 against 95.7 us).  f32 logits leave the
+  // special-function unit idle anyway (32 x 32 rows of 128256: 85.1 without, 86.5 us with them), and rows
+  // off the grid lose nothing (32 x 64 rows of 50257 bf16 logits: 46.5 / 46.9).
+  const bool poly = !is_f32 && (uintptr_t)logits % 16 == 0 && stride_chunk % 8 == 0 && stride_token % 8 == 0;
+  const auto bf16_kernel = poly ? ppl_nll_kernel<uint16_t, true> : ppl_nll_kernel<uint16_t, false>;
   const cudaError_t e = is_f32
-      ? launch_pdl(ppl_nll_kernel<float>, dim3(grid), dim3(kThreads), 0, L.stream, parts, (const float*)logits,
+      ? launch_pdl(ppl_nll_kernel<float, false>, dim3(grid), dim3(kThreads), 0, L.stream, parts, (const float*)logits,
                    num_tokens, vocab, stride_chunk, stride_token, whole, parts, targets, nll, L.status)
-      : launch_pdl(ppl_nll_kernel<uint16_t>, dim3(grid), dim3(kThreads), 0, L.stream, parts,
+      : launch_pdl(bf16_kernel, dim3(grid), dim3(kThreads), 0, L.stream, parts,
                    (const uint16_t*)logits, num_tokens, vocab, stride_chunk, stride_token, whole, parts, targets,
                    nll, L.status);
   if (e != cudaSuccess) return e;

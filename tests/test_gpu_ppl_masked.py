@@ -39,3 +39,20 @@ def test_masked_logits(dtype, lowest, chunks, t, v):
     with np.errstate(invalid="ignore"):
         _, ref = orc.ppl_chunk_scores(x.double().numpy(), tgt)
     np.testing.assert_allclose(nll.cpu().numpy(), ref, atol=TOL, rtol=2e-7)      # (lowest: 3e38 to f32's place)
+
+
+@pytest.mark.parametrize("dtype,v", [(torch.float32, 50257), (torch.float32, 32000), (torch.bfloat16, 50257)])
+def test_one_value_carries_the_sum(dtype, v):
+    """Every exponential of f32 logits, and of rows off the 16-byte grid, is evaluated by ex2 (relative
+    error 2^-22): where one value of magnitude 4 carries the sum, three more roundings to f32 of values
+    below 8 are left, 2^-22 + 3 * 2^-22 in all, wherever in a vector the value lies."""
+    t = 256                                       # enough rows that a row is one CTA, whose threads take vectors in pairs
+    x = torch.full((2, t, v), -40.0, dtype=dtype)
+    x[:, torch.arange(t), torch.arange(t) * 37 % 1000] = 4.0
+    tgt = np.full(t, v - 1, np.int32)
+    nll = torch.full((2, t), -1.0, device="cuda")
+    score = torch.full((2,), -1.0, device="cuda")
+    cc.cc_ppl_chunk_scores(ctx(), x.cuda(), torch.from_numpy(tgt).cuda(), nll, score)
+    assert ctx().poll() == 0
+    _, ref = orc.ppl_chunk_scores(x.double().numpy(), tgt)
+    np.testing.assert_allclose(nll.cpu().numpy(), ref, atol=2.0 ** -20, rtol=2.0 ** -24)   # (the subtraction of -40)
