@@ -195,6 +195,9 @@ cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry
 cudaError_t launch_ppl_scores(const Launch& L, const void* logits, bool is_f32, int num_chunks,
                               int num_tokens, int vocab, int64_t stride_chunk, int64_t stride_token,
                               const int32_t* targets, float* nll, float* score);
+// rows [0, whole) have a CTA each, the others `parts` (a divisor of whole) each; slots: CTAs at a time
+struct PplSplit { int whole, parts; };
+PplSplit ppl_split(int rows, int vocab, int slots);
 cudaError_t launch_select_chunks(const Launch& L, const float* score, int num_chunks, int k,
                                  int32_t* chosen);
 
@@ -208,3 +211,8 @@ cudaError_t run_exp_probe(const Launch& L, bool from_tmem, int iters, long long*
                           double* rate);
 
 }  // namespace cc
+
+// Rules of dispatches as plain C functions, for the tests that run without a GPU.
+extern "C" {
+void ccx_ppl_split(int rows, int vocab, int slots, int* whole, int* parts);
+}

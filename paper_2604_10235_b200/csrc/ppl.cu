@@ -259,19 +259,30 @@ select_chunks_kernel(const float* __restrict__ score, int num_chunks, int k, int
 
 }  // namespace
 
+// A row is a few hundred KB, so whole rows quantise badly: the rows that do not fill a last wave of
+// `slots` CTAs (all of them, when there are few) are split over clusters as wide as that wave allows, not
+// below 8192 values per CTA.  The clusters start at a multiple of their width, so up to seven rows of the
+// full waves are split too; no width is taken that adds a wave with them.  8 x 16 rows of 151936 bf16 logits:
+// 18.8 -> 14 us with three CTAs per row; splitting beyond one wave, or rows of full waves, is slower
+// (cluster scheduling).  Where full waves of 444 were left exactly or nearly, the split used to add a wave:
+// 128256 bf16 logits, 444 rows 31.9 -> 24.2 us, 888 rows 47.7 -> 43.9, 497 rows 32.8 -> 32.0.
+PplSplit ppl_split(int rows, int vocab, int slots) {
+  const int full = rows / slots * slots;
+  PplSplit best{rows, 1};
+  if (rows == full) return best;
+  for (int parts = 2; parts <= kMaxParts && vocab / parts >= 8192; ++parts) {
+    const int whole = full - full % parts;
+    if ((rows - whole) * parts <= full - whole + slots) best = PplSplit{whole, parts};
+  }
+  return best;
+}
+
 cudaError_t launch_ppl_scores(const Launch& L, const void* logits, bool is_f32, int num_chunks,
                               int num_tokens, int vocab, int64_t stride_chunk, int64_t stride_token,
                               const int32_t* targets, float* nll, float* score) {
   const int rows = num_chunks * num_tokens;
-  // A row is a few hundred KB, so whole rows quantise badly: the rows that do not fill a last wave
-  // of CTAs (all of them, when there are few) are split over clusters as wide as that wave allows
-  // (not below 8192 values per CTA).  8 x 16 rows of 151936 bf16 logits: 18.8 -> 14 us with three
-  // CTAs per row; splitting beyond one wave, or rows of full waves, is slower (cluster scheduling).
-  const int slots = L.sm_count * kCtasPerSm;
-  int whole = rows / slots * slots, parts = 1;
-  while (parts < kMaxParts && (rows - whole) * (parts + 1) <= slots && vocab / (parts + 1) >= 8192) ++parts;
-  if (parts == 1) whole = rows;
-  whole -= whole % parts;
+  const PplSplit split = ppl_split(rows, vocab, L.sm_count * kCtasPerSm);
+  const int whole = split.whole, parts = split.parts;
   const unsigned grid = (unsigned)(whole + (rows - whole) * parts);
   // The FMA pipe's exponentials (relative error 8e-5) are for bf16 rows on the 16-byte grid alone, where
   // they take 1.6 % off the call (32 x 64 rows of 128256: 94.2 against 95.7 us).  f32 logits leave the
@@ -297,3 +308,9 @@ cudaError_t launch_select_chunks(const Launch& L, const float* score, int num_ch
 }
 
 }  // namespace cc
+
+extern "C" void ccx_ppl_split(int rows, int vocab, int slots, int* whole, int* parts) {
+  const cc::PplSplit s = cc::ppl_split(rows, vocab, slots);
+  *whole = s.whole;
+  *parts = s.parts;
+}
