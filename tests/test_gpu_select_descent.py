@@ -41,3 +41,24 @@ def test_cut_off_search(kind, n):
                 ref = orc.select_tokens(fused[h], prior, n, budget, 0.5, cap, 2)
                 assert count[h] == keep
                 np.testing.assert_array_equal(idx[h, :keep], ref, err_msg=f"{kind} n={n} B={budget} cap={cap} h={h}")
+
+
+@pytest.mark.parametrize("kind", ["spread", "outlier", "few"])
+@pytest.mark.parametrize("n,hkv,chunk", [(40000, 3, 1), (40961, 40, 1), (131072, 2, 1), (90007, 8, 3)])
+def test_cap_cut_off_by_a_graded_prior_over_several_ctas(kind, n, hkv, chunk):
+    """Both searches of the kernel list and rank candidates (or refine a crowded bin first) in clusters of
+    two and more: the cap's among priors that differ everywhere, then the budget's."""
+    rng = np.random.Generator(np.random.PCG64(n + hkv))
+    fused = _values(kind, rng, hkv, -(-n // chunk))
+    prior = rng.random(n).astype(np.float32)
+    if kind == "outlier":                       # the protected tokens' priors in one bin of the first histogram
+        prior[prior >= 0.5] = (0.5 + rng.random(int((prior >= 0.5).sum())) * 1e-4).astype(np.float32)
+        prior[n // 3] = 1e30
+    _, item_prior = orc.chunk_reduce(np.zeros((1, n), np.float32), prior, chunk, dtype=np.float32)
+    for budget in (n // 4, n // 3):
+        for cap in (0.3, 0.9):
+            idx, count = run_select(fused, prior, n, budget, 0.5, span_ratio=cap, span_min=2, chunk=chunk)
+            for h in range(hkv):
+                ref = orc.select_tokens(fused[h], item_prior, n, budget, 0.5, cap, 2, chunk=chunk)
+                assert count[h] == len(ref) == budget
+                np.testing.assert_array_equal(idx[h], ref, err_msg=f"{kind} n={n} B={budget} cap={cap} h={h}")
