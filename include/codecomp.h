@@ -211,8 +211,11 @@ int cc_compress_layer(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win,
  * are HOST arrays of n_layers device pointers, entry l being what cc_compress_layer takes for
  * layer l.  The descriptor is checked and the workspace carved once; the layers share the
  * workspace, and the intermediates left where cc_workspace_views finds them are those of the last
- * layer.  Results are those of n_layers separate calls; short layers run several to a launch, where
- * the sums of a row's softmax may be added up in another order (last place of an f32 score). */
+ * layer.  Results are those of n_layers separate calls in this order, also where layers share buffers (one
+ * idx scratch for all, a cache compacted into the space of the layer before it).  Layers none of which
+ * writes what another one of them reads or writes may run several to a launch, where the sums of a row's
+ * softmax may be added up in another order (last place of an f32 score); counts, and page tables
+ * made from the same free_pages, may be shared without giving that up. */
 int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
                        const void* const* q_win, const void* const* k, const void* const* v,
                        const float* prior, void* const* k_out, void* const* v_out,

@@ -391,7 +391,8 @@ def cc_exp_rate_probe(ctx: Context, from_tmem: bool, iters: int = 4000, stream=N
 def cc_compress_layers(ctx: Context, desc: Desc, q_win, k, v, prior, k_out, v_out, idx, count,
                        free_pages=None, out_page_table=None, ws=None, stream=None):
     """cc_compress_layer for a list of layers in one call: every tensor argument except ``prior``
-    and ``ws`` is a list with one tensor per layer."""
+    and ``ws`` is a list with one tensor per layer.  Layers may share buffers (an ``idx`` scratch, say);
+    they then run one after the other instead of several to a launch."""
     ws = ctx.workspace(desc) if ws is None else ws
     ctx.call("cc_compress_layers", desc, len(k), q_win, k, v, prior, k_out, v_out, idx, count, free_pages,
              out_page_table, ws, _raw(stream))

@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 
 #include "cc_internal.cuh"
@@ -512,6 +513,78 @@ int take_layer(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, int l, con
   return CC_OK;
 }
 
+// Memory that a layer reads or writes: [lo, hi), of which the first `width` bytes of every `pitch` count
+// (pitch 0: all of it).
+struct Region {
+  uintptr_t lo, hi;
+  size_t pitch, width;
+  int layer;
+  bool written;
+  bool meets(const Region& o) const {
+    if (hi <= o.lo || o.hi <= lo) return false;
+    if (pitch == 0 || pitch != o.pitch) return true;
+    const size_t d = (o.lo % pitch + pitch - lo % pitch) % pitch;      // offset of o's rows behind this one's
+    return d < width || pitch - d < o.width;
+  }
+};
+
+// Whether the layers of `lp` can share their launches: all of them select before the first one
+// compacts, so none may write what another one reads or writes.  (One index scratch for all layers, a cache
+// compacted into the space of the layer before it: such layers run one after the other.)  Writes of the
+// same bytes to the same place do not count: counts, and page tables made from the same list.  Caches of
+// several layers interleaved row by row are apart although their extents overlap.
+bool layers_apart(const BatchTable& bt, const Geometry& g, const LayerPtrs& lp) {
+  Region r[9 * kMaxLayers];
+  int n = 0;
+  auto flat = [&](int layer, bool written, const void* p, size_t bytes) {
+    if (bytes) r[n++] = Region{(uintptr_t)p, (uintptr_t)p + bytes, 0, 0, layer, written};
+  };
+  auto rows = [&](int layer, bool written, const void* p, size_t count, int64_t stride_tok, int64_t stride_head) {
+    if (count == 0) return;
+    const bool by_tok = stride_tok >= stride_head;
+    const size_t outer = (by_tok ? stride_tok : stride_head) * 2, inner = (by_tok ? stride_head : stride_tok) * 2;
+    const size_t n_outer = by_tok ? count : g.hkv, n_inner = by_tok ? g.hkv : count;
+    const size_t width = (n_inner - 1) * inner + kHeadDim * 2;
+    const uintptr_t lo = (uintptr_t)p;
+    r[n++] = Region{lo, lo + (n_outer - 1) * outer + width, width <= outer ? outer : 0, width, layer, written};
+  };
+  const bool paged = bt.page_size > 0;
+  const size_t in_rows = paged ? (size_t)g.pool_pages * bt.page_size : bt.n_tot;
+  const size_t out_rows = bt.b_tot == 0 ? 0 : paged ? in_rows : bt.b_tot;
+  const int64_t out_tok = paged ? g.kv_stride_tok : g.out_stride_tok, out_head = paged ? g.kv_stride_head : g.out_stride_head;
+  const int64_t q_seq = bt.num_seqs > 1 && g.q_stride_seq > 0 ? g.q_stride_seq : g.q_stride_row * g.window;
+  const size_t q_bytes = 2 * ((bt.num_seqs - 1) * q_seq + (g.window - 1) * g.q_stride_row + (g.hq - 1) * g.q_stride_head + kHeadDim);
+  size_t pages = 0;
+  for (int s = 0; paged && s < bt.num_seqs; ++s) pages += (bt.seq[s].keep + bt.page_size - 1) / bt.page_size;
+  for (int l = 0; l < lp.n; ++l) {
+    flat(l, false, lp.q[l], q_bytes);
+    if (lp.k_out[l] != lp.k[l] || !paged) rows(l, false, lp.k[l], in_rows, g.kv_stride_tok, g.kv_stride_head);
+    if (lp.v_out[l] != lp.v[l] || !paged) rows(l, false, lp.v[l], in_rows, g.kv_stride_tok, g.kv_stride_head);
+    rows(l, true, lp.k_out[l], out_rows, out_tok, out_head);
+    rows(l, true, lp.v_out[l], out_rows, out_tok, out_head);
+    flat(l, true, lp.idx[l], (size_t)g.hkv * bt.b_tot * sizeof(int32_t));
+    if (l == 0 || lp.count[l] != lp.count[l - 1]) flat(l, true, lp.count[l], (size_t)bt.num_seqs * g.hkv * sizeof(int32_t));
+    if (!paged || bt.b_tot == 0 ||
+        (l > 0 && lp.free_pages[l] == lp.free_pages[l - 1] && lp.out_page_table[l] == lp.out_page_table[l - 1])) continue;
+    flat(l, false, lp.free_pages[l], pages * sizeof(int32_t));
+    flat(l, true, lp.out_page_table[l], (size_t)bt.num_seqs * g.out_page_table_stride * sizeof(int32_t));
+  }
+  std::sort(r, r + n, [](const Region& a, const Region& b) { return a.lo < b.lo; });
+  int open[9 * kMaxLayers], n_open = 0;          // regions that reach beyond the start of the one looked at
+  for (int i = 0; i < n; ++i) {
+    int kept = 0;
+    for (int j = 0; j < n_open; ++j) {
+      const Region& o = r[open[j]];
+      if (o.hi <= r[i].lo) continue;
+      if (o.layer != r[i].layer && (o.written || r[i].written) && o.meets(r[i])) return false;
+      open[kept++] = open[j];
+    }
+    n_open = kept;
+    open[n_open++] = i;
+  }
+  return true;
+}
+
 // The fused step of the layers of `lp`; bt is the plan's table repeated for them.
 int compress(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, const BatchTable& bt, const LayerPtrs& lp,
              const float* prior, char* score_ws, char* w, void* stream) {
@@ -572,22 +645,33 @@ int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
   char* w = (char*)ws;
   const int groups = (n_layers + p.group - 1) / p.group;
   BatchTable bt;
-  for (int i = 0; i < groups; ++i) {
-    const int l0 = (int)((long long)n_layers * i / groups), l1 = (int)((long long)n_layers * (i + 1) / groups);
-    LayerPtrs lp;
-    lp.n = l1 - l0;
+  bt.num_seqs = 0;
+  // layers [l0, l1) in one launch per stage
+  auto take = [&](int l0, int l1, LayerPtrs* lp) {
+    lp->n = l1 - l0;
     for (int l = l0; l < l1; ++l) {
       const int e = l - l0, slot = l1 - 1 - l;     // the group's last layer uses the first slot of the workspace
       char* base = slot == 0 ? w : w + p.off_group + (size_t)(slot - 1) * p.off_score_ws;
-      lp.scores[e] = (float*)(base + p.off_scores);
-      lp.fused[e] = (float*)(base + p.off_fused);
-      rc = take_layer(ctx, desc, p, e, q_win[l], k[l], v[l], prior, k_out[l], v_out[l], idx[l], count[l],
-                      free_pages ? free_pages[l] : nullptr, out_page_table ? out_page_table[l] : nullptr, &lp);
+      lp->scores[e] = (float*)(base + p.off_scores);
+      lp->fused[e] = (float*)(base + p.off_fused);
+      const int rc = take_layer(ctx, desc, p, e, q_win[l], k[l], v[l], prior, k_out[l], v_out[l], idx[l], count[l],
+                                free_pages ? free_pages[l] : nullptr, out_page_table ? out_page_table[l] : nullptr, lp);
       if (rc != CC_OK) return rc;
     }
-    if (i == 0 || lp.n * p.bt.num_seqs != bt.num_seqs) repeat_layers(p.bt, lp.n, &bt);
-    rc = compress(ctx, desc, p, bt, lp, prior, w + (lp.n > 1 ? p.off_group_ws : p.off_score_ws), w, stream);
-    if (rc != CC_OK) return rc;
+    return (int)CC_OK;
+  };
+  for (int i = 0; i < groups; ++i) {
+    const int l0 = (int)((long long)n_layers * i / groups), l1 = (int)((long long)n_layers * (i + 1) / groups);
+    LayerPtrs lp;
+    if ((rc = take(l0, l1, &lp)) != CC_OK) return rc;
+    const bool apart = lp.n == 1 || layers_apart(p.bt, p.g, lp);
+    const int step = apart ? lp.n : 1;
+    for (int l = l0; l < l1; l += step) {
+      if (!apart && (rc = take(l, l + step, &lp)) != CC_OK) return rc;
+      if (lp.n * p.bt.num_seqs != bt.num_seqs) repeat_layers(p.bt, lp.n, &bt);
+      rc = compress(ctx, desc, p, bt, lp, prior, w + (lp.n > 1 ? p.off_group_ws : p.off_score_ws), w, stream);
+      if (rc != CC_OK) return rc;
+    }
   }
   return CC_OK;
 }

@@ -42,3 +42,73 @@ def test_groups_of_layers_equal_separate_calls(layers, w, lens):
             rows = base + idx[h]
             assert torch.equal(ko[:, h].view(torch.int16), k[l][rows, h].view(torch.int16))
             assert torch.equal(vo[:, h].view(torch.int16), v[l][rows, h].view(torch.int16))
+
+
+@pytest.mark.parametrize("shared", ["idx", "idx_and_count", "all_outputs", "previous_k", "previous_v", "free_list",
+                                    "interleaved", "interleaved_in_place"])
+def test_layers_that_share_buffers(shared):
+    """What layers compute when they run one after the other, bit for bit where the sharing makes them run
+    so, whoever shares what: scratch outputs, caches compacted into the space of the layer before, one page
+    list; caches interleaved row by row share nothing."""
+    from gpu_util import bf16_dev, ctx, desc_for
+    paged = shared in ("free_list", "interleaved_in_place")
+    wl = gen.Workload("share", 43, 1, 8, 2, 128, 32, gen.POOL_MAX, 7, 0, seq_lens=(700, 300), budget_frac=0.4,
+                      page_size=16 if paged else 0)
+    layers, hkv, b_tot = 5, 2, sum(wl.budgets)
+    xs = [gen.make_layer(wl, layer=l) for l in range(layers)]
+    if paged:
+        for x in xs[1:]:
+            gen.repage(x, xs[0])
+    rows = xs[0].k.shape[0]
+    stride = max(-(-b // 16) for b in wl.budgets) if paged else 0
+    woven = shared.startswith("interleaved")
+    pt = torch.from_numpy(xs[0].page_table).cuda() if paged else None
+    d = desc_for(wl, cc.CC_MODE_BF16, page_table=pt, out_pt_stride=stride, pool_pages=xs[0].pool_pages)
+    if woven:                                    # [token][layer][head][channel]
+        d.c.kv_stride_tok = d.c.out_stride_tok = layers * hkv * 128
+    prior = torch.from_numpy(xs[0].prior).cuda()
+    q = [bf16_dev(x.q_win) for x in xs]
+
+    def cache(attr):
+        made = [bf16_dev(getattr(x, attr)) for x in xs]
+        return list(torch.stack(made, 1).unbind(1)) if woven else made
+
+    def empty_cache():
+        if woven:
+            return list(torch.zeros((b_tot, layers, hkv, 128), dtype=torch.bfloat16, device="cuda").unbind(1))
+        return [torch.zeros((b_tot, hkv, 128), dtype=torch.bfloat16, device="cuda") for _ in xs]
+
+    def buffers():
+        k, v = cache("k"), cache("v")
+        ko, vo = (k, v) if paged else (empty_cache(), empty_cache())
+        idx = [torch.full((hkv, b_tot), -9, dtype=torch.int32, device="cuda") for _ in xs]
+        count = [torch.full((2, hkv), -9, dtype=torch.int32, device="cuda") for _ in xs]
+        free = opt = None
+        if paged:
+            free = [torch.from_numpy(xs[0].free_pages).cuda()] * layers
+            opt = [torch.full((2, stride), -9, dtype=torch.int32, device="cuda")] * layers
+        if shared.startswith("idx") or shared == "all_outputs":
+            idx = idx[:1] * layers
+        if shared in ("idx_and_count", "all_outputs"):
+            count = count[:1] * layers
+        if shared == "all_outputs":
+            ko, vo = ko[:1] * layers, vo[:1] * layers
+        if shared == "previous_k":               # the last layer's into a buffer of its own
+            ko = [ko[0]] + [t[:b_tot] for t in k[:-1]]
+        if shared == "previous_v":
+            vo = [vo[0]] + [t[100:100 + b_tot] for t in v[:-1]]
+        return k, v, ko, vo, idx, count, free, opt
+
+    one, all_ = buffers(), buffers()
+    ws = ctx().workspace(d)
+    for l in range(layers):
+        cc.cc_compress_layer(ctx(), d, q[l], *(t[l] for t in one[:2]), prior, *(t[l] if t else None for t in one[2:]), ws)
+    assert ctx().poll() == 0
+    cc.cc_compress_layers(ctx(), d, q, *all_[:2], prior, *all_[2:], ws)
+    assert ctx().poll() == 0
+    together = paged or woven                    # several layers to a launch: ties that f32 rounding decides may swap
+    for a, b in zip(one, all_):
+        for s, t in zip(a or [], b or []):
+            if s.dtype == torch.bfloat16:
+                s, t = s.view(torch.int16), t.view(torch.int16)
+            assert torch.equal(s, t) or (together and (s != t).float().mean() <= 0.01)
