@@ -140,6 +140,10 @@ int cc_poll_status(cc_ctx* ctx, void* stream, int* device_status);
 /* Bytes of device workspace (256-byte aligned) that any entry point below needs for `desc`.
  * Returns 0 if the descriptor is invalid. */
 size_t cc_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc);
+/* Bytes that cc_compress_layers can make use of on n_layers layers: given that much instead of
+ * cc_workspace_bytes (which is enough, and never more), it runs short layers several to a launch.  In
+ * between it takes as many layers per launch as fit.  Returns 0 if the descriptor is invalid. */
+size_t cc_layers_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers);
 
 /* A1 - window attention scores (Section 4.5, the equation for A and u(j)), summed over the
  * query heads of each KV head.  q_win, k: device bf16.  scores: device f32 [H_kv][N_tot],
@@ -213,7 +217,8 @@ int cc_compress_layer(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win,
  * workspace, and the intermediates left where cc_workspace_views finds them are those of the last
  * layer.  Results are those of n_layers separate calls in this order, also where layers share buffers (one
  * idx scratch for all, a cache compacted into the space of the layer before it).  Layers none of which
- * writes what another one of them reads or writes may run several to a launch, where the sums of a row's
+ * writes what another one of them reads or writes run several to a launch where the workspace has room
+ * (cc_layers_workspace_bytes), and then the sums of a row's
  * softmax may be added up in another order (last place of an f32 score); counts, and page tables
  * made from the same free_pages, may be shared without giving that up. */
 int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,

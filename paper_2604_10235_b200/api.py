@@ -120,7 +120,7 @@ class LayerCompressor:
             self.v_out = torch.empty((b_tot, hkv, d), dtype=bf, device=dev)
         self.idx = torch.empty((hkv, b_tot), dtype=torch.int32, device=dev)
         self.count = torch.empty((S, hkv), dtype=torch.int32, device=dev)
-        self.ws = ctx.workspace(self.desc)
+        self.ws = ctx.workspace(self.desc, n_layers=1)
         # pinned landing buffers for the results
         if self.paged:
             ps = wl.page_size

@@ -34,7 +34,8 @@ EXPORTS = ("cc_create", "cc_destroy", "cc_status_string", "cc_last_error", "cc_p
            "cc_workspace_bytes", "cc_score_window", "cc_fuse_prior_pool", "cc_topk_select",
            "cc_compact_kv", "cc_compress_layer", "cc_workspace_views", "cc_topk_select_static",
            "cc_structural_score", "cc_plan_budgets", "cc_select_spans", "cc_ppl_chunk_scores",
-           "cc_select_chunks", "cc_exp_rate_probe", "cc_compress_layers")
+           "cc_select_chunks", "cc_exp_rate_probe", "cc_compress_layers",
+           "cc_layers_workspace_bytes")
 CC_STATIC_SELECT_MAX_ITEMS = 1 << 20
 
 
@@ -98,6 +99,8 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.cc_poll_status.argtypes = [vp, vp, C.POINTER(C.c_int)]
     lib.cc_workspace_bytes.argtypes = [vp, dp]
     lib.cc_workspace_bytes.restype = sz
+    lib.cc_layers_workspace_bytes.argtypes = [vp, dp, C.c_int32]
+    lib.cc_layers_workspace_bytes.restype = sz
     lib.cc_score_window.argtypes = [vp, dp, vp, vp, vp, vp, vp, sz, vp]
     lib.cc_fuse_prior_pool.argtypes = [vp, dp, vp, vp, vp, vp]
     lib.cc_topk_select.argtypes = [vp, dp, vp, vp, vp, vp, vp, sz, vp]
@@ -115,7 +118,7 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.cc_compress_layers.argtypes = [vp, dp, C.c_int32] + [vp] * 3 + [vp] + [vp] * 6 + [vp, sz, vp]
     lib.cc_workspace_views.argtypes = [vp, dp, vp, C.POINTER(vp), C.POINTER(vp)]
     for name in EXPORTS:
-        if name not in ("cc_status_string", "cc_last_error", "cc_workspace_bytes"):
+        if name not in ("cc_status_string", "cc_last_error", "cc_workspace_bytes", "cc_layers_workspace_bytes"):
             getattr(lib, name).restype = C.c_int
     lib.addresses = {name: C.cast(getattr(lib, name), vp).value for name in _SPEC}
     if _CALL is None:
@@ -170,14 +173,16 @@ class Context:
             raise CodecompError(rc, self.lib.cc_last_error(self.handle).decode() or
                                 self.lib.cc_status_string(rc).decode())
 
-    def workspace_bytes(self, desc: "Desc") -> int:
-        n = self.lib.cc_workspace_bytes(self.handle, C.byref(desc.c))
+    def workspace_bytes(self, desc: "Desc", n_layers: Optional[int] = None) -> int:
+        """Bytes of workspace for calls on one layer (``n_layers=1``), for ``cc_compress_layers`` on
+        ``n_layers`` of them at full speed, or (None) for any call."""
+        n = self.lib.cc_layers_workspace_bytes(self.handle, C.byref(desc.c), 2 ** 31 - 1 if n_layers is None else n_layers)
         if n == 0:
             raise CodecompError(CC_ERR_INVALID_ARG, self.lib.cc_last_error(self.handle).decode())
         return int(n)
 
-    def workspace(self, desc: "Desc") -> torch.Tensor:
-        return torch.empty(self.workspace_bytes(desc), dtype=torch.uint8,
+    def workspace(self, desc: "Desc", n_layers: Optional[int] = None) -> torch.Tensor:
+        return torch.empty(self.workspace_bytes(desc, n_layers), dtype=torch.uint8,
                            device=f"cuda:{self.device}")
 
     def poll(self, stream: Optional[int] = None) -> int:
@@ -279,7 +284,7 @@ def _ptr(t: Optional[torch.Tensor]) -> C.c_void_p:
 
 
 def cc_score_window(ctx: Context, desc: Desc, q_win, k, scores, lse=None, ws=None, stream=None):
-    ws = ctx.workspace(desc) if ws is None else ws
+    ws = ctx.workspace(desc, 1) if ws is None else ws
     ctx.call("cc_score_window", desc, q_win, k, scores, lse, ws, _raw(stream))
 
 
@@ -288,7 +293,7 @@ def cc_fuse_prior_pool(ctx: Context, desc: Desc, scores, prior, fused, stream=No
 
 
 def cc_topk_select(ctx: Context, desc: Desc, fused, prior, idx, count, ws=None, stream=None):
-    ws = ctx.workspace(desc) if ws is None else ws
+    ws = ctx.workspace(desc, 1) if ws is None else ws
     ctx.call("cc_topk_select", desc, fused, prior, idx, count, ws, _raw(stream))
 
 
@@ -375,7 +380,7 @@ def cc_select_spans(starts, ends, scores, protected, n: int, budget: int, span_r
 
 def cc_compress_layer(ctx: Context, desc: Desc, q_win, k, v, prior, k_out, v_out, idx, count,
                       free_pages=None, out_page_table=None, ws=None, stream=None):
-    ws = ctx.workspace(desc) if ws is None else ws
+    ws = ctx.workspace(desc, 1) if ws is None else ws
     ctx.call("cc_compress_layer", desc, q_win, k, v, prior, k_out, v_out, idx, count, free_pages,
              out_page_table, ws, _raw(stream))
 
@@ -393,7 +398,7 @@ def cc_compress_layers(ctx: Context, desc: Desc, q_win, k, v, prior, k_out, v_ou
     """cc_compress_layer for a list of layers in one call: every tensor argument except ``prior``
     and ``ws`` is a list with one tensor per layer.  Layers may share buffers (an ``idx`` scratch, say);
     they then run one after the other instead of several to a launch."""
-    ws = ctx.workspace(desc) if ws is None else ws
+    ws = ctx.workspace(desc, len(k)) if ws is None else ws
     ctx.call("cc_compress_layers", desc, len(k), q_win, k, v, prior, k_out, v_out, idx, count, free_pages,
              out_page_table, ws, _raw(stream))
 

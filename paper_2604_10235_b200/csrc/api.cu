@@ -46,18 +46,14 @@ struct Plan {
   Geometry g;
   // workspace layout (byte offsets)
   size_t off_scores, off_fused, off_score_ws, off_select_ws, total;
-  // cc_compress_layers runs up to `group` layers per launch; their intermediates follow `total`:
-  // scores and fused values of the layers after the first, then the score kernel's statistics
-  int group;
-  size_t off_group, off_group_ws, grand_total;
 };
 
 // Layers per launch of cc_compress_layers.  Launches that share a prologue, a pipeline fill and a tail
 // are what short prompts gain from most, and a fuller last wave pays even where the keys of a launch
 // no longer fit L2 (nothing here is bound by reading them twice).  96 MB of keys and 16 layers -> 256 MB
 // and 32 layers per launch, us: 32 layers x 4096 tokens x 8 heads 461 -> 442, 32 x 8192 with 32 query
-// tokens 434 -> 359, 8 x 32768 507 -> 405.  The workspace, which a call on one layer gets too, grows by
-// a 32nd of the limit, 8 MB; 512 MB and more gain another 0 to 3 %.
+// tokens 434 -> 359, 8 x 32768 507 -> 405.  The workspace of such a call grows by a 32nd of the limit,
+// 8 MB; 512 MB and more gain another 0 to 3 %.
 constexpr size_t kGroupKeyBytes = 256u << 20;
 int layers_per_launch(const cc_layer_desc* d, const BatchTable& bt, const Geometry& g) {
   if (d->compute_mode != CC_MODE_BF16 || d->fill_mode != CC_FILL_ATTENTION || bt.n_tot == 0 || bt.b_tot == 0 ||
@@ -211,16 +207,29 @@ int build_plan(cc_ctx* ctx, const cc_layer_desc* d, Plan* p) {
   off += align256(sw);
   p->off_select_ws = off; off += align256(select_ws_bytes(bt, g));
   p->total = off > 256 ? off : 256;
-  p->group = layers_per_launch(d, bt, g);
-  p->off_group = p->total;
-  p->off_group_ws = p->off_group + (size_t)(p->group - 1) * p->off_score_ws;
-  p->grand_total = p->total;
-  if (p->group > 1) {
-    BatchTable all;
-    repeat_layers(bt, p->group, &all);
-    p->grand_total = p->off_group_ws + align256(score_tc_ws_bytes(all, g, ctx->sm_count));
-  }
   return CC_OK;
+}
+
+// A call on several layers runs `layers` of them per launch.  Their intermediates follow those of a call on
+// one layer: scores and fused values of the layers after the first, then the score kernel's statistics.
+struct Group {
+  int layers;
+  size_t off_layers, off_score_ws, total;
+};
+
+// n_layers layers in as few launches as the limits and ws_bytes of workspace allow, spread evenly.
+Group plan_group(const cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, int n_layers, size_t ws_bytes) {
+  Group q{1, p.total, p.off_score_ws, p.total};
+  BatchTable all;
+  for (int limit = layers_per_launch(d, p.bt, p.g); limit > 1; --limit) {
+    const int launches = (n_layers - 1) / limit + 1, layers = (n_layers - 1) / launches + 1;
+    if (layers < 2) break;
+    repeat_layers(p.bt, layers, &all);
+    const size_t off_ws = p.total + (size_t)(layers - 1) * p.off_score_ws;
+    const size_t total = off_ws + align256(score_tc_ws_bytes(all, p.g, ctx->sm_count));
+    if (total <= ws_bytes) return Group{layers, p.total, off_ws, total};
+  }
+  return q;
 }
 
 int check_ws(cc_ctx* ctx, size_t need, void* ws, size_t ws_bytes) {
@@ -400,7 +409,13 @@ int cc_poll_status(cc_ctx* ctx, void* stream, int* device_status) {
 size_t cc_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc) {
   Plan p;
   if (build_plan(const_cast<cc_ctx*>(ctx), desc, &p) != CC_OK) return 0;
-  return p.grand_total;
+  return p.total;
+}
+
+size_t cc_layers_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers) {
+  Plan p;
+  if (build_plan(const_cast<cc_ctx*>(ctx), desc, &p) != CC_OK) return 0;
+  return n_layers > 1 ? plan_group(ctx, desc, p, n_layers, SIZE_MAX).total : p.total;
 }
 
 int cc_score_window(cc_ctx* ctx, const cc_layer_desc* desc, const void* q_win, const void* k,
@@ -641,9 +656,10 @@ int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
     return fail(ctx, CC_ERR_INVALID_ARG, "NULL pointer array");
   if (p.bt.page_size > 0 && (!free_pages || !out_page_table))
     return fail(ctx, CC_ERR_INVALID_ARG, "paged compaction needs free_pages and out_page_table");
-  if ((rc = check_ws(ctx, p.grand_total, ws, ws_bytes)) != CC_OK) return rc;
+  if ((rc = check_ws(ctx, p.total, ws, ws_bytes)) != CC_OK) return rc;
   char* w = (char*)ws;
-  const int groups = (n_layers + p.group - 1) / p.group;
+  const Group group = plan_group(ctx, desc, p, n_layers, ws_bytes);
+  const int groups = (n_layers - 1) / group.layers + 1;
   BatchTable bt;
   bt.num_seqs = 0;
   // layers [l0, l1) in one launch per stage
@@ -651,7 +667,7 @@ int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
     lp->n = l1 - l0;
     for (int l = l0; l < l1; ++l) {
       const int e = l - l0, slot = l1 - 1 - l;     // the group's last layer uses the first slot of the workspace
-      char* base = slot == 0 ? w : w + p.off_group + (size_t)(slot - 1) * p.off_score_ws;
+      char* base = slot == 0 ? w : w + group.off_layers + (size_t)(slot - 1) * p.off_score_ws;
       lp->scores[e] = (float*)(base + p.off_scores);
       lp->fused[e] = (float*)(base + p.off_fused);
       const int rc = take_layer(ctx, desc, p, e, q_win[l], k[l], v[l], prior, k_out[l], v_out[l], idx[l], count[l],
@@ -669,7 +685,7 @@ int cc_compress_layers(cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers,
     for (int l = l0; l < l1; l += step) {
       if (!apart && (rc = take(l, l + step, &lp)) != CC_OK) return rc;
       if (lp.n * p.bt.num_seqs != bt.num_seqs) repeat_layers(p.bt, lp.n, &bt);
-      rc = compress(ctx, desc, p, bt, lp, prior, w + (lp.n > 1 ? p.off_group_ws : p.off_score_ws), w, stream);
+      rc = compress(ctx, desc, p, bt, lp, prior, w + (lp.n > 1 ? group.off_score_ws : p.off_score_ws), w, stream);
       if (rc != CC_OK) return rc;
     }
   }

@@ -112,3 +112,40 @@ def test_layers_that_share_buffers(shared):
             if s.dtype == torch.bfloat16:
                 s, t = s.view(torch.int16), t.view(torch.int16)
             assert torch.equal(s, t) or (together and (s != t).float().mean() <= 0.01)
+
+
+@pytest.mark.parametrize("layers,room", [(7, 1), (7, 2), (7, 3), (7, 7), (33, 33), (40, 33), (1, 1)])
+def test_workspace_of_some_layers(layers, room):
+    """One layer's workspace is what its own call needs; cc_compress_layers keeps inside what it is given, be that
+    one layer's, some layers' or all layers', and refuses less than one layer's."""
+    from gpu_util import bf16_dev, ctx, desc_for
+    wl = gen.Workload("room", 44, 1, 8, 2, 128, 32, gen.POOL_MAX, 7, 300, n=1500)
+    xs = [gen.make_layer(wl, layer=l) for l in range(3)]
+    d = desc_for(wl, cc.CC_MODE_BF16)
+    n_bytes = ctx().workspace_bytes(d, room)
+    one_layer = ctx().workspace_bytes(d, 1)
+    stats = 256 * 8 * 150                        # (maximum, sum) of 128 rows per CTA and (sequence, head)
+    assert one_layer <= 2 * 4 * 2 * 1500 + stats + 2 * 1500 + 4 * 256 and one_layer <= n_bytes <= ctx().workspace_bytes(d)
+    assert ctx().lib.cc_workspace_bytes(ctx().handle, d.c) == one_layer
+    full = torch.full((n_bytes + 4096,), 0x5A, dtype=torch.uint8, device="cuda")
+    prior = torch.from_numpy(xs[0].prior).cuda()
+    q, k, v = ([bf16_dev(getattr(xs[l % 3], a)) for l in range(layers)] for a in ("q_win", "k", "v"))
+
+    def outputs(n):
+        ko = torch.zeros((n, 300, 2, 128), dtype=torch.bfloat16, device="cuda")
+        return (list(ko), list(torch.zeros_like(ko)),
+                list(torch.full((n, 2, 300), -9, dtype=torch.int32, device="cuda")),
+                list(torch.full((n, 1, 2), -9, dtype=torch.int32, device="cuda")))
+
+    one, all_ = outputs(3), outputs(layers)
+    for l in range(3):
+        cc.cc_compress_layer(ctx(), d, q[l % layers], k[l % layers], v[l % layers], prior, *(t[l] for t in one))
+    cc.cc_compress_layers(ctx(), d, q, k, v, prior, *all_, ws=full[:n_bytes])
+    assert ctx().poll() == 0
+    assert bool((full[n_bytes:] == 0x5A).all())
+    for l in range(layers):
+        same = [torch.equal(s[l].view(torch.int16), t[l % 3].view(torch.int16)) for s, t in zip(all_, one)]
+        assert all(same) or (room > 1 and (all_[2][l] != one[2][l % 3]).float().mean() <= 0.01)
+    with pytest.raises(cc.CodecompError) as e:
+        cc.cc_compress_layers(ctx(), d, q, k, v, prior, *all_, ws=full[:one_layer - 256])
+    assert e.value.status == cc.CC_ERR_WORKSPACE
