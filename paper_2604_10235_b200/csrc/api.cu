@@ -13,6 +13,7 @@
 struct cc_ctx {
   int device;
   int sm_count;
+  cc::SelectRoom select_room;
   cc::DeviceStatus* d_status;
   cc::DeviceStatus* h_status;   // pinned
   long long* d_probe;           // scratch of cc_exp_rate_probe: two words per SM
@@ -55,9 +56,9 @@ struct Plan {
 // tokens 434 -> 359, 8 x 32768 507 -> 405.  The workspace of such a call grows by a 32nd of the limit,
 // 8 MB; 512 MB and more gain another 0 to 3 %.
 constexpr size_t kGroupKeyBytes = 256u << 20;
-int layers_per_launch(const cc_layer_desc* d, const BatchTable& bt, const Geometry& g) {
+int layers_per_launch(const cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, const Geometry& g) {
   if (d->compute_mode != CC_MODE_BF16 || d->fill_mode != CC_FILL_ATTENTION || bt.n_tot == 0 || bt.b_tot == 0 ||
-      select_cluster_size(bt, g.hkv) == 0)
+      select_shape(bt, g.hkv, ctx->select_room, true).cluster == 0)
     return 1;
   const size_t key_bytes = (size_t)bt.n_tot * g.hkv * kHeadDim * 2;
   size_t n = kGroupKeyBytes / key_bytes;
@@ -221,7 +222,7 @@ struct Group {
 Group plan_group(const cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, int n_layers, size_t ws_bytes) {
   Group q{1, p.total, p.off_score_ws, p.total};
   BatchTable all;
-  for (int limit = layers_per_launch(d, p.bt, p.g); limit > 1; --limit) {
+  for (int limit = layers_per_launch(ctx, d, p.bt, p.g); limit > 1; --limit) {
     const int launches = (n_layers - 1) / limit + 1, layers = (n_layers - 1) / launches + 1;
     if (layers < 2) break;
     repeat_layers(p.bt, layers, &all);
@@ -281,11 +282,11 @@ int run_fuse(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const float* sc
 
 int run_select(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const LayerPtrs& lp, const float* prior,
                char* ws, void* stream) {
-  const int cluster = select_cluster_size(p.bt, p.g.hkv);
+  const SelectShape shape = select_shape(p.bt, p.g.hkv, ctx->select_room, false);
   cudaError_t e;
-  if (cluster > 0)
+  if (shape.cluster > 0)
     e = launch_select_cluster(make_launch(ctx, stream), p.bt, p.g, d->force_threshold, false,
-                              d->pool_kind, d->pool_size, d->alpha, d->beta, lp, prior, cluster);
+                              d->pool_kind, d->pool_size, d->alpha, d->beta, lp, prior, shape);
   else
     e = launch_select(make_launch(ctx, stream), p.bt, p.g, d->force_threshold, lp.fused[0], prior, lp.idx[0],
                       lp.count[0], ws + p.off_select_ws);
@@ -294,10 +295,10 @@ int run_select(cc_ctx* ctx, const cc_layer_desc* d, const Plan& p, const LayerPt
 }
 
 // pooling + prior fusion + selection in one launch (items of every sequence fit a cluster)
-int run_fuse_select(cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, const Geometry& g, int cluster,
+int run_fuse_select(cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, const Geometry& g, SelectShape shape,
                     const LayerPtrs& lp, const float* prior, void* stream) {
   cudaError_t e = launch_select_cluster(make_launch(ctx, stream), bt, g, d->force_threshold, true, d->pool_kind,
-                                        d->pool_size, d->alpha, d->beta, lp, prior, cluster);
+                                        d->pool_size, d->alpha, d->beta, lp, prior, shape);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "fuse + select launch");
   return CC_OK;
 }
@@ -348,7 +349,8 @@ int cc_create(cc_ctx** out, int device) {
   bool ok = cudaMalloc(&ctx->d_status, sizeof(cc::DeviceStatus)) == cudaSuccess &&
             cudaMemset(ctx->d_status, 0, sizeof(cc::DeviceStatus)) == cudaSuccess &&
             cudaMalloc(&ctx->d_probe, 2 * 256 * sizeof(long long)) == cudaSuccess &&
-            cudaMallocHost(&ctx->h_status, sizeof(cc::DeviceStatus)) == cudaSuccess;
+            cudaMallocHost(&ctx->h_status, sizeof(cc::DeviceStatus)) == cudaSuccess &&
+            cc::query_select_room(&ctx->select_room) == cudaSuccess;
   if (ok) {
     cudaDriverEntryPointQueryResult qres;
     ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ctx->encode_tiled, cudaEnableDefault,
@@ -612,9 +614,9 @@ int compress(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, const BatchT
   int rc;
   const bool nearest = desc->fill_mode == CC_FILL_NEAREST;   // the scores play no part then
   if (!nearest && (rc = run_score(ctx, desc, bt, p.g, lp, nullptr, score_ws, stream)) != CC_OK) return rc;
-  const int cluster = select_cluster_size(bt, p.g.hkv);
-  if (cluster > 0 && !nearest) {
-    if ((rc = run_fuse_select(ctx, desc, bt, p.g, cluster, lp, prior, stream)) != CC_OK) return rc;
+  const SelectShape shape = nearest ? SelectShape{0, 0} : select_shape(bt, p.g.hkv, ctx->select_room, true);
+  if (shape.cluster > 0) {
+    if ((rc = run_fuse_select(ctx, desc, bt, p.g, shape, lp, prior, stream)) != CC_OK) return rc;
   } else {
     if ((rc = run_fuse(ctx, desc, p, lp.scores[0], prior, lp.fused[0], stream)) != CC_OK) return rc;
     if ((rc = run_select(ctx, desc, p, lp, prior, w, stream)) != CC_OK) return rc;

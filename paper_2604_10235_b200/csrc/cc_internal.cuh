@@ -174,14 +174,17 @@ cudaError_t launch_select(const Launch& L, const BatchTable& bt, const Geometry&
                           int32_t* idx, int32_t* count, void* ws);
 
 // cluster kernel: items resident in shared memory, optionally starting from the raw scores
-// (pooling and prior fusion done in the same launch).  select_cluster_size returns the CTAs per
-// (sequence, head) to use, or 0 when a sequence has too many items for it.
-int select_cluster_size(const BatchTable& bt, int hkv);
+// (pooling and prior fusion done in the same launch)
+struct SelectShape { int cluster, threads; };   // CTAs per (sequence, head), threads per CTA
+struct SelectRoom { int one[4], two[4]; };      // CTAs at a time in clusters of 1, 2, 4, 8: one per SM, in pairs
+cudaError_t query_select_room(SelectRoom* room);   // of the current device
+// (cluster 0: a sequence has too many items for the kernel)
+SelectShape select_shape(const BatchTable& bt, int hkv, const SelectRoom& room, bool fused_input);
 // (reads scores, fused, idx and count of the layers)
 cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const Geometry& g,
                                   float force_threshold, bool fused_input, int pool_kind,
                                   int pool_size, float alpha, float beta, const LayerPtrs& lp,
-                                  const float* prior, int cluster);
+                                  const float* prior, SelectShape shape);
 
 // variant of launch_select whose scratch is a static device array (no workspace argument)
 int64_t select_static_capacity();
@@ -215,4 +218,6 @@ cudaError_t run_exp_probe(const Launch& L, bool from_tmem, int iters, long long*
 // Rules of dispatches as plain C functions, for the tests that run without a GPU.
 extern "C" {
 void ccx_ppl_split(int rows, int vocab, int slots, int* whole, int* parts);
+void ccx_select_shape(int max_items, int num_seqs, int hkv, int chunk, int fused_input, const int* one, const int* two,
+                      int* cluster, int* threads);
 }

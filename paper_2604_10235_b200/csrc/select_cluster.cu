@@ -764,10 +764,6 @@ size_t cluster_smem_bytes(int slots, int threads, bool staging) {
   return (b + 15) / 16 * 16;
 }
 
-struct Shape {
-  int cluster, threads;      // CTAs per (sequence, head), threads per CTA
-};
-
 template <bool FUSED, bool CHUNKED>
 cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, int threads,
                          size_t smem) {
@@ -777,6 +773,14 @@ cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& 
   return launch_pdl(kern, dim3(P.cluster, g.hkv, bt.num_seqs), dim3(threads), smem, L.stream, P.cluster, bt, P);
 }
 
+// Two CTAs of 512 threads share an SM when their shared memory (and 1 KB that each is charged besides)
+// fits its 228 KB.
+constexpr size_t kPairSmem = (228 * 1024 - 2 * 1024) / 2;
+
+int steps_per_warp(int max_items, int cluster, int threads) {
+  return max_items > 0 ? (max_items + cluster * threads - 1) / (cluster * threads) : 1;
+}
+
 // Time of a launch with clusters of 1 << lc CTAs of `threads` threads, in us, from launches of one wave
 // on a B200 (n = 2048 .. 131072 items, 2 .. 256 problems): a constant that grows with what the
 // exchanges of wider clusters cost, something for the barriers of 1024 threads (less than in replays
@@ -784,44 +788,71 @@ cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& 
 // 0.48 (0.6) us per item of a thread of 512 (1024).  A chunk's tokens count a fifth of an item each.
 // A CTA of 1024 threads fills an SM, CTAs of 512 share it in pairs; a cluster sits inside one GPC, so
 // fewer CTAs run at a time in wide ones.
-double launch_cost(const BatchTable& bt, int hkv, int lc, int threads) {
+double launch_cost(const BatchTable& bt, int hkv, const SelectRoom& room, bool staging, int lc, int threads) {
   static const double base[4] = {6.1, 7.7, 7.8, 8.6};
-  static const int room[4] = {148, 148, 128, 96};
   const int c = 1 << lc;
   const double per_thread = (bt.max_items + (bt.chunk > 1 ? 0.2 * bt.chunk * bt.max_items : 0.0)) / (double)(c * threads);
-  const int ctas = bt.num_seqs * hkv * c, fit = threads == 512 ? 2 * room[lc] : room[lc];
+  const size_t smem = cluster_smem_bytes(steps_per_warp(bt.max_items, c, threads) * threads, threads, staging);
+  const int ctas = bt.num_seqs * hkv * c, fit = threads == 512 && smem <= kPairSmem ? room.two[lc] : room.one[lc];
   const int waves = (ctas + fit - 1) / fit;
-  const double slope = threads == 1024 ? 0.6 : (ctas > room[lc] ? 0.96 : 0.48);
+  const double slope = threads == 1024 ? 0.6 : (ctas > room.one[lc] ? 0.96 : 0.48);
   return waves * (base[lc] + (threads == 512 ? 0.0 : bt.chunk > 1 ? 1.0 : lc == 0 ? 0.8 : 0.3) + slope * per_thread);
-}
-
-// The cheapest shape; cluster 0 when a sequence has more items than the widest cluster holds.
-Shape select_shape(const BatchTable& bt, int hkv) {
-  if (bt.max_items <= 0) return Shape{1, 512};
-  Shape best{0, 0};
-  double best_us = 1e30;
-  for (int lc = 0; lc <= 3; ++lc)
-    for (int threads = 512; threads <= 1024; threads += 512) {
-      // a warp's run has at most 32 steps; CTAs of 512 threads are to fit an SM in pairs
-      if ((bt.max_items + (threads << lc) - 1) / (threads << lc) > 32) continue;
-      const double us = launch_cost(bt, hkv, lc, threads);
-      if (us < best_us) { best_us = us; best = Shape{1 << lc, threads}; }
-    }
-  return best;
 }
 
 }  // namespace
 
-int select_cluster_size(const BatchTable& bt, int hkv) { return select_shape(bt, hkv).cluster; }
+// CTAs that run at a time, in clusters of 1, 2, 4, 8: how many SMs the GPCs of a part have is not the same
+// on all parts, so the runtime is asked, once per context.  (148, 148, 132, 120 on the part at hand; 296, 296,
+// 284, 264 in pairs.)
+cudaError_t query_select_room(SelectRoom* room) {
+  auto one = select_cluster_kernel<true, false, 1024>;
+  auto two = select_cluster_kernel<true, false, 512>;
+  cudaError_t e = allow_smem(one);
+  if (e == cudaSuccess) e = allow_smem(two);
+  for (int lc = 0; lc <= 3 && e == cudaSuccess; ++lc) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << lc;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << lc);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = kSmemPerCta;
+    e = cudaOccupancyMaxActiveClusters(&room->one[lc], one, &cfg);
+    if (e != cudaSuccess) break;
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = kPairSmem;
+    e = cudaOccupancyMaxActiveClusters(&room->two[lc], two, &cfg);
+    room->one[lc] <<= lc;
+    room->two[lc] <<= lc;
+  }
+  return e;
+}
+
+// The cheapest shape; cluster 0 when a sequence has more items than the widest cluster holds.
+SelectShape select_shape(const BatchTable& bt, int hkv, const SelectRoom& room, bool fused_input) {
+  if (bt.max_items <= 0) return SelectShape{1, 512};
+  SelectShape best{0, 0};
+  double best_us = 1e30;
+  for (int lc = 0; lc <= 3; ++lc)
+    for (int threads = 512; threads <= 1024; threads += 512) {
+      if (room.one[lc] <= 0 || room.two[lc] <= 0) continue;
+      if (steps_per_warp(bt.max_items, 1 << lc, threads) > 32) continue;   // a warp's run has at most 32 steps
+      const double us = launch_cost(bt, hkv, room, fused_input && bt.chunk == 1, lc, threads);
+      if (us < best_us) { best_us = us; best = SelectShape{1 << lc, threads}; }
+    }
+  return best;
+}
 
 cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const Geometry& g,
                                   float force_threshold, bool fused_input, int pool_kind,
                                   int pool_size, float alpha, float beta, const LayerPtrs& lp,
-                                  const float* prior, int cluster) {
-  const Shape sh = select_shape(bt, g.hkv);
+                                  const float* prior, SelectShape sh) {
   ClusterParams P;
   P.cluster = sh.cluster;
-  P.per = bt.max_items > 0 ? (bt.max_items + sh.cluster * sh.threads - 1) / (sh.cluster * sh.threads) : 1;
+  P.per = steps_per_warp(bt.max_items, sh.cluster, sh.threads);
   P.hkv = g.hkv;
   P.theta = force_threshold;
   P.pool_kind = pool_kind;
@@ -844,3 +875,16 @@ cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const G
 }
 
 }  // namespace cc
+
+extern "C" void ccx_select_shape(int max_items, int num_seqs, int hkv, int chunk, int fused_input, const int* one,
+                                 const int* two, int* cluster, int* threads) {
+  static thread_local cc::BatchTable bt;
+  bt.max_items = max_items;
+  bt.num_seqs = num_seqs;
+  bt.chunk = chunk;
+  cc::SelectRoom room;
+  for (int i = 0; i < 4; ++i) { room.one[i] = one[i]; room.two[i] = two[i]; }
+  const cc::SelectShape sh = cc::select_shape(bt, hkv, room, fused_input != 0);
+  *cluster = sh.cluster;
+  *threads = sh.threads;
+}

@@ -21,3 +21,36 @@ def test_split_rows_of_chunk_scoring_never_add_a_wave(vocab, slots):
             assert p == 1
         elif rows < slots:                         # few rows: all of them, as far as one wave allows
             assert p == max(1, min(8, slots // rows, vocab // 8192))
+
+
+FULL = (148, 148, 132, 120), (296, 296, 284, 264)
+
+
+def _shape(items, seqs=1, hkv=8, chunk=1, fused=1, room=FULL):
+    one, two = ((C.c_int * 4)(*r) for r in room)
+    cluster, threads = C.c_int(), C.c_int()
+    binding.load_library().ccx_select_shape(items, seqs, hkv, chunk, fused, one, two, C.byref(cluster), C.byref(threads))
+    return cluster.value, threads.value
+
+
+@pytest.mark.parametrize("seqs,hkv", [(1, 1), (1, 8), (8, 8), (32, 8), (64, 32)])
+@pytest.mark.parametrize("chunk", [1, 10])
+def test_shape_of_the_selection_follows_the_device(seqs, hkv, chunk):
+    """Every shape holds its items (32 steps per warp) and uses a width that the device has room for, whatever
+    its number of SMs per GPC; items beyond the widest cluster are left to the other kernel."""
+    for items in (1, 513, 2048, 16384, 16385, 35784, 65536, 131072, 131073, 262144):
+        for room in (FULL, ((148, 148, 0, 0), (296, 296, 0, 0)), ((20, 20, 16, 8), (40, 40, 32, 16))):
+            cluster, threads = _shape(items, seqs, hkv, chunk, 1, room)
+            if cluster == 0:
+                assert items > 32 * 1024 * max(1 << i for i in range(4) if room[0][i])
+                continue
+            assert cluster in (1, 2, 4, 8) and threads in (512, 1024) and room[0][cluster.bit_length() - 1] > 0
+            assert cluster * threads * 32 >= items
+    assert _shape(262145, seqs, hkv, chunk)[0] == 0 and _shape(0, seqs, hkv, chunk) == (1, 512)
+
+
+def test_a_wave_of_wide_clusters_is_as_wide_as_the_device():
+    """Fourteen problems of 65536 items: 112 CTAs in clusters of eight are one wave where 120 run at a time and
+    two where 96 do, and then narrower clusters are cheaper."""
+    assert _shape(65536, 7, 2)[0] == 8
+    assert _shape(65536, 7, 2, room=((148, 148, 128, 96), (296, 296, 256, 192)))[0] == 4
