@@ -60,8 +60,7 @@ struct __align__(16) Shared {
   Cand own[kCand];                              // this CTA's candidates (peers read them)
   Cand all[kCand];                              // the cluster's, in rank order
   unsigned sub[256];                            // weights of the candidates by their next bits
-  unsigned n_own[2];                            // length of `own`, per search: the peers may still be reading the
-                                                // first search's when this CTA begins the second
+  unsigned n_own;                               // its length (peers read it)
   unsigned xchg[2][kMaxCluster][kWords];        // [buffer copy][source CTA][word]: written by the peers
   unsigned warp_x[2][kWords][kMaxWarps];        // block reductions, alternating
   unsigned bcast[4];
@@ -186,11 +185,10 @@ struct Cut {
 
 // Finds T such that weight(key > T) < R <= weight(key >= T), 1 <= R <= total weight of the
 // eligible items, whose keys lie in [kmin, kmax].  get(li, key, len) tells whether the local
-// item li is eligible; a warp calls it for its items [lo, hi) 32 at a time.  n_own: this search's
-// counter, 0 in every CTA of the cluster since before the last cluster barrier.
+// item li is eligible; a warp calls it for its items [lo, hi) 32 at a time.
 template <int THREADS, class Get>
 __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned kmin, unsigned kmax, unsigned max_len,
-                        bool allow_whole, unsigned* n_own, Get get) {
+                        bool allow_whole, Get get) {
   Shared& sm = *c.sm;
   const int lane = threadIdx.x & 31;
   const unsigned range = kmax - kmin;
@@ -234,6 +232,9 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       if (top == 32 || (kk >> top) == (prefix >> top)) atomicAdd(&h[(kk >> shift) & ((1u << bits) - 1u)], len);
     }
     c.sync_all();
+    // Only now have all peers read what an earlier search left here.  (A second counter cleared at the
+    // kernel's start did as well, and cost 0.3 us: 35784 tokens x 4 heads 43.4 -> 43.7.)
+    if (threadIdx.x == 0) sm.n_own = 0;
     // Thread t < kBins / 4 owns four bins, counted from the top, so a forward scan walks the keys
     // down; a peer's four are one 16-byte load (the exchange is paid per request: 4-byte loads by
     // all threads made this step 4 us long in clusters of eight), and all peers' are requested
@@ -321,13 +322,13 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     for (int li = lo + lane; li < hi; li += 32) {
       unsigned key, len;
       if (!get(li, key, len)) continue;
-      if ((((key - kmin) << sh) >> shift) == (prefix >> shift)) sm.own[atomicAdd(n_own, 1u)] = Cand{key, len};
+      if ((((key - kmin) << sh) >> shift) == (prefix >> shift)) sm.own[atomicAdd(&sm.n_own, 1u)] = Cand{key, len};
     }
     c.sync_all();
     unsigned first[kMaxCluster + 1];        // places of the CTAs' lists in the common one
     first[0] = 0;
 #pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) first[r + 1] = r < c.C ? *c.peer(n_own, r) : 0u;
+    for (int r = 0; r < kMaxCluster; ++r) first[r + 1] = r < c.C ? *c.peer(&sm.n_own, r) : 0u;
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r) first[r + 1] += first[r];
     const unsigned total = first[kMaxCluster];
@@ -457,7 +458,6 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 
 #pragma unroll 1
   for (int i = threadIdx.x; i < kBins; i += THREADS) sm.hist[0][i] = 0;
-  if (threadIdx.x < 2) sm.n_own[threadIdx.x] = 0;
   // Totals collected while loading: protected weight, key range of the unprotected items (of all
   // items when a cap may still strip some of their protection), range of the protected items'
   // priors when there is a cap
@@ -626,7 +626,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     if (!first && forced_tokens >= keep) break;       // protected items alone fill the budget: first B in order
     const unsigned cap = (unsigned)q.span_cap;
     cut = find_cut(c, lo, hi, first ? cap + 1u : keep - forced_tokens, first ? pri_lo : key_lo, first ? pri_hi : key_hi,
-                   (unsigned)cs, !first, &sm.n_own[stage - 1], [&](int li, unsigned& key, unsigned& len) {
+                   (unsigned)cs, !first, [&](int li, unsigned& key, unsigned& len) {
                      if ((flags[li] != 0) != first) return false;
                      key = first ? mono_key(item_prior(li)) : keys[li];
                      len = item_len(li);
