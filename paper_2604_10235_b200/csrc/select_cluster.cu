@@ -232,9 +232,6 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       if (top == 32 || (kk >> top) == (prefix >> top)) atomicAdd(&h[(kk >> shift) & ((1u << bits) - 1u)], len);
     }
     c.sync_all();
-    // Only now have all peers read what an earlier search left here.  (A second counter cleared at the
-    // kernel's start did as well, and cost 0.3 us: 35784 tokens x 4 heads 43.4 -> 43.7.)
-    if (threadIdx.x == 0) sm.n_own = 0;
     // Thread t < kBins / 4 owns four bins, counted from the top, so a forward scan walks the keys
     // down; a peer's four are one 16-byte load (the exchange is paid per request: 4-byte loads by
     // all threads made this step 4 us long in clusters of eight), and all peers' are requested
@@ -316,7 +313,11 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
   }
   unsigned gt_before = below, eq_before = 0;
   if (rank_keys) {
-
+    // Behind this search's histograms all peers have read what an earlier search left in the counter.
+    // (A counter per search cleared at the kernel's start, or the clearing right behind the histogram's
+    // barrier, cost 0.2-0.3 us on one shape or another.)
+    if (threadIdx.x == 0) sm.n_own = 0;
+    __syncthreads();
     // the bin's keys, listed per CTA and read by all of them in rank order
 #pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32) {
