@@ -66,8 +66,8 @@ class cc_layer_desc(C.Structure):
 
 
 _LIB = None
-_CALL = None          # the extension's call(fn, spec, *args): see csrc/py_call.cpp
-# arguments of the entry points that are called through it, after the context and the descriptor
+_BIND = None          # the extension's bind(name, address, spec): see csrc/py_call.cpp
+# arguments of the entry points that are called through it
 _SPEC = {"cc_score_window": b"iittttwi", "cc_fuse_prior_pool": b"iittti", "cc_topk_select": b"iittttwi",
          "cc_topk_select_static": b"iitttti", "cc_compact_kv": b"iippttttti",
          "cc_compress_layer": b"iittptttttttwi", "cc_compress_layers": b"iiiLLLtLLLLLLwi",
@@ -76,7 +76,7 @@ _SPEC = {"cc_score_window": b"iittttwi", "cc_fuse_prior_pool": b"iittti", "cc_to
 
 def load_library(path: Optional[str] = None) -> C.CDLL:
     """Loads (building first if the sources are newer) the in-tree shared library."""
-    global _LIB, _CALL
+    global _LIB, _BIND
     if _LIB is not None and path is None:
         return _LIB
     if path is None:
@@ -120,12 +120,12 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     for name in EXPORTS:
         if name not in ("cc_status_string", "cc_last_error", "cc_workspace_bytes", "cc_layers_workspace_bytes"):
             getattr(lib, name).restype = C.c_int
-    lib.addresses = {name: C.cast(getattr(lib, name), vp).value for name in _SPEC}
-    if _CALL is None:
+    if _BIND is None:
         loader = importlib.machinery.ExtensionFileLoader("_cccall", _build.CALL_PATH)
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_cccall", loader))
         loader.exec_module(module)
-        _CALL = module.call
+        _BIND = module.bind
+    lib.calls = {name: _BIND(name, C.cast(getattr(lib, name), vp).value, spec) for name, spec in _SPEC.items()}
     if path == _build.LIB_PATH:
         _LIB = lib
     return lib
@@ -153,7 +153,7 @@ class Context:
 
     def call(self, name: str, desc: "Desc", *args) -> None:
         """Calls entry point ``name`` with this context, the descriptor and the arguments."""
-        rc = _CALL(self.lib.addresses[name], _SPEC[name], self.handle.value, C.addressof(desc.c), *args)
+        rc = self.lib.calls[name](self.handle.value, C.addressof(desc.c), *args)
         if rc:
             self.check(rc)
 
@@ -264,11 +264,17 @@ class Desc:
         return sum((n + ch - 1) // ch for n in self.lens)
 
 
+# the current stream without a Stream object around it, where this torch has the function
+_CURRENT_RAW = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _raw(stream: Optional[int]) -> int:
     """The stream as an integer; None is torch's current stream."""
-    if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    return stream
+    if stream is not None:
+        return stream
+    if _CURRENT_RAW is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _CURRENT_RAW(torch.cuda.current_device())
 
 
 def _stream(stream: Optional[int]) -> C.c_void_p:
@@ -325,15 +331,14 @@ def cc_ppl_chunk_scores(ctx: Context, logits: torch.Tensor, targets: torch.Tenso
     chunks, t, v = logits.shape
     assert logits.stride(2) == 1
     dtype = CC_F32 if logits.dtype == torch.float32 else CC_BF16
-    rc = _CALL(ctx.lib.addresses["cc_ppl_chunk_scores"], _SPEC["cc_ppl_chunk_scores"], ctx.handle.value, logits,
-               dtype, chunks, t, v, logits.stride(0), logits.stride(1), targets, nll, score, _raw(stream))
+    rc = ctx.lib.calls["cc_ppl_chunk_scores"](ctx.handle.value, logits, dtype, chunks, t, v, logits.stride(0),
+                                              logits.stride(1), targets, nll, score, _raw(stream))
     if rc:
         ctx.check(rc)
 
 
 def cc_select_chunks(ctx: Context, score: torch.Tensor, k: int, chosen: torch.Tensor, stream=None):
-    rc = _CALL(ctx.lib.addresses["cc_select_chunks"], _SPEC["cc_select_chunks"], ctx.handle.value, score,
-               score.numel(), k, chosen, _raw(stream))
+    rc = ctx.lib.calls["cc_select_chunks"](ctx.handle.value, score, score.numel(), k, chosen, _raw(stream))
     if rc:
         ctx.check(rc)
 

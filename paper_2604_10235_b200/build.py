@@ -12,7 +12,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB_DIR = os.path.join(HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libcodecomp.so")
-CALL_PATH = os.path.join(LIB_DIR, "_cccall.so")        # Python extension that marshals the calls
+# Python extension that marshals the calls; the suffix names the interpreter it is built for
+CALL_PATH = os.path.join(LIB_DIR, "_cccall" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["api.cu", "score_simt.cu", "score_tc.cu", "fuse_pool.cu", "select.cu", "select_cluster.cu", "compact.cu",
            "str_score.cu", "planner.cu", "ppl.cu", "exp_probe.cu"]
 
@@ -47,7 +48,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         common += ["-Xptxas", "-v"]
     call = [nvcc, "-shared", "-cudart", "none", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
-            "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "py_call.cpp"), "-o", CALL_PATH]
+            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), os.path.join(CSRC, "py_call.cpp"), "-o", CALL_PATH]
     procs = [("py_call.cpp", subprocess.Popen(call, stdout=subprocess.PIPE, stderr=subprocess.STDOUT,
                                               text=True))]
     objs = []

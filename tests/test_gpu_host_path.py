@@ -138,3 +138,15 @@ def test_v_in_place_needs_page_locked_memory():
         comp.run_host(*host, v_in_place=True)
     with pytest.raises(ValueError):                          # the binding refuses pageable memory too
         cc.cc_compact_kv(ctx(), comp.desc, comp.k, host[2], comp.idx, comp.k_out, comp.v_out)
+
+
+def test_calls_go_to_the_current_stream_whichever_way_it_is_read(monkeypatch):
+    from paper_2604_10235_b200 import binding
+    side = torch.cuda.Stream()
+    for stream in (torch.cuda.current_stream(), side):
+        with torch.cuda.stream(stream):
+            assert binding._raw(None) == stream.cuda_stream
+            with monkeypatch.context() as m:
+                m.setattr(binding, "_CURRENT_RAW", None)
+                assert binding._raw(None) == stream.cuda_stream
+            assert binding._raw(77) == 77
