@@ -19,3 +19,12 @@ def test_scores_of_cut_tiles_and_short_problems(w, hq, hkv, lens, page, causal):
     wl = gen.Workload("spans", 27, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1,
                       page_size=page, causal=causal)
     check_against_oracle(wl, gen.make_layer(wl, layer=sum(lens), with_v=False), cc.CC_MODE_BF16, 2e-3)
+
+
+@pytest.mark.parametrize("w,hq,hkv", [(16, 2, 2), (32, 2, 2), (96, 2, 2), (112, 2, 2), (36, 8, 2), (56, 8, 2), (68, 8, 2),
+                                      (48, 28, 4), (100, 8, 2), (50, 28, 4), (64, 28, 4)])
+@pytest.mark.parametrize("lens,page", [((20000,), 0), ((500, 130, 77) * 3, 16)])
+def test_scores_where_the_last_block_of_rows_is_not_full(w, hq, hkv, lens, page):
+    """16 to 448 rows, one to four blocks of 128, the last of which has 0 to 3 warps without rows."""
+    wl = gen.Workload("padded", 28, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1, page_size=page)
+    check_against_oracle(wl, gen.make_layer(wl, layer=w, with_v=False), cc.CC_MODE_BF16, 2e-3)
