@@ -602,6 +602,7 @@ def host_time_per_layer(ctx, rank):
     outs_v = [torch.empty_like(comp.v_out) for _ in range(n)]
     idxs = [torch.empty_like(comp.idx) for _ in range(n)]
     cnts = [torch.empty_like(comp.count) for _ in range(n)]
+    ws = ctx.workspace(comp.desc, n)
     out = {}
     for name in ("per_call", "all_layers"):
         best = None
@@ -615,7 +616,7 @@ def host_time_per_layer(ctx, rank):
             else:
                 cc.cc_compress_layers(ctx, comp.desc, [x[0] for x in layers], [x[1] for x in layers],
                                       [x[2] for x in layers], layers[0][3], outs_k, outs_v, idxs, cnts,
-                                      ws=comp.ws)
+                                      ws=ws)
             t1 = time.perf_counter()
             torch.cuda.synchronize()
             t2 = time.perf_counter()
