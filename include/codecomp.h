@@ -245,8 +245,9 @@ int cc_structural_score(cc_ctx* ctx, const cc_layer_desc* desc, const int32_t* i
 /* Chunk selection (Section 4.1 "Query-Conditioned Chunk Selection").  logits holds, for every
  * candidate chunk i and query position t, the model's V next-token logits given prefix + C_i and
  * the earlier query tokens: element (i, t, v) at logits[i * stride_chunk + t * stride_token + v]
- * (device, CC_BF16 or CC_F32; strides in elements; rows that all start on 16-byte boundaries
- * are read with vector loads, others value by value, several times slower); targets: device
+ * (device, CC_BF16 or CC_F32; strides in elements; rows may start anywhere: only the values before
+ * the first and after the last 16-byte boundary of a row are read one by one; masked logits may be
+ * -inf or the lowest value of the type, a row of nothing else gives NaN); targets: device
  * i32 [num_tokens], the query tokens q_t.  nll: device f32 [num_chunks][num_tokens] receives
  * -log p(q_t | ...) = logsumexp(row) - row[q_t]; score: device f32 [num_chunks] receives their
  * mean s_i^ppl.  A token id outside [0, V) gives NaN and CC_ERR_DEVICE_FLAG in the status word.

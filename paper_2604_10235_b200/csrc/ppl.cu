@@ -208,11 +208,11 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
   }
   if (threadIdx.x == 0) {
     const int target = targets[t];
-    float out = __int_as_float(0x7fc00000);                   // NaN for an invalid token id
-    if (target >= 0 && target < vocab)
-      out = ((all.m > kNoMax ? all.m : -INFINITY) + log2f(all.s)) * kLn2 - Vec<T>::one(x + target);
-    else
+    float out = __int_as_float(0x7fc00000);                   // NaN for an invalid token id or a row of masked logits
+    if (target < 0 || target >= vocab)
       report_error(status, CC_ERR_DEVICE_FLAG, 600);
+    else if (all.m > kNoMax)
+      out = (all.m + log2f(all.s)) * kLn2 - Vec<T>::one(x + target);
     nll[row] = out;
   }
 }
