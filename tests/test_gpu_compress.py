@@ -180,8 +180,8 @@ def test_span_cap_ragged_paged_and_chunked(mode, tol):
 @pytest.mark.parametrize("n,pool,k", [(140000, gen.POOL_MAX, 7), (140000, gen.POOL_AVG, 5),
                                       (270000, gen.POOL_MAX, 7)])
 def test_more_items_than_a_cluster_stages_or_holds(n, pool, k):
-    """140000 items: more than 16 per thread of the widest cluster, so the cluster kernel pools
-    straight from global memory instead of staging the raw scores.  270000 items: more than a
+    """140000 items: slices of 18 steps per warp of the widest cluster, pooled in parts that go through
+    the two staging buffers in turn.  270000 items: more than a
     cluster holds (262144), so the fused call and cc_topk_select take the single-CTA selection
     kernel and the stand-alone pooling kernel instead."""
     wl = gen.Workload("long", 36, 1, 2, 1, 128, 8, pool, k, 9000, n=n)
