@@ -141,7 +141,7 @@ int cc_poll_status(cc_ctx* ctx, void* stream, int* device_status);
  * Returns 0 if the descriptor is invalid. */
 size_t cc_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc);
 /* Bytes that cc_compress_layers can make use of on n_layers layers: given that much instead of
- * cc_workspace_bytes (which is enough, and never more), it runs short layers several to a launch.  In
+ * cc_workspace_bytes (which is enough, and never larger), it runs short layers several to a launch.  In
  * between it takes as many layers per launch as fit.  Returns 0 if the descriptor is invalid. */
 size_t cc_layers_workspace_bytes(const cc_ctx* ctx, const cc_layer_desc* desc, int32_t n_layers);
 

@@ -10,8 +10,8 @@
 // raises the maximum; the threads' pairs are merged with shuffles.  With 2-byte logits the issue
 // slots come close to the memory time, so scaling and sums are packed f32x2 operations, maxima of
 // bf16 logits are taken on the packed words, and (POLY) one pair of exponentials in eight is evaluated
-// on the FMA pipe.  32 x 64 rows of 128256 logits: bf16 90 us = 5.84 TB/s (93 us with scalar
-// arithmetic), f32 154 us = 6.8 TB/s.  Keeping the loads of the next batch in flight during the
+// on the FMA pipe.  32 x 64 rows of 128256 logits, replayed: bf16 85 us = 6.2 TB/s (scalar
+// arithmetic: 3 us more), f32 150 us = 7.0 TB/s.  Keeping the loads of the next batch in flight during the
 // arithmetic needs 64 registers and costs a resident CTA: slower for bf16 (97 us).
 #include <cooperative_groups.h>
 #include <float.h>
