@@ -52,6 +52,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -84,45 +89,78 @@ __device__ __forceinline__ uint64_t ex2_pair_fma(uint64_t x) {
   return pack2(__int_as_float(r0), __int_as_float(r1));
 }
 
-#ifndef CC_POLY_EVERY
-#define CC_POLY_EVERY 3
-#endif
-constexpr int kPolyEvery = CC_POLY_EVERY;        // one pair in this many takes the polynomial path
+// 2^x on the FMA pipe for x = v * c + off given by its place y = (x + kSatLow) / kSatSpan on a scale that the multiply-add
+// saturates to [0, 1]: both clamps (2^-124 below, 2^124 above) come with the scaling.  kSatSpan is an integer for which
+// kScale / kSatSpan is exact in f32, and offsets are multiples of kSatSpan / 1024, for which off / kSatSpan is:
+// what remains is the rounding of y, 4e-6 in x on either side (with other spans and offsets the roundings of the
+// constants moved all scores by 2e-6).
+constexpr float kScale = 0.12751743f;            // log2(e) / sqrt(128)
+constexpr float kSatLow = 124.0f, kSatSpan = 248.0f, kSatScale = kScale / kSatSpan;
+__device__ __forceinline__ float sat_grid(float x) { return rintf(x * (1024.0f / kSatSpan)) * (kSatSpan / 1024.0f); }
+__device__ __forceinline__ float sat_offset(float off) { return fmaf(off, 1.0f / kSatSpan, 0.5f); }
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+  float d;
+  asm("fma.rn.ftz.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t ex2_pair_sat(float y0, float y1) {
+  const uint64_t y = pack2(y0, y1), span = pack2(kSatSpan, kSatSpan), bias = pack2(kEx2Magic - kSatLow, kEx2Magic - kSatLow);
+  const uint64_t t = fma2(y, span, bias);             // magic + x, rounded to an integer
+  const uint64_t f = fma2(y, span, sub2(bias, t));    // x - n
+  uint64_t p = fma2(f, pack2(kEx2C3, kEx2C3), pack2(kEx2C2, kEx2C2));
+  p = fma2(p, f, pack2(kEx2C1, kEx2C1));
+  p = fma2(p, f, pack2(kEx2C0, kEx2C0));
+  float p0, p1, t0, t1;
+  unpack2(p, p0, p1);
+  unpack2(t, t0, t1);
+  int r0, r1;
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
+  return pack2(__int_as_float(r0), __int_as_float(r1));
+}
 
-// acc += 2^(v * c + off) over the first kWidth of 32 values; off is one pair for all of them or
-// read per value from shared memory (off_col: shared-space address of the first value's offset).
-// Of every kPolyEvery pairs one goes to the FMA pipe, the
-// others to the special-function unit.
-template <bool kPerColumn, int kWidth>
-__device__ __forceinline__ void exp_accumulate(const uint32_t (&v)[32], uint64_t c2, uint64_t off2,
-                                               uint32_t off_col, uint64_t (&acc)[4]) {
+// Of every three pairs one takes the polynomial path, the middle one, and the two paths have a sum each: the
+// special-function unit is the fuller pipe (one pair in four: +3 to 5 % on the score kernel, six of sixteen: +5 %), and the
+// order of the source decides how well it stays fed (polynomials bunched together: +3 to 7 %, three sums for the
+// special-function path: +1 %).
+__device__ __forceinline__ constexpr bool poly_pair(int pair) { return pair % 3 == 1; }
+
+// acc += 2^(v * kScale + off) over the first kWidth of 32 values; off per value from shared memory (off_col: shared-space address of
+// the first one, so that the loads need no address arithmetic).  Arguments up to 64.
+template <int kWidth>
+__device__ __forceinline__ void exp_accumulate_columns(const uint32_t (&v)[32], uint32_t off_col, uint64_t (&acc)[2]) {
+  const uint64_t c2 = pack2(kScale, kScale);
 #pragma unroll
   for (int i = 0; i < kWidth; i += 4) {
-    uint64_t o[2] = {off2, off2};
-    if (kPerColumn) {
-      // off_col is the shared-space address of the offsets: a shared-space load at a constant
-      // distance from it needs no address arithmetic per load
-      float4 L;
-      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                   : "=f"(L.x), "=f"(L.y), "=f"(L.z), "=f"(L.w)
-                   : "r"(off_col + (uint32_t)(i * 4)));
-      o[0] = pack2(L.x, L.y);
-      o[1] = pack2(L.z, L.w);
-    }
+    float4 L;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(L.x), "=f"(L.y), "=f"(L.z), "=f"(L.w)
+                 : "r"(off_col + (uint32_t)(i * 4)));
+    const uint64_t o[2] = {pack2(L.x, L.y), pack2(L.z, L.w)};
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const int pair = (i >> 1) + k;
       const uint64_t x = fma2(pack2(__uint_as_float(v[i + 2 * k]), __uint_as_float(v[i + 2 * k + 1])), c2, o[k]);
-      if (pair % kPolyEvery == kPolyEvery - 1) acc[3] = add2(acc[3], ex2_pair_fma(x));
-      else acc[pair % 3] = add2(acc[pair % 3], ex2_pair_sfu(x));
+      if (poly_pair((i >> 1) + k)) acc[1] = add2(acc[1], ex2_pair_fma(x));
+      else acc[0] = add2(acc[0], ex2_pair_sfu(x));
     }
   }
 }
-__device__ __forceinline__ float acc_total(const uint64_t (&acc)[4]) {
-  float a, b, c, d;
+// The same with c = kScale and one offset for all values (none: 0), a multiple of kSatSpan / 1024, whose os = sat_offset(off).
+// Arguments above 124 saturate: 2^124, or more up to infinity.
+template <bool kOffset, int kWidth>
+__device__ __forceinline__ void exp_accumulate(const uint32_t (&v)[32], uint64_t off2, float os, uint64_t (&acc)[2]) {
+  const uint64_t c2 = pack2(kScale, kScale);
+#pragma unroll
+  for (int pair = 0; pair < kWidth / 2; ++pair) {
+    const float a = __uint_as_float(v[2 * pair]), b = __uint_as_float(v[2 * pair + 1]);
+    if (poly_pair(pair)) acc[1] = add2(acc[1], ex2_pair_sat(fma_sat(a, kSatScale, os), fma_sat(b, kSatScale, os)));
+    else acc[0] = add2(acc[0], ex2_pair_sfu(kOffset ? fma2(pack2(a, b), c2, off2) : mul2(pack2(a, b), c2)));
+  }
+}
+__device__ __forceinline__ float acc_total(const uint64_t (&acc)[2]) {
+  float a, b;
   unpack2(add2(acc[0], acc[1]), a, b);
-  unpack2(add2(acc[2], acc[3]), c, d);
-  return (a + b) + (c + d);
+  return a + b;
 }
 
 }  // namespace cc

@@ -26,7 +26,7 @@
 // passes (16 per clock on the special-function unit against 8192 tensor flops per clock), and
 // what counts is that the unit never idles: a warp reads 32 columns at a time, so it needs few
 // registers and four warps fit per scheduler; scaling and accumulation use packed f32x2
-// instructions; one pair of exponentials in kPolyEvery is evaluated on the FMA pipe instead
+// instructions; one pair of exponentials in three is evaluated on the FMA pipe instead
 // (round to nearest integer, degree-3 polynomial for the fraction, exponent patched in by
 // integer arithmetic; relative error 8e-5).
 //
@@ -62,7 +62,6 @@ constexpr int kBufs = 4;                                  // accumulator buffers
 constexpr int kSets = 4;                                  // epilogue warp sets, one per buffer
 constexpr uint32_t kMiscBytes = 20480;
 constexpr uint32_t kSmemLimit = 232448;                   // 227 KB
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 struct TcParams {
@@ -290,9 +289,8 @@ __device__ __forceinline__ bool warp_wait(const Pipe& p, uint64_t* bar, uint32_t
 // ------------------------------------------------------------------ the four drains
 // One accumulator buffer through a warp, 32 columns at a time.  The common forms and the masked ones
 // are loops of their own, so that the common ones hold no range tests and no moves of values that
-// only the others overwrite.  Bound by the exponentials and the issue slots around them: 14.7
-// (pass 1) and 14.3 (pass 2) exponentials per clock per SM on 131072 tokens x 8 heads, against 20.1 for
-// the arithmetic and the reads alone; 176 and 177 instructions per chunk over all warps of the CTA.
+// only the others overwrite.  Bound by the exponentials and the issue slots around them: the arithmetic and the reads alone reach 20.1
+// per clock per SM.
 __device__ __forceinline__ void hand_back(uint32_t empty_bar, int lane) {
   tc_fence_before();
   __syncwarp();
@@ -300,36 +298,49 @@ __device__ __forceinline__ void hand_back(uint32_t empty_bar, int lane) {
 }
 
 // pass 1, all 128 keys count.  The reference of the exponentials only has to be near the row
-// maximum, not equal to it: it is replaced when a value lies more than 2^64 above it.
-__device__ __forceinline__ void drain_keys(uint32_t addr, uint32_t empty_bar, int lane, float c, uint64_t c2,
-                                           float& m_run, float& l_run) {
-  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+// maximum, not equal to it: it is replaced when a value lies more than 2^64 above it.  Only the first
+// chunk of a row and the last of an item look at their maximum beforehand, a serial stretch of 16 instructions, a
+// vote and a branch before the first exponential; what the chunks in between add is
+// looked at before the buffer goes back, and when it is above kRedo (exponentials saturate at 2^124) nothing
+// has been changed and the answer is false: the caller goes through the item again, chunk by chunk.  (Together
+// with the saturating scale of the polynomial's arguments, the score stage of 32768 tokens x 8 heads of 256 rows -2.9 %,
+// 65536 x 4 of 448 -3.5 %, 32 x 2200 x 8 of 512 -2.8 %, 131072 x 8 of 256 -3.8 %.)
+constexpr float kRedo = 1.1805916e21f;     // 2^70
+__device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, int lane, float& m_run, float& l_run) {
+  uint64_t acc[2] = {0ull, 0ull};
+  float m = m_run, l = l_run;
+  bool look = __any_sync(0xffffffffu, m == -INFINITY);
 #pragma unroll 1
   for (int cc0 = 0; cc0 < kTileKeys; cc0 += 32) {
     uint32_t v[32];
     tmem_ld32(addr + (uint32_t)cc0, v);
     tmem_wait_ld();
-    if (cc0 + 32 == kTileKeys) hand_back(empty_bar, lane);
-    const float mx = max32(v) * c;
-    const bool renew = m_run == -INFINITY || mx > m_run + 64.0f;
-    if (__any_sync(0xffffffffu, renew)) {
-      if (renew) {
-        if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
-        acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
-        m_run = mx;
+    if (look) {
+      if (cc0 + 32 == kTileKeys) {
+        if (__any_sync(0xffffffffu, !(acc_total(acc) < kRedo))) return false;
+        hand_back(empty_bar, lane);
       }
+      const float mx = max32(v) * kScale;
+      if (m == -INFINITY || mx > m + 64.0f) {
+        const float ref = sat_grid(mx);
+        if (m > -INFINITY) l = (l + acc_total(acc)) * ex2(m - ref);
+        acc[0] = acc[1] = 0ull;
+        m = ref;
+      }
+      __syncwarp();
     }
-    exp_accumulate<false, 32>(v, c2, pack2(-m_run, -m_run), 0u, acc);
+    look = cc0 + 64 == kTileKeys;
+    exp_accumulate<true, 32>(v, pack2(-m, -m), sat_offset(-m), acc);
   }
-  l_run += acc_total(acc);
+  m_run = m;
+  l_run = l + acc_total(acc);
+  return true;
 }
 
 // pass 1, keys from valid_r on (a bound of the thread's own) do not count
 // (returns the row's new reference and sum)
-__device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empty_bar, int lane, float c, int valid_r,
-                                                 float m_run, float l_run) {
-  const uint64_t c2 = pack2(c, c);
-  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+__device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empty_bar, int lane, int valid_r, float m_run, float l_run) {
+  uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
   for (int cc0 = 0; cc0 < kTileKeys; cc0 += 32) {
     uint32_t v[32];
@@ -341,45 +352,42 @@ __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empt
 #pragma unroll
     for (int i = 0; i < 32; ++i)
       if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
-    const float mx = max32(v) * c;
+    const float mx = sat_grid(max32(v) * kScale);
     if (m_run == -INFINITY || mx > m_run + 64.0f) {
       if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
-      acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
+      acc[0] = acc[1] = 0ull;
       m_run = mx;
     }
-    exp_accumulate<false, 32>(v, c2, pack2(-m_run, -m_run), 0u, acc);
+    exp_accumulate<true, 32>(v, pack2(-m_run, -m_run), sat_offset(-m_run), acc);
   }
   return make_float2(m_run, l_run + acc_total(acc));
 }
 
 // pass 2: nc columns (a multiple of 16), -L_r of the first at shared-space address nl
-__device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, int lane, uint64_t c2, uint32_t nl,
-                                            int nc) {
-  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+__device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, int lane, uint32_t nl, int nc) {
+  uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
   for (int cc0 = 0; cc0 + 32 <= nc; cc0 += 32) {
     uint32_t v[32];
     tmem_ld32(addr + (uint32_t)cc0, v);               // stays inside the 128-column buffer
     tmem_wait_ld();
     if (cc0 + 32 == nc) hand_back(empty_bar, lane);
-    exp_accumulate<true, 32>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
+    exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
   }
   if (nc & 16) {
     uint32_t v[32];
     tmem_ld32(addr + (uint32_t)(nc - 16), v);
     tmem_wait_ld();
     hand_back(empty_bar, lane);
-    exp_accumulate<true, 16>(v, c2, 0ull, nl + 4u * (uint32_t)(nc - 16), acc);
+    exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)(nc - 16), acc);
   }
   return acc_total(acc);
 }
 
 // pass 2, columns before first_col (a bound of the thread's own) do not count
 // (returns the sum)
-__device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty_bar, int lane, float c, uint32_t nl,
-                                                int nc, int first_col) {
-  const uint64_t c2 = pack2(c, c);
-  uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+__device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty_bar, int lane, uint32_t nl, int nc, int first_col) {
+  uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
   for (int cc0 = 0; cc0 < nc; cc0 += 32) {
     uint32_t v[32];
@@ -390,8 +398,8 @@ __device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty
 #pragma unroll
     for (int i = 0; i < 32; ++i)
       if (cc0 + i < first_col) v[i] = 0xc61c4000u;     // -1e4: exponential ~ 0
-    if (cc0 + 32 <= nc) exp_accumulate<true, 32>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
-    else                exp_accumulate<true, 16>(v, c2, 0ull, nl + 4u * (uint32_t)cc0, acc);
+    if (cc0 + 32 <= nc) exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
+    else                exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)cc0, acc);
   }
   return acc_total(acc);
 }
@@ -698,8 +706,6 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int row_in_tile = quad * 32 + lane;
     const int etid = ew * 32 + lane;         // 0..511, unique per epilogue thread
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    const float c = kLog2e / sqrtf((float)kHeadDim);
-    const uint64_t c2 = pack2(c, c);
     TileCursor cur;
     cur.locate(bt, g.hkv, t_begin);
     int cur_problem = -1;
@@ -862,9 +868,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
 #pragma unroll
             for (int rb = 1; rb < 4; ++rb) if (rb == sub) { m_run = run_m[rb]; l_run = run_l[rb]; }
           }
-          if (!edge) {
-            drain_keys(acc_addr, empty_bar, lane, c, c2, m_run, l_run);
-          } else {
+          if (edge || !drain_keys(acc_addr, empty_bar, lane, m_run, l_run)) {
             // keys of the tile this row attends to: the valid ones, or (causal window) those up to the
             // row's own position n - w + t
             int valid_r = valid;
@@ -872,7 +876,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
               const int t_row = (sub * 128 + row_in_tile) / g.group;
               if (t_row < g.window) valid_r = min(valid, n_cur - g.window + t_row + 1 - key0);
             }
-            const float2 st = drain_keys_masked(acc_addr, empty_bar, lane, c, valid_r, m_run, l_run);
+            const float2 st = drain_keys_masked(acc_addr, empty_bar, lane, valid_r, m_run, l_run);
             m_run = st.x;
             l_run = st.y;
           }
@@ -887,12 +891,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           // thread = key (key0 + row_in_tile); columns = the query rows of this chunk
           const int c0 = sub * P.sub_cols;
           const int nc = min(P.sub_cols, P.rows_pad - c0);        // multiple of 16
-          const uint32_t nl = smem_u32(misc->neg_lc + c0);         // -L_r of the item's columns
           // causal window: key j is seen by the rows t >= j - (n - w), i.e. by the columns from
           // G * (j - n + w) on; the columns before it contribute nothing
-          u_acc = edge ? drain_rows_masked(acc_addr, empty_bar, lane, c, nl, nc,
-                                           g.group * (key0 + row_in_tile - n_cur + g.window) - c0)
-                       : drain_rows(acc_addr, empty_bar, lane, c2, nl, nc);
+          const uint32_t nl = smem_u32(misc->neg_lc + c0);         // -L_r of the item's columns
+          u_acc = edge ? drain_rows_masked(acc_addr, empty_bar, lane, nl, nc, g.group * (key0 + row_in_tile - n_cur + g.window) - c0)
+                       : drain_rows(acc_addr, empty_bar, lane, nl, nc);
         }
       }
       if (PASS == 2) {
