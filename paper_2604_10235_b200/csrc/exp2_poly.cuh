@@ -89,14 +89,12 @@ __device__ __forceinline__ uint64_t ex2_pair_fma(uint64_t x) {
   return pack2(__int_as_float(r0), __int_as_float(r1));
 }
 
-// 2^x on the FMA pipe for x = v * c + off given by its place y = (x + kSatLow) / kSatSpan on a scale that the multiply-add
-// saturates to [0, 1]: both clamps (2^-124 below, 2^124 above) come with the scaling.  kSatSpan is an integer for which
-// kScale / kSatSpan is exact in f32, and offsets are multiples of kSatSpan / 1024, for which off / kSatSpan is:
-// what remains is the rounding of y, 4e-6 in x on either side (with other spans and offsets the roundings of the
-// constants moved all scores by 2e-6).
+// 2^x on the FMA pipe for x = v * kScale + off given by its place y = (x + kSatLow) / kSatSpan on a scale that the
+// multiply-add saturates to [0, 1]: both clamps (2^-124 below, 2^124 above) come with the scaling.  kSatSpan is an integer for
+// which kScale / kSatSpan is exact in f32 and kSatLow / kSatSpan is one half: what remains is the rounding of y, 4e-6 in x (a
+// span of 252 had moved all scores by 2e-6).
 constexpr float kScale = 0.12751743f;            // log2(e) / sqrt(128)
 constexpr float kSatLow = 124.0f, kSatSpan = 248.0f, kSatScale = kScale / kSatSpan;
-__device__ __forceinline__ float sat_grid(float x) { return rintf(x * (1024.0f / kSatSpan)) * (kSatSpan / 1024.0f); }
 __device__ __forceinline__ float sat_offset(float off) { return fmaf(off, 1.0f / kSatSpan, 0.5f); }
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   float d;
@@ -119,11 +117,11 @@ __device__ __forceinline__ uint64_t ex2_pair_sat(float y0, float y1) {
   return pack2(__int_as_float(r0), __int_as_float(r1));
 }
 
-// Of every three pairs one takes the polynomial path, the middle one, and the two paths have a sum each: the
-// special-function unit is the fuller pipe (one pair in four: +3 to 5 % on the score kernel, six of sixteen: +5 %), and the
-// order of the source decides how well it stays fed (polynomials bunched together: +3 to 7 %, three sums for the
-// special-function path: +1 %).
-__device__ __forceinline__ constexpr bool poly_pair(int pair) { return pair % 3 == 1; }
+// Of every three pairs one takes the polynomial path, and the two paths have a sum each: the special-function unit is the
+// fuller pipe (one pair in four: +3 to 5 % on the score kernel, six of sixteen: +5 %), and the order of the source decides how
+// well it stays fed (polynomials bunched together: +3 to 7 %).  Which pairs they are decides which values carry the
+// polynomial's error: another choice is as good, but moves scores by 2e-6 and with them some ties at the cut-off.
+__device__ __forceinline__ constexpr bool poly_pair(int pair) { return pair % 3 == 2; }
 
 // acc += 2^(v * kScale + off) over the first kWidth of 32 values; off per value from shared memory (off_col: shared-space address of
 // the first one, so that the loads need no address arithmetic).  Arguments up to 64.
@@ -145,7 +143,7 @@ __device__ __forceinline__ void exp_accumulate_columns(const uint32_t (&v)[32], 
     }
   }
 }
-// The same with c = kScale and one offset for all values (none: 0), a multiple of kSatSpan / 1024, whose os = sat_offset(off).
+// The same with one offset for all values (none: 0), os = sat_offset(off).
 // Arguments above 124 saturate: 2^124, or more up to infinity.
 template <bool kOffset, int kWidth>
 __device__ __forceinline__ void exp_accumulate(const uint32_t (&v)[32], uint64_t off2, float os, uint64_t (&acc)[2]) {

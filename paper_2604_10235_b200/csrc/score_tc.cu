@@ -32,6 +32,7 @@
 //
 // Every wait on an mbarrier is bounded: when the bound is hit the kernel records
 // CC_ERR_TIMEOUT, every role leaves its loop, TMEM is released and the kernel returns.
+#include <cuda_bf16.h>
 #include <string.h>
 
 #include <type_traits>
@@ -60,7 +61,8 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kBufCols = 128;                        // accumulator buffer stride
 constexpr int kBufs = 4;                                  // accumulator buffers in TMEM
 constexpr int kSets = 4;                                  // epilogue warp sets, one per buffer
-constexpr uint32_t kMiscBytes = 20480;
+constexpr uint32_t kMiscBytes = 18432;
+constexpr uint32_t kLBytes = 20, kLFixed = 8 * 16 + kTileKeys * 4;   // -L_r in its two forms: bytes a row, and besides
 constexpr uint32_t kSmemLimit = 232448;                   // 227 KB
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -131,6 +133,10 @@ __device__ __forceinline__ bool mbar_spin(uint32_t bar, uint32_t parity) {
       "D%=:\n\tselp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
   return ok != 0;
+}
+// This thread's stores to shared memory before, the tensor core's reads after.
+__device__ __forceinline__ void fence_proxy_async() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -235,17 +241,19 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t m, uint32_t n) {
 struct Barriers {
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
-  uint64_t q_full, q_empty;
+  uint64_t q_full, q_empty, l_full;
   uint64_t acc_full[kBufs], acc_empty[kBufs];
   uint64_t u_full[8][4];             // pass 2: the other sets' partial sums of (slot, quadrant)
   uint64_t edge_full[2][4];          // ... of a first / last tile of which the CTA has one half
 };
 
 struct Misc {                        // lives in the last kMiscBytes of dynamic shared memory
-  float neg_lc[kMaxRows];            // pass 2: -L_r in the log2 domain (-1e4 for padded rows)
   union {
-    float2 xchg[kSets][kMaxRows];    // (max, sum) hand-over: pass 1 per set, pass 2 while merging
-    float u_part[8][kSets][kTileKeys];   // pass 2: partial column sums, slot = tile & 7
+    float2 xchg[kSets][kMaxRows];    // (max, sum) hand-over: pass 1 per set, pass 2 while merging (the first of them)
+    struct {
+      float u_part[8][kSets - 1][kTileKeys];   // pass 2: partial column sums, slot = tile & 7
+      uint4 ones[2 * kTileKeys];     // pass 2: the other side of the operand with -L_r: 128 keys x 16 channels, (1, 1, 1, 0, ...)
+    };
   };
   float edge_part[2][kTileKeys];     // pass 2: partial column sums of those tiles
   Barriers bar;
@@ -322,10 +330,9 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
       }
       const float mx = max32(v) * kScale;
       if (m == -INFINITY || mx > m + 64.0f) {
-        const float ref = sat_grid(mx);
-        if (m > -INFINITY) l = (l + acc_total(acc)) * ex2(m - ref);
+        if (m > -INFINITY) l = (l + acc_total(acc)) * ex2(m - mx);
         acc[0] = acc[1] = 0ull;
-        m = ref;
+        m = mx;
       }
       __syncwarp();
     }
@@ -352,7 +359,7 @@ __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empt
 #pragma unroll
     for (int i = 0; i < 32; ++i)
       if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
-    const float mx = sat_grid(max32(v) * kScale);
+    const float mx = max32(v) * kScale;
     if (m_run == -INFINITY || mx > m_run + 64.0f) {
       if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
       acc[0] = acc[1] = 0ull;
@@ -363,7 +370,9 @@ __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empt
   return make_float2(m_run, l_run + acc_total(acc));
 }
 
-// pass 2: nc columns (a multiple of 16), -L_r of the first at shared-space address nl
+// pass 2: nc columns (a multiple of 16).  ADDED: the products come with -L_r; otherwise nl is the shared-space address of
+// that of the first column
+template <bool ADDED>
 __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, int lane, uint32_t nl, int nc) {
   uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
@@ -372,14 +381,16 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
     tmem_ld32(addr + (uint32_t)cc0, v);               // stays inside the 128-column buffer
     tmem_wait_ld();
     if (cc0 + 32 == nc) hand_back(empty_bar, lane);
-    exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
+    if (ADDED) exp_accumulate<false, 32>(v, 0ull, 0.5f, acc);
+    else exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
   }
   if (nc & 16) {
     uint32_t v[32];
     tmem_ld32(addr + (uint32_t)(nc - 16), v);
     tmem_wait_ld();
     hand_back(empty_bar, lane);
-    exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)(nc - 16), acc);
+    if (ADDED) exp_accumulate<false, 16>(v, 0ull, 0.5f, acc);
+    else exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)(nc - 16), acc);
   }
   return acc_total(acc);
 }
@@ -474,9 +485,11 @@ __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, 
 // ------------------------------------------------------------------ the kernel
 // CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of
 // that code.  IDLE ones (pass 1) skip the items of warps whose 32 rows all lie behind the last one: one
-// item in four on two of the four schedulers for 448 rows.  65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us,
+// item in four on two of the four schedulers for 448 rows.  ADDED ones (pass 2) have -L_r added by the product, a ninth step of
+// 16 channels (ones x three bf16 that sum to it), instead of reading it from shared memory for every column: eight loads fewer
+// per chunk, and the argument of the polynomial is one saturating multiply-add (see kAddedItems).  65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us,
 // 30000 x 8 of 400 rows 82.2 -> 81.0; with the test in all instantiations the others were 0.2-0.5 % slower.
-template <int PASS, bool CAUSAL, int LAYERS, int HALVES, bool IDLE>
+template <int PASS, bool CAUSAL, int LAYERS, int HALVES, bool IDLE, bool ADDED>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ Geometry g,
                 const __grid_constant__ TcParams P, const __grid_constant__ TcLayers<LAYERS> M,
@@ -488,6 +501,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   uint8_t* q_smem = smem;
   uint8_t* k_smem = smem + q_bytes;
   Misc* misc = reinterpret_cast<Misc*>(k_smem + (size_t)P.n_stages * kStageBytes);
+  // pass 2: -L_r as an operand (rows_pad + 8 rows), in the log2 domain (-1e4 for padded rows), 128 zeros
+  uint4* l_smem = reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(misc) + kMiscBytes);
+  float* neg_lc = reinterpret_cast<float*>(l_smem + P.rows_pad + 8);
   Pipe pipe{misc, status};
 
   // the warp index as a value the compiler knows to be the same in all lanes: the MMA issuer's
@@ -505,6 +521,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     }
     mbar_init(smem_u32(&misc->bar.q_full), 1);
     mbar_init(smem_u32(&misc->bar.q_empty), kIssuers);
+    mbar_init(smem_u32(&misc->bar.l_full), 1);
     for (int i = 0; i < kBufs; ++i) {
       mbar_init(smem_u32(&misc->bar.acc_full[i]), 1);
       mbar_init(smem_u32(&misc->bar.acc_empty[i]), 4);       // the four warps of a set
@@ -522,6 +539,13 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   if (warp == 1) {
     tmem_alloc(smem_u32(&misc->tmem_base), kTmemCols);
     tmem_relinquish();
+  }
+  if (ADDED && threadIdx.x >= 128 && threadIdx.x < 128 + 2 * kTileKeys) {
+    const int i = threadIdx.x - 128;       // 8-row groups of 256 bytes: channels 0-7 of the rows, channels 8-15
+    misc->ones[i] = (i & 8) ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
+    if (i < 8) l_smem[P.rows_pad + i] = make_uint4(0u, 0u, 0u, 0u);
+    if (CAUSAL && i < kTileKeys) neg_lc[P.rows_pad + i] = 0.0f;
+    fence_proxy_async();
   }
   if (PASS == 2) pdl_launch_dependents();
   tc_fence_before();
@@ -649,6 +673,13 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
                     : instr_desc(128, (uint32_t)(P.rows_pad - (P.n_sub - 1) * P.sub_cols));
       const uint32_t empty0 = smem_u32(&misc->bar.empty[0]);
       const uint32_t accf0 = smem_u32(&misc->bar.acc_full[0]);
+      // pass 2: one more step of 16 channels adds -L_r (ones from the keys' side; the rows' side is 16 bytes a row,
+      // the second 8 channels of a group of rows lie on the next group's first and meet zeros)
+      const uint64_t ones_desc = (uint64_t)(((smem_u32(misc->ones) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(16u | (1u << 14)) << 32);
+      const uint64_t l_desc = (uint64_t)(((smem_u32(l_smem) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(8u | (1u << 14)) << 32);
+      // only the first two of its items of a (sequence, head) does an issuer multiply without it: L_r may not be known yet
+      uint32_t l_phase = 0, n_own = 0;
+      bool l_known = false;
       const bool elected = elect_one();
       bool ok = true;
       for (int t = t_begin; t < t_end && ok; ++t) {
@@ -669,6 +700,13 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
             ok = false;
             break;
           }
+          if (ADDED && n_own++ == 2) {
+            if (!warp_wait(pipe, &misc->bar.l_full, l_phase, 23)) {
+              ok = false;
+              break;
+            }
+            l_known = true;
+          }
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + buf * kBufCols;
           const uint32_t idesc = sub == P.n_sub - 1 ? idesc_last : idesc_full;
@@ -681,6 +719,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
               const uint64_t al = PASS == 1 ? ql : kl, bl = PASS == 1 ? kl : ql;
               umma(d_tmem, al | ((uint64_t)a_hi << 32), bl | ((uint64_t)b_hi << 32), idesc, ks > 0);
             }
+            if (ADDED && l_known)
+              umma(d_tmem, ones_desc, l_desc + (uint64_t)((uint32_t)sub * (uint32_t)P.sub_cols), idesc, true);
             umma_commit(accf0 + 8u * buf);
           }
         }
@@ -688,6 +728,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         if (elected) umma_commit(empty0 + 8u * (uint32_t)stage);
         if (++stage == P.n_stages) { stage = 0; phase ^= 1; }
         if (--left == 0 && t + 1 < t_end) {
+          l_known = false;
+          n_own = 0;
+          l_phase ^= 1;      // (without a third item there is no wait; with one the next L_r waits for that item)
           // the next tile belongs to another (sequence, head): Q may be replaced once the
           // multiplications issued so far have read it
           if (elected) umma_commit(smem_u32(&misc->bar.q_empty));
@@ -791,13 +834,24 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           const float lc = m + log2f(l);
           const int gq = row % g.group, tq = row / g.group;     // row = t * G + g
           const bool real = tq < g.window;
-          misc->neg_lc[row] = real ? -lc : -1.0e4f;
+          neg_lc[row] = real ? -lc : -1.0e4f;
+          if (ADDED) {
+            // the same in units of the products, as three bf16 that add up to it (padded rows: far below everything)
+            const float nl = real ? -lc * (1.0f / kScale) : -8.0e4f;
+            const float rest = real ? fmaf(nl, kScale, lc) * (-1.0f / kScale) : 0.0f;       // rounding of the division
+            const __nv_bfloat16 x0 = __float2bfloat16_rn(nl), x1 = __float2bfloat16_rn(nl - __bfloat162float(x0));
+            const __nv_bfloat16 x2 = __float2bfloat16_rn(nl - __bfloat162float(x0) - __bfloat162float(x1) + rest);
+            l_smem[row] = make_uint4((uint32_t)__bfloat16_as_ushort(x0) | (uint32_t)__bfloat16_as_ushort(x1) << 16,
+                                     (uint32_t)__bfloat16_as_ushort(x2), 0u, 0u);
+            fence_proxy_async();
+          }
           if (real && P.lse != nullptr && tb == first_tile)
             P.lse[((int64_t)cur.s * g.hq + cur.h * g.group + gq) * g.window + tq] = lc * kLn2;
         }
         if (ways > 1) epi_barrier();
       }
       epi_barrier();
+      if (ADDED && etid == 0) mbar_arrive(smem_u32(&misc->bar.l_full));
     };
 
     // A set works on every fourth item of the span, item = (tile - t_begin) * n_sub + sub, and
@@ -814,6 +868,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int t_slot = t_begin + (sub_begin > 0 ? 1 : 0);
     const int idle_from = (max(P.rows_pad - quad * 32, 0) + 127) / 128;   // row blocks from here on have no row of this warp
     uint32_t par = 0;
+    bool first_item = true;     // pass 2: of the set in the (sequence, head); these are multiplied without -L_r
     int prob_end = t_begin, first_tile = 0, n_cur = 0;
     float* out = nullptr;
     const uint32_t full_bar = smem_u32(&misc->bar.acc_full[set]);
@@ -841,6 +896,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           const SeqInfo& sq = bt.seq[cur.s];
           first_tile = g.hkv * sq.tile_off + cur.h * sq.n_tiles;
           if (PASS == 2) merge_lse(sq, first_tile, prob_end);
+          first_item = true;
           cur_problem = cur.problem(g.hkv);
           prob_end = min(t_end, first_tile + sq.n_tiles);
           n_cur = sq.n;
@@ -893,9 +949,14 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           const int nc = min(P.sub_cols, P.rows_pad - c0);        // multiple of 16
           // causal window: key j is seen by the rows t >= j - (n - w), i.e. by the columns from
           // G * (j - n + w) on; the columns before it contribute nothing
-          const uint32_t nl = smem_u32(misc->neg_lc + c0);         // -L_r of the item's columns
-          u_acc = edge ? drain_rows_masked(acc_addr, empty_bar, lane, nl, nc, g.group * (key0 + row_in_tile - n_cur + g.window) - c0)
-                       : drain_rows(acc_addr, empty_bar, lane, nl, nc);
+          if (edge)
+            u_acc = drain_rows_masked(acc_addr, empty_bar, lane, smem_u32(neg_lc + (!ADDED || first_item ? c0 : P.rows_pad)), nc,
+                                      g.group * (key0 + row_in_tile - n_cur + g.window) - c0);
+          else if (!ADDED || first_item)
+            u_acc = drain_rows<false>(acc_addr, empty_bar, lane, smem_u32(neg_lc + c0), nc);
+          else
+            u_acc = drain_rows<true>(acc_addr, empty_bar, lane, 0u, nc);
+          first_item = false;
         }
       }
       if (PASS == 2) {
@@ -962,6 +1023,12 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// Items of a CTA from which on pass 2 lets the products add -L_r (ADDED).  The first item of each set cannot have it, and the
+// operand has to be prepared: 20480 tokens x 8 heads of 256 rows (17 items) -0.8 %, 65536 x 4 of 448 -1.3 %, 131072 x 8 -2.0 %,
+// 32 x 2200 x 8 of 512 -2.0 %; level at 7 to 14 items, +0.9 % on 131072 x 2 of 128 rows (14 items) and 12 x 300 x 8 of 512.
+// Spans with cut tiles have few items.
+constexpr int kAddedItems = 16;
+
 struct TcPlan {
   TcParams P;
   size_t smem_bytes;
@@ -998,12 +1065,12 @@ TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count, int laye
   P.grid = units < sm_count ? units : sm_count;
   if (P.grid < 1) P.grid = 1;
   pl.ok = P.rows_pad <= kMaxRows && w_pad <= 256 && g.group <= 256;
-  const uint32_t q_bytes = (uint32_t)P.rows_pad * 256u;
-  int stages = ((int)kSmemLimit - 1024 - (int)kMiscBytes - (int)q_bytes) / (int)kStageBytes;
+  const uint32_t q_bytes = (uint32_t)P.rows_pad * 256u, l_bytes = (uint32_t)P.rows_pad * kLBytes + kLFixed;
+  int stages = ((int)kSmemLimit - 1024 - (int)kMiscBytes - (int)(q_bytes + l_bytes)) / (int)kStageBytes;
   if (stages > kMaxStages) stages = kMaxStages;
   if (stages < 2) pl.ok = false;
   P.n_stages = stages;
-  pl.smem_bytes = 1024 + q_bytes + (size_t)stages * kStageBytes + kMiscBytes;
+  pl.smem_bytes = 1024 + q_bytes + (size_t)stages * kStageBytes + kMiscBytes + l_bytes;
   return pl;
 }
 
@@ -1066,10 +1133,13 @@ cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry&
   }
   // the last row block has a warp without rows (causal calls gain nothing: 10007 tokens x 4 heads 40.0 -> 40.1 us)
   const bool idle = P.rows_pad % 128 != 0 && P.rows_pad % 128 <= 96;
-  auto pass1 = g.causal ? score_tc_kernel<1, true, LAYERS, HALVES, false>
-               : idle   ? score_tc_kernel<1, false, LAYERS, HALVES, true>
-                        : score_tc_kernel<1, false, LAYERS, HALVES, false>;
-  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false> : score_tc_kernel<2, false, LAYERS, HALVES, false>;
+  auto pass1 = g.causal ? score_tc_kernel<1, true, LAYERS, HALVES, false, false>
+               : idle   ? score_tc_kernel<1, false, LAYERS, HALVES, true, false>
+                        : score_tc_kernel<1, false, LAYERS, HALVES, false, false>;
+  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false, false> : score_tc_kernel<2, false, LAYERS, HALVES, false, false>;
+  if (HALVES == 1 && P.total_tiles * P.n_sub >= kAddedItems * P.grid)
+    pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false, HALVES == 1>
+                     : score_tc_kernel<2, false, LAYERS, HALVES, false, HALVES == 1>;
   cudaError_t e = allow_smem(pass1);
   if (e == cudaSuccess) e = allow_smem(pass2);
   if (e != cudaSuccess) return e;

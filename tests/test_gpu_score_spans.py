@@ -28,3 +28,14 @@ def test_scores_where_the_last_block_of_rows_is_not_full(w, hq, hkv, lens, page)
     """16 to 448 rows, one to four blocks of 128, the last of which has 0 to 3 warps without rows."""
     wl = gen.Workload("padded", 28, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1, page_size=page)
     check_against_oracle(wl, gen.make_layer(wl, layer=w, with_v=False), cc.CC_MODE_BF16, 2e-3)
+
+
+# Error budget: the polynomial's 7.8e-5 twice (value and row sum) and f32 products and references below 64, 2^-18.
+@pytest.mark.parametrize("w,hq,hkv", [(16, 8, 8), (12, 32, 8), (16, 56, 8), (50, 32, 8), (96, 32, 8), (64, 56, 8), (128, 32, 8)])
+@pytest.mark.parametrize("lens,page,causal", [((41000,), 0, False), ((5000, 130, 77, 300, 9000, 1, 700, 26000), 16, False),
+                                              ((40000, 300), 0, True)])
+def test_scores_whose_row_sums_the_product_subtracts(w, hq, hkv, lens, page, causal):
+    """Sixteen items per CTA and more, 16 to 512 rows in one to four blocks, problems of one tile up to hundreds."""
+    wl = gen.Workload("added", 30, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1, page_size=page,
+                      causal=causal)
+    check_against_oracle(wl, gen.make_layer(wl, layer=w, with_v=False), cc.CC_MODE_BF16, 2e-4)
