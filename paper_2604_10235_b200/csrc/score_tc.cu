@@ -447,6 +447,12 @@ struct TileCursor {
 // one at weight b * P.weight / grid.
 constexpr int kTileWeight = 4;
 
+// a / b in 32 bits where they fit, which is always but for batches of millions of tiles: the 64-bit division is a call of some
+// hundred instructions, run once per CTA from a cold instruction cache.
+__device__ __forceinline__ long long quotient(long long a, long long b) {
+  if (((a | b) >> 32) == 0) return (unsigned)a / (unsigned)b;
+  return a / b;
+}
 // The unit at weight w, counted over all (sequence, head)s.
 template <int HALVES>
 __device__ long long unit_at(const BatchTable& bt, int hkv, const TcParams& P, long long w) {
@@ -474,7 +480,7 @@ __device__ __forceinline__ int cta_of_unit(const BatchTable& bt, int hkv, const 
   for (int i = 0; i < s; ++i)
     if (bt.seq[i].n_tiles) w += (long long)(bt.seq[i].n_tiles * kTileWeight + P.change) * hkv;
   w += (long long)(bt.seq[s].n_tiles * kTileWeight + P.change) * h + P.change + (long long)(local + 1) * (kTileWeight / HALVES);
-  return (int)((w * P.grid - 1) / P.weight);      // w: the weight behind the unit
+  return (int)quotient(w * P.grid - 1, P.weight);      // w: the weight behind the unit
 }
 
 // A value that is the same in all lanes, in a form in which the compiler knows it: loop bounds and
@@ -514,28 +520,28 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&M.q[0])) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&M.k[0])) : "memory");
   }
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kMaxStages; ++i) {
-      mbar_init(smem_u32(&misc->bar.full[i]), 1);
-      mbar_init(smem_u32(&misc->bar.empty[i]), kIssuers);   // one arrival per MMA issuer
+  if (warp == 0) {               // one or two of each kind per lane: 64 in a row by one thread took 0.2 us
+    if (lane < kMaxStages) {
+      mbar_init(smem_u32(&misc->bar.full[lane]), 1);
+      mbar_init(smem_u32(&misc->bar.empty[lane]), kIssuers);   // one arrival per MMA issuer
     }
-    mbar_init(smem_u32(&misc->bar.q_full), 1);
-    mbar_init(smem_u32(&misc->bar.q_empty), kIssuers);
-    mbar_init(smem_u32(&misc->bar.l_full), 1);
-    for (int i = 0; i < kBufs; ++i) {
-      mbar_init(smem_u32(&misc->bar.acc_full[i]), 1);
-      mbar_init(smem_u32(&misc->bar.acc_empty[i]), 4);       // the four warps of a set
+    if (lane < kBufs) {
+      mbar_init(smem_u32(&misc->bar.acc_full[lane]), 1);
+      mbar_init(smem_u32(&misc->bar.acc_empty[lane]), 4);       // the four warps of a set
     }
-    for (int i = 0; i < 8; ++i)
-      for (int j = 0; j < 4; ++j)        // one arrival per set that hands its partial sums over
-        mbar_init(smem_u32(&misc->bar.u_full[i][j]), P.n_sub > 1 ? P.n_sub - 1 : 1);
-    for (int i = 0; i < 2; ++i)
-      for (int j = 0; j < 4; ++j) mbar_init(smem_u32(&misc->bar.edge_full[i][j]), 1);
-    misc->abort_flag = 0;
+    // one arrival per set that hands its partial sums over
+    mbar_init(smem_u32(&misc->bar.u_full[lane >> 2][lane & 3]), P.n_sub > 1 ? P.n_sub - 1 : 1);
+    if (lane < 8) mbar_init(smem_u32(&misc->bar.edge_full[lane >> 2][lane & 3]), 1);
+    if (lane == 0) {
+      mbar_init(smem_u32(&misc->bar.q_full), 1);
+      mbar_init(smem_u32(&misc->bar.q_empty), kIssuers);
+      mbar_init(smem_u32(&misc->bar.l_full), 1);
+      misc->abort_flag = 0;
+    }
     fence_barrier_init();
   }
   if (warp >= 2 && warp < 4 && lane == 0)      // the ends of the span, computed once (it is a slow piece of code)
-    misc->span[warp - 2] = unit_at<HALVES>(bt, g.hkv, P, (blockIdx.x + warp - 2) * P.weight / P.grid);
+    misc->span[warp - 2] = unit_at<HALVES>(bt, g.hkv, P, quotient((blockIdx.x + warp - 2) * P.weight, P.grid));
   if (warp == 1) {
     tmem_alloc(smem_u32(&misc->tmem_base), kTmemCols);
     tmem_relinquish();
@@ -565,10 +571,12 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   // pass 1, which only produces the row statistics: the TMA and MMA roles of pass 2 start at
   // once (their first K tiles and products overlap the tail of pass 1) and only the epilogue
   // warps, which read the statistics and write the scores, wait.
-  if (PASS == 1) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
+  auto pass1_wait = [] {
+    if (PASS == 1) {
+      pdl_wait();
+      pdl_launch_dependents();
+    }
+  };
 
   if (warp == 0) {
     // ================================================================ TMA producer
@@ -578,6 +586,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     {
       TileCursor cur;
       cur.locate(bt, g.hkv, t_begin);
+      pass1_wait();
       const bool elected = elect_one();
       int stage = 0, cur_problem = -1;
       uint32_t phase = 0, qe_phase = 0;
@@ -653,6 +662,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     {
       TileCursor cur;
       cur.locate(bt, g.hkv, t_begin);
+      pass1_wait();
       int left = cur.n_tiles - cur.local;          // tiles of the current (sequence, head) still to do
       int stage = 0;
       uint32_t phase = 0, qf_phase = 0, item = 0;
@@ -751,6 +761,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     TileCursor cur;
     cur.locate(bt, g.hkv, t_begin);
+    pass1_wait();
     int cur_problem = -1;
     bool dead = false;      // after a failed wait: keep the loop structure (and its barriers), skip the work
     float run_m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -786,69 +797,75 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       epi_barrier();
     };
 
-    // pass 2 (first_tile = the (sequence, head)'s first tile, tb = its first tile in this span):
-    auto merge_lse = [&](const SeqInfo& sq, int first_tile, int tb) {
-      // merge the spans' (max, sum) of the new (sequence, head) into -L_r: the spans are
-      // dealt round-robin to the threads that share a row, all loads of a thread are issued
-      // before the first use, and the threads of a row meet through shared memory
-      epi_barrier();
-      const int b0 = cta_of_unit<HALVES>(bt, g.hkv, P, cur.s, cur.h, 0);
-      const int b1 = cta_of_unit<HALVES>(bt, g.hkv, P, cur.s, cur.h, sq.n_tiles * HALVES - 1);
+    // pass 2: merge the spans' (max, sum) of a (sequence, head) into -L_r.  b0, b1: the first and the last CTA
+    // that have tiles of it; write_lse: this CTA has its first.  A thread takes two neighbouring rows, one 16-byte load
+    // a span; the threads that share a pair of rows take every ways-th span, issue up to kPartLoads loads before they use the
+    // first, and meet through shared memory.  Bound by that latency and by the fetch of its instructions, on the path between
+    // the passes: with a row per thread, rounds of eight loads, a chain of exponentials and the spans looked up on the
+    // way it took 2.5 us on 2048 tokens x 2 heads, 3.1 on 32768 x 8, 4.5 on 10007 x 4 of 448 rows (37 spans), now
+    // 2.1, 2.2 and 3.0; whole calls -2 to -4 %.  (Eight loads: 10007 x 4 +1 %; four: +1 % there, 2048 x 2 level.  A first round on
+    // whatever the buffer holds while pass 1 ends, to have the code at hand: 1.65 us, but late where pass 2 starts late, 10007 x 4 +7 %.)
+    auto merge_lse = [&](int b0, int b1, bool write_lse) {
+      constexpr int kPartLoads = 10;
       const int problem = cur.problem(g.hkv);
-      const int ways = max(1, min(4, kEpiThreads / P.rows_pad));    // threads per row
-      const int per_sweep = kEpiThreads / ways;                     // rows per sweep
-      float2* fold = &misc->xchg[0][0];          // no tile is in flight here, the union is free
-      for (int base = 0; base < P.rows_pad; base += per_sweep) {
-        const int row = base + etid % per_sweep, way = etid / per_sweep;
+      const int pairs = P.rows_pad / 2, ways = min(16, kEpiThreads / pairs);
+      const int way = etid / pairs, pair = etid - way * pairs;
+      float2* fold = &misc->xchg[0][0];          // [ways][rows_pad]; no tile is in flight here, the union is free
+      float m0 = -INFINITY, l0 = 0.f, m1 = -INFINITY, l1 = 0.f;
+      if (way < ways) {
+        const float4* part = reinterpret_cast<const float4*>(P.part + (int64_t)(b0 + way + problem) * P.rows_pad) + pair;
+        const int64_t pitch = (int64_t)ways * pairs;
+#pragma unroll 1
+        for (int b = b0 + way; b <= b1; b += kPartLoads * ways) {
+          float4 o[kPartLoads];
+#pragma unroll
+          for (int k = 0; k < kPartLoads; ++k) {
+            o[k] = b + k * ways <= b1 ? __ldcg(part) : make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
+            part += pitch;
+          }
+          float n0 = m0, n1 = m1;
+#pragma unroll
+          for (int k = 0; k < kPartLoads; ++k) { n0 = fmaxf(n0, o[k].x); n1 = fmaxf(n1, o[k].z); }
+          // (a row without a key in any of the spans so far: m - n is a difference of infinities)
+          l0 = l0 > 0.f ? l0 * ex2(m0 - n0) : 0.f;
+          l1 = l1 > 0.f ? l1 * ex2(m1 - n1) : 0.f;
+#pragma unroll
+          for (int k = 0; k < kPartLoads; ++k) {
+            l0 += o[k].y > 0.f ? o[k].y * ex2(o[k].x - n0) : 0.f;
+            l1 += o[k].w > 0.f ? o[k].w * ex2(o[k].z - n1) : 0.f;
+          }
+          m0 = n0;
+          m1 = n1;
+        }
+      }
+      epi_barrier();                             // all sets are done with the (sequence, head) before
+      if (way < ways) *reinterpret_cast<float4*>(&fold[way * P.rows_pad + 2 * pair]) = make_float4(m0, l0, m1, l1);
+      epi_barrier();
+      const int row = etid;
+      if (row < P.rows_pad) {
         float m = -INFINITY, l = 0.f;
-        if (row < P.rows_pad) {
-          for (int b = b0 + way; b <= b1; b += 8 * ways) {
-            float2 pr[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int bb = b + k * ways;
-              pr[k] = bb <= b1 ? P.part[(int64_t)(bb + problem) * P.rows_pad + row]
-                               : make_float2(-INFINITY, 0.f);
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              if (pr[k].y > 0.f) {
-                const float mn = fmaxf(m, pr[k].x);
-                l = l * ex2(m - mn) + pr[k].y * ex2(pr[k].x - mn);
-                m = mn;
-              }
-            }
-          }
-          if (ways > 1) fold[etid] = make_float2(m, l);
+        for (int k = 0; k < ways; ++k) m = fmaxf(m, fold[k * P.rows_pad + row].x);
+        for (int k = 0; k < ways; ++k) {
+          const float2 o = fold[k * P.rows_pad + row];
+          l += o.y > 0.f ? o.y * ex2(o.x - m) : 0.f;
         }
-        if (ways > 1) epi_barrier();
-        if (row < P.rows_pad && way == 0) {
-          for (int k = 1; k < ways; ++k) {
-            const float2 o = fold[k * per_sweep + etid];
-            if (o.y > 0.f) {
-              const float mn = fmaxf(m, o.x);
-              l = l * ex2(m - mn) + o.y * ex2(o.x - mn);
-              m = mn;
-            }
-          }
-          const float lc = m + log2f(l);
-          const int gq = row % g.group, tq = row / g.group;     // row = t * G + g
-          const bool real = tq < g.window;
-          neg_lc[row] = real ? -lc : -1.0e4f;
-          if (ADDED) {
-            // the same in units of the products, as three bf16 that add up to it (padded rows: far below everything)
-            const float nl = real ? -lc * (1.0f / kScale) : -8.0e4f;
-            const float rest = real ? fmaf(nl, kScale, lc) * (-1.0f / kScale) : 0.0f;       // rounding of the division
-            const __nv_bfloat16 x0 = __float2bfloat16_rn(nl), x1 = __float2bfloat16_rn(nl - __bfloat162float(x0));
-            const __nv_bfloat16 x2 = __float2bfloat16_rn(nl - __bfloat162float(x0) - __bfloat162float(x1) + rest);
-            l_smem[row] = make_uint4((uint32_t)__bfloat16_as_ushort(x0) | (uint32_t)__bfloat16_as_ushort(x1) << 16,
-                                     (uint32_t)__bfloat16_as_ushort(x2), 0u, 0u);
-            fence_proxy_async();
-          }
-          if (real && P.lse != nullptr && tb == first_tile)
-            P.lse[((int64_t)cur.s * g.hq + cur.h * g.group + gq) * g.window + tq] = lc * kLn2;
+        const float lc = m + log2f(l);
+        const bool real = row < P.rows;          // row = t * G + g
+        neg_lc[row] = real ? -lc : -1.0e4f;
+        if (ADDED) {
+          // the same in units of the products, as three bf16 that add up to it (padded rows: far below everything)
+          const float nl = real ? -lc * (1.0f / kScale) : -8.0e4f;
+          const float rest = real ? fmaf(nl, kScale, lc) * (-1.0f / kScale) : 0.0f;       // rounding of the division
+          const __nv_bfloat16 x0 = __float2bfloat16_rn(nl), x1 = __float2bfloat16_rn(nl - __bfloat162float(x0));
+          const __nv_bfloat16 x2 = __float2bfloat16_rn(nl - __bfloat162float(x0) - __bfloat162float(x1) + rest);
+          l_smem[row] = make_uint4((uint32_t)__bfloat16_as_ushort(x0) | (uint32_t)__bfloat16_as_ushort(x1) << 16,
+                                   (uint32_t)__bfloat16_as_ushort(x2), 0u, 0u);
+          fence_proxy_async();
         }
-        if (ways > 1) epi_barrier();
+        if (real && P.lse != nullptr && write_lse) {
+          const int gq = row % g.group, tq = row / g.group;
+          P.lse[((int64_t)cur.s * g.hq + cur.h * g.group + gq) * g.window + tq] = lc * kLn2;
+        }
       }
       epi_barrier();
       if (ADDED && etid == 0) mbar_arrive(smem_u32(&misc->bar.l_full));
@@ -874,7 +891,17 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const uint32_t full_bar = smem_u32(&misc->bar.acc_full[set]);
     const uint32_t empty_bar = smem_u32(&misc->bar.acc_empty[set]);
     const uint32_t acc_addr = lane_addr + (uint32_t)set * kBufCols;
-    if (PASS == 2) pdl_wait();
+    // CTA with the first unit of the span's first (sequence, head), CTA with the last one of its last
+    int b_first = 0, b_last = 0;
+    if (PASS == 2) {
+      if (t_begin < t_end) {
+        TileCursor last;
+        last.locate(bt, g.hkv, t_end - 1);
+        b_first = cta_of_unit<HALVES>(bt, g.hkv, P, cur.s, cur.h, 0);
+        b_last = cta_of_unit<HALVES>(bt, g.hkv, P, last.s, last.h, last.n_tiles * HALVES - 1);
+      }
+      pdl_wait();
+    }
     if (HALVES > 1 && PASS == 1 && sub_end < n_sub && etid < kTileKeys) {
       // pass 2 adds to the scores of the tile this span shares with the next one
       TileCursor last;
@@ -895,7 +922,11 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           }
           const SeqInfo& sq = bt.seq[cur.s];
           first_tile = g.hkv * sq.tile_off + cur.h * sq.n_tiles;
-          if (PASS == 2) merge_lse(sq, first_tile, prob_end);
+          if (PASS == 2) {
+            // (sequence, head)s that begin or end in this span: this CTA is their first or last
+            const bool begins = first_tile * HALVES >= u_begin, ends = (first_tile + sq.n_tiles) * HALVES <= u_end;
+            merge_lse(begins ? (int)blockIdx.x : b_first, ends ? (int)blockIdx.x : b_last, begins);
+          }
           first_item = true;
           cur_problem = cur.problem(g.hkv);
           prob_end = min(t_end, first_tile + sq.n_tiles);

@@ -39,3 +39,11 @@ def test_scores_whose_row_sums_the_product_subtracts(w, hq, hkv, lens, page, cau
     wl = gen.Workload("added", 30, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1, page_size=page,
                       causal=causal)
     check_against_oracle(wl, gen.make_layer(wl, layer=w, with_v=False), cc.CC_MODE_BF16, 2e-4)
+
+
+@pytest.mark.parametrize("w,hq,hkv", [(16, 1, 1), (24, 1, 1), (128, 1, 1), (64, 7, 1), (128, 4, 1)])
+@pytest.mark.parametrize("lens", [(19000,), (40000,), (7, 18500, 200, 21000)])
+def test_scores_of_one_head_spread_over_all_ctas(w, hq, hkv, lens):
+    """Up to 148 spans of a (sequence, head) to merge, 16 to 512 rows: sixteen threads for a pair of rows, or two."""
+    wl = gen.Workload("merge", 31, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1)
+    check_against_oracle(wl, gen.make_layer(wl, layer=w, with_v=False), cc.CC_MODE_BF16, 2e-4)
