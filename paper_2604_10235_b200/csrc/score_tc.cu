@@ -1086,11 +1086,11 @@ TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count, int laye
   P.halves = layers == 1 && P.n_sub % 2 == 0 && P.total_tiles > 2 * sm_count && half * 1.1 < 2 * whole ? 2 : 1;
   int starts = 0;
   for (int s = 0; s < bt.num_seqs; ++s) starts += bt.seq[s].n_tiles > 0;
-  // A start weighs as much as 2500 / rows quarters of a tile (2.4 tiles at 256 rows, 1.2 at 512; spans
-  // that straddle one were 2.3 us late in pass 2): llama3_8b shape 49.0 -> 47.3 us, 32 chunks 188 -> 178;
-  // half and one and a half times that weight gain less.  With few tiles per CTA whole tiles are too
-  // coarse to pay it back.
-  P.change = P.total_tiles >= 4 * sm_count ? (2500 + P.rows_pad / 2) / P.rows_pad : 0;
+  // A start weighs as much as 2000 / rows quarters of a tile (2 tiles at 256 rows, 1 at 512; spans
+  // that straddle one are that late in pass 2): llama3_8b shape 49.0 -> 47.3 us, 32 chunks 188 -> 178.  Against 2500 / rows
+  // 32 chunks -1.2 to -1.6 %, batches of 32 and 16 sequences -1.5 and -1.9 %, the others level; 1500 and 1000: +1 to 3 % on batches
+  // of 448 rows.  With few tiles per CTA whole tiles are too coarse to pay it back.
+  P.change = P.total_tiles >= 4 * sm_count ? (2000 + P.rows_pad / 2) / P.rows_pad : 0;
   P.weight = (long long)P.total_tiles * 4 + (long long)starts * g.hkv * P.change;
   const int units = P.total_tiles * P.halves;
   P.grid = units < sm_count ? units : sm_count;
