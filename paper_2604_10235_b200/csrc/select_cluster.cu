@@ -82,19 +82,24 @@ struct ClusterParams {
   int32_t* count[kMaxLayers];
 };
 
-template <int THREADS>
+// SINGLE: a CTA per (sequence, head), no cluster.  The loops over the peers go, which are unrolled for eight, and with them
+// what a small problem spent most of its time on, the fetch of instructions: 2048 tokens x 2 heads 17.7 -> 16.2 us,
+// 1500 x 8 21.0 -> 19.7, 32 chunks -0.9 %.
+template <int THREADS, bool SINGLE>
 struct Ctx {
-  static constexpr int kWarps = THREADS / 32;
+  static constexpr int kWarps = THREADS / 32, kPeers = SINGLE ? 1 : kMaxCluster;
   Shared* sm;
-  int C, rank;
+  int width, rank_;
+  __device__ int cluster() const { return SINGLE ? 1 : width; }
+  __device__ int rank() const { return SINGLE ? 0 : rank_; }
   unsigned n_xchg, n_red, n_hist;   // exchanges, block reductions, histograms so far (select the copy)
 
   __device__ void sync_all() {
-    if (C > 1) cg::this_cluster().sync(); else __syncthreads();
+    if (!SINGLE) cg::this_cluster().sync(); else __syncthreads();
   }
   template <class T>
   __device__ const T* peer(const T* p, int r) const {
-    if (C == 1) return p;
+    if (SINGLE) return p;
     return cg::this_cluster().map_shared_rank(const_cast<T*>(p), r);
   }
   // Sum of v over the block.  Two copies of the warp totals: a copy is written again only after
@@ -164,8 +169,8 @@ struct Ctx {
   // peer reaches after it has read exchange k - 2.
   __device__ const unsigned (*publish(const unsigned (&w)[kWords]))[kWords] {
     const unsigned bf = n_xchg++ & 1u;
-    if ((int)threadIdx.x < C) {
-      unsigned* dst = C == 1 ? sm->xchg[bf][0] : cg::this_cluster().map_shared_rank(&sm->xchg[bf][rank][0], (int)threadIdx.x);
+    if ((int)threadIdx.x < cluster()) {
+      unsigned* dst = SINGLE ? sm->xchg[bf][0] : cg::this_cluster().map_shared_rank(&sm->xchg[bf][rank()][0], (int)threadIdx.x);
 #pragma unroll
       for (int i = 0; i < kWords; ++i) dst[i] = w[i];
     }
@@ -186,9 +191,10 @@ struct Cut {
 // Finds T such that weight(key > T) < R <= weight(key >= T), 1 <= R <= total weight of the
 // eligible items, whose keys lie in [kmin, kmax].  get(li, key, len) tells whether the local
 // item li is eligible; a warp calls it for its items [lo, hi) 32 at a time.
-template <int THREADS, class Get>
-__device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned kmin, unsigned kmax, unsigned max_len,
+template <int THREADS, bool SINGLE, class Get>
+__device__ Cut find_cut(Ctx<THREADS, SINGLE>& c, int lo, int hi, unsigned R, unsigned kmin, unsigned kmax, unsigned max_len,
                         bool allow_whole, Get get) {
+  constexpr int kPeers = Ctx<THREADS, SINGLE>::kPeers;
   Shared& sm = *c.sm;
   const int lane = threadIdx.x & 31;
   const unsigned range = kmax - kmin;
@@ -200,11 +206,11 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       unsigned key, len;
       if (get(li, key, len)) mine += len;
     }
-    if (c.C == 1) return cut;
+    if (SINGLE) return cut;
     unsigned w[kWords] = {c.block_sum(mine), 0u, 0u, 0u, 0u, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
 #pragma unroll 1
-    for (int r = 0; r < c.rank; ++r) cut.tied_before += x[r][0];
+    for (int r = 0; r < c.rank(); ++r) cut.tied_before += x[r][0];
     return cut;
   }
   if (threadIdx.x < 256) sm.sub[threadIdx.x] = 0;     // (published by the barriers below)
@@ -241,14 +247,14 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     const int b0 = owner ? kBins - kOwn - (int)threadIdx.x * kOwn : 0;
     unsigned n[kOwn] = {0u, 0u, 0u, 0u}, nb[kOwn] = {0u, 0u, 0u, 0u};   // weight per bin: all CTAs, those before this one
     if (owner) {
-      uint4 v[kMaxCluster];
+      uint4 v[kPeers];
 #pragma unroll
-      for (int r = 0; r < kMaxCluster; ++r)
-        v[r] = r < c.C ? *reinterpret_cast<const uint4*>(c.peer(h + b0, r)) : make_uint4(0u, 0u, 0u, 0u);
+      for (int r = 0; r < kPeers; ++r)
+        v[r] = r < c.cluster() ? *reinterpret_cast<const uint4*>(c.peer(h + b0, r)) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int r = 0; r < kMaxCluster; ++r) {
+      for (int r = 0; r < kPeers; ++r) {
         n[0] += v[r].x; n[1] += v[r].y; n[2] += v[r].z; n[3] += v[r].w;
-        if (r < c.rank) { nb[0] += v[r].x; nb[1] += v[r].y; nb[2] += v[r].z; nb[3] += v[r].w; }
+        if (r < c.rank()) { nb[0] += v[r].x; nb[1] += v[r].y; nb[2] += v[r].z; nb[3] += v[r].w; }
       }
     }
     unsigned sum = 0;
@@ -296,11 +302,11 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
     }
     unsigned a0 = 0u, d0 = 0u, f0 = 0u;
     c.block_totals(a0, lo_k, hi_k, d0, f0);
-    if (c.C > 1) {
+    if (!SINGLE) {
       const unsigned w[kWords] = {lo_k, hi_k, 0u, 0u, 0u, 0u};
       const unsigned(*x)[kWords] = c.publish(w);
 #pragma unroll 1
-      for (int r = 0; r < c.C; ++r) {
+      for (int r = 0; r < c.cluster(); ++r) {
         lo_k = min(lo_k, x[r][0]);
         hi_k = max(hi_k, x[r][1]);
       }
@@ -326,17 +332,17 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       if ((((key - kmin) << sh) >> shift) == (prefix >> shift)) sm.own[atomicAdd(&sm.n_own, 1u)] = Cand{key, len};
     }
     c.sync_all();
-    unsigned first[kMaxCluster + 1];        // places of the CTAs' lists in the common one
+    unsigned first[kPeers + 1];        // places of the CTAs' lists in the common one
     first[0] = 0;
 #pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) first[r + 1] = r < c.C ? *c.peer(&sm.n_own, r) : 0u;
+    for (int r = 0; r < kPeers; ++r) first[r + 1] = r < c.cluster() ? *c.peer(&sm.n_own, r) : 0u;
+    unsigned before = 0;                    // (a sum, not first[rank]: that would put the array into local memory)
 #pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) first[r + 1] += first[r];
-    const unsigned total = first[kMaxCluster];
-    unsigned before = 0;
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r)
-      if (r == c.rank) before = first[r];
+    for (int r = 0; r < kPeers; ++r) {
+      if (r < c.rank()) before += first[r + 1];
+      first[r + 1] += first[r];
+    }
+    const unsigned total = first[kPeers];
     const int sub_bits = min(8, shift), sub_shift = shift - sub_bits;
     auto sub_bin = [&](unsigned key) { return (((key - kmin) << sh) >> sub_shift) & ((1u << sub_bits) - 1u); };
     const bool refine = total > 64;         // narrow a long list down by the next bits before ranking
@@ -345,7 +351,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       int r = 0;
       unsigned at = i;
 #pragma unroll
-      for (int k = 1; k < kMaxCluster; ++k)
+      for (int k = 1; k < kPeers; ++k)
         if (i >= first[k]) { r = k; at = i - first[k]; }
       const Cand o = c.peer(sm.own, r)[at];
       sm.all[i] = o;
@@ -398,7 +404,7 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
       if (o.key == cut.T) eq_before += o.len;
     }
   }
-  if (c.C > 1) {
+  if (!SINGLE) {
     c.block_sum2(gt_before, eq_before);
     cut.above_before += gt_before;
     cut.tied_before += eq_before;
@@ -408,19 +414,19 @@ __device__ Cut find_cut(Ctx<THREADS>& c, int lo, int hi, unsigned R, unsigned km
 
 // CHUNKED instantiations rank fixed chunks of bt.chunk tokens; the others are compiled for
 // token-level items only (bt.chunk == 1), which keeps their code short.
-template <bool FUSED, bool CHUNKED, int THREADS>
+template <bool FUSED, bool CHUNKED, int THREADS, bool SINGLE>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ ClusterParams P) {
   extern __shared__ __align__(16) uint8_t dyn[];
   Shared& sm = *reinterpret_cast<Shared*>(dyn);
-  Ctx<THREADS> c;
+  Ctx<THREADS, SINGLE> c;
   c.sm = &sm;
-  c.C = P.cluster;
-  c.rank = P.cluster > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  c.width = P.cluster;
+  c.rank_ = SINGLE ? 0 : (int)cg::this_cluster().block_rank();
   c.n_xchg = c.n_red = c.n_hist = 0;
 
   pdl_launch_dependents();
-  if (c.C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
+  if (!SINGLE) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
   // FUSED runs right after the second score pass, which starts only once the caller's inputs
   // are complete: the token-level path reads the prior before it waits for the scores
   const bool early_prior = FUSED && !CHUNKED;
@@ -429,8 +435,8 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   const int h = blockIdx.y, s = blockIdx.z;
   const SeqInfo& q = bt.seq[s];
   const int m = q.n_items, cs = CHUNKED ? bt.chunk : 1;
-  const int slice = (m + c.C * THREADS - 1) / (c.C * THREADS) * THREADS;     // items per CTA, a multiple of 32
-  const int cta_lo = min(m, c.rank * slice), cta_items = min(m, cta_lo + slice) - cta_lo;
+  const int slice = (m + c.cluster() * THREADS - 1) / (c.cluster() * THREADS) * THREADS;     // items per CTA, a multiple of 32
+  const int cta_lo = min(m, c.rank() * slice), cta_items = min(m, cta_lo + slice) - cta_lo;
   unsigned* keys = reinterpret_cast<unsigned*>(dyn + sizeof(Shared));
   uint8_t* flags = reinterpret_cast<uint8_t*>(keys + P.per * THREADS);
   const float* p = P.prior + q.tok_off;
@@ -640,14 +646,14 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 
   // ---- stage 0: totals of the cluster (the block reduction's barrier also publishes keys and flags)
   c.block_totals(forced_tokens, key_lo, key_hi, pri_lo, pri_hi);
-  if (c.C > 1) {
+  if (!SINGLE) {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // so have the others
     const unsigned w[kWords] = {forced_tokens, key_lo, key_hi, pri_lo, pri_hi, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
     forced_tokens = 0;
 #pragma unroll 1
-    for (int r = 0; r < c.C; ++r) {
-      if (r == c.rank) forced_before = forced_tokens;
+    for (int r = 0; r < c.cluster(); ++r) {
+      if (r == c.rank()) forced_before = forced_tokens;
       forced_tokens += x[r][0];
       key_lo = min(key_lo, x[r][1]);
       key_hi = max(key_hi, x[r][2]);
@@ -697,13 +703,13 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
       forced_before = cut.above_before + min(cut.tied_before, cap - cut.above);
     } else {
       forced_tokens = c.block_sum(kept);
-      if (c.C > 1) {
+      if (!SINGLE) {
         const unsigned w[kWords] = {forced_tokens, 0u, 0u, 0u, 0u, 0u};
         const unsigned(*x)[kWords] = c.publish(w);
         forced_tokens = forced_before = 0;
 #pragma unroll 1
-        for (int r = 0; r < c.C; ++r) {
-          if (r == c.rank) forced_before = forced_tokens;
+        for (int r = 0; r < c.cluster(); ++r) {
+          if (r == c.rank()) forced_before = forced_tokens;
           forced_tokens += x[r][0];
         }
       }
@@ -715,7 +721,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   // last read of a peer's shared memory is done: announce it now, wait for the peers at the
   // very end, and write the indices in between
   // (relaxed: nothing is published by it, so it need not wait for stores in flight)
-  if (c.C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  if (!SINGLE) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
   // ---- stage 3: ordered emission.  Items kept for sure (def) and the tied ones in sequence order,
   // until the budget is full
@@ -791,11 +797,11 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
       if ((dm | tm) >> lane & 1u) emit(lo + k * 32 + lane, tm >> lane & 1u, db, tb);
     }
   }
-  for (int i = (int)keep + c.rank * THREADS + threadIdx.x; i < q.budget; i += c.C * THREADS)
+  for (int i = (int)keep + c.rank() * THREADS + threadIdx.x; i < q.budget; i += c.cluster() * THREADS)
     out[i] = -1;
-  if (c.rank == 0 && threadIdx.x == 0) P.count[q.layer][q.src * P.hkv + h] = (int)keep;
+  if (c.rank() == 0 && threadIdx.x == 0) P.count[q.layer][q.src * P.hkv + h] = (int)keep;
   // no CTA may leave while a peer can still read its shared memory
-  if (c.C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (!SINGLE) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 size_t cluster_smem_bytes(int slots, int threads, bool staging) {
@@ -807,7 +813,10 @@ size_t cluster_smem_bytes(int slots, int threads, bool staging) {
 template <bool FUSED, bool CHUNKED>
 cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, int threads,
                          size_t smem) {
-  auto kern = threads == 512 ? select_cluster_kernel<FUSED, CHUNKED, 512> : select_cluster_kernel<FUSED, CHUNKED, 1024>;
+  auto kern = P.cluster == 1 ? (threads == 512 ? select_cluster_kernel<FUSED, CHUNKED, 512, true>
+                                               : select_cluster_kernel<FUSED, CHUNKED, 1024, true>)
+                             : (threads == 512 ? select_cluster_kernel<FUSED, CHUNKED, 512, false>
+                                               : select_cluster_kernel<FUSED, CHUNKED, 1024, false>);
   const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(P.cluster, g.hkv, bt.num_seqs), dim3(threads), smem, L.stream, P.cluster, bt, P);
@@ -827,9 +836,10 @@ int steps_per_warp(int max_items, int cluster, int threads) {
 // of this kernel alone: behind other kernels its code is cold, which more warps hide better), and
 // 0.48 (0.6) us per item of a thread of 512 (1024).  A chunk's tokens count a fifth of an item each.
 // A CTA of 1024 threads fills an SM, CTAs of 512 share it in pairs; a cluster sits inside one GPC, so
-// fewer CTAs run at a time in wide ones.
+// fewer CTAs run at a time in wide ones.  (One CTA: 6.1 until it had its own code; with 4.8 3500 tokens x 2, 4, 8 heads -4 %,
+// three sequences of up to 3000 -7 %; 5.2: 5000 tokens +1 %, 4.2: 7000 tokens +3 to 6 %.)
 double launch_cost(const BatchTable& bt, int hkv, const SelectRoom& room, bool staging, int lc, int threads) {
-  static const double base[4] = {6.1, 7.7, 7.8, 8.6};
+  static const double base[4] = {4.8, 7.7, 7.8, 8.6};
   const int c = 1 << lc;
   const double per_thread = (bt.max_items + (bt.chunk > 1 ? 0.2 * bt.chunk * bt.max_items : 0.0)) / (double)(c * threads);
   const size_t smem = cluster_smem_bytes(steps_per_warp(bt.max_items, c, threads) * threads, threads, staging);
@@ -845,8 +855,8 @@ double launch_cost(const BatchTable& bt, int hkv, const SelectRoom& room, bool s
 // on all parts, so the runtime is asked, once per context.  (148, 148, 132, 120 on the part at hand; 296, 296,
 // 284, 264 in pairs.)
 cudaError_t query_select_room(SelectRoom* room) {
-  auto one = select_cluster_kernel<true, false, 1024>;
-  auto two = select_cluster_kernel<true, false, 512>;
+  auto one = select_cluster_kernel<true, false, 1024, false>;
+  auto two = select_cluster_kernel<true, false, 512, false>;
   cudaError_t e = allow_smem(one);
   if (e == cudaSuccess) e = allow_smem(two);
   for (int lc = 0; lc <= 3 && e == cudaSuccess; ++lc) {
