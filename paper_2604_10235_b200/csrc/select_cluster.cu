@@ -82,24 +82,25 @@ struct ClusterParams {
   int32_t* count[kMaxLayers];
 };
 
-// SINGLE: a CTA per (sequence, head), no cluster.  The loops over the peers go, which are unrolled for eight, and with them
-// what a small problem spent most of its time on, the fetch of instructions: 2048 tokens x 2 heads 17.7 -> 16.2 us,
-// 1500 x 8 21.0 -> 19.7, 32 chunks -0.9 %.
-template <int THREADS, bool SINGLE>
+// CLUSTER: CTAs per (sequence, head).  The loops over them are unrolled, and in code for eight that only looks how many
+// there are, the fetch of instructions was most of a small problem's time: alone (no cluster, no exchange) 2048 tokens x 2
+// heads 17.7 -> 16.2 us, 1500 x 8 21.0 -> 19.7; in twos and fours 7000 and 10000 tokens x 2, 4, 8 heads -1 to -2 %.  Eight looks
+// all the same: with the number known the registers spill and 14000 tokens take 2 % more.
+template <int THREADS, int CLUSTER>
 struct Ctx {
-  static constexpr int kWarps = THREADS / 32, kPeers = SINGLE ? 1 : kMaxCluster;
+  static constexpr int kWarps = THREADS / 32, kPeers = CLUSTER;
   Shared* sm;
   int width, rank_;
-  __device__ int cluster() const { return SINGLE ? 1 : width; }
-  __device__ int rank() const { return SINGLE ? 0 : rank_; }
+  __device__ int cluster() const { return CLUSTER == kMaxCluster ? width : CLUSTER; }
+  __device__ int rank() const { return CLUSTER == 1 ? 0 : rank_; }
   unsigned n_xchg, n_red, n_hist;   // exchanges, block reductions, histograms so far (select the copy)
 
   __device__ void sync_all() {
-    if (!SINGLE) cg::this_cluster().sync(); else __syncthreads();
+    if (CLUSTER > 1) cg::this_cluster().sync(); else __syncthreads();
   }
   template <class T>
   __device__ const T* peer(const T* p, int r) const {
-    if (SINGLE) return p;
+    if (CLUSTER == 1) return p;
     return cg::this_cluster().map_shared_rank(const_cast<T*>(p), r);
   }
   // Sum of v over the block.  Two copies of the warp totals: a copy is written again only after
@@ -170,7 +171,7 @@ struct Ctx {
   __device__ const unsigned (*publish(const unsigned (&w)[kWords]))[kWords] {
     const unsigned bf = n_xchg++ & 1u;
     if ((int)threadIdx.x < cluster()) {
-      unsigned* dst = SINGLE ? sm->xchg[bf][0] : cg::this_cluster().map_shared_rank(&sm->xchg[bf][rank()][0], (int)threadIdx.x);
+      unsigned* dst = CLUSTER == 1 ? sm->xchg[bf][0] : cg::this_cluster().map_shared_rank(&sm->xchg[bf][rank()][0], (int)threadIdx.x);
 #pragma unroll
       for (int i = 0; i < kWords; ++i) dst[i] = w[i];
     }
@@ -191,10 +192,10 @@ struct Cut {
 // Finds T such that weight(key > T) < R <= weight(key >= T), 1 <= R <= total weight of the
 // eligible items, whose keys lie in [kmin, kmax].  get(li, key, len) tells whether the local
 // item li is eligible; a warp calls it for its items [lo, hi) 32 at a time.
-template <int THREADS, bool SINGLE, class Get>
-__device__ Cut find_cut(Ctx<THREADS, SINGLE>& c, int lo, int hi, unsigned R, unsigned kmin, unsigned kmax, unsigned max_len,
+template <int THREADS, int CLUSTER, class Get>
+__device__ Cut find_cut(Ctx<THREADS, CLUSTER>& c, int lo, int hi, unsigned R, unsigned kmin, unsigned kmax, unsigned max_len,
                         bool allow_whole, Get get) {
-  constexpr int kPeers = Ctx<THREADS, SINGLE>::kPeers;
+  constexpr int kPeers = CLUSTER;
   Shared& sm = *c.sm;
   const int lane = threadIdx.x & 31;
   const unsigned range = kmax - kmin;
@@ -206,7 +207,7 @@ __device__ Cut find_cut(Ctx<THREADS, SINGLE>& c, int lo, int hi, unsigned R, uns
       unsigned key, len;
       if (get(li, key, len)) mine += len;
     }
-    if (SINGLE) return cut;
+    if (CLUSTER == 1) return cut;
     unsigned w[kWords] = {c.block_sum(mine), 0u, 0u, 0u, 0u, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
 #pragma unroll 1
@@ -302,7 +303,7 @@ __device__ Cut find_cut(Ctx<THREADS, SINGLE>& c, int lo, int hi, unsigned R, uns
     }
     unsigned a0 = 0u, d0 = 0u, f0 = 0u;
     c.block_totals(a0, lo_k, hi_k, d0, f0);
-    if (!SINGLE) {
+    if (CLUSTER > 1) {
       const unsigned w[kWords] = {lo_k, hi_k, 0u, 0u, 0u, 0u};
       const unsigned(*x)[kWords] = c.publish(w);
 #pragma unroll 1
@@ -404,7 +405,7 @@ __device__ Cut find_cut(Ctx<THREADS, SINGLE>& c, int lo, int hi, unsigned R, uns
       if (o.key == cut.T) eq_before += o.len;
     }
   }
-  if (!SINGLE) {
+  if (CLUSTER > 1) {
     c.block_sum2(gt_before, eq_before);
     cut.above_before += gt_before;
     cut.tied_before += eq_before;
@@ -414,19 +415,19 @@ __device__ Cut find_cut(Ctx<THREADS, SINGLE>& c, int lo, int hi, unsigned R, uns
 
 // CHUNKED instantiations rank fixed chunks of bt.chunk tokens; the others are compiled for
 // token-level items only (bt.chunk == 1), which keeps their code short.
-template <bool FUSED, bool CHUNKED, int THREADS, bool SINGLE>
+template <bool FUSED, bool CHUNKED, int THREADS, int CLUSTER>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ ClusterParams P) {
   extern __shared__ __align__(16) uint8_t dyn[];
   Shared& sm = *reinterpret_cast<Shared*>(dyn);
-  Ctx<THREADS, SINGLE> c;
+  Ctx<THREADS, CLUSTER> c;
   c.sm = &sm;
   c.width = P.cluster;
-  c.rank_ = SINGLE ? 0 : (int)cg::this_cluster().block_rank();
+  c.rank_ = CLUSTER == 1 ? 0 : (int)cg::this_cluster().block_rank();
   c.n_xchg = c.n_red = c.n_hist = 0;
 
   pdl_launch_dependents();
-  if (!SINGLE) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
+  if (CLUSTER > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
   // FUSED runs right after the second score pass, which starts only once the caller's inputs
   // are complete: the token-level path reads the prior before it waits for the scores
   const bool early_prior = FUSED && !CHUNKED;
@@ -646,7 +647,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 
   // ---- stage 0: totals of the cluster (the block reduction's barrier also publishes keys and flags)
   c.block_totals(forced_tokens, key_lo, key_hi, pri_lo, pri_hi);
-  if (!SINGLE) {
+  if (CLUSTER > 1) {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // so have the others
     const unsigned w[kWords] = {forced_tokens, key_lo, key_hi, pri_lo, pri_hi, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
@@ -703,7 +704,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
       forced_before = cut.above_before + min(cut.tied_before, cap - cut.above);
     } else {
       forced_tokens = c.block_sum(kept);
-      if (!SINGLE) {
+      if (CLUSTER > 1) {
         const unsigned w[kWords] = {forced_tokens, 0u, 0u, 0u, 0u, 0u};
         const unsigned(*x)[kWords] = c.publish(w);
         forced_tokens = forced_before = 0;
@@ -721,7 +722,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   // last read of a peer's shared memory is done: announce it now, wait for the peers at the
   // very end, and write the indices in between
   // (relaxed: nothing is published by it, so it need not wait for stores in flight)
-  if (!SINGLE) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  if (CLUSTER > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
   // ---- stage 3: ordered emission.  Items kept for sure (def) and the tied ones in sequence order,
   // until the budget is full
@@ -801,7 +802,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     out[i] = -1;
   if (c.rank() == 0 && threadIdx.x == 0) P.count[q.layer][q.src * P.hkv + h] = (int)keep;
   // no CTA may leave while a peer can still read its shared memory
-  if (!SINGLE) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (CLUSTER > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 size_t cluster_smem_bytes(int slots, int threads, bool staging) {
@@ -810,16 +811,23 @@ size_t cluster_smem_bytes(int slots, int threads, bool staging) {
   return (b + 15) / 16 * 16;
 }
 
-template <bool FUSED, bool CHUNKED>
-cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, int threads,
-                         size_t smem) {
-  auto kern = P.cluster == 1 ? (threads == 512 ? select_cluster_kernel<FUSED, CHUNKED, 512, true>
-                                               : select_cluster_kernel<FUSED, CHUNKED, 1024, true>)
-                             : (threads == 512 ? select_cluster_kernel<FUSED, CHUNKED, 512, false>
-                                               : select_cluster_kernel<FUSED, CHUNKED, 1024, false>);
+template <bool FUSED, bool CHUNKED, int THREADS, int CLUSTER>
+cudaError_t launch_one(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, size_t smem) {
+  auto kern = select_cluster_kernel<FUSED, CHUNKED, THREADS, CLUSTER>;
   const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(P.cluster, g.hkv, bt.num_seqs), dim3(threads), smem, L.stream, P.cluster, bt, P);
+  return launch_pdl(kern, dim3(CLUSTER, g.hkv, bt.num_seqs), dim3(THREADS), smem, L.stream, CLUSTER, bt, P);
+}
+template <bool FUSED, bool CHUNKED>
+cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, SelectShape sh,
+                         size_t smem) {
+  const bool wide = sh.threads == 1024;
+  switch (sh.cluster) {
+    case 1: return wide ? launch_one<FUSED, CHUNKED, 1024, 1>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 1>(L, bt, g, P, smem);
+    case 2: return wide ? launch_one<FUSED, CHUNKED, 1024, 2>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 2>(L, bt, g, P, smem);
+    case 4: return wide ? launch_one<FUSED, CHUNKED, 1024, 4>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 4>(L, bt, g, P, smem);
+    default: return wide ? launch_one<FUSED, CHUNKED, 1024, 8>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 8>(L, bt, g, P, smem);
+  }
 }
 
 // Two CTAs of 512 threads share an SM when their shared memory (and 1 KB that each is charged besides)
@@ -855,8 +863,8 @@ double launch_cost(const BatchTable& bt, int hkv, const SelectRoom& room, bool s
 // on all parts, so the runtime is asked, once per context.  (148, 148, 132, 120 on the part at hand; 296, 296,
 // 284, 264 in pairs.)
 cudaError_t query_select_room(SelectRoom* room) {
-  auto one = select_cluster_kernel<true, false, 1024, false>;
-  auto two = select_cluster_kernel<true, false, 512, false>;
+  auto one = select_cluster_kernel<true, false, 1024, 8>;
+  auto two = select_cluster_kernel<true, false, 512, 8>;
   cudaError_t e = allow_smem(one);
   if (e == cudaSuccess) e = allow_smem(two);
   for (int lc = 0; lc <= 3 && e == cudaSuccess; ++lc) {
@@ -918,10 +926,10 @@ cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const G
   }
   const size_t smem = cluster_smem_bytes(P.per * sh.threads, sh.threads, fused_input && bt.chunk == 1);
   if (fused_input)
-    return bt.chunk > 1 ? launch_shape<true, true>(L, bt, g, P, sh.threads, smem)
-                        : launch_shape<true, false>(L, bt, g, P, sh.threads, smem);
-  return bt.chunk > 1 ? launch_shape<false, true>(L, bt, g, P, sh.threads, smem)
-                      : launch_shape<false, false>(L, bt, g, P, sh.threads, smem);
+    return bt.chunk > 1 ? launch_shape<true, true>(L, bt, g, P, sh, smem)
+                        : launch_shape<true, false>(L, bt, g, P, sh, smem);
+  return bt.chunk > 1 ? launch_shape<false, true>(L, bt, g, P, sh, smem)
+                      : launch_shape<false, false>(L, bt, g, P, sh, smem);
 }
 
 }  // namespace cc
