@@ -345,7 +345,9 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
 }
 
 // pass 1, keys from valid_r on (a bound of the thread's own) do not count
-// (returns the row's new reference and sum)
+// (returns the row's new reference and sum).  Chunks that no row of the warp attends to are skipped, and in those that all do
+// nothing is masked: with a causal window most are one or the other, and the CTA with the last tiles of a sequence is what a
+// short call waits for (10007 tokens x 4 heads: 7 us of work there, 4.5 to 5.5 elsewhere; score stage 24.1 -> 22.8 us).
 __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empty_bar, int lane, int valid_r, float m_run, float l_run) {
   uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
@@ -355,10 +357,13 @@ __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empt
     tmem_ld32(addr + (uint32_t)cc0, v);
     tmem_wait_ld();
     if (cc0 + 32 == kTileKeys) hand_back(empty_bar, lane);
+    const bool whole = __all_sync(0xffffffffu, cc0 + 32 <= valid_r);
     if (cc0 >= valid_r) continue;
+    if (!whole) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
+      for (int i = 0; i < 32; ++i)
+        if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
+    }
     const float mx = max32(v) * kScale;
     if (m_run == -INFINITY || mx > m_run + 64.0f) {
       if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
@@ -395,9 +400,10 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
   return acc_total(acc);
 }
 
-// pass 2, columns before first_col (a bound of the thread's own) do not count
-// (returns the sum)
-__device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty_bar, int lane, uint32_t nl, int nc, int first_col) {
+// pass 2, columns before first_col (a bound of the thread's own) do not count, and nothing does for a thread without a key
+// (returns the sum).  Skips and masks as above.
+__device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty_bar, int lane, uint32_t nl, int nc, int first_col,
+                                                   bool key) {
   uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
   for (int cc0 = 0; cc0 < nc; cc0 += 32) {
@@ -406,9 +412,12 @@ __device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty
     tmem_ld32(addr + (uint32_t)cc0, v);
     tmem_wait_ld();
     if (cc0 + 32 >= nc) hand_back(empty_bar, lane);
+    if (!__any_sync(0xffffffffu, key && cc0 + 32 > first_col)) continue;
+    if (!__all_sync(0xffffffffu, !key || cc0 >= first_col)) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (cc0 + i < first_col) v[i] = 0xc61c4000u;     // -1e4: exponential ~ 0
+      for (int i = 0; i < 32; ++i)
+        if (cc0 + i < first_col) v[i] = 0xc61c4000u;     // -1e4: exponential ~ 0
+    }
     if (cc0 + 32 <= nc) exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
     else                exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)cc0, acc);
   }
@@ -982,7 +991,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           // G * (j - n + w) on; the columns before it contribute nothing
           if (edge)
             u_acc = drain_rows_masked(acc_addr, empty_bar, lane, smem_u32(neg_lc + (!ADDED || first_item ? c0 : P.rows_pad)), nc,
-                                      g.group * (key0 + row_in_tile - n_cur + g.window) - c0);
+                                      g.group * (key0 + row_in_tile - n_cur + g.window) - c0, row_in_tile < valid);
           else if (!ADDED || first_item)
             u_acc = drain_rows<false>(acc_addr, empty_bar, lane, smem_u32(neg_lc + c0), nc);
           else
