@@ -320,8 +320,8 @@ int check_compact(cc_ctx* ctx, const cc_layer_desc* d, const BatchTable& bt, con
   return CC_OK;
 }
 
-int run_compact(cc_ctx* ctx, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp, void* stream) {
-  cudaError_t e = launch_compact(make_launch(ctx, stream), bt, g, lp);
+int run_compact(cc_ctx* ctx, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp, bool alone, void* stream) {
+  cudaError_t e = launch_compact(make_launch(ctx, stream), bt, g, lp, alone);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "compact launch");
   return CC_OK;
 }
@@ -505,7 +505,7 @@ int cc_compact_kv(cc_ctx* ctx, const cc_layer_desc* desc, const void* k, const v
   lp.idx[0] = const_cast<int32_t*>(idx);
   lp.free_pages[0] = free_pages;
   lp.out_page_table[0] = out_page_table;
-  return run_compact(ctx, p.bt, p.g, lp, stream);
+  return run_compact(ctx, p.bt, p.g, lp, true, stream);
 }
 
 namespace {
@@ -626,7 +626,7 @@ int compress(cc_ctx* ctx, const cc_layer_desc* desc, const Plan& p, const BatchT
     if ((rc = check_compact(ctx, desc, p.bt, lp.k[l], lp.v[l], lp.k_out[l], lp.v_out[l], lp.free_pages[l],
                             lp.out_page_table[l])) != CC_OK)
       return rc;
-  return run_compact(ctx, bt, p.g, lp, stream);
+  return run_compact(ctx, bt, p.g, lp, false, stream);
 }
 
 }  // namespace

@@ -192,7 +192,8 @@ cudaError_t launch_select_static(const Launch& L, const BatchTable& bt, const Ge
                                  float force_threshold, const float* fused, const float* prior,
                                  int32_t* idx, int32_t* count, int device);
 
-cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp);
+// alone: not behind the other stages of a call
+cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp, bool alone);
 
 // chunk selection by query-conditioned perplexity (Section 4.1)
 cudaError_t launch_ppl_scores(const Launch& L, const void* logits, bool is_f32, int num_chunks,

@@ -150,7 +150,7 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
 
 }  // namespace
 
-cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp) {
+cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry& g, const LayerPtrs& lp, bool alone) {
   CompactPtrs P = {};
   for (int l = 0; l < lp.n; ++l) {
     P.k[l] = (const uint16_t*)lp.k[l];
@@ -179,7 +179,11 @@ cudaError_t launch_compact(const Launch& L, const BatchTable& bt, const Geometry
   for (int s = 0; s < bt.num_seqs; ++s)
     blocks += max((int64_t)1, (((int64_t)bt.seq[s].keep << hc_shift) + kRowsPerBlock - 1) / kRowsPerBlock);
   dim3 grid((unsigned)blocks);
-  auto kern = hpg >= 4 ? compact_kernel<4> : (hpg >= 2 ? compact_kernel<2> : compact_kernel<1>);
+  // Rows in flight per thread against threads per SM (80 registers for four rows, 48 for two: 768 and 1280 threads).  Replayed alone
+  // four rows win: ragged batch 43.3 against 44.0 us, 32 chunks 41.5 against 43.8.  Behind the score stage, with the clock
+  // that stage leaves, two do: all layers 423 -> 416 us, ragged batch 477 -> 472, 32 chunks 244 -> 241.  (One row 420, 32-byte
+  // loads one row at a time 417; blocks of 128 threads level, of 512 slower.)
+  auto kern = hpg >= 4 && alone ? compact_kernel<4> : (hpg >= 2 ? compact_kernel<2> : compact_kernel<1>);
   return launch_pdl(kern, grid, dim3(kThreads), 0, L.stream, 1, bt, g, P, L.status, hpg, hc_shift);
 }
 
