@@ -86,7 +86,7 @@ constexpr int kSmemPerCta = 232448;      // 227 KB
 template <class... KArgs>
 cudaError_t allow_smem(void (*kernel)(KArgs...)) {
   struct Seen { const void* kernel; int device; };
-  static thread_local Seen seen[64];
+  static thread_local Seen seen[96];
   static thread_local int n_seen = 0;
   int device = -1;
   cudaError_t e = cudaGetDevice(&device);
@@ -94,7 +94,7 @@ cudaError_t allow_smem(void (*kernel)(KArgs...)) {
   for (int i = 0; i < n_seen; ++i)
     if (seen[i].kernel == (const void*)kernel && seen[i].device == device) return cudaSuccess;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
-  if (e == cudaSuccess && n_seen < 64) seen[n_seen++] = Seen{(const void*)kernel, device};
+  if (e == cudaSuccess && n_seen < 96) seen[n_seen++] = Seen{(const void*)kernel, device};
   return e;
 }
 

@@ -49,7 +49,7 @@ constexpr int kMaxCluster = 8;
 constexpr int kMaxWarps = 32;
 constexpr int kStep = 4;                  // items a thread pools per part of the slice
 constexpr int kMaxHalf = 32;              // half of the widest pooling window, rounded up
-constexpr int kWords = 6;                 // words of an exchange
+constexpr int kWords = 3;                 // words of an exchange
 
 struct Cand {
   unsigned key, len;
@@ -132,23 +132,19 @@ struct Ctx {
     a = __reduce_add_sync(0xffffffffu, lane < warp ? w[0][lane] : 0u);
     b = __reduce_add_sync(0xffffffffu, lane < warp ? w[1][lane] : 0u);
   }
-  // Sum of a, minimum of b, maximum of e, minimum of d, maximum of f over the block.
-  __device__ void block_totals(unsigned& a, unsigned& b, unsigned& e, unsigned& d, unsigned& f) {
+  // Sum of a, minimum of b, maximum of e over the block.
+  __device__ void block_totals(unsigned& a, unsigned& b, unsigned& e) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned(*w)[kMaxWarps] = sm->warp_x[n_red++ & 1u];
     a = __reduce_add_sync(0xffffffffu, a);
     b = __reduce_min_sync(0xffffffffu, b);
     e = __reduce_max_sync(0xffffffffu, e);
-    d = __reduce_min_sync(0xffffffffu, d);
-    f = __reduce_max_sync(0xffffffffu, f);
-    if (lane == 0) { w[0][warp] = a; w[1][warp] = b; w[2][warp] = e; w[3][warp] = d; w[4][warp] = f; }
+    if (lane == 0) { w[0][warp] = a; w[1][warp] = b; w[2][warp] = e; }
     __syncthreads();
     const int i = lane < kWarps ? lane : 0;
     a = __reduce_add_sync(0xffffffffu, lane < kWarps ? w[0][i] : 0u);
     b = __reduce_min_sync(0xffffffffu, w[1][i]);
     e = __reduce_max_sync(0xffffffffu, w[2][i]);
-    d = __reduce_min_sync(0xffffffffu, w[3][i]);
-    f = __reduce_max_sync(0xffffffffu, w[4][i]);
   }
   // Exclusive prefix sum over the threads of the block.
   __device__ unsigned block_scan(unsigned v) {
@@ -208,7 +204,7 @@ __device__ Cut find_cut(Ctx<THREADS, CLUSTER>& c, int lo, int hi, unsigned R, un
       if (get(li, key, len)) mine += len;
     }
     if (CLUSTER == 1) return cut;
-    unsigned w[kWords] = {c.block_sum(mine), 0u, 0u, 0u, 0u, 0u};
+    unsigned w[kWords] = {c.block_sum(mine), 0u, 0u};
     const unsigned(*x)[kWords] = c.publish(w);
 #pragma unroll 1
     for (int r = 0; r < c.rank(); ++r) cut.tied_before += x[r][0];
@@ -301,10 +297,10 @@ __device__ Cut find_cut(Ctx<THREADS, CLUSTER>& c, int lo, int hi, unsigned R, un
       lo_k = min(lo_k, key);
       hi_k = max(hi_k, key);
     }
-    unsigned a0 = 0u, d0 = 0u, f0 = 0u;
-    c.block_totals(a0, lo_k, hi_k, d0, f0);
+    unsigned a0 = 0u;
+    c.block_totals(a0, lo_k, hi_k);
     if (CLUSTER > 1) {
-      const unsigned w[kWords] = {lo_k, hi_k, 0u, 0u, 0u, 0u};
+      const unsigned w[kWords] = {lo_k, hi_k, 0u};
       const unsigned(*x)[kWords] = c.publish(w);
 #pragma unroll 1
       for (int r = 0; r < c.cluster(); ++r) {
@@ -414,8 +410,10 @@ __device__ Cut find_cut(Ctx<THREADS, CLUSTER>& c, int lo, int hi, unsigned R, un
 }
 
 // CHUNKED instantiations rank fixed chunks of bt.chunk tokens; the others are compiled for
-// token-level items only (bt.chunk == 1), which keeps their code short.
-template <bool FUSED, bool CHUNKED, int THREADS, int CLUSTER>
+// token-level items only (bt.chunk == 1), which keeps their code short.  CAPPED ones (any sequence of the launch has a
+// cap on its protected tokens, and all CHUNKED ones) hold the search for the cap; without it whole calls on 2000 to 70000
+// tokens take 1 to 3 % less.
+template <bool FUSED, bool CHUNKED, bool CAPPED, int THREADS, int CLUSTER>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ ClusterParams P) {
   extern __shared__ __align__(16) uint8_t dyn[];
@@ -428,10 +426,9 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 
   pdl_launch_dependents();
   if (CLUSTER > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
-  // FUSED runs right after the second score pass, which starts only once the caller's inputs
-  // are complete: the token-level path reads the prior before it waits for the scores
-  const bool early_prior = FUSED && !CHUNKED;
-  if (!early_prior) pdl_wait();
+  // FUSED runs right after the second score pass, which starts only once the caller's inputs are complete and all that was
+  // enqueued before the call has ended: what the priors decide, it does before it waits for the scores
+  if (!FUSED) pdl_wait();
 
   const int h = blockIdx.y, s = blockIdx.z;
   const SeqInfo& q = bt.seq[s];
@@ -454,228 +451,230 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     const int i = cta_lo + li;
     return (unsigned)(min(q.n, (i + 1) * cs) - i * cs);
   };
-  auto item_prior = [&](int li) -> float {
-    const int i = cta_lo + li;
-    if (cs == 1) return p[i];
-    float pr = p[(int64_t)i * cs];
-    const int end = min(q.n, (i + 1) * cs);
-#pragma unroll 1
-    for (int j = i * cs + 1; j < end; ++j) pr = fmaxf(pr, p[j]);
-    return pr;
-  };
-
 #pragma unroll 1
   for (int i = threadIdx.x; i < kBins; i += THREADS) sm.hist[0][i] = 0;
-  // Totals collected while loading: protected weight, key range of the unprotected items (of all
-  // items when a cap may still strip some of their protection), range of the protected items'
-  // priors when there is a cap
-  const bool capped = q.span_cap >= 0;
+
+  // ---- priors: parked in the key slots, with the protected flags, the protected weight and, when there is a cap, the range
+  // of the protected items' priors (loads are issued four or eight at a time)
+  const bool capped = CAPPED && q.span_cap >= 0;
   unsigned forced_tokens = 0, forced_before = 0;              // before: in the CTAs before this one
-  unsigned key_lo = 0xffffffffu, key_hi = 0u, pri_lo = 0xffffffffu, pri_hi = 0u;
-  auto tally = [&](unsigned key, float pr, unsigned len) {
+  unsigned pri_lo = 0xffffffffu, pri_hi = 0u;
+  const bool flags_later = FUSED && !CHUNKED && !capped;      // with the scores, four to a word
+  auto park = [&](int li, float pr) {
     const bool forced = pr >= theta;
-    if (forced) {
-      forced_tokens += len;
-      if (capped) {
-        const unsigned pk = mono_key(pr);
-        pri_lo = min(pri_lo, pk);
-        pri_hi = max(pri_hi, pk);
-      }
+    keys[li] = __float_as_uint(pr);
+    if (flags_later) return;
+    flags[li] = forced ? 1 : 0;
+    if (!forced) return;
+    forced_tokens += item_len(li);
+    if (capped) {
+      const unsigned pk = mono_key(pr);
+      pri_lo = min(pri_lo, pk);
+      pri_hi = max(pri_hi, pk);
     }
-    if (!forced || capped) {
-      key_lo = min(key_lo, key);
-      key_hi = max(key_hi, key);
-    }
-    return forced;
   };
-  // ---- load: keys and protected flags of the CTA's slice (coalesced over the block)
-  if (FUSED) {
-    const float* u = P.scores[q.layer] + (int64_t)h * bt.n_tot + q.tok_off;
-    const int half = (cs == 1 && P.pool_kind != CC_POOL_NONE) ? P.pool_size / 2 : 0;
-    auto fuse = [&](float val, float pr) {
-      return mono_key(__fadd_rn(__fmul_rn(P.alpha, val), __fmul_rn(P.beta, pr)));
-    };
-    // Keys and flags of four items in place of their parked priors.  Bound, like the pooling above it, by issue slots (26
-    // items a thread: 1.2 us a part of four): bounds as one unsigned compare, two taps per step, and the cap's
-    // prior range on its own took the load of a 52437-token sequence by two CTAs from 10.9 to 8.4 us, the call on 2048
-    // tokens x 2 heads 18.7 -> 18.2, 10007 x 4 38.9 -> 38.4, 32768 x 8 -0.9 %.  (Walking the slice four items to a lane in the search
-    // as well: 65536-token batches -0.5 %, small calls +1 to 2 %.)
-    auto store4 = [&](int l4, const float (&v)[4], float4 pr) {
-      const uint4 k4 = make_uint4(fuse(v[0], pr.x), fuse(v[1], pr.y), fuse(v[2], pr.z), fuse(v[3], pr.w));
-      const int left = cta_items - l4;
-      const unsigned key[4] = {k4.x, k4.y, k4.z, k4.w};
-      const float pri[4] = {pr.x, pr.y, pr.z, pr.w};
-      unsigned f = 0;
+  auto parked = [&](int li) -> float { return __uint_as_float(keys[li]); };
+  if (cs == 1) {
+#pragma unroll 1
+    for (int t0 = threadIdx.x; t0 < cta_items; t0 += 4 * THREADS) {
+      float b[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool forced = j < left && pri[j] >= theta;
-        if (forced) f |= 1u << (8 * j);
-        const bool counts = j < left && (capped || !forced);
-        key_lo = min(key_lo, counts ? key[j] : 0xffffffffu);
-        key_hi = max(key_hi, counts ? key[j] : 0u);
-      }
-      forced_tokens += __popc(f);
-      if (capped && f) {
-#pragma unroll 1
-        for (int j = 0; j < 4; ++j) {
-          if (!(f >> (8 * j) & 1u)) continue;
-          const unsigned pk = mono_key(reinterpret_cast<const float*>(keys)[l4 + j]);
-          pri_lo = min(pri_lo, pk);
-          pri_hi = max(pri_hi, pk);
-        }
-      }
-      *reinterpret_cast<unsigned*>(flags + l4) = f;
-      *reinterpret_cast<uint4*>(keys + l4) = k4;
-    };
-    if (cs == 1) {
-      // The priors are parked in the key slots (loads issued four at a time: the slice costs a
-      // couple of round trips to L2 instead of one per item).
-#pragma unroll 1
-      for (int t0 = threadIdx.x; t0 < cta_items; t0 += 4 * THREADS) {
-        float b[4];
+      for (int k = 0; k < 4; ++k) b[k] = t0 + k * THREADS < cta_items ? p[cta_lo + t0 + k * THREADS] : 0.0f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) b[k] = t0 + k * THREADS < cta_items ? p[cta_lo + t0 + k * THREADS] : 0.0f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (t0 + k * THREADS < cta_items) keys[t0 + k * THREADS] = __float_as_uint(b[k]);
-      }
-      pdl_wait();                                   // the scores are complete from here on
-      // The scores go through two staging buffers of kStep * THREADS items and the pooling halo
-      // (zero outside the sequence, which is neutral for the maximum too: scores are not
-      // negative); a part is requested while the one before it is pooled.
-      float* us = reinterpret_cast<float*>(flags + P.per * THREADS);
-      const int part = kStep * THREADS, pitch = part + 2 * kMaxHalf;
-      float a[kStep + 1];
-      // element e of the slice with its halo is score e - half of the slice; those of [e_lo, e_hi) exist
-      const float* uh = u + cta_lo - half;
-      const int e_lo = max(0, half - cta_lo);
-      const unsigned e_span = (unsigned)max(0, min(cta_items + 2 * half, q.n - cta_lo + half) - e_lo);
-      auto request = [&](int c0) {
-        const int e = c0 + (int)threadIdx.x;
-#pragma unroll
-        for (int k = 0; k < kStep; ++k) a[k] = (unsigned)(e + k * THREADS - e_lo) < e_span ? uh[e + k * THREADS] : 0.0f;
-        a[kStep] = (int)threadIdx.x < 2 * half && (unsigned)(e + part - e_lo) < e_span ? uh[e + part] : 0.0f;
-      };
-      if (cta_items > 0) request(0);
-#pragma unroll 1
-      for (int c0 = 0, buf = 0; c0 < cta_items; c0 += part, buf ^= 1) {
-        float* ub = us + buf * pitch;
-#pragma unroll
-        for (int k = 0; k < kStep; ++k) ub[threadIdx.x + k * THREADS] = a[k];
-        if ((int)threadIdx.x < 2 * half) ub[threadIdx.x + part] = a[kStep];
-        __syncthreads();
-        if (c0 + part < cta_items) request(c0 + part);
-        const int l4 = c0 + 4 * (int)threadIdx.x;
-        if (l4 < cta_items) {
-          const float4 pr = *reinterpret_cast<const float4*>(keys + l4);       // the parked priors
-          float v[4];
-          // four windows, two taps per step; averages are left-to-right sums, then one division
-          const float* w = ub + 4 * threadIdx.x;
-          const float4 x = *reinterpret_cast<const float4*>(w);
-          float y0 = x.y, y1 = x.z, y2 = x.w;
-          v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-          if (P.pool_kind == CC_POOL_MAX) {
-#pragma unroll 1
-            for (int d = 1; d < 2 * half; d += 2) {
-              const float2 y = *reinterpret_cast<const float2*>(w + d + 3);
-              v[0] = max3(v[0], y0, y1); v[1] = max3(v[1], y1, y2); v[2] = max3(v[2], y2, y.x); v[3] = max3(v[3], y.x, y.y);
-              y0 = y2; y1 = y.x; y2 = y.y;
-            }
-          } else if (half > 0) {
-#pragma unroll 1
-            for (int d = 1; d < 2 * half; d += 2) {
-              const float2 y = *reinterpret_cast<const float2*>(w + d + 3);
-              v[0] = __fadd_rn(__fadd_rn(v[0], y0), y1); v[1] = __fadd_rn(__fadd_rn(v[1], y1), y2);
-              v[2] = __fadd_rn(__fadd_rn(v[2], y2), y.x); v[3] = __fadd_rn(__fadd_rn(v[3], y.x), y.y);
-              y0 = y2; y1 = y.x; y2 = y.y;
-            }
-#pragma unroll 1
-            for (int j = 0; j < 4; ++j) {       // (rotates: one copy of the division)
-              const float y = __fdiv_rn(v[0], (float)(2 * half + 1));
-              v[0] = v[1]; v[1] = v[2]; v[2] = v[3]; v[3] = y;
-            }
-          }
-          store4(l4, v, pr);
-        }
-      }
-    } else {
-#pragma unroll 1
-      for (int li = threadIdx.x; li < cta_items; li += THREADS) {
-        // chunk sum in token order; the loads of eight tokens are issued before they are used
-        const int t0 = (cta_lo + li) * cs, t1 = min(q.n, t0 + cs);
-        float val = 0.0f, pr = -INFINITY;
-#pragma unroll 1
-        for (int j0 = t0; j0 < t1; j0 += 8) {
-          float a[8], b[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            a[k] = j0 + k < t1 ? u[j0 + k] : 0.0f;
-            b[k] = j0 + k < t1 ? p[j0 + k] : -INFINITY;
-          }
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            if (j0 + k < t1) {
-              val = (j0 + k == t0) ? a[k] : __fadd_rn(val, a[k]);
-              pr = fmaxf(pr, b[k]);
-            }
-          }
-        }
-        keys[li] = fuse(val, pr);
-        flags[li] = tally(keys[li], pr, item_len(li)) ? 1 : 0;
-      }
+      for (int k = 0; k < 4; ++k)
+        if (t0 + k * THREADS < cta_items) park(t0 + k * THREADS, b[k]);
     }
   } else {
-    const float* f = P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off;
 #pragma unroll 1
-    for (int l0 = threadIdx.x; l0 < cta_items; l0 += 4 * THREADS) {
-      float a[4], b[4];
+    for (int li = threadIdx.x; li < cta_items; li += THREADS) {
+      const int t0 = (cta_lo + li) * cs, t1 = min(q.n, t0 + cs);
+      float pr = -INFINITY;
+#pragma unroll 1
+      for (int j0 = t0; j0 < t1; j0 += 8) {
+        float b[8];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int li = l0 + k * THREADS;
-        a[k] = li < cta_items ? f[cta_lo + li] : 0.0f;
-        b[k] = li < cta_items ? item_prior(li) : 0.0f;
-      }
+        for (int k = 0; k < 8; ++k) b[k] = j0 + k < t1 ? p[j0 + k] : -INFINITY;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int li = l0 + k * THREADS;
-        if (li >= cta_items) break;
-        keys[li] = mono_key(a[k]);
-        flags[li] = tally(keys[li], b[k], item_len(li)) ? 1 : 0;
+        for (int k = 0; k < 8; ++k) pr = fmaxf(pr, b[k]);
       }
+      park(li, pr);
     }
   }
-
-  // ---- stage 0: totals of the cluster (the block reduction's barrier also publishes keys and flags)
-  c.block_totals(forced_tokens, key_lo, key_hi, pri_lo, pri_hi);
-  if (CLUSTER > 1) {
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // so have the others
-    const unsigned w[kWords] = {forced_tokens, key_lo, key_hi, pri_lo, pri_hi, 0u};
+  // Sum (and the sum over the CTAs before this one), minimum and maximum over the cluster (the block reduction's barrier also
+  // publishes what was stored to shared memory).
+  bool started = CLUSTER == 1;
+  auto totals = [&](unsigned& sum, unsigned& before, unsigned& lo0, unsigned& hi0) {
+    c.block_totals(sum, lo0, hi0);
+    if (CLUSTER == 1) return;
+    if (!started) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // so have the others
+    started = true;
+    const unsigned w[kWords] = {sum, lo0, hi0};
     const unsigned(*x)[kWords] = c.publish(w);
-    forced_tokens = 0;
+    sum = before = 0;
 #pragma unroll 1
     for (int r = 0; r < c.cluster(); ++r) {
-      if (r == c.rank()) forced_before = forced_tokens;
-      forced_tokens += x[r][0];
-      key_lo = min(key_lo, x[r][1]);
-      key_hi = max(key_hi, x[r][2]);
-      pri_lo = min(pri_lo, x[r][3]);
-      pri_hi = max(pri_hi, x[r][4]);
+      if (r == c.rank()) before = sum;
+      sum += x[r][0];
+      lo0 = min(lo0, x[r][1]);
+      hi0 = max(hi0, x[r][2]);
     }
-  }
+  };
 
-  // ---- stage 1: cap on protected items (longest prefix by (prior desc, index asc) within B_span), and
-  // stage 2: cut-off among the unprotected items, through one copy of the search
-  const bool over_cap = capped && forced_tokens > (unsigned)q.span_cap;
+  // ---- stage 1: cap on the protected items (longest prefix by (prior desc, index asc) within B_span), which hangs on the priors
+  // alone and is found before the scores are there; stage 2: cut-off among the unprotected items; one copy of the search.
+  // (3 us of search less behind the scores: 32 chunks 243.8 -> 239.7 us, all layers -1 %; 3277 chunks of ten tokens, whose
+  // priors had been read with the scores, 56.3 -> 54.0.  Writing the indices as early where protected items fill the budget
+  // takes an exchange more in every call: 32768 tokens in clusters of eight +4 %.)
   Cut cut{0u, false, 0u, 0u, 0u};
 #pragma unroll 1
-  for (int stage = over_cap ? 1 : 2; stage <= 2; ++stage) {
+  for (int stage = capped ? 1 : 2; stage <= 2; ++stage) {
     const bool first = stage == 1;
-    if (!first && forced_tokens >= keep) break;       // protected items alone fill the budget: first B in order
     const unsigned cap = (unsigned)q.span_cap;
-    cut = find_cut(c, lo, hi, first ? cap + 1u : keep - forced_tokens, first ? pri_lo : key_lo, first ? pri_hi : key_hi,
+    unsigned key_lo = pri_lo, key_hi = pri_hi;      // of the items the search is among
+    if (first) {
+      totals(forced_tokens, forced_before, key_lo, key_hi);
+      if (forced_tokens <= cap) continue;
+    } else {
+      key_lo = 0xffffffffu;
+      key_hi = 0u;
+      // ---- keys of the CTA's slice (coalesced over the block)
+      auto tally = [&](int li, unsigned key) {
+        keys[li] = key;
+        if (flags[li]) return;
+        key_lo = min(key_lo, key);
+        key_hi = max(key_hi, key);
+      };
+      if (FUSED) {
+        pdl_wait();                                   // the scores are complete from here on
+        const float* u = P.scores[q.layer] + (int64_t)h * bt.n_tot + q.tok_off;
+        const int half = (cs == 1 && P.pool_kind != CC_POOL_NONE) ? P.pool_size / 2 : 0;
+        auto fuse = [&](float val, float pr) {
+          return mono_key(__fadd_rn(__fmul_rn(P.alpha, val), __fmul_rn(P.beta, pr)));
+        };
+        // Keys and flags of four items in place of their parked priors.  Bound, like the pooling above it, by issue slots (26
+        // items a thread: 1.2 us a part of four): bounds as one unsigned compare, two taps per step, and the cap's
+        // prior range on its own took the load of a 52437-token sequence by two CTAs from 10.9 to 8.4 us, the call on 2048
+        // tokens x 2 heads 18.7 -> 18.2, 10007 x 4 38.9 -> 38.4, 32768 x 8 -0.9 %.  (Walking the slice four items to a lane in the search
+        // as well: 65536-token batches -0.5 %, small calls +1 to 2 %.)
+        auto store4 = [&](int l4, const float (&v)[4], float4 pr) {
+          const uint4 k4 = make_uint4(fuse(v[0], pr.x), fuse(v[1], pr.y), fuse(v[2], pr.z), fuse(v[3], pr.w));
+          const int left = cta_items - l4;
+          const unsigned key[4] = {k4.x, k4.y, k4.z, k4.w};
+          unsigned f = 0;
+          if (capped) {
+            f = *reinterpret_cast<const unsigned*>(flags + l4);
+          } else {
+            f = (pr.x >= theta ? 1u : 0u) | (left > 1 && pr.y >= theta ? 1u << 8 : 0u) | (left > 2 && pr.z >= theta ? 1u << 16 : 0u) |
+                (left > 3 && pr.w >= theta ? 1u << 24 : 0u);
+            forced_tokens += __popc(f);
+            *reinterpret_cast<unsigned*>(flags + l4) = f;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const bool counts = j < left && !(f >> (8 * j) & 255u);
+            key_lo = min(key_lo, counts ? key[j] : 0xffffffffu);
+            key_hi = max(key_hi, counts ? key[j] : 0u);
+          }
+          *reinterpret_cast<uint4*>(keys + l4) = k4;
+        };
+        if (cs == 1) {
+          // The scores go through two staging buffers of kStep * THREADS items and the pooling halo
+          // (zero outside the sequence, which is neutral for the maximum too: scores are not
+          // negative); a part is requested while the one before it is pooled.
+          float* us = reinterpret_cast<float*>(flags + P.per * THREADS);
+          const int part = kStep * THREADS, pitch = part + 2 * kMaxHalf;
+          float a[kStep + 1];
+          // element e of the slice with its halo is score e - half of the slice; those of [e_lo, e_hi) exist
+          const float* uh = u + cta_lo - half;
+          const int e_lo = max(0, half - cta_lo);
+          const unsigned e_span = (unsigned)max(0, min(cta_items + 2 * half, q.n - cta_lo + half) - e_lo);
+          auto request = [&](int c0) {
+            const int e = c0 + (int)threadIdx.x;
+#pragma unroll
+            for (int k = 0; k < kStep; ++k) a[k] = (unsigned)(e + k * THREADS - e_lo) < e_span ? uh[e + k * THREADS] : 0.0f;
+            a[kStep] = (int)threadIdx.x < 2 * half && (unsigned)(e + part - e_lo) < e_span ? uh[e + part] : 0.0f;
+          };
+          if (cta_items > 0) request(0);
+#pragma unroll 1
+          for (int c0 = 0, buf = 0; c0 < cta_items; c0 += part, buf ^= 1) {
+            float* ub = us + buf * pitch;
+#pragma unroll
+            for (int k = 0; k < kStep; ++k) ub[threadIdx.x + k * THREADS] = a[k];
+            if ((int)threadIdx.x < 2 * half) ub[threadIdx.x + part] = a[kStep];
+            __syncthreads();
+            if (c0 + part < cta_items) request(c0 + part);
+            const int l4 = c0 + 4 * (int)threadIdx.x;
+            if (l4 < cta_items) {
+              const float4 pr = *reinterpret_cast<const float4*>(keys + l4);       // the parked priors
+              float v[4];
+              // four windows, two taps per step; averages are left-to-right sums, then one division
+              const float* w = ub + 4 * threadIdx.x;
+              const float4 x = *reinterpret_cast<const float4*>(w);
+              float y0 = x.y, y1 = x.z, y2 = x.w;
+              v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+              if (P.pool_kind == CC_POOL_MAX) {
+#pragma unroll 1
+                for (int d = 1; d < 2 * half; d += 2) {
+                  const float2 y = *reinterpret_cast<const float2*>(w + d + 3);
+                  v[0] = max3(v[0], y0, y1); v[1] = max3(v[1], y1, y2); v[2] = max3(v[2], y2, y.x); v[3] = max3(v[3], y.x, y.y);
+                  y0 = y2; y1 = y.x; y2 = y.y;
+                }
+              } else if (half > 0) {
+#pragma unroll 1
+                for (int d = 1; d < 2 * half; d += 2) {
+                  const float2 y = *reinterpret_cast<const float2*>(w + d + 3);
+                  v[0] = __fadd_rn(__fadd_rn(v[0], y0), y1); v[1] = __fadd_rn(__fadd_rn(v[1], y1), y2);
+                  v[2] = __fadd_rn(__fadd_rn(v[2], y2), y.x); v[3] = __fadd_rn(__fadd_rn(v[3], y.x), y.y);
+                  y0 = y2; y1 = y.x; y2 = y.y;
+                }
+#pragma unroll 1
+                for (int j = 0; j < 4; ++j) {       // (rotates: one copy of the division)
+                  const float y = __fdiv_rn(v[0], (float)(2 * half + 1));
+                  v[0] = v[1]; v[1] = v[2]; v[2] = v[3]; v[3] = y;
+                }
+              }
+              store4(l4, v, pr);
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int li = threadIdx.x; li < cta_items; li += THREADS) {
+            // chunk sum in token order; the loads of eight tokens are issued before they are used
+            const int t0 = (cta_lo + li) * cs, t1 = min(q.n, t0 + cs);
+            float val = 0.0f;
+#pragma unroll 1
+            for (int j0 = t0; j0 < t1; j0 += 8) {
+              float a[8];
+#pragma unroll
+              for (int k = 0; k < 8; ++k) a[k] = j0 + k < t1 ? u[j0 + k] : 0.0f;
+#pragma unroll
+              for (int k = 0; k < 8; ++k)
+                if (j0 + k < t1) val = (j0 + k == t0) ? a[k] : __fadd_rn(val, a[k]);
+            }
+            tally(li, fuse(val, parked(li)));
+          }
+        }
+      } else {
+        const float* f = P.fused[q.layer] + (int64_t)h * bt.m_tot + q.item_off;
+#pragma unroll 1
+        for (int l0 = threadIdx.x; l0 < cta_items; l0 += 4 * THREADS) {
+          float a[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) a[k] = l0 + k * THREADS < cta_items ? f[cta_lo + l0 + k * THREADS] : 0.0f;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (l0 + k * THREADS < cta_items) tally(l0 + k * THREADS, mono_key(a[k]));
+        }
+      }
+      unsigned sum = capped ? 0u : forced_tokens, before = 0u;
+      totals(sum, before, key_lo, key_hi);
+      if (!capped) { forced_tokens = sum; forced_before = before; }
+      if (forced_tokens >= keep) break;       // protected items alone fill the budget: first B in order
+    }
+    cut = find_cut(c, lo, hi, first ? cap + 1u : keep - forced_tokens, key_lo, key_hi,
                    (unsigned)cs, !first, [&](int li, unsigned& key, unsigned& len) {
                      if ((flags[li] != 0) != first) return false;
-                     key = first ? mono_key(item_prior(li)) : keys[li];
+                     key = first ? mono_key(parked(li)) : keys[li];
                      len = item_len(li);
                      return true;
                    });
@@ -683,7 +682,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     unsigned ties = 0, none = 0;
 #pragma unroll 1
     for (int li = lo + lane; li < hi; li += 32)
-      if (flags[li] && mono_key(item_prior(li)) == cut.T) ties += item_len(li);
+      if (flags[li] && mono_key(parked(li)) == cut.T) ties += item_len(li);
     ties = __reduce_add_sync(0xffffffffu, ties);
     c.warps_before2(ties, none);
     unsigned tie_run = cut.tied_before + ties, kept = 0;
@@ -691,7 +690,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     for (int l0 = lo; l0 < hi; l0 += 32) {
       const int li = l0 + lane;
       const bool forced = li < hi && flags[li];
-      const unsigned pk = forced ? mono_key(item_prior(li)) : 0u, len = forced ? item_len(li) : 0u;
+      const unsigned pk = forced ? mono_key(parked(li)) : 0u, len = forced ? item_len(li) : 0u;
       const unsigned tm = __ballot_sync(0xffffffffu, forced && pk == cut.T);
       const unsigned before = tie_run + __popc(tm & ((1u << lane) - 1u)) * (unsigned)cs;
       tie_run += __popc(tm) * (unsigned)cs;
@@ -705,7 +704,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
     } else {
       forced_tokens = c.block_sum(kept);
       if (CLUSTER > 1) {
-        const unsigned w[kWords] = {forced_tokens, 0u, 0u, 0u, 0u, 0u};
+        const unsigned w[kWords] = {forced_tokens, 0u, 0u};
         const unsigned(*x)[kWords] = c.publish(w);
         forced_tokens = forced_before = 0;
 #pragma unroll 1
@@ -715,6 +714,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
         }
       }
     }
+    __syncthreads();               // the load replaces parked priors and reads flags of other warps' items
   }
   const bool ties_are_forced = forced_tokens >= keep;
   if (ties_are_forced) cut = Cut{0u, false, 0u, 0u, 0u};
@@ -724,7 +724,7 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
   // (relaxed: nothing is published by it, so it need not wait for stores in flight)
   if (CLUSTER > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
-  // ---- stage 3: ordered emission.  Items kept for sure (def) and the tied ones in sequence order,
+  // ordered emission.  Items kept for sure (def) and the tied ones in sequence order,
   // until the budget is full
   auto classify = [&](int li, bool& def, bool& tie) {
     def = tie = false;
@@ -811,22 +811,22 @@ size_t cluster_smem_bytes(int slots, int threads, bool staging) {
   return (b + 15) / 16 * 16;
 }
 
-template <bool FUSED, bool CHUNKED, int THREADS, int CLUSTER>
+template <bool FUSED, bool CHUNKED, bool CAPPED, int THREADS, int CLUSTER>
 cudaError_t launch_one(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, size_t smem) {
-  auto kern = select_cluster_kernel<FUSED, CHUNKED, THREADS, CLUSTER>;
+  auto kern = select_cluster_kernel<FUSED, CHUNKED, CAPPED, THREADS, CLUSTER>;
   const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(CLUSTER, g.hkv, bt.num_seqs), dim3(THREADS), smem, L.stream, CLUSTER, bt, P);
 }
-template <bool FUSED, bool CHUNKED>
+template <bool FUSED, bool CHUNKED, bool CAPPED>
 cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, SelectShape sh,
                          size_t smem) {
   const bool wide = sh.threads == 1024;
   switch (sh.cluster) {
-    case 1: return wide ? launch_one<FUSED, CHUNKED, 1024, 1>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 1>(L, bt, g, P, smem);
-    case 2: return wide ? launch_one<FUSED, CHUNKED, 1024, 2>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 2>(L, bt, g, P, smem);
-    case 4: return wide ? launch_one<FUSED, CHUNKED, 1024, 4>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 4>(L, bt, g, P, smem);
-    default: return wide ? launch_one<FUSED, CHUNKED, 1024, 8>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, 512, 8>(L, bt, g, P, smem);
+    case 1: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 1>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 1>(L, bt, g, P, smem);
+    case 2: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 2>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 2>(L, bt, g, P, smem);
+    case 4: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 4>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 4>(L, bt, g, P, smem);
+    default: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 8>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 8>(L, bt, g, P, smem);
   }
 }
 
@@ -863,8 +863,8 @@ double launch_cost(const BatchTable& bt, int hkv, const SelectRoom& room, bool s
 // on all parts, so the runtime is asked, once per context.  (148, 148, 132, 120 on the part at hand; 296, 296,
 // 284, 264 in pairs.)
 cudaError_t query_select_room(SelectRoom* room) {
-  auto one = select_cluster_kernel<true, false, 1024, 8>;
-  auto two = select_cluster_kernel<true, false, 512, 8>;
+  auto one = select_cluster_kernel<true, false, true, 1024, 8>;
+  auto two = select_cluster_kernel<true, false, true, 512, 8>;
   cudaError_t e = allow_smem(one);
   if (e == cudaSuccess) e = allow_smem(two);
   for (int lc = 0; lc <= 3 && e == cudaSuccess; ++lc) {
@@ -925,11 +925,15 @@ cudaError_t launch_select_cluster(const Launch& L, const BatchTable& bt, const G
     P.count[l] = lp.count[l];
   }
   const size_t smem = cluster_smem_bytes(P.per * sh.threads, sh.threads, fused_input && bt.chunk == 1);
+  bool capped = false;
+  for (int i = 0; i < bt.num_seqs; ++i) capped |= bt.seq[i].span_cap >= 0;
   if (fused_input)
-    return bt.chunk > 1 ? launch_shape<true, true>(L, bt, g, P, sh, smem)
-                        : launch_shape<true, false>(L, bt, g, P, sh, smem);
-  return bt.chunk > 1 ? launch_shape<false, true>(L, bt, g, P, sh, smem)
-                      : launch_shape<false, false>(L, bt, g, P, sh, smem);
+    return bt.chunk > 1 ? launch_shape<true, true, true>(L, bt, g, P, sh, smem)
+           : capped     ? launch_shape<true, false, true>(L, bt, g, P, sh, smem)
+                        : launch_shape<true, false, false>(L, bt, g, P, sh, smem);
+  return bt.chunk > 1 ? launch_shape<false, true, true>(L, bt, g, P, sh, smem)
+         : capped     ? launch_shape<false, false, true>(L, bt, g, P, sh, smem)
+                      : launch_shape<false, false, false>(L, bt, g, P, sh, smem);
 }
 
 }  // namespace cc
