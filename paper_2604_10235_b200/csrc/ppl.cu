@@ -100,7 +100,11 @@ template <> struct Vec<float> {
     }
     return fmaxf(m0, m1);
   }
-  __device__ static float one(const float* p) { return *p; }
+  __device__ static float one(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+  }
 };
 template <> struct Vec<uint16_t> {       // bf16 bit patterns
   uint4 a;
@@ -115,8 +119,23 @@ template <> struct Vec<uint16_t> {       // bf16 bit patterns
     for (int u = 0; u < kN; ++u) m = max_bf16x2(max_bf16x2(m, max_bf16x2(r[u].a.x, r[u].a.y)), max_bf16x2(r[u].a.z, r[u].a.w));
     return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
   }
-  __device__ static float one(const uint16_t* p) { return __uint_as_float((uint32_t)*p << 16); }
+  __device__ static float one(const uint16_t* p) {
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __uint_as_float((uint32_t)v << 16);
+  }
 };
+// The pairs of kLanes neighbouring lanes as one, in all of them: the maximum first, so that every lane has a single exponential.
+template <int kLanes>
+__device__ __forceinline__ void merge_lanes(Running& r) {
+  float top = r.m;
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  float sum = r.s * ex2(r.m - top);
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  r = Running{top, sum};
+}
 // adds a batch of vectors
 template <bool POLY, typename T, int kN>
 __device__ __forceinline__ void add_batch(Running& run, const Vec<T> (&r)[kN]) {
@@ -153,16 +172,21 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
   const int row = split ? whole + ((int)blockIdx.x - whole) / parts : (int)blockIdx.x;
   const int n_parts = split ? parts : 1;
   if (split) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
-  pdl_wait();
   const int chunk = row / num_tokens, t = row % num_tokens;
   const T* x = logits + (int64_t)chunk * stride_chunk + (int64_t)t * stride_token;
   Running r{kNoMax, 0.f};
+  // The target is asked for before the row, its logit before the last vectors of it: both at the end, one after the other, and a
+  // chain of sixteen merges by one thread, kept a CTA 2 us after its row was read, in waves that all end together.
+  const bool writer = part == 0 && threadIdx.x == 0;
+  int target = -1;
   const int head = min(vocab, (int)((16u - (unsigned)((uintptr_t)x & 15u)) & 15u) / (int)sizeof(T));
   const T* xv = x + head;
   const int n_vec = (vocab - head) / kVecWidth;
   int i = (int)((int64_t)n_vec * part / n_parts) + threadIdx.x;
   const int i_end = (int)((int64_t)n_vec * (part + 1) / n_parts);
   constexpr int kB = kBatch<T>;
+  pdl_wait();
+  if (writer) asm volatile("ld.global.s32 %0, [%1];" : "=r"(target) : "l"(targets + t));
   for (; i + (kB - 1) * kThreads < i_end; i += kB * kThreads) {
     Vec<T> raw[kB];
 #pragma unroll
@@ -175,6 +199,8 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
       add_batch<POLY, T, kGroup>(r, taken);
     }
   }
+  const bool known = writer && target >= 0 && target < vocab;
+  const float at_target = known ? Vec<T>::one(x + target) : 0.0f;
   for (; i < i_end; i += kThreads) {
     Vec<T> raw[1];
     raw[0].load(xv + (int64_t)i * kVecWidth);
@@ -187,15 +213,16 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
       r.merge(Vec<T>::one(x + (j < head ? j : tail + j - head)) * kLog2e, 1.0f);
   }
 
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    r.merge(__shfl_xor_sync(0xffffffffu, r.m, o), __shfl_xor_sync(0xffffffffu, r.s, o));
+  merge_lanes<32>(r);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) { sm_m[warp] = r.m; sm_s[warp] = r.s; }
   __syncthreads();
   Running all{kNoMax, 0.f};
-  if (threadIdx.x == 0)
-    for (int w = 0; w < kThreads / 32; ++w) all.merge(sm_m[w], sm_s[w]);
+  if (warp == 0) {
+    static_assert(kThreads / 32 == 16, "a half warp merges the warps' pairs");
+    all = Running{sm_m[lane & 15], sm_s[lane & 15]};
+    merge_lanes<16>(all);
+  }
   if (split) {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // the first CTA has started
     if (threadIdx.x == 0)
@@ -206,13 +233,12 @@ ppl_nll_kernel(const T* __restrict__ logits, int num_tokens, int vocab, int64_t 
     if (threadIdx.x == 0)
       for (int k = 1; k < parts; ++k) all.merge(sm_part[k].x, sm_part[k].y);
   }
-  if (threadIdx.x == 0) {
-    const int target = targets[t];
+  if (writer) {
     float out = __int_as_float(0x7fc00000);                   // NaN for an invalid token id or a row of masked logits
-    if (target < 0 || target >= vocab)
+    if (!known)
       report_error(status, CC_ERR_DEVICE_FLAG, 600);
     else if (all.m > kNoMax)
-      out = (all.m + log2f(all.s)) * kLn2 - Vec<T>::one(x + target);
+      out = (all.m + log2f(all.s)) * kLn2 - at_target;
     nll[row] = out;
   }
 }
