@@ -47,7 +47,6 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
                const __grid_constant__ CompactPtrs P, DeviceStatus* status, int heads_per_group,
                int hc_shift) {
   pdl_launch_dependents();
-  pdl_wait();
   int s = 0, local = blockIdx.x;              // sequence of this block, block index within it
   for (; s < bt.num_seqs - 1; ++s) {
     const int nb = max(1, ((bt.seq[s].keep << hc_shift) + kRowsPerBlock - 1) / kRowsPerBlock);
@@ -64,6 +63,14 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
   const int ps = bt.page_size;
   // page sizes are powers of two in practice: shifts instead of divisions then
   const int ps_shift = (ps > 0 && (ps & (ps - 1)) == 0) ? __ffs(ps) - 1 : -1;
+  const int units = q.keep << hc_shift;          // fits: keep * heads indexes an int32 array
+  const int hc_mask = (1 << hc_shift) - 1;
+  const int u = local * kRowsPerBlock + grp;
+  const int slot = u >> hc_shift;
+  const int h0 = (u & hc_mask) * heads_per_group;
+  const int64_t head_step = ps == 0 ? g.out_stride_head : g.kv_stride_head;
+  const int32_t* ip = idx + (int64_t)h0 * bt.b_tot + q.idx_off + slot;
+  pdl_wait();                                    // all of the above is arithmetic on the parameters
 
   // the block with index 0 of each sequence also publishes the sequence's new page table
   if (ps > 0 && local == 0) {
@@ -78,16 +85,10 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
     }
   }
 
-  const int units = q.keep << hc_shift;          // fits: keep * heads indexes an int32 array
-  const int hc_mask = (1 << hc_shift) - 1;
-  const int64_t head_step = ps == 0 ? g.out_stride_head : g.kv_stride_head;
   const int32_t* pt = ps > 0 ? g.page_table + (int64_t)q.src * g.page_table_stride : nullptr;
-  const int u = local * kRowsPerBlock + grp;
   if (u < units) {
     uint16_t* __restrict__ k_out = P.k_out[q.layer];
     uint16_t* __restrict__ v_out = P.v_out[q.layer];
-    const int slot = u >> hc_shift;
-    const int h0 = (u & hc_mask) * heads_per_group;
     int64_t dst0;                                  // destination row of (slot, head 0)
     if (ps == 0) {
       dst0 = ((int64_t)q.idx_off + slot) * g.out_stride_tok;
@@ -100,7 +101,6 @@ compact_kernel(const __grid_constant__ BatchTable bt, const Geometry g,
       }
       dst0 = ((int64_t)page * ps + (slot - pg * ps)) * g.kv_stride_tok;
     }
-    const int32_t* ip = idx + (int64_t)h0 * bt.b_tot + q.idx_off + slot;
 #pragma unroll 1
     for (int hh = 0; hh < heads_per_group; hh += kUnroll) {
       int tok[kUnroll];
