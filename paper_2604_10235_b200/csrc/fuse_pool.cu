@@ -77,7 +77,6 @@ nearest_fill_kernel(const __grid_constant__ BatchTable bt, int hkv, float theta,
   __shared__ unsigned mask[kNearWords];
   __shared__ int s_before, s_after;            // closest protected tokens outside the tile
   pdl_launch_dependents();
-  pdl_wait();
   const int s = blockIdx.y;
   const SeqInfo& q = bt.seq[s];
   const int n = q.n, lo = blockIdx.x * kNearTile;
@@ -85,15 +84,19 @@ nearest_fill_kernel(const __grid_constant__ BatchTable bt, int hkv, float theta,
   const float* p = prior + q.tok_off;
   const int t = threadIdx.x, lane = t & 31, word = t >> 5, j = lo + t;
   if (t == 0) { s_before = -1; s_after = 2 * n; }
-  const unsigned m = __ballot_sync(0xffffffffu, j < n && p[j] >= theta);
+  pdl_wait();
+  // the tile's priors and those of its neighbours, where the search nearly always ends, are asked for together
+  const float own = j < n ? p[j] : 0.0f;
+  const float left = lo > 0 ? p[j - kNearTile] : 0.0f, right = j + kNearTile < n ? p[j + kNearTile] : 0.0f;
+  const unsigned m = __ballot_sync(0xffffffffu, j < n && own >= theta);
   if (lane == 0) mask[word] = m;
   // outside the tile: the last protected token before lo, the first one from lo + kNearTile on
   bool need_b = lo > 0, need_a = lo + kNearTile < n;
   for (int step = 1; need_b || need_a; ++step) {
     __syncthreads();
     const int jb = lo - step * kNearTile + t, ja = lo + step * kNearTile + t;
-    if (need_b && p[jb] >= theta) atomicMax(&s_before, jb);
-    if (need_a && ja < n && p[ja] >= theta) atomicMin(&s_after, ja);
+    if (need_b && (step == 1 ? left : p[jb]) >= theta) atomicMax(&s_before, jb);
+    if (need_a && ja < n && (step == 1 ? right : p[ja]) >= theta) atomicMin(&s_after, ja);
     __syncthreads();
     need_b = need_b && s_before < 0 && lo - (step + 1) * kNearTile >= 0;
     need_a = need_a && s_after >= n && lo + (step + 1) * kNearTile < n;

@@ -426,10 +426,6 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 
   pdl_launch_dependents();
   if (CLUSTER > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA has started
-  // FUSED runs right after the second score pass, which starts only once the caller's inputs are complete and all that was
-  // enqueued before the call has ended: what the priors decide, it does before it waits for the scores
-  if (!FUSED) pdl_wait();
-
   const int h = blockIdx.y, s = blockIdx.z;
   const SeqInfo& q = bt.seq[s];
   const int m = q.n_items, cs = CHUNKED ? bt.chunk : 1;
@@ -454,6 +450,9 @@ select_cluster_kernel(const __grid_constant__ BatchTable bt, const __grid_consta
 #pragma unroll 1
   for (int i = threadIdx.x; i < kBins; i += THREADS) sm.hist[0][i] = 0;
 
+  // FUSED runs right after the second score pass, which starts only once the caller's inputs are complete and all that was
+  // enqueued before the call has ended: what the priors decide, it does before it waits for the scores
+  if (!FUSED) pdl_wait();
   // ---- priors: parked in the key slots, with the protected flags, the protected weight and, when there is a cap, the range
   // of the protected items' priors (loads are issued four or eight at a time)
   const bool capped = CAPPED && q.span_cap >= 0;
