@@ -46,10 +46,11 @@ SM_MAX_MHZ = 1965.0
 # Exponentials per clock per SM that the arithmetic units allow, from unit counts: 16 special-
 # function results and 128 fp32 FMA lanes per clock.  An exponential on the special-function
 # path also takes 2 FMA-lane operations (scale-and-shift of the logit, accumulation), one on the
-# polynomial path 9 (scale with both clamps, three for the range reduction, three for the cubic, exponent
+# polynomial path 10 (scale, clamp, three for the range reduction, three for the cubic, exponent
 # insertion, accumulation).  With a fraction p on the polynomial path both pipes are full when
-# (1 - p) / 16 = (2 (1 - p) + 9 p) / 128, p = 2/5: 16 / (3/5) = 26.7 per clock per SM.
-ALU_EXP_PER_CLK_SM = 26.7
+# (1 - p) / 16 = (2 (1 - p) + 10 p) / 128, p = 3/8: 16 / (5/8) = 25.6 per clock per SM.  (The kernel's
+# clamps come with its scaling by now: 9 operations would make it 26.7.)
+ALU_EXP_PER_CLK_SM = 25.6
 
 
 def score_kernel_roofline(work, peaks, score_seconds):
@@ -63,7 +64,7 @@ def score_kernel_roofline(work, peaks, score_seconds):
         roof = {"bound": "alu", "achieved": 2.0 * work["exps"] / score_seconds / 1e9,
                 "peak": alu_peak / 1e9, "unit": "Gexp/s",
                 "peak_source": "unit counts: 16 SFU results + 128 FMA lanes per clock per SM, "
-                               "148 SMs, 1965 MHz (26.7 exponentials per clock per SM)"}
+                               "148 SMs, 1965 MHz (25.6 exponentials per clock per SM)"}
     elif t_f >= t_b:
         roof = {"bound": "tensor", "achieved": work["flops"] / score_seconds / 1e12,
                 "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
