@@ -8,11 +8,13 @@
 namespace cc {
 
 constexpr float kEx2Magic = 12582912.0f;         // 1.5 * 2^23: adding it rounds to the nearest integer
-// degree-3 minimax polynomial of 2^f on [-0.5, 0.5], relative error 7.8e-5
-constexpr float kEx2C3 = 0.05516434833407402f;
-constexpr float kEx2C2 = 0.24259322881698608f;
-constexpr float kEx2C1 = 0.693260669708252f;
-constexpr float kEx2C0 = 0.9999293088912964f;
+// 2^f on [-0.5, 0.5] by the cubic with the least mean error among those within 7.8e-5 of it (relative; a linear program over
+// 2001 points).  The mean is what stays in a row's sum: 2.6e-6, against 5.8e-6 of an earlier fit and 8e-5 as the
+// least maximum with a mean of zero.
+constexpr float kEx2C3 = 0.05528990179300308f;
+constexpr float kEx2C2 = 0.24261438846588135f;
+constexpr float kEx2C1 = 0.6932293772697449f;
+constexpr float kEx2C0 = 0.9999241828918457f;
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -89,32 +91,32 @@ __device__ __forceinline__ uint64_t ex2_pair_fma(uint64_t x) {
   return pack2(__int_as_float(r0), __int_as_float(r1));
 }
 
-// 2^x on the FMA pipe for x = v * kScale + off given by its place y = (x + kSatLow) / kSatSpan on a scale that the
-// multiply-add saturates to [0, 1]: both clamps (2^-124 below, 2^124 above) come with the scaling.  kSatSpan is an integer for
-// which kScale / kSatSpan is exact in f32 and kSatLow / kSatSpan is one half: what remains is the rounding of y, 4e-6 in x (a
-// span of 252 had moved all scores by 2e-6).
 constexpr float kScale = 0.12751743f;            // log2(e) / sqrt(128)
-constexpr float kSatLow = 124.0f, kSatSpan = 248.0f, kSatScale = kScale / kSatSpan;
-__device__ __forceinline__ float sat_offset(float off) { return fmaf(off, 1.0f / kSatSpan, 0.5f); }
-__device__ __forceinline__ float fma_sat(float a, float b, float c) {
-  float d;
-  asm("fma.rn.ftz.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t ex2_pair_sat(float y0, float y1) {
-  const uint64_t y = pack2(y0, y1), span = pack2(kSatSpan, kSatSpan), bias = pack2(kEx2Magic - kSatLow, kEx2Magic - kSatLow);
-  const uint64_t t = fma2(y, span, bias);             // magic + x, rounded to an integer
-  const uint64_t f = fma2(y, span, sub2(bias, t));    // x - n
+// 2^(v * kScale - m) for a pair on the FMA pipe, m an integer of at most kMaxRef in size.  Then kEx2Magic - m is exact, and
+// the product takes part unrounded in both steps: n is the integer nearest to the exact argument, and the remainder, at most one
+// half, is rounded once, to 2^-25.  (An argument rounded at its own size is good to 2^-20 between -16 and -32.  Its place on a scale of
+// 248 powers of two, from a saturating multiply-add that clamps on both sides, is good to 2^-18 only and has a bias per reference.
+// Score stages are 0.3 to 0.6 % faster with that, and 1 % slower with arguments rounded at their own size.  Against 64 bits, geometric
+// means over 17 shapes x 4 inputs: log-sums 1.45e-6 with arguments of their own size, 1.47e-6 with the scale, 1.14e-6 now;
+// scores 3.70e-6, 3.71e-6, 3.66e-6 in norm.)
+// The clamp below, at -124, is on the value; the caller sees to it that arguments stay under 127.
+constexpr float kMaxRef = 1048576.0f;
+struct PolyRef { float bias, low; };
+__device__ __forceinline__ PolyRef poly_ref(float m) { return PolyRef{kEx2Magic - m, (m - 124.0f) * (1.0f / kScale)}; }
+__device__ __forceinline__ uint64_t ex2_pair_scaled(float v0, float v1, const PolyRef& r) {
+  const uint64_t v = pack2(fmaxf(v0, r.low), fmaxf(v1, r.low)), c2 = pack2(kScale, kScale), bias = pack2(r.bias, r.bias);
+  const uint64_t t = fma2(v, c2, bias);             // magic + n
+  const uint64_t f = fma2(v, c2, sub2(bias, t));    // v * kScale - m - n
   uint64_t p = fma2(f, pack2(kEx2C3, kEx2C3), pack2(kEx2C2, kEx2C2));
   p = fma2(p, f, pack2(kEx2C1, kEx2C1));
   p = fma2(p, f, pack2(kEx2C0, kEx2C0));
   float p0, p1, t0, t1;
   unpack2(p, p0, p1);
   unpack2(t, t0, t1);
-  int r0, r1;
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
-  return pack2(__int_as_float(r0), __int_as_float(r1));
+  int e0, e1;
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(e0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(e1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
+  return pack2(__int_as_float(e0), __int_as_float(e1));
 }
 
 // Of every three pairs one takes the polynomial path, and the two paths have a sum each: the special-function unit is the
@@ -143,17 +145,35 @@ __device__ __forceinline__ void exp_accumulate_columns(const uint32_t (&v)[32], 
     }
   }
 }
-// The same with one offset for all values (none: 0), os = sat_offset(off).
-// Arguments above 124 saturate: 2^124, or more up to infinity.
-template <bool kOffset, int kWidth>
-__device__ __forceinline__ void exp_accumulate(const uint32_t (&v)[32], uint64_t off2, float os, uint64_t (&acc)[2]) {
-  const uint64_t c2 = pack2(kScale, kScale);
+// The same with one offset for all values, any number.
+__device__ __forceinline__ void exp_accumulate_any(const uint32_t (&v)[32], float off, uint64_t (&acc)[2]) {
+  const uint64_t c2 = pack2(kScale, kScale), off2 = pack2(off, off);
+#pragma unroll
+  for (int pair = 0; pair < 16; ++pair) {
+    const uint64_t x = fma2(pack2(__uint_as_float(v[2 * pair]), __uint_as_float(v[2 * pair + 1])), c2, off2);
+    if (poly_pair(pair)) acc[1] = add2(acc[1], ex2_pair_fma(x));
+    else acc[0] = add2(acc[0], ex2_pair_sfu(x));
+  }
+}
+// acc += 2^(v * kScale - m) over the first kWidth of 32 values, m an integer of at most kMaxRef in size (kRef false: 0),
+// r = poly_ref(m).
+template <bool kRef, int kWidth>
+__device__ __forceinline__ void exp_accumulate(const uint32_t (&v)[32], float m, const PolyRef& r, uint64_t (&acc)[2]) {
+  const uint64_t c2 = pack2(kScale, kScale), off2 = pack2(-m, -m);
 #pragma unroll
   for (int pair = 0; pair < kWidth / 2; ++pair) {
     const float a = __uint_as_float(v[2 * pair]), b = __uint_as_float(v[2 * pair + 1]);
-    if (poly_pair(pair)) acc[1] = add2(acc[1], ex2_pair_sat(fma_sat(a, kSatScale, os), fma_sat(b, kSatScale, os)));
-    else acc[0] = add2(acc[0], ex2_pair_sfu(kOffset ? fma2(pack2(a, b), c2, off2) : mul2(pack2(a, b), c2)));
+    if (poly_pair(pair)) acc[1] = add2(acc[1], ex2_pair_scaled(a, b, r));
+    else acc[0] = add2(acc[0], ex2_pair_sfu(kRef ? fma2(pack2(a, b), c2, off2) : mul2(pack2(a, b), c2)));
   }
+}
+// The largest of limit and the values that take the polynomial path.
+__device__ __forceinline__ float poly_max(const uint32_t (&v)[32], float limit) {
+#pragma unroll
+  for (int pair = 0; pair < 16; ++pair)
+    if (poly_pair(pair))
+      asm("max.f32 %0, %0, %1, %2;" : "+f"(limit) : "f"(__uint_as_float(v[2 * pair])), "f"(__uint_as_float(v[2 * pair + 1])));
+  return limit;
 }
 __device__ __forceinline__ float acc_total(const uint64_t (&acc)[2]) {
   float a, b;

@@ -306,17 +306,17 @@ __device__ __forceinline__ void hand_back(uint32_t empty_bar, int lane) {
 }
 
 // pass 1, all 128 keys count.  The reference of the exponentials only has to be near the row
-// maximum, not equal to it: it is replaced when a value lies more than 2^64 above it.  Only the first
+// maximum, not equal to it: it is replaced when a value lies more than 2^64 above it.  It is an integer, for the sake of
+// the polynomial's arguments.  Only the first
 // chunk of a row and the last of an item look at their maximum beforehand, a serial stretch of 16 instructions, a
-// vote and a branch before the first exponential; what the chunks in between add is
-// looked at before the buffer goes back, and when it is above kRedo (exponentials saturate at 2^124) nothing
-// has been changed and the answer is false: the caller goes through the item again, chunk by chunk.  (Together
-// with the saturating scale of the polynomial's arguments, the score stage of 32768 tokens x 8 heads of 256 rows -2.9 %,
-// 65536 x 4 of 448 -3.5 %, 32 x 2200 x 8 of 512 -2.8 %, 131072 x 8 of 256 -3.8 %.)
+// vote and a branch before the first exponential.  Of the chunks in between, sums and the largest polynomial argument (which
+// would wrap silently above 128) are looked at before the buffer goes back, and when they are too large, or the reference
+// is, nothing has been changed and the answer is false: the caller goes through the item again, chunk by chunk.
 constexpr float kRedo = 1.1805916e21f;     // 2^70
 __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, int lane, float& m_run, float& l_run) {
   uint64_t acc[2] = {0ull, 0ull};
-  float m = m_run, l = l_run;
+  float m = m_run, l = l_run, top = -INFINITY;
+  PolyRef r = poly_ref(m);
   bool look = __any_sync(0xffffffffu, m == -INFINITY);
 #pragma unroll 1
   for (int cc0 = 0; cc0 < kTileKeys; cc0 += 32) {
@@ -324,20 +324,25 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
     tmem_ld32(addr + (uint32_t)cc0, v);
     tmem_wait_ld();
     if (look) {
+      const float mx = max32(v) * kScale;
       if (cc0 + 32 == kTileKeys) {
-        if (__any_sync(0xffffffffu, !(acc_total(acc) < kRedo))) return false;
+        const bool fine = acc_total(acc) < kRedo && fmaf(top, kScale, -m) < 100.0f && fmaxf(fabsf(m), mx) < kMaxRef;
+        if (!__all_sync(0xffffffffu, fine)) return false;
         hand_back(empty_bar, lane);
       }
-      const float mx = max32(v) * kScale;
       if (m == -INFINITY || mx > m + 64.0f) {
-        if (m > -INFINITY) l = (l + acc_total(acc)) * ex2(m - mx);
+        const float ref = rintf(mx);
+        if (m > -INFINITY) l = (l + acc_total(acc)) * ex2(m - ref);
         acc[0] = acc[1] = 0ull;
-        m = mx;
+        m = ref;
+        r = poly_ref(m);
       }
       __syncwarp();
+    } else {
+      top = poly_max(v, top);
     }
     look = cc0 + 64 == kTileKeys;
-    exp_accumulate<true, 32>(v, pack2(-m, -m), sat_offset(-m), acc);
+    exp_accumulate<true, 32>(v, m, r, acc);
   }
   m_run = m;
   l_run = l + acc_total(acc);
@@ -345,7 +350,7 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
 }
 
 // pass 1, keys from valid_r on (a bound of the thread's own) do not count
-// (returns the row's new reference and sum).  Chunks that no row of the warp attends to are skipped, and in those that all do
+// (returns the row's new reference and sum); logits of any size.  Chunks that no row of the warp attends to are skipped, and in those that all do
 // nothing is masked: with a causal window most are one or the other, and the CTA with the last tiles of a sequence is what a
 // short call waits for (10007 tokens x 4 heads: 7 us of work there, 4.5 to 5.5 elsewhere; score stage 24.1 -> 22.8 us).
 __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empty_bar, int lane, int valid_r, float m_run, float l_run) {
@@ -366,11 +371,12 @@ __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empt
     }
     const float mx = max32(v) * kScale;
     if (m_run == -INFINITY || mx > m_run + 64.0f) {
-      if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - mx);
+      const float ref = rintf(mx);
+      if (m_run > -INFINITY) l_run = (l_run + acc_total(acc)) * ex2(m_run - ref);
       acc[0] = acc[1] = 0ull;
-      m_run = mx;
+      m_run = ref;
     }
-    exp_accumulate<true, 32>(v, pack2(-m_run, -m_run), sat_offset(-m_run), acc);
+    exp_accumulate_any(v, -m_run, acc);
   }
   return make_float2(m_run, l_run + acc_total(acc));
 }
@@ -386,7 +392,7 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
     tmem_ld32(addr + (uint32_t)cc0, v);               // stays inside the 128-column buffer
     tmem_wait_ld();
     if (cc0 + 32 == nc) hand_back(empty_bar, lane);
-    if (ADDED) exp_accumulate<false, 32>(v, 0ull, 0.5f, acc);
+    if (ADDED) exp_accumulate<false, 32>(v, 0.0f, poly_ref(0.0f), acc);
     else exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
   }
   if (nc & 16) {
@@ -394,7 +400,7 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
     tmem_ld32(addr + (uint32_t)(nc - 16), v);
     tmem_wait_ld();
     hand_back(empty_bar, lane);
-    if (ADDED) exp_accumulate<false, 16>(v, 0ull, 0.5f, acc);
+    if (ADDED) exp_accumulate<false, 16>(v, 0.0f, poly_ref(0.0f), acc);
     else exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)(nc - 16), acc);
   }
   return acc_total(acc);
@@ -502,7 +508,7 @@ __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, 
 // that code.  IDLE ones (pass 1) skip the items of warps whose 32 rows all lie behind the last one: one
 // item in four on two of the four schedulers for 448 rows.  ADDED ones (pass 2) have -L_r added by the product, a ninth step of
 // 16 channels (ones x three bf16 that sum to it), instead of reading it from shared memory for every column: eight loads fewer
-// per chunk, and the argument of the polynomial is one saturating multiply-add (see kAddedItems).  65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us,
+// per chunk  (see kAddedItems).  65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us,
 // 30000 x 8 of 400 rows 82.2 -> 81.0; with the test in all instantiations the others were 0.2-0.5 % slower.
 template <int PASS, bool CAUSAL, int LAYERS, int HALVES, bool IDLE, bool ADDED>
 __global__ void __launch_bounds__(kThreads, 1)
