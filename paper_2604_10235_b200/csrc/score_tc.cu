@@ -349,6 +349,9 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
   return true;
 }
 
+// Stands for a product that does not count: minus infinity, since a row's own logits may lie anywhere.
+constexpr uint32_t kMasked = 0xff800000u;
+
 // pass 1, keys from valid_r on (a bound of the thread's own) do not count
 // (returns the row's new reference and sum); logits of any size.  Chunks that no row of the warp attends to are skipped, and in those that all do
 // nothing is masked: with a causal window most are one or the other, and the CTA with the last tiles of a sequence is what a
@@ -367,7 +370,7 @@ __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empt
     if (!whole) {
 #pragma unroll
       for (int i = 0; i < 32; ++i)
-        if (cc0 + i >= valid_r) v[i] = 0xc61c4000u;  // -1e4: its exponential underflows to 0
+        if (cc0 + i >= valid_r) v[i] = kMasked;
     }
     const float mx = max32(v) * kScale;
     if (m_run == -INFINITY || mx > m_run + 64.0f) {
@@ -422,7 +425,7 @@ __device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty
     if (!__all_sync(0xffffffffu, !key || cc0 >= first_col)) {
 #pragma unroll
       for (int i = 0; i < 32; ++i)
-        if (cc0 + i < first_col) v[i] = 0xc61c4000u;     // -1e4: exponential ~ 0
+        if (cc0 + i < first_col) v[i] = kMasked;
     }
     if (cc0 + 32 <= nc) exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
     else                exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)cc0, acc);

@@ -112,7 +112,8 @@ def test_rises_in_columns_of_the_polynomial(at, jump):
 
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("at", [0, 31, 36, 100, 127, 128 + 80, 640 + 120])
-@pytest.mark.parametrize("logit,rest", [(7.0e5, 0.0), (1.5e6, 0.0), (3.0e7, 0.0)])
+@pytest.mark.parametrize("logit,rest", [(7.0e5, 0.0), (1.5e6, 0.0), (3.0e7, 0.0), (-1.0e3, -1.2e3), (-7.3e5, -1.0e6),
+                                        (-1.0e6, -4.0e6)])
 def test_logits_of_any_size(at, logit, rest, causal):
     """References around and beyond 2^20: the one key has all of every row that attends to it.  Its scores are good to half a unit
     in the last place of the f32 row statistic and to one of the product, in powers of two."""
