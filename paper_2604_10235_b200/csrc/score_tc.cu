@@ -61,8 +61,6 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kBufCols = 128;                        // accumulator buffer stride
 constexpr int kBufs = 4;                                  // accumulator buffers in TMEM
 constexpr int kSets = 4;                                  // epilogue warp sets, one per buffer
-constexpr uint32_t kMiscBytes = 18432;
-constexpr uint32_t kLBytes = 20, kLFixed = 8 * 16 + kTileKeys * 4;   // -L_r in its two forms: bytes a row, and besides
 constexpr uint32_t kSmemLimit = 232448;                   // 227 KB
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -247,7 +245,7 @@ struct Barriers {
   uint64_t edge_full[2][4];          // ... of a first / last tile of which the CTA has one half
 };
 
-struct Misc {                        // lives in the last kMiscBytes of dynamic shared memory
+struct Misc {                        // behind the ring of K tiles in dynamic shared memory
   union {
     float2 xchg[kSets][kMaxRows];    // (max, sum) hand-over: pass 1 per set, pass 2 while merging (the first of them)
     struct {
@@ -255,13 +253,16 @@ struct Misc {                        // lives in the last kMiscBytes of dynamic 
       uint4 ones[2 * kTileKeys];     // pass 2: the other side of the operand with -L_r: 128 keys x 16 channels, (1, 1, 1, 0, ...)
     };
   };
-  float edge_part[2][kTileKeys];     // pass 2: partial column sums of those tiles
+  union {
+    float edge_part[2][kTileKeys];   // pass 2: partial column sums of cut tiles
+    float zeros[kTileKeys];          // pass 2, products with -L_r (no tile is cut then): offsets of none
+  };
   Barriers bar;
   long long span[2];                 // first unit of the CTA, first unit behind it
   uint32_t tmem_base;
   volatile int abort_flag;
 };
-static_assert(sizeof(Misc) <= kMiscBytes, "Misc does not fit");
+static_assert(sizeof(Misc) % 16 == 0, "the operand behind Misc starts on 16 bytes");
 
 struct Pipe {
   Misc* misc;
@@ -525,9 +526,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   uint8_t* q_smem = smem;
   uint8_t* k_smem = smem + q_bytes;
   Misc* misc = reinterpret_cast<Misc*>(k_smem + (size_t)P.n_stages * kStageBytes);
-  // pass 2: -L_r as an operand (rows_pad + 8 rows), in the log2 domain (-1e4 for padded rows), 128 zeros
-  uint4* l_smem = reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(misc) + kMiscBytes);
-  float* neg_lc = reinterpret_cast<float*>(l_smem + P.rows_pad + 8);
+  // pass 2: -L_r in the log2 domain (-1e4 for padded rows), before it (ADDED) as an operand (rows_pad + 8 rows)
+  uint4* l_smem = reinterpret_cast<uint4*>(misc + 1);
+  float* neg_lc = reinterpret_cast<float*>(ADDED ? l_smem + P.rows_pad + 8 : l_smem);
   Pipe pipe{misc, status};
 
   // the warp index as a value the compiler knows to be the same in all lanes: the MMA issuer's
@@ -568,7 +569,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int i = threadIdx.x - 128;       // 8-row groups of 256 bytes: channels 0-7 of the rows, channels 8-15
     misc->ones[i] = (i & 8) ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
     if (i < 8) l_smem[P.rows_pad + i] = make_uint4(0u, 0u, 0u, 0u);
-    if (CAUSAL && i < kTileKeys) neg_lc[P.rows_pad + i] = 0.0f;
+    if (CAUSAL && i < kTileKeys) misc->zeros[i] = 0.0f;
     fence_proxy_async();
   }
   if (PASS == 2) pdl_launch_dependents();
@@ -999,7 +1000,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           // causal window: key j is seen by the rows t >= j - (n - w), i.e. by the columns from
           // G * (j - n + w) on; the columns before it contribute nothing
           if (edge)
-            u_acc = drain_rows_masked(acc_addr, empty_bar, lane, smem_u32(neg_lc + (!ADDED || first_item ? c0 : P.rows_pad)), nc,
+            u_acc = drain_rows_masked(acc_addr, empty_bar, lane, smem_u32(!ADDED || first_item ? neg_lc + c0 : misc->zeros), nc,
                                       g.group * (key0 + row_in_tile - n_cur + g.window) - c0, row_in_tile < valid);
           else if (!ADDED || first_item)
             u_acc = drain_rows<false>(acc_addr, empty_bar, lane, smem_u32(neg_lc + c0), nc);
@@ -1078,9 +1079,29 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 // Spans with cut tiles have few items.
 constexpr int kAddedItems = 16;
 
+// Shared memory of a launch: Q, a ring of as many K tiles as there is room for, Misc, and in pass 2 the row statistics.  Each
+// launch has the ring that its own needs leave: 5 tiles at 176 rows, 4 at 304 (320 in pass 1), 3 at 432 (448 in pass 1).
+struct Ring {
+  int stages;
+  size_t smem_bytes;
+};
+Ring ring_of(int rows_pad, size_t l_bytes) {
+  const size_t fixed = 1024 + (size_t)rows_pad * 256 + sizeof(Misc) + l_bytes;
+  const int stages = fixed < kSmemLimit ? (int)((kSmemLimit - fixed) / kStageBytes) : 0;
+  const int n = stages < kMaxStages ? stages : kMaxStages;
+  return Ring{n, fixed + (size_t)n * kStageBytes};
+}
+Ring ring_pass1(int rows_pad) { return ring_of(rows_pad, 0); }
+Ring ring_pass2(int rows_pad, bool added) { return ring_of(rows_pad, (size_t)rows_pad * 4 + (added ? (size_t)(rows_pad + 8) * 16 : 0)); }
+// Whether pass 2 lets the products add -L_r (ADDED): with items enough (kAddedItems), and not where the operand costs the ring a tile
+// (64, 304, 432 rows): 131072 tokens x 8 heads of 64 rows 86.6 with it and 84.9 us without, 65536 x 8 of 304 rows 102.6 and 102.0,
+// of 432 130.3 and 129.7.
+bool adds_statistic(int rows_pad, int items, int grid) {
+  return items >= kAddedItems * grid && ring_pass2(rows_pad, true).stages == ring_pass2(rows_pad, false).stages;
+}
+
 struct TcPlan {
   TcParams P;
-  size_t smem_bytes;
   bool ok;
 };
 
@@ -1114,12 +1135,7 @@ TcPlan make_plan(const BatchTable& bt, const Geometry& g, int sm_count, int laye
   P.grid = units < sm_count ? units : sm_count;
   if (P.grid < 1) P.grid = 1;
   pl.ok = P.rows_pad <= kMaxRows && w_pad <= 256 && g.group <= 256;
-  const uint32_t q_bytes = (uint32_t)P.rows_pad * 256u, l_bytes = (uint32_t)P.rows_pad * kLBytes + kLFixed;
-  int stages = ((int)kSmemLimit - 1024 - (int)kMiscBytes - (int)(q_bytes + l_bytes)) / (int)kStageBytes;
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages < 2) pl.ok = false;
-  P.n_stages = stages;
-  pl.smem_bytes = 1024 + q_bytes + (size_t)stages * kStageBytes + kMiscBytes + l_bytes;
+  if (ring_pass2(P.rows_pad, false).stages < 2) pl.ok = false;
   return pl;
 }
 
@@ -1186,7 +1202,8 @@ cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry&
                : idle   ? score_tc_kernel<1, false, LAYERS, HALVES, true, false>
                         : score_tc_kernel<1, false, LAYERS, HALVES, false, false>;
   auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false, false> : score_tc_kernel<2, false, LAYERS, HALVES, false, false>;
-  if (HALVES == 1 && P.total_tiles * P.n_sub >= kAddedItems * P.grid)
+  const bool added = HALVES == 1 && adds_statistic(P.rows_pad, P.total_tiles * P.n_sub, P.grid);
+  if (added)
     pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false, HALVES == 1>
                      : score_tc_kernel<2, false, LAYERS, HALVES, false, HALVES == 1>;
   cudaError_t e = allow_smem(pass1);
@@ -1195,10 +1212,13 @@ cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry&
 
   P.n_sub = (P.rows_pad + 127) / 128;
   P.sub_cols = 0;
-  e = launch_pdl(pass1, dim3(P.grid), dim3(kThreads), pl.smem_bytes, L.stream, 1, bt, g, P, M, L.status);
+  const Ring ring1 = ring_pass1(P.rows_pad), ring2 = ring_pass2(P.rows_pad, added);
+  P.n_stages = ring1.stages;
+  e = launch_pdl(pass1, dim3(P.grid), dim3(kThreads), ring1.smem_bytes, L.stream, 1, bt, g, P, M, L.status);
   if (e != cudaSuccess) return e;
   P.sub_cols = ((P.rows_pad + P.n_sub - 1) / P.n_sub + 15) / 16 * 16;
-  return launch_pdl(pass2, dim3(P.grid), dim3(kThreads), pl.smem_bytes, L.stream, 1, bt, g, P, M, L.status);
+  P.n_stages = ring2.stages;
+  return launch_pdl(pass2, dim3(P.grid), dim3(kThreads), ring2.smem_bytes, L.stream, 1, bt, g, P, M, L.status);
 }
 
 }  // namespace
@@ -1221,3 +1241,11 @@ cudaError_t launch_score_tc(const Launch& L, const BatchTable& bt, const Geometr
 }
 
 }  // namespace cc
+
+extern "C" void ccx_score_ring(int rows_pad, int items, int grid, int* pass1, int* pass2, int* added, size_t* smem_bytes) {
+  *added = cc::adds_statistic(rows_pad, items, grid);
+  const cc::Ring one = cc::ring_pass1(rows_pad), two = cc::ring_pass2(rows_pad, *added != 0);
+  *pass1 = one.stages;
+  *pass2 = two.stages;
+  *smem_bytes = one.smem_bytes > two.smem_bytes ? one.smem_bytes : two.smem_bytes;
+}

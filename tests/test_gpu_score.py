@@ -64,7 +64,7 @@ def test_scores_tiny_config(mode, tol):
 @pytest.mark.parametrize("w,hq,hkv,page", [(96, 8, 2, 0), (48, 14, 2, 16)])
 def test_scores_three_stage_ring(w, hq, hkv, page):
     """Row counts of 384 and 336: the shared-memory ring of the tensor-core kernel has three K
-    stages then (four below 295 rows, two above 413), and 40000 keys give every CTA more tiles than
+    stages then (four below 313 rows, two above 440, in pass 2), and 40000 keys give every CTA more tiles than
     the ring has stages, so it wraps."""
     wl = gen.Workload("ring3", 26, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 1,
                       seq_lens=(40000,), budget_frac=0.1, page_size=page)

@@ -54,3 +54,16 @@ def test_a_wave_of_wide_clusters_is_as_wide_as_the_device():
     two where 96 do, and then narrower clusters are cheaper."""
     assert _shape(65536, 7, 2)[0] == 8
     assert _shape(65536, 7, 2, room=((148, 148, 128, 96), (296, 296, 256, 192)))[0] == 4
+
+
+@pytest.mark.parametrize("items", [1, 40])
+def test_row_statistics_cost_the_ring_of_k_tiles_nothing(items):
+    """As many tiles of 32 KB as Q, 20 KB of hand-over buffers and 2 KB of statistics leave of 227 KB, whatever else a launch holds."""
+    ring = binding.load_library().ccx_score_ring
+    for rows in range(16, 513, 16):
+        one, two, added, smem = C.c_int(), C.c_int(), C.c_int(), C.c_size_t()
+        ring(rows, items * 148, 148, C.byref(one), C.byref(two), C.byref(added), C.byref(smem))
+        least = min(6, (232448 - 1024 - 20480 - 256 * rows) // 32768)
+        assert one.value >= two.value >= least >= 2, rows
+        assert one.value <= 6 and smem.value <= 232448
+        assert items == 40 or not added.value
