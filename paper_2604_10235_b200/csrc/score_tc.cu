@@ -44,15 +44,11 @@ namespace cc {
 
 namespace {
 
-#ifndef CC_ISSUERS
-#define CC_ISSUERS 2
-#endif
-constexpr int kIssuers = CC_ISSUERS;                      // 1 or 2
+constexpr int kIssuers = 2;                               // MMA issuers: items go to them in pairs, one per epilogue set and turn
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (1 + kIssuers + kEpiWarps) * 32; // TMA, the MMA issuers, 16 epilogue warps
-constexpr int kMmaWarpB = 2 + kEpiWarps;                  // second MMA issuer (the last warp), if any
-static_assert(kIssuers == 1 || kIssuers == 2, "every warp of the CTA needs a role");
-static_assert(kThreads / 32 == kMmaWarpB + kIssuers - 1, "warps 0, 1, the epilogue warps, the second issuer");
+constexpr int kMmaWarpB = 2 + kEpiWarps;                  // second MMA issuer (the last warp)
+static_assert(kThreads / 32 == kMmaWarpB + 1, "warps 0, 1, the epilogue warps, the second issuer");
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kMaxStages = 6;
 constexpr uint32_t kPanelBytes = kTileKeys * 128;        // one 64-channel half of a K tile
@@ -665,7 +661,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         if (++stage == P.n_stages) { stage = 0; phase ^= 1; }
       }
     }
-  } else if (warp == 1 || (kIssuers == 2 && warp == kMmaWarpB)) {
+  } else if (warp == 1 || warp == kMmaWarpB) {
     // ================================================================ MMA issuers
     // The whole warp walks the items and waits; one elected lane issues the multiplications.  With
     // all of it inside `if (lane == 0)` the compiler cannot know that the operands of tcgen05.mma
@@ -706,7 +702,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
       // the second 8 channels of a group of rows lie on the next group's first and meet zeros)
       const uint64_t ones_desc = (uint64_t)(((smem_u32(misc->ones) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(16u | (1u << 14)) << 32);
       const uint64_t l_desc = (uint64_t)(((smem_u32(l_smem) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(8u | (1u << 14)) << 32);
-      // only the first two of its items of a (sequence, head) does an issuer multiply without it: L_r may not be known yet
+      // only the first two of its items of a (sequence, head), the first of each set, does an issuer multiply without it: L_r may not be known yet
       uint32_t l_phase = 0, n_own = 0;
       bool l_known = false;
       const bool elected = elect_one();
@@ -722,7 +718,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         const uint32_t k_lo = k_lo0 + (uint32_t)stage * (kStageBytes >> 4);
 #pragma unroll 1
         for (int sub = t == t_begin ? sub_begin : 0; sub < (t == t_end - 1 ? sub_end : P.n_sub); ++sub, ++item) {
-          if (kIssuers == 2 && (int)((item >> 1) & 1u) != my_half) continue;
+          if ((int)((item >> 1) & 1u) != my_half) continue;
           const uint32_t buf = item & (kBufs - 1);
           const uint32_t par = ((item >> 2) & 1u) ^ 1u;
           if (!warp_wait(pipe, &misc->bar.acc_empty[buf], par, 22)) {

@@ -1,9 +1,11 @@
 """Rules that choose the form of a launch, as plain functions of sizes (no GPU)."""
 import ctypes as C
+import os
+import re
 
 import pytest
 
-from paper_2604_10235_b200 import binding
+from paper_2604_10235_b200 import binding, build
 
 
 @pytest.mark.parametrize("vocab", [5000, 32000, 50257, 151936])
@@ -67,3 +69,10 @@ def test_row_statistics_cost_the_ring_of_k_tiles_nothing(items):
         assert one.value >= two.value >= least >= 2, rows
         assert one.value <= 6 and smem.value <= 232448
         assert items == 40 or not added.value
+
+
+def test_no_switch_of_a_build_changes_a_kernel():
+    """What is tested is what is built: no constant of the sources can be set from the compiler's command line."""
+    for name in os.listdir(build.CSRC):
+        with open(os.path.join(build.CSRC, name)) as f:
+            assert not re.search(r"^\s*#\s*(ifn?def|if|elif)\b", f.read(), re.M), name
