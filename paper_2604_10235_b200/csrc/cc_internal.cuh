@@ -221,5 +221,6 @@ extern "C" {
 void ccx_ppl_split(int rows, int vocab, int slots, int* whole, int* parts);
 void ccx_select_shape(int max_items, int num_seqs, int hkv, int chunk, int fused_input, const int* one, const int* two,
                       int* cluster, int* threads);
+int ccx_select_has_shape(int chunk, int cluster, int threads);
 void ccx_score_ring(int rows_pad, int items, int grid, int* pass1, int* pass2, int* added, size_t* smem_bytes);
 }

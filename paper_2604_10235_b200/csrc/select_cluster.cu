@@ -817,15 +817,26 @@ cudaError_t launch_one(const Launch& L, const BatchTable& bt, const Geometry& g,
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(CLUSTER, g.hkv, bt.num_seqs), dim3(THREADS), smem, L.stream, CLUSTER, bt, P);
 }
+// Shapes there is code for: those that are the cheapest (launch_cost) for some batch on 148 SMs.  Of the ones with 512 threads
+// these are a CTA alone, for short sequences, and clusters of four and eight for chunks; the others lost to 1024 threads or to
+// another width on each of 400000 batches (1 to 10^6 items, 1 to 128 sequences, 1 to 32 heads, chunks of 1 to 64 tokens).
+constexpr bool has_shape(bool chunked, int cluster, int threads) {
+  return threads == 1024 || cluster == 1 || (chunked && cluster >= 4);
+}
+template <bool FUSED, bool CHUNKED, bool CAPPED, int CLUSTER>
+cudaError_t launch_width(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, int threads, size_t smem) {
+  if (threads == 1024) return launch_one<FUSED, CHUNKED, CAPPED, 1024, CLUSTER>(L, bt, g, P, smem);
+  if constexpr (has_shape(CHUNKED, CLUSTER, 512)) return launch_one<FUSED, CHUNKED, CAPPED, 512, CLUSTER>(L, bt, g, P, smem);
+  return cudaErrorInvalidConfiguration;
+}
 template <bool FUSED, bool CHUNKED, bool CAPPED>
 cudaError_t launch_shape(const Launch& L, const BatchTable& bt, const Geometry& g, const ClusterParams& P, SelectShape sh,
                          size_t smem) {
-  const bool wide = sh.threads == 1024;
   switch (sh.cluster) {
-    case 1: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 1>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 1>(L, bt, g, P, smem);
-    case 2: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 2>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 2>(L, bt, g, P, smem);
-    case 4: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 4>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 4>(L, bt, g, P, smem);
-    default: return wide ? launch_one<FUSED, CHUNKED, CAPPED, 1024, 8>(L, bt, g, P, smem) : launch_one<FUSED, CHUNKED, CAPPED, 512, 8>(L, bt, g, P, smem);
+    case 1: return launch_width<FUSED, CHUNKED, CAPPED, 1>(L, bt, g, P, sh.threads, smem);
+    case 2: return launch_width<FUSED, CHUNKED, CAPPED, 2>(L, bt, g, P, sh.threads, smem);
+    case 4: return launch_width<FUSED, CHUNKED, CAPPED, 4>(L, bt, g, P, sh.threads, smem);
+    default: return launch_width<FUSED, CHUNKED, CAPPED, 8>(L, bt, g, P, sh.threads, smem);
   }
 }
 
@@ -863,7 +874,7 @@ double launch_cost(const BatchTable& bt, int hkv, const SelectRoom& room, bool s
 // 284, 264 in pairs.)
 cudaError_t query_select_room(SelectRoom* room) {
   auto one = select_cluster_kernel<true, false, true, 1024, 8>;
-  auto two = select_cluster_kernel<true, false, true, 512, 8>;
+  auto two = select_cluster_kernel<true, true, true, 512, 8>;
   cudaError_t e = allow_smem(one);
   if (e == cudaSuccess) e = allow_smem(two);
   for (int lc = 0; lc <= 3 && e == cudaSuccess; ++lc) {
@@ -895,7 +906,7 @@ SelectShape select_shape(const BatchTable& bt, int hkv, const SelectRoom& room, 
   double best_us = 1e30;
   for (int lc = 0; lc <= 3; ++lc)
     for (int threads = 512; threads <= 1024; threads += 512) {
-      if (room.one[lc] <= 0 || room.two[lc] <= 0) continue;
+      if (!has_shape(bt.chunk > 1, 1 << lc, threads) || room.one[lc] <= 0 || room.two[lc] <= 0) continue;
       if (steps_per_warp(bt.max_items, 1 << lc, threads) > 32) continue;   // a warp's run has at most 32 steps
       const double us = launch_cost(bt, hkv, room, fused_input && bt.chunk == 1, lc, threads);
       if (us < best_us) { best_us = us; best = SelectShape{1 << lc, threads}; }
@@ -948,4 +959,7 @@ extern "C" void ccx_select_shape(int max_items, int num_seqs, int hkv, int chunk
   const cc::SelectShape sh = cc::select_shape(bt, hkv, room, fused_input != 0);
   *cluster = sh.cluster;
   *threads = sh.threads;
+}
+extern "C" int ccx_select_has_shape(int chunk, int cluster, int threads) {
+  return cc::has_shape(chunk > 1, cluster, threads);
 }

@@ -51,6 +51,20 @@ def test_shape_of_the_selection_follows_the_device(seqs, hkv, chunk):
     assert _shape(262145, seqs, hkv, chunk)[0] == 0 and _shape(0, seqs, hkv, chunk) == (1, 512)
 
 
+@pytest.mark.parametrize("chunk", [1, 4, 33])
+def test_every_shape_of_the_selection_is_one_that_is_chosen(chunk):
+    """Each shape that is compiled is the cheapest for some batch on this device, and whatever the device no other is chosen."""
+    has = binding.load_library().ccx_select_has_shape
+    compiled = {(c, t) for c in (1, 2, 4, 8) for t in (512, 1024) if has(chunk, c, t)}
+    sizes = sorted({int(1.07 ** i) for i in range(186)} | {16385, 65537})
+    problems = [(1, 1), (1, 8), (2, 8), (5, 4), (8, 8), (19, 8), (32, 8), (64, 32)]
+    chosen = {_shape(items, s, h, chunk) for items in sizes for s, h in problems}
+    assert chosen - {(0, 0)} == compiled
+    for room in (((148, 148, 0, 0), (296, 296, 0, 0)), ((20, 20, 16, 8), (40, 40, 32, 16)), ((132, 132, 132, 132), (264,) * 4),
+                 ((16, 64, 128, 144), (16, 64, 200, 280))):
+        assert {_shape(items, s, h, chunk, 1, room) for items in sizes for s, h in problems} - {(0, 0)} <= compiled
+
+
 def test_a_wave_of_wide_clusters_is_as_wide_as_the_device():
     """Fourteen problems of 65536 items: 112 CTAs in clusters of eight are one wave where 120 run at a time and
     two where 96 do, and then narrower clusters are cheaper."""
