@@ -70,6 +70,21 @@ __device__ __forceinline__ uint64_t ex2_pair_sfu(uint64_t x) {
   unpack2(x, a, b);
   return pack2(ex2(a), ex2(b));
 }
+__device__ __forceinline__ uint64_t ex2_cubic(uint64_t f) {
+  uint64_t p = fma2(f, pack2(kEx2C3, kEx2C3), pack2(kEx2C2, kEx2C2));
+  p = fma2(p, f, pack2(kEx2C1, kEx2C1));
+  return fma2(p, f, pack2(kEx2C0, kEx2C0));
+}
+// p * 2^n: n (low mantissa bits of t) shifted into the exponent field by one multiply-add
+__device__ __forceinline__ uint64_t ex2_insert(uint64_t p, uint64_t t) {
+  float p0, p1, t0, t1;
+  unpack2(p, p0, p1);
+  unpack2(t, t0, t1);
+  int r0, r1;
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
+  return pack2(__int_as_float(r0), __int_as_float(r1));
+}
 // 2^x for a pair on the FMA pipe (packed form of ex2_poly, same clamp)
 __device__ __forceinline__ uint64_t ex2_pair_fma(uint64_t x) {
   float a, b;
@@ -77,46 +92,49 @@ __device__ __forceinline__ uint64_t ex2_pair_fma(uint64_t x) {
   x = pack2(fmaxf(a, -125.0f), fmaxf(b, -125.0f));
   const uint64_t magic = pack2(kEx2Magic, kEx2Magic);
   const uint64_t t = add2(x, magic);
-  const uint64_t f = sub2(x, sub2(t, magic));
-  uint64_t p = fma2(f, pack2(kEx2C3, kEx2C3), pack2(kEx2C2, kEx2C2));
-  p = fma2(p, f, pack2(kEx2C1, kEx2C1));
-  p = fma2(p, f, pack2(kEx2C0, kEx2C0));
-  float p0, p1, t0, t1;
-  unpack2(p, p0, p1);
-  unpack2(t, t0, t1);
-  // p * 2^n: n (low mantissa bits of t) shifted into the exponent field by one multiply-add
-  int r0, r1;
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(r1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
-  return pack2(__int_as_float(r0), __int_as_float(r1));
+  return ex2_insert(ex2_cubic(sub2(x, sub2(t, magic))), t);
 }
 
 constexpr float kScale = 0.12751743f;            // log2(e) / sqrt(128)
-// 2^(v * kScale - m) for a pair on the FMA pipe, m an integer of at most kMaxRef in size.  Then kEx2Magic - m is exact, and
-// the product takes part unrounded in both steps: n is the integer nearest to the exact argument, and the remainder, at most one
-// half, is rounded once, to 2^-25.  (An argument rounded at its own size is good to 2^-20 between -16 and -32.  Its place on a scale of
-// 248 powers of two, from a saturating multiply-add that clamps on both sides, is good to 2^-18 only and has a bias per reference.
-// Score stages are 0.3 to 0.6 % faster with that, and 1 % slower with arguments rounded at their own size.  Against 64 bits, geometric
-// means over 17 shapes x 4 inputs: log-sums 1.45e-6 with arguments of their own size, 1.47e-6 with the scale, 1.14e-6 now;
-// scores 3.70e-6, 3.71e-6, 3.66e-6 in norm.)
-// The clamp below, at -124, is on the value; the caller sees to it that arguments stay under 127.
-constexpr float kMaxRef = 1048576.0f;
-struct PolyRef { float bias, low; };
-__device__ __forceinline__ PolyRef poly_ref(float m) { return PolyRef{kEx2Magic - m, (m - 124.0f) * (1.0f / kScale)}; }
-__device__ __forceinline__ uint64_t ex2_pair_scaled(float v0, float v1, const PolyRef& r) {
-  const uint64_t v = pack2(fmaxf(v0, r.low), fmaxf(v1, r.low)), c2 = pack2(kScale, kScale), bias = pack2(r.bias, r.bias);
-  const uint64_t t = fma2(v, c2, bias);             // magic + n
-  const uint64_t f = fma2(v, c2, sub2(bias, t));    // v * kScale - m - n
-  uint64_t p = fma2(f, pack2(kEx2C3, kEx2C3), pack2(kEx2C2, kEx2C2));
-  p = fma2(p, f, pack2(kEx2C1, kEx2C1));
-  p = fma2(p, f, pack2(kEx2C0, kEx2C0));
-  float p0, p1, t0, t1;
-  unpack2(p, p0, p1);
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+  float d;
+  asm("fma.rn.ftz.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+// Two forms of 2^x for a pair on the FMA pipe, x given by the product v, for the two passes of the score kernel.  An argument
+// rounded at its own size is good to 2^-20 between -16 and -32; its place on one scale of 248 powers of two, from a saturating
+// multiply-add that clamps on both sides, is good to 2^-18 only and has a bias per reference, which is why neither form computes with one.
+// Against 64 bits, geometric means over 17 shapes x 4 inputs: log-sums of rows 1.45e-6 with arguments of their own size, 1.47e-6
+// from that scale, 1.14e-6 now; scores 3.70e-6, 3.71e-6, 3.66e-6 in norm.  The calls take 0 to 0.4 % more than with that scale, 1 % at the
+// power limit; with arguments of their own size in pass 1 1.5 %, with the clamps as minima and maxima 0.7 %.
+//
+// Pass 1: acc + 2^(v * kScale - m), m an integer of at most kMaxRef in size.  n comes from the place of the argument on a scale that
+// ends at -127 and 124 (the rounding there, 2^-10 at most and 2^-16 for references below 64, moves the border between one n and the next and nothing else).  The remainder takes the
+// unrounded product and is rounded once, to 2^-25, since kEx2Magic - m is exact.  2^n is a factor of its own, 0 for n = -127:
+// whatever the cubic makes of a remainder outside [-1/2, 1/2], where the scale has saturated, counts nothing below and is 2^124
+// or more above.  (Only where the cubic overflows, below -2^43, the product with 0 is no number; the caller looks for that.)
+constexpr float kMaxRef = 4096.0f;
+constexpr float kPlaceLow = 127.0f, kPlaceSpan = 251.0f;
+struct PolyRef { float bias, place; };
+__device__ __forceinline__ PolyRef poly_ref(float m) { return PolyRef{kEx2Magic - m, (kPlaceLow - m) * (1.0f / kPlaceSpan)}; }
+__device__ __forceinline__ uint64_t ex2_pair_scaled(float v0, float v1, const PolyRef& r, uint64_t acc) {
+  const uint64_t y = pack2(fma_sat(v0, kScale / kPlaceSpan, r.place), fma_sat(v1, kScale / kPlaceSpan, r.place));
+  const uint64_t t = fma2(y, pack2(kPlaceSpan, kPlaceSpan), pack2(kEx2Magic - kPlaceLow, kEx2Magic - kPlaceLow));    // magic + n
+  const uint64_t p = ex2_cubic(fma2(pack2(v0, v1), pack2(kScale, kScale), sub2(pack2(r.bias, r.bias), t)));
+  float t0, t1;
   unpack2(t, t0, t1);
-  int e0, e1;
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(e0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(e1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
-  return pack2(__int_as_float(e0), __int_as_float(e1));
+  int s0, s1;                                      // n in the exponent field, 127 + n
+  asm("mad.lo.s32 %0, %1, 8388608, 1065353216;" : "=r"(s0) : "r"(__float_as_int(t0)));
+  asm("mad.lo.s32 %0, %1, 8388608, 1065353216;" : "=r"(s1) : "r"(__float_as_int(t1)));
+  return fma2(p, pack2(__int_as_float(s0), __int_as_float(s1)), acc);
+}
+// Pass 2: 2^(v * kScale) for arguments of at most 0 (taken as 0 above).  The scale ends at -124 and 0 and is counted from its upper end,
+// so the place is the argument rounded at its own size (kScale / kDepth is exact in f32).
+constexpr float kDepth = 124.0f;
+__device__ __forceinline__ uint64_t ex2_pair_below(float v0, float v1) {
+  const uint64_t y = pack2(fma_sat(v0, -kScale / kDepth, 0.0f), fma_sat(v1, -kScale / kDepth, 0.0f)), span = pack2(-kDepth, -kDepth);
+  const uint64_t magic = pack2(kEx2Magic, kEx2Magic), t = fma2(y, span, magic);
+  return ex2_insert(ex2_cubic(fma2(y, span, sub2(magic, t))), t);
 }
 
 // Of every three pairs one takes the polynomial path, and the two paths have a sum each: the special-function unit is the
@@ -155,25 +173,35 @@ __device__ __forceinline__ void exp_accumulate_any(const uint32_t (&v)[32], floa
     else acc[0] = add2(acc[0], ex2_pair_sfu(x));
   }
 }
-// acc += 2^(v * kScale - m) over the first kWidth of 32 values, m an integer of at most kMaxRef in size (kRef false: 0),
-// r = poly_ref(m).
-template <bool kRef, int kWidth>
+// acc += 2^(v * kScale - m) over 32 values, m an integer of at most kMaxRef in size, r = poly_ref(m).
 __device__ __forceinline__ void exp_accumulate(const uint32_t (&v)[32], float m, const PolyRef& r, uint64_t (&acc)[2]) {
   const uint64_t c2 = pack2(kScale, kScale), off2 = pack2(-m, -m);
 #pragma unroll
-  for (int pair = 0; pair < kWidth / 2; ++pair) {
+  for (int pair = 0; pair < 16; ++pair) {
     const float a = __uint_as_float(v[2 * pair]), b = __uint_as_float(v[2 * pair + 1]);
-    if (poly_pair(pair)) acc[1] = add2(acc[1], ex2_pair_scaled(a, b, r));
-    else acc[0] = add2(acc[0], ex2_pair_sfu(kRef ? fma2(pack2(a, b), c2, off2) : mul2(pack2(a, b), c2)));
+    if (poly_pair(pair)) acc[1] = ex2_pair_scaled(a, b, r, acc[1]);
+    else acc[0] = add2(acc[0], ex2_pair_sfu(fma2(pack2(a, b), c2, off2)));
   }
 }
-// The largest of limit and the values that take the polynomial path.
-__device__ __forceinline__ float poly_max(const uint32_t (&v)[32], float limit) {
+// acc += 2^(v * kScale) over the first kWidth of 32 values, arguments of at most 0.
+template <int kWidth>
+__device__ __forceinline__ void exp_accumulate_below(const uint32_t (&v)[32], uint64_t (&acc)[2]) {
+  const uint64_t c2 = pack2(kScale, kScale);
+#pragma unroll
+  for (int pair = 0; pair < kWidth / 2; ++pair) {
+    const float a = __uint_as_float(v[2 * pair]), b = __uint_as_float(v[2 * pair + 1]);
+    if (poly_pair(pair)) acc[1] = add2(acc[1], ex2_pair_below(a, b));
+    else acc[0] = add2(acc[0], ex2_pair_sfu(mul2(pack2(a, b), c2)));
+  }
+}
+// The largest size of the values that take the polynomial path.
+__device__ __forceinline__ float poly_reach(const uint32_t (&v)[32]) {
+  float reach = 0.0f;
 #pragma unroll
   for (int pair = 0; pair < 16; ++pair)
     if (poly_pair(pair))
-      asm("max.f32 %0, %0, %1, %2;" : "+f"(limit) : "f"(__uint_as_float(v[2 * pair])), "f"(__uint_as_float(v[2 * pair + 1])));
-  return limit;
+      asm("max.f32 %0, %0, %1, %2;" : "+f"(reach) : "f"(fabsf(__uint_as_float(v[2 * pair]))), "f"(fabsf(__uint_as_float(v[2 * pair + 1]))));
+  return reach;
 }
 __device__ __forceinline__ float acc_total(const uint64_t (&acc)[2]) {
   float a, b;

@@ -63,7 +63,7 @@ exp_probe_kernel(long long* out, int iters, float m) {
     } else {
       m = m == 7.0f ? 0.0f : m + 1.0f;     // new arguments every round
     }
-    exp_accumulate<true, 32>(v, m, poly_ref(m), acc);
+    exp_accumulate(v, m, poly_ref(m), acc);
   }
   const long long t1 = clock64();
   const float total = acc_total(acc);

@@ -304,15 +304,16 @@ __device__ __forceinline__ void hand_back(uint32_t empty_bar, int lane) {
 
 // pass 1, all 128 keys count.  The reference of the exponentials only has to be near the row
 // maximum, not equal to it: it is replaced when a value lies more than 2^64 above it.  It is an integer, for the sake of
-// the polynomial's arguments.  Only the first
-// chunk of a row and the last of an item look at their maximum beforehand, a serial stretch of 16 instructions, a
-// vote and a branch before the first exponential.  Of the chunks in between, sums and the largest polynomial argument (which
-// would wrap silently above 128) are looked at before the buffer goes back, and when they are too large, or the reference
-// is, nothing has been changed and the answer is false: the caller goes through the item again, chunk by chunk.
+// the polynomial's arguments.  Only the first chunk of a row and the last of an item look at their maximum beforehand, a serial stretch
+// of 16 instructions, a vote and a branch before the first exponential.  The sums of the others, which grow beyond 2^70 or are no numbers
+// where a value is out of the arithmetic's range, and the ranges of the reference and of the last chunk are looked at before the
+// buffer goes back; when one is not as it should be, nothing has been changed and the answer is false: the caller goes through
+// the item again, chunk by chunk.
 constexpr float kRedo = 1.1805916e21f;     // 2^70
+constexpr float kMaxProduct = 1.0995116e12f;     // 2^40
 __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, int lane, float& m_run, float& l_run) {
   uint64_t acc[2] = {0ull, 0ull};
-  float m = m_run, l = l_run, top = -INFINITY;
+  float m = m_run, l = l_run;
   PolyRef r = poly_ref(m);
   bool look = __any_sync(0xffffffffu, m == -INFINITY);
 #pragma unroll 1
@@ -323,7 +324,7 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
     if (look) {
       const float mx = max32(v) * kScale;
       if (cc0 + 32 == kTileKeys) {
-        const bool fine = acc_total(acc) < kRedo && fmaf(top, kScale, -m) < 100.0f && fmaxf(fabsf(m), mx) < kMaxRef;
+        const bool fine = acc_total(acc) < kRedo && fmaxf(fabsf(m), mx) < kMaxRef && poly_reach(v) < kMaxProduct;
         if (!__all_sync(0xffffffffu, fine)) return false;
         hand_back(empty_bar, lane);
       }
@@ -335,11 +336,9 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
         r = poly_ref(m);
       }
       __syncwarp();
-    } else {
-      top = poly_max(v, top);
     }
     look = cc0 + 64 == kTileKeys;
-    exp_accumulate<true, 32>(v, m, r, acc);
+    exp_accumulate(v, m, r, acc);
   }
   m_run = m;
   l_run = l + acc_total(acc);
@@ -392,7 +391,7 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
     tmem_ld32(addr + (uint32_t)cc0, v);               // stays inside the 128-column buffer
     tmem_wait_ld();
     if (cc0 + 32 == nc) hand_back(empty_bar, lane);
-    if (ADDED) exp_accumulate<false, 32>(v, 0.0f, poly_ref(0.0f), acc);
+    if (ADDED) exp_accumulate_below<32>(v, acc);
     else exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
   }
   if (nc & 16) {
@@ -400,7 +399,7 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
     tmem_ld32(addr + (uint32_t)(nc - 16), v);
     tmem_wait_ld();
     hand_back(empty_bar, lane);
-    if (ADDED) exp_accumulate<false, 16>(v, 0.0f, poly_ref(0.0f), acc);
+    if (ADDED) exp_accumulate_below<16>(v, acc);
     else exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)(nc - 16), acc);
   }
   return acc_total(acc);
