@@ -231,12 +231,22 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t m, uint32_t n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
+// Operands of the step of 16 channels that adds -L_r: ones from the keys' side; the rows' side is 16 bytes a row, the second 8
+// channels of a group of rows lie on the next group's first and meet zeros.
+__device__ __forceinline__ uint64_t ones_desc(const void* ones) {
+  return (uint64_t)(((smem_u32(ones) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(16u | (1u << 14)) << 32);
+}
+__device__ __forceinline__ uint64_t stat_desc(const void* rows) {
+  return (uint64_t)(((smem_u32(rows) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(8u | (1u << 14)) << 32);
+}
+
 // ------------------------------------------------------------------ shared state
 struct Barriers {
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
   uint64_t q_full, q_empty, l_full;
   uint64_t acc_full[kBufs], acc_empty[kBufs];
+  uint64_t late_full[kBufs];         // ADDED: -L_r has been added to the first item of the set in the (sequence, head)
   uint64_t u_full[8][4];             // pass 2: the other sets' partial sums of (slot, quadrant)
   uint64_t edge_full[2][4];          // ... of a first / last tile of which the CTA has one half
 };
@@ -249,10 +259,7 @@ struct Misc {                        // behind the ring of K tiles in dynamic sh
       uint4 ones[2 * kTileKeys];     // pass 2: the other side of the operand with -L_r: 128 keys x 16 channels, (1, 1, 1, 0, ...)
     };
   };
-  union {
-    float edge_part[2][kTileKeys];   // pass 2: partial column sums of cut tiles
-    float zeros[kTileKeys];          // pass 2, products with -L_r (no tile is cut then): offsets of none
-  };
+  float edge_part[2][kTileKeys];     // pass 2: partial column sums of cut tiles
   Barriers bar;
   long long span[2];                 // first unit of the CTA, first unit behind it
   uint32_t tmem_base;
@@ -407,6 +414,7 @@ __device__ __forceinline__ float drain_rows(uint32_t addr, uint32_t empty_bar, i
 
 // pass 2, columns before first_col (a bound of the thread's own) do not count, and nothing does for a thread without a key
 // (returns the sum).  Skips and masks as above.
+template <bool ADDED>
 __device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty_bar, int lane, uint32_t nl, int nc, int first_col,
                                                    bool key) {
   uint64_t acc[2] = {0ull, 0ull};
@@ -423,8 +431,13 @@ __device__ __forceinline__ float drain_rows_masked(uint32_t addr, uint32_t empty
       for (int i = 0; i < 32; ++i)
         if (cc0 + i < first_col) v[i] = kMasked;
     }
-    if (cc0 + 32 <= nc) exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
-    else                exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)cc0, acc);
+    if (ADDED) {
+      if (cc0 + 32 <= nc) exp_accumulate_below<32>(v, acc);
+      else                exp_accumulate_below<16>(v, acc);
+    } else {
+      if (cc0 + 32 <= nc) exp_accumulate_columns<32>(v, nl + 4u * (uint32_t)cc0, acc);
+      else                exp_accumulate_columns<16>(v, nl + 4u * (uint32_t)cc0, acc);
+    }
   }
   return acc_total(acc);
 }
@@ -521,9 +534,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
   uint8_t* q_smem = smem;
   uint8_t* k_smem = smem + q_bytes;
   Misc* misc = reinterpret_cast<Misc*>(k_smem + (size_t)P.n_stages * kStageBytes);
-  // pass 2: -L_r in the log2 domain (-1e4 for padded rows), before it (ADDED) as an operand (rows_pad + 8 rows)
+  // pass 2: -L_r, as an operand (ADDED; rows_pad + 8 rows) or in the log2 domain (-1e4 for padded rows)
   uint4* l_smem = reinterpret_cast<uint4*>(misc + 1);
-  float* neg_lc = reinterpret_cast<float*>(ADDED ? l_smem + P.rows_pad + 8 : l_smem);
+  float* neg_lc = reinterpret_cast<float*>(misc + 1);
   Pipe pipe{misc, status};
 
   // the warp index as a value the compiler knows to be the same in all lanes: the MMA issuer's
@@ -542,6 +555,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     if (lane < kBufs) {
       mbar_init(smem_u32(&misc->bar.acc_full[lane]), 1);
       mbar_init(smem_u32(&misc->bar.acc_empty[lane]), 4);       // the four warps of a set
+      mbar_init(smem_u32(&misc->bar.late_full[lane]), 1);
     }
     // one arrival per set that hands its partial sums over
     mbar_init(smem_u32(&misc->bar.u_full[lane >> 2][lane & 3]), P.n_sub > 1 ? P.n_sub - 1 : 1);
@@ -564,7 +578,6 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int i = threadIdx.x - 128;       // 8-row groups of 256 bytes: channels 0-7 of the rows, channels 8-15
     misc->ones[i] = (i & 8) ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
     if (i < 8) l_smem[P.rows_pad + i] = make_uint4(0u, 0u, 0u, 0u);
-    if (CAUSAL && i < kTileKeys) misc->zeros[i] = 0.0f;
     fence_proxy_async();
   }
   if (PASS == 2) pdl_launch_dependents();
@@ -697,11 +710,9 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
                     : instr_desc(128, (uint32_t)(P.rows_pad - (P.n_sub - 1) * P.sub_cols));
       const uint32_t empty0 = smem_u32(&misc->bar.empty[0]);
       const uint32_t accf0 = smem_u32(&misc->bar.acc_full[0]);
-      // pass 2: one more step of 16 channels adds -L_r (ones from the keys' side; the rows' side is 16 bytes a row,
-      // the second 8 channels of a group of rows lie on the next group's first and meet zeros)
-      const uint64_t ones_desc = (uint64_t)(((smem_u32(misc->ones) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(16u | (1u << 14)) << 32);
-      const uint64_t l_desc = (uint64_t)(((smem_u32(l_smem) & 0x3FFFFu) >> 4) | (8u << 16)) | ((uint64_t)(8u | (1u << 14)) << 32);
-      // only the first two of its items of a (sequence, head), the first of each set, does an issuer multiply without it: L_r may not be known yet
+      // pass 2: one more step adds -L_r, but for the first two of an issuer's items of a (sequence, head), the first of each set:
+      // L_r may not be known yet, and the set takes that step itself
+      const uint64_t ones = ones_desc(misc->ones), stat = stat_desc(l_smem);
       uint32_t l_phase = 0, n_own = 0;
       bool l_known = false;
       const bool elected = elect_one();
@@ -744,7 +755,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
               umma(d_tmem, al | ((uint64_t)a_hi << 32), bl | ((uint64_t)b_hi << 32), idesc, ks > 0);
             }
             if (ADDED && l_known)
-              umma(d_tmem, ones_desc, l_desc + (uint64_t)((uint32_t)sub * (uint32_t)P.sub_cols), idesc, true);
+              umma(d_tmem, ones, stat + (uint64_t)((uint32_t)sub * (uint32_t)P.sub_cols), idesc, true);
             umma_commit(accf0 + 8u * buf);
           }
         }
@@ -865,9 +876,10 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         }
         const float lc = m + log2f(l);
         const bool real = row < P.rows;          // row = t * G + g
-        neg_lc[row] = real ? -lc : -1.0e4f;
-        if (ADDED) {
-          // the same in units of the products, as three bf16 that add up to it (padded rows: far below everything)
+        if (!ADDED) {
+          neg_lc[row] = real ? -lc : -1.0e4f;
+        } else {
+          // in units of the products, as three bf16 that add up to it (padded rows: far below everything)
           const float nl = real ? -lc * (1.0f / kScale) : -8.0e4f;
           const float rest = real ? fmaf(nl, kScale, lc) * (-1.0f / kScale) : 0.0f;       // rounding of the division
           const __nv_bfloat16 x0 = __float2bfloat16_rn(nl), x1 = __float2bfloat16_rn(nl - __bfloat162float(x0));
@@ -899,7 +911,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int t_slot = t_begin + (sub_begin > 0 ? 1 : 0);
     const int idle_from = (max(P.rows_pad - quad * 32, 0) + 127) / 128;   // row blocks from here on have no row of this warp
     uint32_t par = 0;
-    bool first_item = true;     // pass 2: of the set in the (sequence, head); these are multiplied without -L_r
+    bool first_item = true;     // ADDED: of the set in the (sequence, head); these come without -L_r
+    uint32_t late_par = 0;
     int prob_end = t_begin, first_tile = 0, n_cur = 0;
     float* out = nullptr;
     const uint32_t full_bar = smem_u32(&misc->bar.acc_full[set]);
@@ -955,6 +968,24 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         dead = !warp_wait(pipe, &misc->bar.acc_full[set], par, 30);
       }
       par ^= 1u;
+      if (ADDED && first_item) {
+        // The step that the issuer could not take, so that all items are rounded alike and equal keys have equal scores.  (With the
+        // offset added to the product when it is read, keys of these items differed from their equals in the last places;
+        // the calls take 0 to 0.4 % more, 32768 tokens x 8 heads 55.8 -> 56.0 us.)
+        if (!dead) {
+          tc_fence_after();
+          if ((ew & 3) == 0 && elect_one()) {
+            const int c0 = sub * P.sub_cols;
+            umma(tmem_base + (uint32_t)set * kBufCols, ones_desc(misc->ones), stat_desc(l_smem) + (uint64_t)(uint32_t)c0,
+                 instr_desc(128, (uint32_t)min(P.sub_cols, P.rows_pad - c0)), true);
+            umma_commit(smem_u32(&misc->bar.late_full[set]));
+          }
+          __syncwarp();
+          dead = !warp_wait(pipe, &misc->bar.late_full[set], late_par, 35);
+        }
+        late_par ^= 1u;
+        first_item = false;
+      }
       float u_acc = 0.f;
       if (!dead) {
         tc_fence_after();
@@ -995,13 +1026,10 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
           // causal window: key j is seen by the rows t >= j - (n - w), i.e. by the columns from
           // G * (j - n + w) on; the columns before it contribute nothing
           if (edge)
-            u_acc = drain_rows_masked(acc_addr, empty_bar, lane, smem_u32(!ADDED || first_item ? neg_lc + c0 : misc->zeros), nc,
-                                      g.group * (key0 + row_in_tile - n_cur + g.window) - c0, row_in_tile < valid);
-          else if (!ADDED || first_item)
-            u_acc = drain_rows<false>(acc_addr, empty_bar, lane, smem_u32(neg_lc + c0), nc);
+            u_acc = drain_rows_masked<ADDED>(acc_addr, empty_bar, lane, smem_u32(neg_lc + c0), nc,
+                                             g.group * (key0 + row_in_tile - n_cur + g.window) - c0, row_in_tile < valid);
           else
-            u_acc = drain_rows<true>(acc_addr, empty_bar, lane, 0u, nc);
-          first_item = false;
+            u_acc = drain_rows<ADDED>(acc_addr, empty_bar, lane, smem_u32(neg_lc + c0), nc);
         }
       }
       if (PASS == 2) {
@@ -1068,7 +1096,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Items of a CTA from which on pass 2 lets the products add -L_r (ADDED).  The first item of each set cannot have it, and the
+// Items of a CTA from which on pass 2 lets the products add -L_r (ADDED).  The first item of each set gets it late, and the
 // operand has to be prepared: 20480 tokens x 8 heads of 256 rows (17 items) -0.8 %, 65536 x 4 of 448 -1.3 %, 131072 x 8 -2.0 %,
 // 32 x 2200 x 8 of 512 -2.0 %; level at 7 to 14 items, +0.9 % on 131072 x 2 of 128 rows (14 items) and 12 x 300 x 8 of 512.
 // Spans with cut tiles have few items.
@@ -1087,7 +1115,7 @@ Ring ring_of(int rows_pad, size_t l_bytes) {
   return Ring{n, fixed + (size_t)n * kStageBytes};
 }
 Ring ring_pass1(int rows_pad) { return ring_of(rows_pad, 0); }
-Ring ring_pass2(int rows_pad, bool added) { return ring_of(rows_pad, (size_t)rows_pad * 4 + (added ? (size_t)(rows_pad + 8) * 16 : 0)); }
+Ring ring_pass2(int rows_pad, bool added) { return ring_of(rows_pad, added ? (size_t)(rows_pad + 8) * 16 : (size_t)rows_pad * 4); }
 // Whether pass 2 lets the products add -L_r (ADDED): with items enough (kAddedItems), and not where the operand costs the ring a tile
 // (64, 304, 432 rows): 131072 tokens x 8 heads of 64 rows 86.6 with it and 84.9 us without, 65536 x 8 of 304 rows 102.6 and 102.0,
 // of 432 130.3 and 129.7.

@@ -2,6 +2,7 @@
 at before the first and the last 32 keys of a tile only, and a tile whose other keys overflow it is gone through again."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import codecomp_oracle as orc
 from paper_2604_10235_b200 import binding as cc
@@ -29,5 +30,34 @@ def test_scores_of_rows_that_rise(w, hq, hkv, at, jump):
     k = orc.bf16_bits_to_f64(x.k).astype(np.float32)
     k[:, :, 0] = 0.0
     k[at, :, 0] = jump * np.sqrt(128.0) / 4.0
+    x.k = gen.f32_to_bf16_bits(k)
+    check_against_oracle(wl, x, cc.CC_MODE_BF16, TOL)
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("w", [16, 64, 96, 128])
+def test_rises_in_later_tiles_of_a_span(w, causal):
+    """Seventeen tiles per CTA, one to four row blocks.  Every 23 tiles, so mostly well inside a span: heads 0 to 3 have four
+    tiles of keys 57 powers of two up, which the reference stays below, and in the next one, which the set that had the first of
+    them goes through again, a key 72 up, in the chunk of the head's number; 3 % of a row is left to the keys of before, whose
+    sum has to come through that.  Heads 4 to 7 rise by 72 and, in the set's next tile of that row block, by 80 more."""
+    n, hkv, every = 40000, 8, 23
+    tiles = -(-n // 128)
+    assert tiles * hkv > 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    wl = gen.Workload("later", 37, 1, 32, hkv, 128, w, gen.POOL_MAX, 7, 1, n=n, causal=causal)
+    x = gen.make_layer(wl, layer=w, with_v=False)
+    q = orc.bf16_bits_to_f64(x.q_win).astype(np.float32)
+    q[..., 0] = 4.0
+    x.q_win = gen.f32_to_bf16_bits(q)
+    k = orc.bf16_bits_to_f64(x.k).astype(np.float32) * 0.25
+    k[:, :, 0] = 0.0
+    up = np.log(2.0) * np.sqrt(128.0) / 4.0      # one power of two, in channel 0 of a key
+    for tile in range(2, tiles - 8, every):
+        for h in range(4):
+            k[tile * 128:(tile + 4) * 128, h, 0] = 57.0 * up
+            k[(tile + 4) * 128 + 32 * h + 11, h, 0] = 72.0 * up
+        for h in range(4, 8):
+            k[tile * 128 + 32 * (h - 4) + 11, h, 0] = 72.0 * up
+            k[(tile + 4) * 128 + 32 * ((h - 3) % 4) + 11, h, 0] = 152.0 * up
     x.k = gen.f32_to_bf16_bits(k)
     check_against_oracle(wl, x, cc.CC_MODE_BF16, TOL)

@@ -1,12 +1,14 @@
 """Score parity where the tensor-core kernel cuts tiles at their middle between two CTAs (few tiles
 per SM: fewer than half a tile each, a last or first half, several problems in a span), contiguous,
 paged and causal, and where a span holds many short problems."""
+import numpy as np
 import pytest
 
+from oracle import codecomp_oracle as orc
 from paper_2604_10235_b200 import binding as cc
 from paper_2604_10235_b200 import inputs as gen
 
-from test_gpu_score import check_against_oracle
+from test_gpu_score import check_against_oracle, run_scores
 
 pytestmark = pytest.mark.gpu
 
@@ -39,6 +41,27 @@ def test_scores_whose_row_sums_the_product_subtracts(w, hq, hkv, lens, page, cau
     wl = gen.Workload("added", 30, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1, page_size=page,
                       causal=causal)
     check_against_oracle(wl, gen.make_layer(wl, layer=w, with_v=False), cc.CC_MODE_BF16, 2e-4)
+
+
+@pytest.mark.parametrize("w,hq,hkv", [(16, 8, 8), (12, 32, 8), (50, 32, 8), (96, 32, 8), (128, 32, 8)])
+@pytest.mark.parametrize("lens,page,causal", [((41000,), 0, False), ((5000, 130, 77, 300, 9000, 1, 700, 26000), 16, False),
+                                              ((40000, 300), 0, True)])
+def test_equal_keys_have_equal_scores(w, hq, hkv, lens, page, causal):
+    """The tie rule (equal values: the lower index first) decides among equal keys, so nothing else may: wherever a key lies in its
+    tile, in the span of its CTA and in the sequence, its score is the same bit for bit, as long as the same rows attend to it."""
+    wl = gen.Workload("equal", 36, 1, hq, hkv, 128, w, gen.POOL_MAX, 7, 0, seq_lens=lens, budget_frac=0.1, page_size=page,
+                      causal=causal)
+    x = gen.make_layer(wl, layer=w, with_v=False)
+    period = 61                                  # a prime: every key falls on every place of a tile
+    for s, n in enumerate(lens):
+        rows = orc.paged_rows(x.page_table[s], n, page) if page else np.arange(x.tok_offsets[s], x.tok_offsets[s] + n)
+        x.k[rows] = x.k[rows[:period]][np.arange(n) % period]
+    u, _ = run_scores(wl, x, cc.CC_MODE_BF16, want_lse=False)
+    for s, n in enumerate(lens):
+        lo = int(x.tok_offsets[s])
+        seen = n - w + 1 if causal else n        # keys that all rows attend to
+        own = u[:, lo:lo + seen]
+        np.testing.assert_array_equal(own, own[:, np.arange(seen) % period])
 
 
 @pytest.mark.parametrize("w,hq,hkv", [(16, 1, 1), (24, 1, 1), (128, 1, 1), (64, 7, 1), (128, 4, 1)])
