@@ -355,10 +355,10 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
 // Stands for a product that does not count: minus infinity, since a row's own logits may lie anywhere.
 constexpr uint32_t kMasked = 0xff800000u;
 
-// pass 1, keys from valid_r on (a bound of the thread's own) do not count
-// (returns the row's new reference and sum); logits of any size.  Chunks that no row of the warp attends to are skipped, and in those that all do
-// nothing is masked: with a causal window most are one or the other, and the CTA with the last tiles of a sequence is what a
-// short call waits for (10007 tokens x 4 heads: 7 us of work there, 4.5 to 5.5 elsewhere; score stage 24.1 -> 22.8 us).
+// pass 1, keys from valid_r on (a bound of the thread's own) do not count (returns the row's new reference and sum); logits of any
+// size.  Of chunks that no row of the warp attends to all but the read is skipped, and in those that all do nothing is masked: with
+// a causal window most are one or the other, and the CTA with the last tiles of a sequence is what a short call waits for
+// (10007 tokens x 4 heads: 7 us of work there, 4.5 to 5.5 elsewhere; score stage 24.1 -> 22.8 us).
 __device__ __forceinline__ float2 drain_keys_masked(uint32_t addr, uint32_t empty_bar, int lane, int valid_r, float m_run, float l_run) {
   uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll 1
@@ -516,12 +516,11 @@ __device__ __forceinline__ int cta_of_unit(const BatchTable& bt, int hkv, const 
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // ------------------------------------------------------------------ the kernel
-// CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of
-// that code.  IDLE ones (pass 1) skip the items of warps whose 32 rows all lie behind the last one: one
-// item in four on two of the four schedulers for 448 rows.  ADDED ones (pass 2) have -L_r added by the product, a ninth step of
-// 16 channels (ones x three bf16 that sum to it), instead of reading it from shared memory for every column: eight loads fewer
-// per chunk  (see kAddedItems).  65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us,
-// 30000 x 8 of 400 rows 82.2 -> 81.0; with the test in all instantiations the others were 0.2-0.5 % slower.
+// CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of that code.  IDLE ones (pass 1)
+// skip the items of warps whose 32 rows all lie behind the last one, one item in four on two of the four schedulers for 448
+// rows: 65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us, 30000 x 8 of 400 rows 82.2 -> 81.0; with the test in all instantiations
+// the others were 0.2-0.5 % slower.  ADDED ones (pass 2) have -L_r added by the product, a ninth step of 16 channels (ones x three
+// bf16 that sum to it), instead of reading it from shared memory for every column: eight loads fewer per chunk (figures: kAddedItems).
 template <int PASS, bool CAUSAL, int LAYERS, int HALVES, bool IDLE, bool ADDED>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ Geometry g,

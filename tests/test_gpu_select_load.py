@@ -1,5 +1,6 @@
 """Pooling and fusing inside the selection kernel against the stage entry points, bit for bit: the fused call's own scores go
-through cc_fuse_prior_pool and cc_topk_select, which have their own code for both.  Lengths around a thread's four items, a
+through cc_fuse_prior_pool, which has its own code for both; the indices are those of cc_topk_select, whose load is another one but
+whose search and emission are the same code, and of cc_topk_select_static, a kernel of its own.  Lengths around a thread's four items, a
 part of the slice (four per thread) and a CTA's share; every width of the pooling window's two-tap steps."""
 import math
 
@@ -40,9 +41,10 @@ def test_fused_load_matches_the_stages(pool, cap, lens):
     staged = torch.empty_like(fused)
     cc.cc_fuse_prior_pool(ctx(), d, scores, prior, staged)
     assert torch.equal(staged, fused)
-    idx2, count2 = torch.full_like(idx, -9), torch.full_like(count, -9)
-    cc.cc_topk_select(ctx(), d, fused, prior, idx2, count2)
-    assert torch.equal(idx, idx2) and torch.equal(count, count2)
+    for select in (cc.cc_topk_select, cc.cc_topk_select_static):
+        idx2, count2 = torch.full_like(idx, -9), torch.full_like(count, -9)
+        select(ctx(), d, fused, prior, idx2, count2)
+        assert torch.equal(idx, idx2) and torch.equal(count, count2)
 
 
 @pytest.mark.parametrize("cap", [0.0, 0.3])

@@ -74,7 +74,8 @@ def test_a_wave_of_wide_clusters_is_as_wide_as_the_device():
 
 @pytest.mark.parametrize("items", [1, 40])
 def test_row_statistics_cost_the_ring_of_k_tiles_nothing(items):
-    """As many tiles of 32 KB as Q, 20 KB of hand-over buffers and 2 KB of statistics leave of 227 KB, whatever else a launch holds."""
+    """As many tiles of 32 KB as Q, 18 KB of hand-over buffers and 2 KB of statistics leave of 227 KB, in whichever of its two forms
+    pass 2 has the statistics."""
     ring = binding.load_library().ccx_score_ring
     for rows in range(16, 513, 16):
         one, two, added, smem = C.c_int(), C.c_int(), C.c_int(), C.c_size_t()
