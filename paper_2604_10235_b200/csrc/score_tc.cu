@@ -315,10 +315,14 @@ __device__ __forceinline__ void hand_back(uint32_t empty_bar, int lane) {
 // of 16 instructions, a vote and a branch before the first exponential.  The sums of the others, which grow beyond 2^70 or are no numbers
 // where a value is out of the arithmetic's range, and the ranges of the reference and of the last chunk are looked at before the
 // buffer goes back; when one is not as it should be, nothing has been changed and the answer is false: the caller goes through
-// the item again, chunk by chunk.
+// the item again, chunk by chunk.  HALF: only the lanes in `real` decide; the others
+// multiply whatever lies behind the rows of Q, keys among it, whose products with keys are large where a channel of all keys is
+// (300 in two channels, 65536 tokens: 8 heads of 48 rows 49.7 -> 46.7 us, causal 59 -> 50, 4 of 448 rows causal 80 -> 74; without
+// such channels 48 rows +1 us).
 constexpr float kRedo = 1.1805916e21f;     // 2^70
 constexpr float kMaxProduct = 1.0995116e12f;     // 2^40
-__device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, int lane, float& m_run, float& l_run) {
+template <bool HALF>
+__device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, int lane, unsigned real, float& m_run, float& l_run) {
   uint64_t acc[2] = {0ull, 0ull};
   float m = m_run, l = l_run;
   PolyRef r = poly_ref(m);
@@ -332,7 +336,11 @@ __device__ __forceinline__ bool drain_keys(uint32_t addr, uint32_t empty_bar, in
       const float mx = max32(v) * kScale;
       if (cc0 + 32 == kTileKeys) {
         const bool fine = acc_total(acc) < kRedo && fmaxf(fabsf(m), mx) < kMaxRef && poly_reach(v) < kMaxProduct;
-        if (!__all_sync(0xffffffffu, fine)) return false;
+        if (HALF) {
+          if (__ballot_sync(0xffffffffu, !fine) & real) return false;
+        } else if (!__all_sync(0xffffffffu, fine)) {
+          return false;
+        }
         hand_back(empty_bar, lane);
       }
       if (m == -INFINITY || mx > m + 64.0f) {
@@ -516,12 +524,13 @@ __device__ __forceinline__ int cta_of_unit(const BatchTable& bt, int hkv, const 
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // ------------------------------------------------------------------ the kernel
-// CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of that code.  IDLE ones (pass 1)
+// CAUSAL instantiations carry the masked copies of the epilogue loops; the others have none of that code.  PAD (pass 1): 1 ones
 // skip the items of warps whose 32 rows all lie behind the last one, one item in four on two of the four schedulers for 448
 // rows: 65536 tokens x 4 heads of 448 rows 92.8 -> 91.9 us, 30000 x 8 of 400 rows 82.2 -> 81.0; with the test in all instantiations
-// the others were 0.2-0.5 % slower.  ADDED ones (pass 2) have -L_r added by the product, a ninth step of 16 channels (ones x three
+// the others were 0.2-0.5 % slower.  2 ones know of warps with rows in half of their lanes besides (448 rows +1.5 % with that test).
+// ADDED ones (pass 2) have -L_r added by the product, a ninth step of 16 channels (ones x three
 // bf16 that sum to it), instead of reading it from shared memory for every column: eight loads fewer per chunk (figures: kAddedItems).
-template <int PASS, bool CAUSAL, int LAYERS, int HALVES, bool IDLE, bool ADDED>
+template <int PASS, bool CAUSAL, int LAYERS, int HALVES, int PAD, bool ADDED>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ Geometry g,
                 const __grid_constant__ TcParams P, const __grid_constant__ TcLayers<LAYERS> M,
@@ -909,6 +918,8 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
     const int cut_first = sub_begin > 0 ? t_begin : -1, cut_last = sub_end < n_sub ? t_end - 1 : -1;
     const int t_slot = t_begin + (sub_begin > 0 ? 1 : 0);
     const int idle_from = (max(P.rows_pad - quad * 32, 0) + 127) / 128;   // row blocks from here on have no row of this warp
+    // lanes of a warp that have a row in the last block of rows (a multiple of 16 in all), if any do
+    const unsigned last_rows = P.rows_pad - (n_sub - 1) * 128 - quad * 32 >= 32 ? ~0u : 0xffffu;
     uint32_t par = 0;
     bool first_item = true;     // ADDED: of the set in the (sequence, head); these come without -L_r
     uint32_t late_par = 0;
@@ -990,7 +1001,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
         tc_fence_after();
         const bool edge = PASS == 1 ? valid < kTileKeys || (CAUSAL && key0 + kTileKeys > n_cur - g.window + 1)
                                     : CAUSAL && key0 + kTileKeys > n_cur - g.window + 1;
-        if (IDLE && sub >= idle_from) {
+        if (PAD && sub >= idle_from) {
           hand_back(empty_bar, lane);
         } else if (PASS == 1) {
           // thread = query row (sub * 128 + row_in_tile); columns = the 128 keys of the tile
@@ -999,7 +1010,7 @@ score_tc_kernel(const __grid_constant__ BatchTable bt, const __grid_constant__ G
 #pragma unroll
             for (int rb = 1; rb < 4; ++rb) if (rb == sub) { m_run = run_m[rb]; l_run = run_l[rb]; }
           }
-          if (edge || !drain_keys(acc_addr, empty_bar, lane, m_run, l_run)) {
+          if (edge || !drain_keys<PAD == 2>(acc_addr, empty_bar, lane, sub == n_sub - 1 ? last_rows : ~0u, m_run, l_run)) {
             // keys of the tile this row attends to: the valid ones, or (causal window) those up to the
             // row's own position n - w + t
             int valid_r = valid;
@@ -1218,16 +1229,18 @@ cudaError_t launch_passes(const Launch& L, const BatchTable& bt, const Geometry&
     if (r != CUDA_SUCCESS) { *drv_err = (int)r; return cudaErrorUnknown; }
     M.scores[l] = lp.scores[l];
   }
-  // the last row block has a warp without rows (causal calls gain nothing: 10007 tokens x 4 heads 40.0 -> 40.1 us)
-  const bool idle = P.rows_pad % 128 != 0 && P.rows_pad % 128 <= 96;
-  auto pass1 = g.causal ? score_tc_kernel<1, true, LAYERS, HALVES, false, false>
-               : idle   ? score_tc_kernel<1, false, LAYERS, HALVES, true, false>
-                        : score_tc_kernel<1, false, LAYERS, HALVES, false, false>;
-  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false, false> : score_tc_kernel<2, false, LAYERS, HALVES, false, false>;
+  // PAD: the last block of rows is not full; a warp has rows in half of its lanes, or some warps have none (causal calls gain nothing
+  // from a form of their own for that: 10007 tokens x 4 heads of 448 rows level)
+  const int pad = P.rows_pad % 32 != 0 ? 2 : P.rows_pad % 128 != 0 ? 1 : 0;
+  auto pass1 = g.causal ? (pad ? score_tc_kernel<1, true, LAYERS, HALVES, 2, false> : score_tc_kernel<1, true, LAYERS, HALVES, 0, false>)
+               : pad == 2 ? score_tc_kernel<1, false, LAYERS, HALVES, 2, false>
+               : pad == 1 ? score_tc_kernel<1, false, LAYERS, HALVES, 1, false>
+                          : score_tc_kernel<1, false, LAYERS, HALVES, 0, false>;
+  auto pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, 0, false> : score_tc_kernel<2, false, LAYERS, HALVES, 0, false>;
   const bool added = HALVES == 1 && adds_statistic(P.rows_pad, P.total_tiles * P.n_sub, P.grid);
   if (added)
-    pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, false, HALVES == 1>
-                     : score_tc_kernel<2, false, LAYERS, HALVES, false, HALVES == 1>;
+    pass2 = g.causal ? score_tc_kernel<2, true, LAYERS, HALVES, 0, HALVES == 1>
+                     : score_tc_kernel<2, false, LAYERS, HALVES, 0, HALVES == 1>;
   cudaError_t e = allow_smem(pass1);
   if (e == cudaSuccess) e = allow_smem(pass2);
   if (e != cudaSuccess) return e;
