@@ -118,6 +118,21 @@ def test_keys_far_below_in_columns_of_the_polynomial(at, depth):
     check_against_oracle(wl, one_key(wl, at, depth, 0.0), cc.CC_MODE_BF16, TOL)
 
 
+def check_one_key_with_all_of_every_row(n, at, logit, rest, causal, ulps):
+    wl = gen.Workload("huge", 34, 1, 8, 2, 128, 64, gen.POOL_MAX, 7, 1, n=n, causal=causal)
+    x = one_key(wl, at, logit, rest)
+    d = cc.Desc(8, 2, 64, n=n, budget=1, causal=causal)
+    q, k = (torch.from_numpy(a.view(np.int16)).view(torch.bfloat16).cuda() for a in (x.q_win, x.k))
+    u, lse = scores(d, q, k, (1, 8, 64))
+    assert np.isfinite(u).all() and np.isfinite(lse).all()
+    off = 0.5 * np.spacing(np.float32(abs(logit) / LN2)) + ulps * SCALE * np.spacing(np.float32(abs(logit) * np.sqrt(128.0))) + 4e-4
+    assert np.abs(np.log2(u[:, at] / 256.0)).max() < off
+    assert u.sum() - u[:, at].sum() < 256.0 * 2e-4
+    bits = orc.bf16_bits_to_f64(x.q_win).reshape(64, 8, 128), orc.bf16_bits_to_f64(x.k)[at]
+    ref = np.einsum("whd,hd->hw", bits[0], np.repeat(bits[1], 4, axis=0)) / np.sqrt(128.0)
+    np.testing.assert_allclose(lse[0], ref, rtol=1e-6, atol=0.2)
+
+
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("at", [0, 31, 36, 100, 127, 128 + 80, 640 + 120])
 @pytest.mark.parametrize("logit,rest", [(2.8e3, 0.0), (2.9e3, 0.0), (7.0e5, 0.0), (3.0e7, 0.0), (-1.0e3, -1.2e3),
@@ -125,15 +140,13 @@ def test_keys_far_below_in_columns_of_the_polynomial(at, depth):
 def test_logits_of_any_size(at, logit, rest, causal):
     """References around 2^12 and far beyond, others far below: the one key has all of every row that attends to it.  Its scores are good to half a unit
     in the last place of the f32 row statistic and to one of the product, in powers of two."""
-    wl = gen.Workload("huge", 34, 1, 8, 2, 128, 64, gen.POOL_MAX, 7, 1, n=1000, causal=causal)
-    x = one_key(wl, at, logit, rest)
-    d = cc.Desc(8, 2, 64, n=1000, budget=1, causal=causal)
-    q, k = (torch.from_numpy(a.view(np.int16)).view(torch.bfloat16).cuda() for a in (x.q_win, x.k))
-    u, lse = scores(d, q, k, (1, 8, 64))
-    assert np.isfinite(u).all() and np.isfinite(lse).all()
-    off = 0.5 * np.spacing(np.float32(abs(logit) / LN2)) + SCALE * np.spacing(np.float32(abs(logit) * np.sqrt(128.0))) + 4e-4
-    assert np.abs(np.log2(u[:, at] / 256.0)).max() < off
-    assert u.sum() - u[:, at].sum() < 256.0 * 2e-4
-    bits = orc.bf16_bits_to_f64(x.q_win).reshape(64, 8, 128), orc.bf16_bits_to_f64(x.k)[at]
-    ref = np.einsum("whd,hd->hw", bits[0], np.repeat(bits[1], 4, axis=0)) / np.sqrt(128.0)
-    np.testing.assert_allclose(lse[0], ref, rtol=1e-6, atol=0.2)
+    check_one_key_with_all_of_every_row(1000, at, logit, rest, causal, 1)
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("at", [5, 10 * 128 + 100, 41000, 79900])
+@pytest.mark.parametrize("logit,rest", [(2.8e3, 0.0), (7.0e5, 0.0), (-2.8e3, -4.0e3), (-7.3e5, -1.0e6), (0.0, -1.0e9)])
+def test_logits_of_any_size_in_a_long_call(at, logit, rest, causal):
+    """The same where the product subtracts the row statistic (sixteen items per CTA and more): a rounding of it and one of its
+    three parts' sum besides, each of at most a unit of the product."""
+    check_one_key_with_all_of_every_row(80000, at, logit, rest, causal, 3)
